@@ -317,7 +317,8 @@ int32_t geer_checked_build(void);
 
 /* Synchronise `stream`, then read the first recorded bounds violation: *site
  * (0: none; 1 forward tile, 2 forward list range, 3 forward item, 4 backward
- * tile, 5 backward list range, 6 backward item, 7 duplicated pair's super-tile)
+ * tile, 5 backward list range, 6 backward item, 7 duplicated pair's super-tile, 8 a ray hit a list entry that the
+ * forward's sub-tile bound dropped: the checked build walks those too)
  * and *index (the offending value). A violation read is cleared, with its
  * status bit. Always GEER_OK with *site = 0 in libgeer.so. */
 geer_status geer_bounds_violation(geer_workspace *ws, uint32_t *site, int64_t *index, void *stream);

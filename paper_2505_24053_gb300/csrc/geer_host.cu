@@ -113,17 +113,24 @@ bool flag_intervals(const float4 *tab, int n, int32_t z[2], int32_t w[2]) {
 // Super-tile grid of each camera (binning is by super-tiles of S x S tiles; the
 // render filters a super-tile's list down to its tile). Free layouts take the
 // smallest S in 4..8 that keeps every super-tile id below 256 (one radix pass),
-// else 4. Slot layouts take S = 4 and the slot's own tile ids, so that every
-// launch shape depends on the slot count only.
+// else 4. Slot layouts take S = kSlotSuper and ids from the slot's tile count, so that
+// every launch shape depends on the slot count only. (A batch of the serving
+// mix, 2M Gaussians: 3128 us with S = 4, 2991 with 5, 2986 with 6, 2933 with 8; with an
+// id per tile of the slots the emission's counters did not fit shared memory: 5133.)
+constexpr int kSlotSuper = 8;
+
 void assign_super(DevCam *cams, int n, int64_t slot_tiles, int32_t &S, int64_t &n_stiles) {
     if (slot_tiles > 0) {
-        S = 4;
+        S = kSlotSuper;
+        // ceil(x / S) ceil(y / S) <= (xy + (S - 1)(x + y) + (S - 1)^2) / S^2 and x + y <= xy + 1, so
+        // that a slot of T tiles has at most T / S + 1 super-tiles, whatever its shape
+        const int64_t per_slot = slot_tiles / S + 1;
         for (int ci = 0; ci < n; ++ci) {
             DevCam &d = cams[ci];
             d.stiles_x = (int32_t)ceil_div(d.tiles_x, S);
-            d.stile_base = (int32_t)(ci * slot_tiles);
+            d.stile_base = (int32_t)(ci * per_slot);
         }
-        n_stiles = n * slot_tiles;
+        n_stiles = n * per_slot;
         return;
     }
     S = 4;
@@ -301,7 +308,9 @@ size_t layout(const Caps &c, char *base, geer_workspace *ws) {
     size_t o_k1 = L.take(sizeof(uint32_t) * c.pairs);
     size_t o_v0 = L.take(sizeof(uint32_t) * c.pairs);
     size_t o_v1 = L.take(sizeof(uint32_t) * c.pairs);
-    size_t o_srg = L.take(sizeof(uint4) * c.pairs);
+    size_t o_sm0 = L.take(2 * sizeof(uint32_t) * c.pairs);
+    size_t o_sm1 = L.take(2 * sizeof(uint32_t) * c.pairs);
+    size_t o_sa = L.take(2 * sizeof(uint32_t) * (c.pairs / 32 + 1));
     const int64_t groups = ceil_div(c.sort_tiles, kGroupTiles) + 1;
     size_t o_th = L.take(sizeof(uint32_t) * kRadix * c.sort_tiles);
     size_t o_gs = L.take(sizeof(uint32_t) * kRadix * groups);
@@ -344,7 +353,9 @@ size_t layout(const Caps &c, char *base, geer_workspace *ws) {
         ws->d_keys[1] = reinterpret_cast<uint32_t *>(base + o_k1);
         ws->d_vals[0] = reinterpret_cast<uint32_t *>(base + o_v0);
         ws->d_vals[1] = reinterpret_cast<uint32_t *>(base + o_v1);
-        ws->d_sranges = reinterpret_cast<uint4 *>(base + o_srg);
+        ws->d_smask[0] = reinterpret_cast<uint32_t *>(base + o_sm0);
+        ws->d_smask[1] = reinterpret_cast<uint32_t *>(base + o_sm1);
+        ws->d_sany = reinterpret_cast<uint32_t *>(base + o_sa);
         ws->d_tile_hist = reinterpret_cast<uint32_t *>(base + o_th);
         ws->d_group_sum = reinterpret_cast<uint32_t *>(base + o_gs);
         ws->d_group_excl = reinterpret_cast<uint32_t *>(base + o_ge);

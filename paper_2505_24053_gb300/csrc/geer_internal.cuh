@@ -10,7 +10,7 @@ namespace geer {
 
 constexpr int kTile = 16;                   // BEAP tile edge in rays (a camera sub-frustum)
 constexpr int kTilePix = kTile * kTile;
-constexpr int kTileWarps = kTilePix / 32;    // warps of a tile's rays (one byte each in the hit record)
+constexpr int kTileWarps = kTilePix / 32;    // warps of a tile's rays: 8 x 4 each in the forward, 16 x 2 in the backward and the hit record (a byte each)
 constexpr uint8_t kRegionCentral = 0, kRegionPeripheral = 1, kRegionNone = 255;  // native evaluation regions
 constexpr int64_t kHitEntries = 2048;      // tile-list entries per tile whose hit bytes are recorded
 // Forward checkpoints: the rays' (T, C) at the end of the first forward batch
@@ -72,6 +72,7 @@ enum CheckSite : uint32_t {
     kSiteBwdList = 5,     // render backward: super-tile list range
     kSiteBwdItem = 6,     // render backward: item id (record gather, accumulator scatter)
     kSiteDupSuper = 7,    // duplicate: super-tile id of an emitted pair
+    kSiteFwdCull = 8,     // render forward: a ray hit a list entry that its sub-tile's bound dropped (checked build only)
 };
 
 // Guard of an index that comes from an earlier kernel (or from the caller's
@@ -187,61 +188,14 @@ __device__ __forceinline__ void cp_async4(float *smem, const float *gmem) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(gmem) : "memory");
 }
 
-// Bulk (TMA engine) copies into shared memory that complete on an mbarrier.
-__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-
-// Arrive once on the barrier, announcing `bytes` more to be written by bulk copies.
-__device__ __forceinline__ void mbar_arrive_expect(uint64_t *bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(bytes)
-                 : "memory");
-}
-
-// bytes (a multiple of 16, both addresses 16-byte aligned) from global to this
-// CTA's shared memory; completion is counted on bar.
-__device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
-                     smem_u32(dst)),
-                 "l"(src), "r"(bytes), "r"(smem_u32(bar))
-                 : "memory");
-}
-
-// Orders this thread's earlier generic accesses of shared memory before later
-// bulk copies into it.
-__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
-
-// Waits for the barrier's phase `parity` to complete, at most `limit` polls;
-// false if it did not (the caller records a timeout and goes on).
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, uint32_t limit) {
-    for (uint32_t it = 0; it < limit; ++it) {
-        uint32_t done;
-        asm volatile(
-            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-            : "=r"(done)
-            : "r"(smem_u32(bar)), "r"(parity)
-            : "memory");
-        if (done) return true;
-    }
-    return false;
-}
-
 __device__ __forceinline__ void unpack_ranges(const uint4 r4, int rg[8]) {
     rg[0] = (int)(r4.x & 0xffff); rg[1] = (int)(r4.x >> 16); rg[2] = (int)(r4.y & 0xffff); rg[3] = (int)(r4.y >> 16);
     rg[4] = (int)(r4.z & 0xffff); rg[5] = (int)(r4.z >> 16); rg[6] = (int)(r4.w & 0xffff); rg[7] = (int)(r4.w >> 16);
 }
 
-// Association of tile (cx, cy) with an item: the column test takes the arc kind
-// of the tile's rows (cos(phi) >= 0: direct, < 0: shifted) and the row test that
-// of its columns; col / row are the tile's table entries (z, w: the tile has rays
-// with cos >= 0 / cos <= 0).
-__device__ __forceinline__ bool tile_assoc(const float4 &col, const float4 &row, int cx, int cy, const int rg[8]) {
-    bool aok = (row.z != 0.0f && cx >= rg[0] && cx < rg[1]) || (row.w != 0.0f && cx >= rg[2] && cx < rg[3]);
-    bool bok = (col.z != 0.0f && cy >= rg[4] && cy < rg[5]) || (col.w != 0.0f && cy >= rg[6] && cy < rg[7]);
-    return aok && bok;
-}
+// A sorted pair's association with the S x S tiles of its super-tile, one bit per
+// tile (row by row): one 32-bit word up to S = 5, two beyond.
+__host__ __device__ inline int mask_words(int S) { return S * S > 32 ? 2 : 1; }
 
 // Schedule bucket of a cost c (a tile's pair count, a backward unit's steps):
 // larger costs first, four buckets per octave, zero cost last.
@@ -326,7 +280,8 @@ struct geer_workspace {
     float4 *d_Cfin;         // [cap_pixels] composited colour before the background (tiles with checkpoints)
     int bwd_grid;           // persistent backward blocks
     int train_grid;         // persistent blocks of the fused forward + L1 + backward render
-    uint4 *d_sranges;       // [cap_pairs] association ranges of the sorted pairs' items (in list order)
+    uint32_t *d_smask[2];   // [cap_pairs][mask_words] tile masks of the pairs (ping-pong with d_keys / d_vals)
+    uint32_t *d_sany;       // [cap_pairs / 32 + 1][mask_words] the sorted pairs' masks of 32 or'd together
     uint2 *d_srange;        // [cap_tiles] super-tile [start, end) in the sorted pairs, followed by [cap_tiles] u32 counts
     uint32_t *d_last;       // [cap_pixels] list entries walked per ray
     float *d_Tfin;          // [cap_pixels] final transmittance (for the backward)

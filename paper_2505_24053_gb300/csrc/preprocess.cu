@@ -819,17 +819,61 @@ __global__ void __launch_bounds__(kPrepThreads) k_gather_counts(const DevCam *__
     if (threadIdx.x == 0) bs_super[blockIdx.x] = stot;
 }
 
+// Bits [lo, hi) of the S tile columns (or rows) that start at base.
+__device__ __forceinline__ uint32_t span_bits(int lo, int hi, int base, int S) {
+    const int l = min(max(lo - base, 0), S), h = min(max(hi - base, 0), S);
+    return h > l ? (1u << h) - (1u << l) : 0u;
+}
+
+// The tile mask of an item and super-tile (sx, sy): bit j * S + i for its tile
+// (sx S + i, sy S + j). A tile (x, y) is associated when (x in X0 and row y has rays
+// with cos(phi) >= 0, or x in X1 and row y has rays with cos(phi) <= 0), and likewise
+// for its row in Y0 / Y1 with the column's flags.
+__device__ __forceinline__ uint64_t tile_mask_general(const DevCam &cam, const int rg[8], int sx, int sy, int S) {
+    const int x0 = sx * S, y0 = sy * S;
+    const uint32_t X0 = span_bits(rg[0], rg[1], x0, S), Y0 = span_bits(rg[4], rg[5], y0, S);
+    const uint32_t X1 = span_bits(rg[2], rg[3], x0, S), Y1 = span_bits(rg[6], rg[7], y0, S);
+    const uint32_t zc = span_bits(cam.zc[0], cam.zc[1], x0, S), zr = span_bits(cam.zr[0], cam.zr[1], y0, S);
+    const uint32_t wc = span_bits(0, cam.wc[0], x0, S) | span_bits(cam.wc[1], cam.tiles_x, x0, S);
+    const uint32_t wr = span_bits(0, cam.wr[0], y0, S) | span_bits(cam.wr[1], cam.tiles_y, y0, S);
+    uint64_t m = 0;
+    for (int j = 0; j < S; ++j) {
+        const uint32_t a = (zr >> j & 1u ? X0 : 0u) | (wr >> j & 1u ? X1 : 0u);
+        const uint32_t b = (Y0 >> j & 1u ? zc : 0u) | (Y1 >> j & 1u ? wc : 0u);
+        m |= (uint64_t)(a & b) << (j * S);
+    }
+    return m;
+}
+
+// The same for a rectangle (is_rect): columns [xlo, xhi) x rows [ylo, yhi). every:
+// bit j * S of every row j.
+__device__ __forceinline__ uint64_t tile_mask_rect(uint32_t xr, uint32_t yr, int sx, int sy, int S, uint64_t every) {
+    const uint32_t cols = span_bits((int)(xr & 0xffff), (int)(xr >> 16), sx * S, S);
+    const uint32_t rows = span_bits((int)(yr & 0xffff), (int)(yr >> 16), sy * S, S);
+    // rows is a run of ones [l, h): the bits every has in [l S, h S), each times cols
+    const int l = __ffs(rows) - 1, h = 32 - __clz(rows);
+    const uint64_t upto = h * S < 64 ? (1ull << (h * S)) - 1ull : ~0ull;
+    return rows ? (every & upto & ~((1ull << (l * S)) - 1ull)) * cols : 0ull;
+}
+
+__device__ __forceinline__ void put_mask(uint32_t *out, int64_t i, int words, uint64_t m) {
+    if (words == 1) out[i] = (uint32_t)m;
+    else reinterpret_cast<uint2 *>(out)[i] = make_uint2((uint32_t)m, (uint32_t)(m >> 32));
+}
+
 // DuplicateWithKeys in depth order, at super-tile granularity: item i of the
 // depth-sorted list emits one (global super-tile, item) pair per super-tile
-// holding an associated tile, in row-major order, and counts the pairs per
-// super-tile. Items whose association is a rectangle are emitted by the whole
-// warp together (lane j writes output j: coalesced); others loop per thread.
+// holding an associated tile, in row-major order, with its tile mask (what the
+// renders' list fills test: one bit of a 4-byte load, where the 16 bytes of ranges
+// cost an unpacking and eight comparisons), and counts the pairs per super-tile.
+// Items whose association is a rectangle are emitted by the whole warp together
+// (lane j writes output j: coalesced); others loop per thread.
 __global__ void __launch_bounds__(kPrepThreads) k_duplicate(
     const DevCam *__restrict__ cams, const float4 *__restrict__ ttab, int64_t n, int S,
     const uint32_t *__restrict__ sorted0, const uint32_t *__restrict__ sorted1, const uint4 *__restrict__ ranges,
     const uint32_t *__restrict__ count, uint32_t *__restrict__ misc, const uint32_t *__restrict__ blocksum,
-    uint32_t *__restrict__ okeys,
-    uint32_t *__restrict__ ovals, uint32_t *__restrict__ scount, int nst, int64_t cap) {
+    uint32_t *__restrict__ okeys, uint32_t *__restrict__ ovals, uint32_t *__restrict__ omask,
+    uint32_t *__restrict__ scount, int nst, int64_t cap) {
     grid_dep_sync();
     __shared__ uint32_t wsum[kPrepThreads / 32];
     extern __shared__ uint32_t sh[];  // per-super-tile pair counts when they fit (nst <= kSmemTiles)
@@ -843,11 +887,15 @@ __global__ void __launch_bounds__(kPrepThreads) k_duplicate(
     uint32_t item = 0, cnt = 0;
     int rg[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     int ci = 0;
+    uint32_t xr = 0, yr = 0;  // the direct column and row ranges, packed
     bool rect = true;
     if (i < L) {
         item = sorted_id[i];
         ci = (int)(item / (uint32_t)n);
-        unpack_ranges(ranges[item], rg);
+        const uint4 r4 = ranges[item];
+        xr = r4.x;
+        yr = r4.z;
+        unpack_ranges(r4, rg);
         rect = is_rect(cams[ci], rg);
         cnt = super_count(cams[ci], S, rg, count[item], rect);
     }
@@ -871,6 +919,9 @@ __global__ void __launch_bounds__(kPrepThreads) k_duplicate(
         uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
         if (lane >= o) incl += y;
     }
+    const int words = mask_words(S);
+    uint64_t every = 0;
+    for (int j = 0; j < S; ++j) every |= 1ull << (j * S);
     const uint32_t wtot = __shfl_sync(0xffffffffu, incl, 31);
     const uint32_t sb = (uint32_t)(cam.stile_base + sy0 * cam.stiles_x + sx0);
     for (uint32_t j0 = 0; j0 < wtot; j0 += 32) {
@@ -889,12 +940,16 @@ __global__ void __launch_bounds__(kPrepThreads) k_duplicate(
         const int o_sx = __shfl_sync(0xffffffffu, cam.stiles_x, lo);
         const uint32_t o_item = __shfl_sync(0xffffffffu, item, lo);
         const int64_t o_off = __shfl_sync(0xffffffffu, off, lo);
+        const uint32_t o_xr = __shfl_sync(0xffffffffu, xr, lo), o_yr = __shfl_sync(0xffffffffu, yr, lo);
+        const uint32_t o_s = __shfl_sync(0xffffffffu, (uint32_t)sx0 | (uint32_t)sy0 << 16, lo);
         if (j < wtot) {
             const uint32_t k = j - (o_incl - o_cnt);
             const uint32_t ky = k / (uint32_t)o_rw, kx = k - ky * (uint32_t)o_rw;
             const uint32_t st = o_sb + ky * (uint32_t)o_sx + kx;
             okeys[o_off + k] = st;
             ovals[o_off + k] = o_item;
+            put_mask(omask, o_off + k, words,
+                     tile_mask_rect(o_xr, o_yr, (int)(o_s & 0xffff) + (int)kx, (int)(o_s >> 16) + (int)ky, S, every));
             if (in_bounds(st, (uint64_t)nst, kSiteDupSuper, misc)) atomicAdd(smem ? &sh[st] : &scount[st], 1u);
         }
     }
@@ -907,6 +962,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_duplicate(
                 const uint32_t st = (uint32_t)(cam.stile_base + sy * cam.stiles_x + sx);
                 okeys[o] = st;
                 ovals[o] = item;
+                put_mask(omask, o, words, tile_mask_general(cam, rg, sx, sy, S));
                 if (in_bounds(st, (uint64_t)nst, kSiteDupSuper, misc)) atomicAdd(smem ? &sh[st] : &scount[st], 1u);
                 ++o;
             }
@@ -1186,7 +1242,7 @@ cudaError_t launch_duplicate(const geer_workspace *ws, cudaStream_t s) {
         const size_t smem = ws->n_stiles <= kSmemTiles ? sizeof(uint32_t) * ws->n_stiles : 0;
         launch_k(k_duplicate, dim3((unsigned)m), dim3(kPrepThreads), smem, s, ws->d_cams, ws->d_tile_tab,
                  ws->n_gauss, ws->super_size, ws->d_iid[0], ws->d_iid[1], ws->d_ranges, ws->d_count, ws->d_misc,
-                 ws->d_blocksum2, ws->d_keys[0], ws->d_vals[0], scount, (int)ws->n_stiles, ws->cap_pairs);
+                 ws->d_blocksum2, ws->d_keys[0], ws->d_vals[0], ws->d_smask[0], scount, (int)ws->n_stiles, ws->cap_pairs);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }

@@ -1,12 +1,14 @@
 // render.cu -- the per-ray render (Algorithm 1 per-CSF loop: Cano_Ray, Dist,
 // BlendInOrder) and its backward (App. C, RenderCUDA stage).
 //
-// A BEAP tile (a camera sub-frustum) of 16 x 16 rays is processed by 16 / ROWS
-// blocks of ROWS x 16 threads, one thread per ray, tiles taken in the order of
-// descending pair count (the costliest first). The forward builds the tile's
-// depth-ordered list on the fly from its super-tile's list (association test per
-// entry), stages the records through shared memory in batches of BATCH and every
-// ray walks them front to back with the closed-form ray integral (Sec. 3.1):
+// A BEAP tile (a camera sub-frustum) of 16 x 16 rays is processed by one block,
+// one thread per ray, tiles taken in the order of descending pair count (the
+// costliest first). A warp holds the 8 x 4 rays of one sub-tile (each half-warp
+// 4 x 4 of them). The forward builds the tile's depth-ordered list on the fly
+// from its super-tile's list (association test per entry), stages the records
+// through shared memory in batches of BATCH, tests each entry once per sub-tile
+// with a conservative bound (cull_keep) and every ray walks its sub-tile's
+// entries front to back with the closed-form ray integral (Sec. 3.1):
 //   d_u = W d, m_u = o_u x d_u, kappa = |m_u|^2 / |d_u|^2,
 //   alpha = min(alpha_max, sigma exp(-kappa / 2)),
 // skipping alpha < alpha_min and Gaussians whose closest approach lies behind
@@ -19,36 +21,15 @@
 namespace geer {
 namespace {
 
-#ifndef GEER_FWD_ROWS
-#define GEER_FWD_ROWS 16
-#endif
-#ifndef GEER_FWD_BATCH
-#define GEER_FWD_BATCH 256
-#endif
-#ifndef GEER_FWD_UNROLL
-#define GEER_FWD_UNROLL 4
-#endif
 #ifndef GEER_FWD_MINB
 #define GEER_FWD_MINB 4  // resident forward blocks per SM the registers must allow
-#endif
-#ifndef GEER_FWD_BULK
-#define GEER_FWD_BULK 0  // 1: the forward stages its records with bulk copies (TMA engine) on an mbarrier
-#endif
-constexpr uint32_t kBarPolls = 1u << 22;  // bound of a wait on a shared-memory barrier
-constexpr int kFwdUnroll = GEER_FWD_UNROLL;
-#ifndef GEER_SCAN
-#define GEER_SCAN 4
-#endif
-constexpr int kScan = GEER_SCAN;  // super-list loads in flight per thread in a list fill
-#ifndef GEER_BWD_ROWS
-#define GEER_BWD_ROWS 16
-#endif
-#ifndef GEER_BWD_BATCH
-#define GEER_BWD_BATCH 256
 #endif
 #ifndef GEER_BWD_MINB
 #define GEER_BWD_MINB 4
 #endif
+constexpr int kBatch = 256;    // list entries staged per batch (one per thread)
+constexpr int kFwdUnroll = 4;  // list entries evaluated together
+constexpr int kScan = 4;       // super-list loads in flight per thread in a list fill
 constexpr float kNegHalfLog2e = -0.72134752044448170f;  // -log2(e) / 2
 
 // A load of data written earlier in the same launch (CG: through L2, never a
@@ -57,6 +38,22 @@ template <bool CG, typename T>
 __device__ __forceinline__ T ld_cg(const T *p) {
     if constexpr (CG) return __ldcg(p);
     else return *p;
+}
+
+// 2^x. The hardware's approximation, as exp2f uses it for x >= -126 (every hit's
+// exponent argument: alpha_min and above), without exp2f's scaling below that.
+__device__ __forceinline__ float ex2(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// 1/x for a normal x, within 1 ulp: __fdividef(1, x) without its range scaling
+// (a times it gives __fdividef(a, x) bit for bit for divisors in [2^-126, 2^126)).
+__device__ __forceinline__ float rcp(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
 }
 
 __device__ __forceinline__ int find_cam(const DevCam *cams, int ncams, int t) {
@@ -87,7 +84,7 @@ __device__ __forceinline__ Eval evaluate(const float4 &a, const float4 &b, const
     const float mm = v.m0 * v.m0 + v.m1 * v.m1 + v.m2 * v.m2;
     v.dd = v.du0 * v.du0 + v.du1 * v.du1 + v.du2 * v.du2;
     v.od = c.y * v.du0 + c.z * v.du1 + c.w * v.du2;
-    v.kappa = __fdividef(mm, v.dd);
+    v.kappa = mm * rcp(v.dd);
     v.arg = fmaf(v.kappa, kNegHalfLog2e, e.x);
     v.hit = !(v.arg < log2_amin || v.od >= 0.0f);
     return v;
@@ -120,78 +117,165 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
     return m;
 }
 
-// Tile (cx, cy)'s list is its super-tile's depth-ordered list filtered by the
-// association test (sranges: the association ranges of the sorted pairs, in
-// list order): appends the entries of [pos, end) that pass until s_id holds at
-// least `want` entries or the list ends. Each step loads kScan x kThreads
-// entries at once (independent loads: a sparse tile's scan is bound by their
-// latency) and appends them in sub-steps of kThreads while s_id holds fewer than
-// `want`, so that s_id never takes more than want - 1 + kThreads entries; the
-// entries of sub-steps it did not take are read again by the next call.
-// Block-uniform (pos, end, s_cnt, want are the same in every thread); s_id is
-// visible on return. s_wcnt holds kScan x kThreads / 32 counts.
-template <int kThreads>
-__device__ __forceinline__ void fill_list(const uint32_t *__restrict__ svals, const uint4 *__restrict__ sranges,
-                                          const float4 &col, const float4 &row, int cx, int cy, uint32_t &pos,
-                                          uint32_t end, int want, uint32_t *s_id, uint32_t *s_pos, int &s_cnt,
-                                          uint32_t *s_wcnt) {
-    constexpr int kWarps = kThreads / 32;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    while (s_cnt < want && pos < end) {
-        uint4 raw[kScan];
-        uint32_t id[kScan];
+// A tile's super-tile list and its bit in the entries' masks.
+struct TileList {
+    const uint32_t *vals;  // item ids
+    const uint32_t *mask;  // the mask word that holds the tile's bit, `words` apart
+    const uint32_t *any;   // the same word of the groups' masks (32 entries each, aligned), `words` apart
+    int words, shift;
+    uint2 sr;              // [begin, end)
+};
+
+struct FillSmem {
+    uint32_t wcnt[2][kScan * kTileWarps];  // a step writes one set while the slowest warp still reads the other
+    uint32_t cut, taken;
+    uint8_t grp[32];
+};
+
+constexpr uint32_t kChunk = 256;                // super-list entries that a fill takes or leaves together
+constexpr uint32_t kLook = 31 * kChunk;         // entries of a step that skips empty groups of 32
+constexpr uint32_t kSparse = 4;                 // tile entries of a step at or below which the next ones skip
+
+// Inclusive (incl) and exclusive prefix of a step's 32 counts, one per lane.
+__device__ __forceinline__ uint32_t scan_counts(const uint32_t *wcnt, uint32_t &incl) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t c = wcnt[lane];
+    incl = c;
 #pragma unroll
-        for (int r = 0; r < kScan; ++r) {
-            const uint32_t i = pos + (uint32_t)(r * kThreads) + threadIdx.x;
-            raw[r] = make_uint4(0u, 0u, 0u, 0u);
-            id[r] = 0u;
-            if (i < end) {
-                raw[r] = sranges[i];
-                id[r] = svals[i];
-            }
-        }
-        uint32_t bal[kScan];
-#pragma unroll
-        for (int r = 0; r < kScan; ++r) {
-            const uint32_t i = pos + (uint32_t)(r * kThreads) + threadIdx.x;
-            bool ok = false;
-            if (i < end) {
-                int rg[8];
-                unpack_ranges(raw[r], rg);
-                ok = tile_assoc(col, row, cx, cy, rg);
-            }
-            bal[r] = __ballot_sync(0xffffffffu, ok);
-            if (lane == 0) s_wcnt[r * kWarps + warp] = __popc(bal[r]);
-        }
-        __syncthreads();
-        int cnt = s_cnt;
-        uint32_t adv = 0;
-#pragma unroll
-        for (int r = 0; r < kScan; ++r) {
-            if (cnt >= want) break;  // block-uniform: every thread reads the same counts
-            uint32_t base = 0, tot = 0;
-#pragma unroll
-            for (int w = 0; w < kWarps; ++w) {
-                const uint32_t c = s_wcnt[r * kWarps + w];
-                base += w < warp ? c : 0u;
-                tot += c;
-            }
-            if (bal[r] >> lane & 1u) {
-                const int k = cnt + (int)(base + __popc(bal[r] & lanemask_lt()));
-                s_id[k] = id[r];
-                if (s_pos) s_pos[k] = pos + (uint32_t)(r * kThreads) + threadIdx.x;
-            }
-            cnt += (int)tot;
-            adv += kThreads;
-        }
-        __syncthreads();
-        s_cnt = cnt;
-        pos += adv;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
     }
+    return incl - c;
 }
 
-// Moves the s_cnt - cnt entries not yet consumed (fewer than kThreads) to the front.
-template <int kThreads>
+// A tile's list is its super-tile's depth-ordered list filtered by its mask bit:
+// appends the entries of [pos, end) that pass, in chunks of 256 super-list entries
+// counted from the list's start, until s_id holds at least `want` entries or the
+// list ends (so that s_id never takes more than want - 1 + 256; the chunks set the
+// batches and with them the checkpoints' places). Each step loads kScan x 256
+// entries at once (independent loads: the scan is bound by their latency); chunks it
+// did not take are read again by the next call. After a step with hardly an entry
+// of the tile, a step looks at the or'd masks of 248 groups of 32 entries and reads
+// those of at most 32 groups that hold one (the serving scene's sparsest tiles own
+// 1 entry in 400 of an 800K-entry list: 1.1 ms of a batch's 2.9 were one such
+// block's scan). Block-uniform (pos, sparse, want and s_cnt are the same in every
+// thread); s_id is visible on return.
+__device__ __forceinline__ void fill_list(const TileList &tl, uint32_t &pos, bool &sparse, int want, uint32_t *s_id,
+                                          uint32_t *s_pos, int &s_cnt, FillSmem &sf) {
+    constexpr int kWarps = kTileWarps;
+    static_assert(kScan * kWarps == 32 && kChunk == kTilePix, "a warp scans a step's counts with a lane each");
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t end = tl.sr.y;
+    if (s_cnt >= want || pos >= end) return;
+    for (int par = 0; s_cnt < want && pos < end; par ^= 1) {
+        uint32_t id[kScan], at[kScan], bal[kScan], incl;
+        if (!sparse) {
+#pragma unroll
+            for (int r = 0; r < kScan; ++r) {
+                at[r] = pos + (uint32_t)r * kChunk + threadIdx.x;
+                bal[r] = at[r] < end ? tl.mask[(size_t)at[r] * tl.words] : 0u;
+                id[r] = at[r] < end ? tl.vals[at[r]] : 0u;
+            }
+#pragma unroll
+            for (int r = 0; r < kScan; ++r) {
+                bal[r] = __ballot_sync(0xffffffffu, bal[r] >> tl.shift & 1u);
+                if (lane == 0) sf.wcnt[par][r * kWarps + warp] = __popc(bal[r]);
+            }
+            __syncthreads();
+            const uint32_t excl = scan_counts(sf.wcnt[par], incl);
+            uint32_t taken = 0;
+            sparse = __shfl_sync(0xffffffffu, incl, 31) <= kSparse;
+#pragma unroll
+            for (int r = 0; r < kScan; ++r) {
+                const uint32_t base = __shfl_sync(0xffffffffu, excl, r * kWarps + warp);
+                const uint32_t upto = __shfl_sync(0xffffffffu, incl, r * kWarps + kWarps - 1);
+                if (s_cnt + (int)taken >= want) break;  // block-uniform: every warp scans the same counts
+                if (bal[r] >> lane & 1u) {
+                    const int k = s_cnt + (int)(base + __popc(bal[r] & lanemask_lt()));
+                    s_id[k] = id[r];
+                    if (s_pos) s_pos[k] = at[r];
+                }
+                taken = upto;
+                pos += kChunk;
+            }
+            s_cnt += (int)taken;
+            continue;
+        }
+        // the groups of [pos, pos + kLook) that hold an entry of the tile
+        const uint32_t g0 = pos >> 5, lim = min(pos + kLook, end);
+        const uint32_t g = g0 + threadIdx.x;
+        const bool any = (g << 5) < lim && (tl.any[(size_t)g * tl.words] >> tl.shift & 1u);
+        const uint32_t b = __ballot_sync(0xffffffffu, any);
+        if (lane == 0) sf.wcnt[par][warp] = __popc(b);
+        if (threadIdx.x == 0) sf.taken = 0u;
+        __syncthreads();
+        uint32_t pre = 0, n = 0;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) {
+            const uint32_t c = sf.wcnt[par][w];
+            pre += w < warp ? c : 0u;
+            n += c;
+        }
+        if (n > 32u) {  // dense again
+            sparse = false;
+            continue;
+        }
+        if (any) sf.grp[pre + __popc(b & lanemask_lt())] = (uint8_t)threadIdx.x;
+        par ^= 1;
+        __syncthreads();
+        const uint32_t gs = (uint32_t)lane < n ? (g0 + sf.grp[lane]) << 5 : 0xffffffffu;
+#pragma unroll
+        for (int r = 0; r < kScan; ++r) {
+            const uint32_t first = __shfl_sync(0xffffffffu, gs, r * kWarps + warp);
+            at[r] = first + (uint32_t)lane;
+            const bool in = first != 0xffffffffu && at[r] >= pos && at[r] < lim;
+            bal[r] = in ? tl.mask[(size_t)at[r] * tl.words] : 0u;
+            id[r] = in ? tl.vals[at[r]] : 0u;
+        }
+#pragma unroll
+        for (int r = 0; r < kScan; ++r) {
+            bal[r] = __ballot_sync(0xffffffffu, bal[r] >> tl.shift & 1u);
+            if (lane == 0) sf.wcnt[par][r * kWarps + warp] = __popc(bal[r]);
+        }
+        __syncthreads();
+        const uint32_t excl = scan_counts(sf.wcnt[par], incl);
+        const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+        uint32_t rank[kScan], stop = lim;
+#pragma unroll
+        for (int r = 0; r < kScan; ++r)
+            rank[r] = __shfl_sync(0xffffffffu, excl, r * kWarps + warp) + __popc(bal[r] & lanemask_lt());
+        const bool cuts = s_cnt + (int)total >= want;
+        if (cuts) {  // the chunk of entry number `want` is the last one to take
+#pragma unroll
+            for (int r = 0; r < kScan; ++r)
+                if ((bal[r] >> lane & 1u) && rank[r] == (uint32_t)(want - s_cnt) - 1u) sf.cut = (at[r] - pos) / kChunk;
+            __syncthreads();
+            stop = pos + (sf.cut + 1u) * kChunk;
+        }
+#pragma unroll
+        for (int r = 0; r < kScan; ++r) {
+            const bool take = (bal[r] >> lane & 1u) && at[r] < stop;
+            if (take) {
+                s_id[s_cnt + (int)rank[r]] = id[r];
+                if (s_pos) s_pos[s_cnt + (int)rank[r]] = at[r];
+            }
+            if (cuts) {  // how many that is
+                const uint32_t most = __reduce_max_sync(0xffffffffu, take ? rank[r] + 1u : 0u);
+                if (lane == 0 && most) atomicMax(&sf.taken, most);
+            }
+        }
+        if (cuts) __syncthreads();
+        s_cnt += cuts ? (int)sf.taken : (int)total;
+        pos = cuts ? stop : pos + kLook;
+    }
+    __syncthreads();
+}
+
+// The same filter walking the super-tile list backwards: appends the passing
+// entries of [beg, pos) in descending position order (the tile list read back to
+// front) until s_id holds at least kBatch entries or pos reaches beg.
+// Moves the s_cnt - cnt entries not yet consumed (fewer than 256) to the front.
 __device__ __forceinline__ void shift_list(uint32_t *s_id, uint32_t *s_pos, int cnt, int &s_cnt) {
     const int rem = s_cnt - cnt;
     uint32_t keep = 0, keep_pos = 0;
@@ -209,21 +293,18 @@ __device__ __forceinline__ void shift_list(uint32_t *s_id, uint32_t *s_pos, int 
 
 // The same filter walking the super-tile list backwards: appends the passing
 // entries of [beg, pos) in descending position order (the tile list read back to
-// front) until s_id holds at least BATCH entries or pos reaches beg.
-template <int kThreads, int BATCH>
-__device__ __forceinline__ void fill_list_rev(const uint32_t *__restrict__ svals, const uint4 *__restrict__ sranges,
-                                              const float4 &col, const float4 &row, int cx, int cy, uint32_t &pos,
-                                              uint32_t beg, uint32_t *s_id, int &s_cnt, uint32_t *s_wcnt) {
+// front) until s_id holds at least kBatch entries or pos reaches beg.
+__device__ __forceinline__ void fill_list_rev(const TileList &tl, uint32_t &pos, uint32_t beg, uint32_t *s_id,
+                                              int &s_cnt, uint32_t *s_wcnt) {
+    constexpr int kThreads = kTilePix;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    while (s_cnt < BATCH && pos > beg) {
+    while (s_cnt < kBatch && pos > beg) {
         bool ok = false;
         uint32_t id = 0;
         if (pos - beg > threadIdx.x) {
             const uint32_t i = pos - 1 - threadIdx.x;
-            int rg[8];
-            unpack_ranges(sranges[i], rg);
-            ok = tile_assoc(col, row, cx, cy, rg);
-            if (ok) id = svals[i];
+            ok = tl.mask[(size_t)i * tl.words] >> tl.shift & 1u;
+            if (ok) id = tl.vals[i];
         }
         const uint32_t bal = __ballot_sync(0xffffffffu, ok);
         if (lane == 0) s_wcnt[warp] = __popc(bal);
@@ -243,37 +324,253 @@ __device__ __forceinline__ void fill_list_rev(const uint32_t *__restrict__ svals
 }
 
 // Shared-memory working set of one block's walk over its tile's list.
-template <int kThreads, int BATCH>
 struct WalkSmem {
-    float4 rec[BATCH * 4];           // records of the current batch
-    uint32_t id[BATCH + kThreads];   // tile-list entries found by the filter (item ids)
-    uint32_t pos[BATCH + kThreads];  // their positions in the super-tile list (forward)
-    uint2 hit[BATCH];                // per entry: one byte per warp of the tile, nonzero if a ray hit it
-    uint32_t wcnt[kScan * kThreads / 32];
+    float4 rec[(kBatch + 1) * 4];       // records of the current batch; forward: the last one is never hit
+    uint32_t id[kBatch + kTilePix];     // tile-list entries found by the filter (item ids)
+    uint32_t pos[kBatch + kTilePix];    // their positions in the super-tile list (forward)
+    uint2 hit[kBatch];                  // per entry: one byte per backward warp (16 x 2 rays), nonzero if a ray hit it
+    uint16_t list[kTileWarps][kBatch + kFwdUnroll];  // forward: each sub-tile's entries of the batch (byte offsets in rec)
+    float4 conic[kBatch * 2];           // forward: the entries' quadratics
+    float4 sub[kTileWarps];             // forward: the sub-tiles' rectangles (centre, half sizes) in the tile's chart
+    float2 ray[kTileWarps][32];         // forward: their rays' points there
+    float4 frame[3];                    // forward: the chart's axes c, e1, e2 (splat: the reference angles)
+    uint32_t ext[2];                    // forward: the largest |x|, |y| of the tile's rays (FP32 bits)
+    FillSmem fill;
     uint32_t maxlast, walkpos;       // the tile's last contributor and its super-list position + 1
     uint32_t nck, next_ck;           // forward: checkpoints recorded, list index of the next one
-    uint32_t wacc[kThreads];         // forward: each thread's count of backward steps
+    uint32_t wacc[kTilePix];         // forward: each thread's count of backward steps
     uint32_t ckw[kCkptMax];          // forward: the counts at the checkpoints (work: then the walk's)
     uint32_t ckB[kCkptMax];          // forward: the checkpoints' tile-list indices
     uint32_t work, pend;             // forward: a checkpoint's count of backward steps; its index + 1 while due
     int cam;
-    uint64_t bar;                    // forward with bulk staging: the batch's records have landed
 };
 
-// Copies item `id`'s 64-byte record into shared memory (4 x 16 B). An id beyond
-// the items (a guard failure) stages a record that no ray hits: W = 0 gives
-// kappa = 0/0 and o_u . d_u = 0 (the exact integral's test fails), and
-// log2(sigma) = -inf fails the splat alpha's.
-__device__ __forceinline__ void stage_record(float4 *dst, const Record *__restrict__ rec, uint32_t id, uint64_t items,
-                                             uint32_t site, uint32_t *misc) {
+// Item `id`'s 64-byte record (4 x 16 B). An id beyond the items (a guard failure)
+// gives a record that no ray hits: W = 0 gives kappa = 0/0 and o_u . d_u = 0 (the
+// exact integral's test fails), and log2(sigma) = -inf fails the splat alpha's.
+__device__ __forceinline__ void load_record(float4 q[4], const Record *__restrict__ rec, uint32_t id, uint64_t items,
+                                            uint32_t site, uint32_t *misc) {
     if (in_bounds(id, items, site, misc)) {
         const float4 *src = reinterpret_cast<const float4 *>(rec + id);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) dst[k] = src[k];
+        for (int k = 0; k < 4; ++k) q[k] = src[k];
     } else {
-        dst[0] = dst[1] = dst[2] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        dst[3] = make_float4(-INFINITY, 0.0f, 0.0f, 0.0f);
+        q[0] = q[1] = q[2] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        q[3] = make_float4(-INFINITY, 0.0f, 0.0f, 0.0f);
     }
+}
+
+// ---- Sub-tile culling -------------------------------------------------------
+// A ray hits an entry where kappa = |o_u x W d|^2 / |W d|^2 <= kappa_max =
+// 2 ln(sigma / alpha_min). kappa does not depend on d's length: with d scaled to
+// c + x e1 + y e2 (the tile's chart: c its central direction, e1 and e2 orthonormal
+// to it) that is Q(x, y) = |o_u x W d|^2 - kappa_max |W d|^2 <= 0, a quadratic in
+// (x, y). No ray of a sub-tile hits the entry when a lower bound of Q over the
+// rectangle of its rays' points is positive: the tangent plane's least value
+// (valid for a convex Q) at the rectangle's point nearest the conic's centre, or,
+// when Q is not convex, at the rectangle's centre with the curvature subtracted.
+// A conic that covers only a few rays' share of the rectangle is also evaluated
+// at all 32 rays.
+//
+// A thread computes one entry's quadratic (~130 instructions), each warp then tests
+// 32 entries at a time against its sub-tile, a lane per entry (~35 instructions,
+// ~210 more for the rays), where evaluating one entry costs a warp ~50 whether or
+// not a ray of it hits. Of the 1M-Gaussian fisheye scene's (entry, sub-tile) pairs
+// 28% have a ray that hits and 38% pass the test, of the 500k shell's 17% and 23%
+// (36% without the rays; 70% in the corner tiles that end its launch, 9% with
+// them). us a pass with the tile masks of the lists, before and after: 500k shell
+// at 1024 x 1024 305 -> 262, 4096 Gaussians at 128 x 128 131 -> 118.5.
+//
+// The test never drops what evaluate() / evaluate_splat() calls a hit: e bounds
+// the FP32 errors of both sides. evaluate(): W d carries 4 ulp of |W| |d|, which
+// o_u x multiplies by |o_u|; kappa, its exponent argument and the quotient a few
+// ulp each (in kappa_max's margin); the chart point 8 ulp of the direction. Q: 67
+// ulp of the squared magnitudes it is built from. Entries of extreme scale (where
+// the quotient under- or overflows) are always kept.
+struct Conic {
+    float q0, gx, gy, a, b, c;  // Q(x, y) = q0 + 2 gx x + 2 gy y + a x^2 + 2 b x y + c y^2
+    float e;                    // error bound: out where the lower bound exceeds e
+};
+
+template <bool SPLAT>
+__device__ __forceinline__ Conic cull_conic(const float4 q[4], const float4 *frame, const uint32_t *ext,
+                                            float log2_amin) {
+    Conic v;
+    const float hx = __uint_as_float(ext[0]), hy = __uint_as_float(ext[1]);
+    // kappa_max, with the rounding of the hit test's exponent argument in it
+    const float km = fmaf(fmaxf(q[3].x - log2_amin, 0.0f), 1.38632f, 2e-5f);
+    if (SPLAT) {
+        constexpr float kTwoPi = 6.28318530717959f, kInvTwoPi = 0.159154943091895f;
+        float dt = frame[0].x - q[0].x, dp = frame[0].y - q[0].y;
+        dt = fmaf(-kTwoPi, rintf(dt * kInvTwoPi), dt);
+        dp = fmaf(-kTwoPi, rintf(dp * kInvTwoPi), dp);
+        v.a = q[0].z;
+        v.b = q[0].w;
+        v.c = q[1].x;
+        v.gx = fmaf(v.a, dt, v.b * dp);
+        v.gy = fmaf(v.b, dt, v.c * dp);
+        v.q0 = fmaf(v.gx, dt, v.gy * dp) - km;
+        const float s = fabsf(dt) + hx, t = fabsf(dp) + hy, ab = fabsf(v.b);
+        const float as = fmaf(v.a, s, ab * t), ct = fmaf(v.c, t, ab * s);
+        v.e = 8e-6f * fmaf(as, s, ct * t) + 8e-6f * (as + ct) + 1e-10f * (v.a + v.c + 2.0f * ab);
+        if (!(s < 3.14f && t < 3.14f)) v.e = INFINITY;  // a wrap of the difference inside the tile: kept
+        return v;
+    }
+    const float4 &A = q[0], &B = q[1], &C = q[2];  // W00 W01 W02 W10 | W11 W12 W20 W21 | W22 ou0 ou1 ou2
+    const float ox = C.y, oy = C.z, oz = C.w;
+    const float4 f0 = frame[0], f1 = frame[1], f2 = frame[2];
+    const auto row0 = [&](const float4 &f) { return fmaf(A.x, f.x, fmaf(A.y, f.y, A.z * f.z)); };
+    const auto row1 = [&](const float4 &f) { return fmaf(A.w, f.x, fmaf(B.x, f.y, B.y * f.z)); };
+    const auto row2 = [&](const float4 &f) { return fmaf(B.z, f.x, fmaf(B.w, f.y, C.x * f.z)); };
+    const float u0 = row0(f0), u1 = row1(f0), u2 = row2(f0);  // W d at the chart's origin
+    const float v0 = row0(f1), v1 = row1(f1), v2 = row2(f1);  // and its x
+    const float w0 = row0(f2), w1 = row1(f2), w2 = row2(f2);  // and y derivatives
+    const float m0 = oy * u2 - oz * u1, m1 = oz * u0 - ox * u2, m2 = ox * u1 - oy * u0;  // the same of o_u x W d
+    const float k0 = oy * v2 - oz * v1, k1 = oz * v0 - ox * v2, k2 = ox * v1 - oy * v0;
+    const float l0 = oy * w2 - oz * w1, l1 = oz * w0 - ox * w2, l2 = ox * w1 - oy * w0;
+    const float mm = m0 * m0 + m1 * m1 + m2 * m2, kk = k0 * k0 + k1 * k1 + k2 * k2, ll = l0 * l0 + l1 * l1 + l2 * l2;
+    v.q0 = fmaf(-km, u0 * u0 + u1 * u1 + u2 * u2, mm);
+    v.gx = fmaf(-km, u0 * v0 + u1 * v1 + u2 * v2, m0 * k0 + m1 * k1 + m2 * k2);
+    v.gy = fmaf(-km, u0 * w0 + u1 * w1 + u2 * w2, m0 * l0 + m1 * l1 + m2 * l2);
+    v.a = fmaf(-km, v0 * v0 + v1 * v1 + v2 * v2, kk);
+    v.b = fmaf(-km, v0 * w0 + v1 * w1 + v2 * w2, k0 * l0 + k1 * l1 + k2 * l2);
+    v.c = fmaf(-km, w0 * w0 + w1 * w1 + w2 * w2, ll);
+    // the errors, from |W| |d| (n), |o_u| and the largest |m| of the tile (bm)
+    const float r0 = A.x * A.x + A.y * A.y + A.z * A.z, r1 = A.w * A.w + B.x * B.x + B.y * B.y,
+                r2 = B.z * B.z + B.w * B.w + C.x * C.x;
+    const float sk = sqrtf(km), n = sqrtf((r0 + r1 + r2) * fmaf(hx, hx, fmaf(hy, hy, 1.001f)));
+    const float on = sqrtf(ox * ox + oy * oy + oz * oz), bm = sqrtf(mm) + hx * sqrtf(kk) + hy * sqrtf(ll);
+    const float cc = 2e-6f * n * (on + sk);
+    v.e = fmaf(cc, fmaf(2.0f * sk, n, cc), 4e-6f * fmaf(bm, fmaf(on, n, bm), km * n * n));
+    if (!(n < 1e18f && fminf(r0, fminf(r1, r2)) > 1e-30f)) v.e = INFINITY;  // extreme scales: kept
+    return v;
+}
+
+// Whether a ray in the rectangle r (centre x, y, half sizes) may hit the entry.
+// few: the conic covers the share of about eight rays or less.
+__device__ __forceinline__ bool cull_keep(const Conic &v, const float4 &r, bool &few) {
+    const float det = fmaf(v.a, v.c, -v.b * v.b);
+    const bool convex = v.a > 0.0f && v.c > 0.0f && det > 1e-6f * v.a * v.c;
+    float x = r.x, y = r.y;
+    few = false;
+    if (convex) {  // the point of the rectangle nearest the conic's centre (any point serves)
+        const float id = __fdividef(1.0f, det);
+        const float cx = (v.b * v.gy - v.c * v.gx) * id, cy = (v.b * v.gx - v.a * v.gy) * id;
+        x = fminf(fmaxf(cx, r.x - r.z), r.x + r.z);
+        y = fminf(fmaxf(cy, r.y - r.w), r.y + r.w);
+        // its area is pi w / sqrt(det), w = -Q at the centre, the rectangle's 4 r.z r.w
+        const float w = -fmaf(v.gx, cx, fmaf(v.gy, cy, v.q0));
+        few = w * w * id < 0.1f * r.z * r.z * r.w * r.w;
+    }
+    const float hx = fmaf(v.a, x, fmaf(v.b, y, v.gx)), hy = fmaf(v.b, x, fmaf(v.c, y, v.gy));  // half gradient
+    // Q at (x, y) = q0 + (gx + hx) x + (gy + hy) y; the tangent plane's least value over the rectangle
+    const float at = fmaf(v.gx + hx, x, fmaf(v.gy + hy, y, v.q0));
+    float low = at + 2.0f * (fmaf(hx, r.x - x, hy * (r.y - y)) - fmaf(fabsf(hx), r.z, fabsf(hy) * r.w));
+    if (!convex)
+        low += fminf(v.a, 0.0f) * r.z * r.z + fminf(v.c, 0.0f) * r.w * r.w - 2.0f * fabsf(v.b) * r.z * r.w;
+    return !(low > v.e);  // a NaN keeps the entry
+}
+
+// The least Q over the sub-tile's rays (a NaN where there is no ray).
+__device__ __forceinline__ bool cull_keep_rays(const Conic &v, const float2 *ray) {
+    float low = NAN;
+#pragma unroll 8
+    for (int k = 0; k < 32; k += 2) {
+        const float4 r = *reinterpret_cast<const float4 *>(ray + k);
+        low = fminf(low, fmaf(r.x, fmaf(v.a, r.x, fmaf(2.0f * v.b, r.y, 2.0f * v.gx)),
+                              fmaf(r.y, fmaf(v.c, r.y, 2.0f * v.gy), v.q0)));
+        low = fminf(low, fmaf(r.z, fmaf(v.a, r.z, fmaf(2.0f * v.b, r.w, 2.0f * v.gx)),
+                              fmaf(r.w, fmaf(v.c, r.w, 2.0f * v.gy), v.q0)));
+    }
+    return !(low > v.e);
+}
+constexpr int kRaysFrom = 6;  // entries of 32 for which testing all rays is cheaper than evaluating them
+
+// The tile's chart, its sub-tiles' rectangles and rays there (block-wide, ends in a
+// barrier). c: the mean direction of the tile's rays; e1 and e2: the projection of
+// the x axis (of the y axis for a c near the x axis) and the normal to it. The
+// rectangles carry 8 ulp of rounding. A sub-tile with a ray more than ~84 degrees
+// from c, or without rays, gets infinite half sizes (its low is -infinity or NaN:
+// its test never drops an entry). Splat: the rays' screen angles about the first
+// ray's.
+template <bool SPLAT>
+__device__ __forceinline__ void sub_tiles(WalkSmem &sm, bool inside, float dx, float dy, float dz) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float x, y;
+    bool bad = false;
+    if (threadIdx.x < 2) sm.ext[threadIdx.x] = 0u;
+    if (SPLAT) {
+        if (threadIdx.x == 0) sm.frame[0] = make_float4(dx, dy, 0.0f, 0.0f);  // the tile's first ray is in the image
+        __syncthreads();
+        x = dx - sm.frame[0].x;
+        y = dy - sm.frame[0].y;
+    } else {
+        const float len = sqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz))), inv = inside && len > 0.0f ? 1.0f / len : 0.0f;
+        float s0 = dx * inv, s1 = dy * inv, s2 = dz * inv;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+            s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+            s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+        }
+        if (lane == 0) sm.sub[warp] = make_float4(s0, s1, s2, 0.0f);
+        __syncthreads();
+        if (warp == 0) {
+            const float4 t = sm.sub[lane & (kTileWarps - 1)];
+            float c0 = t.x, c1 = t.y, c2 = t.z;
+#pragma unroll
+            for (int o = kTileWarps / 2; o > 0; o >>= 1) {
+                c0 += __shfl_xor_sync(0xffffffffu, c0, o);
+                c1 += __shfl_xor_sync(0xffffffffu, c1, o);
+                c2 += __shfl_xor_sync(0xffffffffu, c2, o);
+            }
+            const float ic = rsqrtf(fmaf(c0, c0, fmaf(c1, c1, c2 * c2)));
+            c0 *= ic;
+            c1 *= ic;
+            c2 *= ic;
+            // a e1 (or e2) = axis - c (c . axis), normalised; the other one by the cross product
+            const bool ax = fabsf(c0) < 0.9f;
+            const float p = ax ? c0 : c1;
+            float a0 = fmaf(-c0, p, ax ? 1.0f : 0.0f), a1 = fmaf(-c1, p, ax ? 0.0f : 1.0f), a2 = -c2 * p;
+            const float ia = rsqrtf(fmaf(a0, a0, fmaf(a1, a1, a2 * a2)));
+            a0 *= ia;
+            a1 *= ia;
+            a2 *= ia;
+            if (lane == 0) {
+                sm.frame[0] = make_float4(c0, c1, c2, 0.0f);
+                sm.frame[1] = make_float4(a0, a1, a2, 0.0f);
+                sm.frame[2] = make_float4(c1 * a2 - c2 * a1, c2 * a0 - c0 * a2, c0 * a1 - c1 * a0, 0.0f);
+            }
+        }
+        __syncthreads();
+        const float4 c = sm.frame[0], e1 = sm.frame[1], e2 = sm.frame[2];
+        const float dc = fmaf(dx, c.x, fmaf(dy, c.y, dz * c.z)), idc = 1.0f / dc;
+        x = fmaf(dx, e1.x, fmaf(dy, e1.y, dz * e1.z)) * idc;
+        y = fmaf(dx, e2.x, fmaf(dy, e2.y, dz * e2.z)) * idc;
+        bad = !(dc > 0.1f * len);
+    }
+    const unsigned in = __ballot_sync(0xffffffffu, inside);
+    const bool ok = in && !__any_sync(0xffffffffu, inside && bad);
+    float x0 = inside ? x : INFINITY, x1 = inside ? x : -INFINITY, y0 = inside ? y : INFINITY, y1 = inside ? y : -INFINITY;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        x0 = fminf(x0, __shfl_xor_sync(0xffffffffu, x0, o));
+        x1 = fmaxf(x1, __shfl_xor_sync(0xffffffffu, x1, o));
+        y0 = fminf(y0, __shfl_xor_sync(0xffffffffu, y0, o));
+        y1 = fmaxf(y1, __shfl_xor_sync(0xffffffffu, y1, o));
+    }
+    sm.ray[warp][lane] = ok && inside ? make_float2(x, y) : make_float2(NAN, NAN);
+    if (lane == 0) {
+        const float mx = fmaxf(fabsf(x0), fabsf(x1)), my = fmaxf(fabsf(y0), fabsf(y1));
+        sm.sub[warp] = ok ? make_float4(0.5f * (x0 + x1), 0.5f * (y0 + y1), 0.5f * (x1 - x0) + (1e-6f * mx + 1e-7f),
+                                        0.5f * (y1 - y0) + (1e-6f * my + 1e-7f))
+                          : make_float4(0.0f, 0.0f, INFINITY, INFINITY);
+        if (ok) {  // (an atomic max of non-negative FP32 bits)
+            atomicMax(&sm.ext[0], __float_as_uint(mx * 1.00001f + 1e-6f));
+            atomicMax(&sm.ext[1], __float_as_uint(my * 1.00001f + 1e-6f));
+        }
+    }
+    __syncthreads();
 }
 
 // A tile's super-tile list range must lie within the sorted pairs; a guard
@@ -284,6 +581,16 @@ __device__ __forceinline__ uint2 checked_range(uint2 sr, int64_t cap_pairs, uint
     return sr;
 }
 
+// A thread's ray in the forward: warp w holds sub-tile w's 8 x 4 rays (two columns
+// of four sub-tiles). Compact warps meet fewer footprints than rows do: a disc of
+// radius r pixels meets (8 + 2r)(4 + 2r) placements of an 8 x 4 warp,
+// (16 + 2r)(2 + 2r) of a 16 x 2 one. The backward's warps hold 16 x 2 rays (ray =
+// thread): the order of its sums, and with it the last digits of ill-conditioned
+// gradients (needles close to a camera), stays what it is.
+__device__ __forceinline__ int fwd_ray(int tid) {
+    return ((tid >> 6) * 4 + ((tid >> 3) & 3)) * kTile + ((tid >> 5) & 1) * 8 + (tid & 7);
+}
+
 // Per-ray forward state (n_eval: entries evaluated, set when the walk ends).
 struct FwdRay {
     float T, cr, cg, cb;
@@ -291,74 +598,63 @@ struct FwdRay {
     bool done;
 };
 
-// Composites list entries [j0, j1) of the staged batch into ray state f, front
-// to back (App. B.1 colour equation), until the ray terminates: kFwdUnroll
-// entries are evaluated together (independent work for the scheduler on long
-// walks), then composited strictly in list order. Entry j of the batch has
-// tile-list index n_list + j. hit_b: the ray's warp's hit byte of entry 0 (8
-// bytes per entry).
+// Composites the sub-tile's entries of the staged batch (list: n byte offsets of
+// their records, padded to a multiple of kFwdUnroll with a record that no ray
+// hits) into ray state f, front to back (App. B.1 colour equation), until the
+// ray terminates: kFwdUnroll entries are evaluated together (independent work for
+// the scheduler on long walks), then composited strictly in list order. Entry j
+// of the batch has tile-list index n_list + j. hit_b: the hit byte of entry 0 of the
+// ray's backward warp (8 bytes per entry).
 template <bool SPLAT>
-__device__ __forceinline__ void walk_entries(const float4 *srec, int j0, int j1, uint32_t n_list, uint8_t *hit_b,
-                                             const Params &p, float log2_amin, float dx, float dy, float dz,
-                                             FwdRay &f) {
-    int j = j0;
-    for (; j + kFwdUnroll <= j1 && !f.done; j += kFwdUnroll) {
+__device__ __forceinline__ void walk_entries(const float4 *srec, const uint16_t *list, int n, uint32_t n_list, uint32_t *misc,
+                                             uint8_t *hit_b, const Params &p, float log2_amin, float dx, float dy,
+                                             float dz, FwdRay &f) {
+    static_assert(kFwdUnroll == 4, "four 16-bit offsets per shared load");
+    for (int k = 0; k < n && !f.done; k += kFwdUnroll) {
+        const uint2 o2 = *reinterpret_cast<const uint2 *>(list + k);
+        uint32_t off[kFwdUnroll] = {o2.x & 0xffffu, o2.x >> 16, o2.y & 0xffffu, o2.y >> 16};
+        const uint32_t drop = GEER_CHECKED ? (off[0] & 1u) | (off[1] & 1u) << 1 | (off[2] & 1u) << 2 | (off[3] & 1u) << 3 : 0u;
+#pragma unroll
+        for (int u = 0; u < kFwdUnroll; ++u) off[u] &= ~(GEER_CHECKED ? 1u : 0u);
         Eval v[kFwdUnroll];
         float4 e[kFwdUnroll];
 #pragma unroll
         for (int u = 0; u < kFwdUnroll; ++u) {
-            const float4 a = srec[(j + u) * 4 + 0];  // W00 W01 W02 W10
-            const float4 b = srec[(j + u) * 4 + 1];  // W11 W12 W20 W21
-            const float4 c = srec[(j + u) * 4 + 2];  // W22 ou0 ou1 ou2
-            e[u] = srec[(j + u) * 4 + 3];            // log2 sigma, r, g, b
+            const float4 *r = reinterpret_cast<const float4 *>(reinterpret_cast<const char *>(srec) + off[u]);
+            const float4 a = r[0];  // W00 W01 W02 W10
+            const float4 b = r[1];  // W11 W12 W20 W21
+            const float4 c = r[2];  // W22 ou0 ou1 ou2
+            e[u] = r[3];            // log2 sigma, r, g, b
             v[u] = SPLAT ? evaluate_splat(a, b, e[u], dx, dy, log2_amin) : evaluate(a, b, c, e[u], dx, dy, dz, log2_amin);
         }
         // after the group's record loads (a byte store may alias them); the
-        // same value from every lane of the warp: no race
+        // same value from every lane: no race
 #pragma unroll
         for (int u = 0; u < kFwdUnroll; ++u)
-            if (v[u].hit) hit_b[(j + u) * 8] = 1;
+            if (v[u].hit) hit_b[off[u] >> 3] = 1;
+        // branch-free per entry (predicated updates): with data-dependent branches
+        // the four steps cost a reconvergence each
 #pragma unroll
         for (int u = 0; u < kFwdUnroll; ++u) {
-            if (!v[u].hit) continue;
-            const float alpha = fminf(exp2f(v[u].arg), p.alpha_max);
+            const float alpha = fminf(ex2(v[u].arg), p.alpha_max);
             const float Tn = f.T * (1.0f - alpha);
-            if (Tn < p.T_min) {
+            const uint32_t at = n_list + (off[u] >> 6) + 1u;
+            const bool live = v[u].hit && !f.done;
+            if (GEER_CHECKED && live && (drop >> u & 1u)) in_bounds(n_list + (off[u] >> 6), 0u, kSiteFwdCull, misc);
+            if (live && Tn < p.T_min) {
                 f.done = true;
-                f.n_eval = n_list + (uint32_t)(j + u) + 1u;  // entries up to this one
-                break;
+                f.n_eval = at;  // entries up to this one
             }
-            const float wgt = alpha * f.T;
-            f.cr = fmaf(wgt, e[u].y, f.cr);
-            f.cg = fmaf(wgt, e[u].z, f.cg);
-            f.cb = fmaf(wgt, e[u].w, f.cb);
-            f.T = Tn;
-            ++f.n_applied;
-            f.last = n_list + (uint32_t)(j + u) + 1u;
+            if (live && !(Tn < p.T_min)) {
+                const float wgt = alpha * f.T;
+                f.cr = fmaf(wgt, e[u].y, f.cr);
+                f.cg = fmaf(wgt, e[u].z, f.cg);
+                f.cb = fmaf(wgt, e[u].w, f.cb);
+                f.T = Tn;
+                ++f.n_applied;
+                f.last = at;
+            }
         }
-    }
-    for (; j < j1 && !f.done; ++j) {
-        const float4 a = srec[j * 4 + 0];
-        const float4 b = srec[j * 4 + 1];
-        const float4 c = srec[j * 4 + 2];
-        const float4 e = srec[j * 4 + 3];
-        const Eval v = SPLAT ? evaluate_splat(a, b, e, dx, dy, log2_amin) : evaluate(a, b, c, e, dx, dy, dz, log2_amin);
-        if (!v.hit) continue;
-        hit_b[j * 8] = 1;
-        const float alpha = fminf(exp2f(v.arg), p.alpha_max);
-        const float Tn = f.T * (1.0f - alpha);
-        if (Tn < p.T_min) {
-            f.done = true;
-            f.n_eval = n_list + (uint32_t)j + 1u;
-            break;
-        }
-        const float wgt = alpha * f.T;
-        f.cr = fmaf(wgt, e.y, f.cr);
-        f.cg = fmaf(wgt, e.z, f.cg);
-        f.cb = fmaf(wgt, e.w, f.cb);
-        f.T = Tn;
-        ++f.n_applied;
-        f.last = n_list + (uint32_t)j + 1u;
     }
 }
 
@@ -370,76 +666,83 @@ __device__ __forceinline__ void walk_entries(const float4 *srec, int j0, int j1,
 // 0 .. maxlast - 1.
 // SPLAT: the splat alpha (GEER_ALPHA_SPLAT) in place of the ray integral;
 // (dx, dy) then carry the ray's screen angles.
-template <int kThreads, int BATCH, bool SPLAT>
-__device__ __forceinline__ void forward_walk(WalkSmem<kThreads, BATCH> &sm, const uint32_t *__restrict__ svals,
-                                             const uint4 *__restrict__ sranges, const Record *__restrict__ rec,
-                                             const Params &p, const float4 &col, const float4 &row, int cx, int cy,
-                                             uint2 sr, float dx, float dy, float dz, uint2 *__restrict__ hit_rec,
+template <bool SPLAT>
+__device__ __forceinline__ void forward_walk(WalkSmem &sm, const TileList &tl, const Record *__restrict__ rec,
+                                             const Params &p, float dx, float dy, float dz,
+                                             uint2 *__restrict__ hit_rec,
                                              uint32_t *__restrict__ id_rec, int64_t hit_entries, uint64_t items,
                                              uint32_t *misc,
                                              float4 *__restrict__ ckpt, uint2 *__restrict__ ckpt_at,
                                              FwdRay &f) {
-    const int tid = threadIdx.x;
-    uint8_t *const hit_b = reinterpret_cast<uint8_t *>(sm.hit) + (tid >> 5);  // this warp's byte of entry 0
+    constexpr int kThreads = kTilePix;
+    static_assert(kBatch == kThreads, "one record per thread and batch");
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    uint8_t *const hit_b = reinterpret_cast<uint8_t *>(sm.hit) + fwd_ray(tid) / 32;  // the ray's byte of entry 0
+    sub_tiles<SPLAT>(sm, !f.done, dx, dy, dz);
     if (tid == 0) {
         sm.maxlast = 0u;
-        sm.walkpos = sr.x;
+        sm.walkpos = tl.sr.x;
         sm.nck = 0u;
         sm.next_ck = ckpt ? kCkptFirst : 0xffffffffu;
         sm.work = 0u;
         sm.pend = 0u;
     }
+    if (tid < 4) sm.rec[kBatch * 4 + tid] = make_float4(tid == 3 ? -INFINITY : 0.0f, 0.0f, 0.0f, 0.0f);
     sm.wacc[tid] = 0u;
     const float log2_amin = log2f(p.alpha_min);
-    uint32_t pos = sr.x, n_list = 0;
-    int s_cnt = 0, want = BATCH < 64 ? BATCH : 64;
-#if GEER_FWD_BULK
-    static_assert(BATCH <= kThreads, "one record per thread and batch");
-    uint32_t parity = 0;
-    if (tid == 0) mbar_init(&sm.bar, kThreads);
-#endif
+    uint32_t pos = tl.sr.x, n_list = 0;
+    bool sparse = false;
+    int s_cnt = 0, want = 64;
     while (true) {
         if (__syncthreads_count(f.done) == kThreads) break;
-        // batches grow 64, 128, ... BATCH: most rays of a dense scene stop early
-        fill_list<kThreads>(svals, sranges, col, row, cx, cy, pos, sr.y, want, sm.id, sm.pos, s_cnt, sm.wcnt);
-        want = min(2 * want, BATCH);
-        const int cnt = min(s_cnt, BATCH);
+        // batches grow 64, 128, ... kBatch: most rays of a dense scene stop early
+        fill_list(tl, pos, sparse, want, sm.id, sm.pos, s_cnt, sm.fill);
+        want = min(2 * want, kBatch);
+        const int cnt = min(s_cnt, kBatch);
         if (cnt == 0) break;
-#if GEER_FWD_BULK
-        // every thread arrives once; thread r < cnt copies record r (64 B) with the
-        // TMA engine and announces its bytes
-        fence_proxy_async();
-        if (tid < cnt) {
-            const uint32_t id = sm.id[tid];
-            if (in_bounds(id, items, kSiteFwdItem, misc)) {
-                mbar_arrive_expect(&sm.bar, (uint32_t)sizeof(Record));
-                bulk_g2s(sm.rec + tid * 4, rec + id, (uint32_t)sizeof(Record), &sm.bar);
-            } else {
-                stage_record(sm.rec + tid * 4, rec, id, items, kSiteFwdItem, misc);
-                mbar_arrive_expect(&sm.bar, 0u);
-            }
+        if (tid < cnt) {  // entry tid: its record and quadratic
+            float4 q[4];
+            load_record(q, rec, sm.id[tid], items, kSiteFwdItem, misc);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) sm.rec[tid * 4 + k] = q[k];
+            const Conic v = cull_conic<SPLAT>(q, sm.frame, sm.ext, log2_amin);
+            sm.conic[2 * tid] = make_float4(v.q0, v.gx, v.gy, v.a);
+            sm.conic[2 * tid + 1] = make_float4(v.b, v.c, v.e, 0.0f);
             sm.hit[tid] = make_uint2(0u, 0u);
-        } else {
-            mbar_arrive_expect(&sm.bar, 0u);
         }
         __syncthreads();
-        if (!mbar_wait(&sm.bar, parity, kBarPolls)) atomicOr(misc + kMiscStatus, kStatusTimeout);
-        parity ^= 1u;
-#else
-        for (int r = tid; r < cnt; r += kThreads) {
-            stage_record(sm.rec + r * 4, rec, sm.id[r], items, kSiteFwdItem, misc);
-            sm.hit[r] = make_uint2(0u, 0u);
+        if (!__all_sync(0xffffffffu, f.done)) {
+            // the entries this warp's rays may hit, in list order
+            uint16_t *const list = sm.list[warp];
+            const float4 rect = sm.sub[warp];
+            int n = 0;
+            for (int g = 0; g < cnt; g += 32) {
+                bool keep = false, few = false;
+                Conic v{};
+                if (g + lane < cnt) {
+                    const float4 u = sm.conic[2 * (g + lane)], w = sm.conic[2 * (g + lane) + 1];
+                    v = Conic{u.x, u.y, u.z, u.w, w.x, w.y, w.z};
+                    keep = cull_keep(v, rect, few);
+                }
+                if (__popc(__ballot_sync(0xffffffffu, keep && few)) >= kRaysFrom)
+                    keep = keep && cull_keep_rays(v, sm.ray[warp]);
+                // (the checked build walks the dropped entries too, marked, to see that no ray hits one)
+                const bool walk = GEER_CHECKED ? g + lane < cnt : keep;
+                const uint32_t b = __ballot_sync(0xffffffffu, walk);
+                if (walk) list[n + __popc(b & lanemask_lt())] = (uint16_t)((g + lane) * 64 + (keep ? 0 : 1));
+                n += __popc(b);
+            }
+            if (lane < kFwdUnroll) list[n + lane] = (uint16_t)(kBatch * 64);
+            __syncwarp();
+            walk_entries<SPLAT>(sm.rec, list, n, n_list, misc, hit_b, p, log2_amin, dx, dy, dz, f);
         }
-        __syncthreads();
-#endif
-        if (!f.done) walk_entries<SPLAT>(sm.rec, 0, cnt, n_list, hit_b, p, log2_amin, dx, dy, dz, f);
         // a checkpoint for the backward: every ray's (T, C) in front of tile-list
         // entry n_list + cnt and where that entry's search starts in the super-tile list
         // (its state lives in shared memory, advanced by thread 0 after the next
         // barrier: the walk's registers are at their limit)
         const uint32_t nck = sm.nck;
         const bool ck = n_list + (uint32_t)cnt >= sm.next_ck && nck < (uint32_t)kCkptMax;
-        if (ck) ckpt[(size_t)nck * kTilePix + tid] = make_float4(f.T, f.cr, f.cg, f.cb);
+        if (ck) ckpt[(size_t)nck * kTilePix + fwd_ray(tid)] = make_float4(f.T, f.cr, f.cg, f.cb);
         // the tile's last contributor so far and where it lies in the super-tile list
         const uint32_t wl = __reduce_max_sync(0xffffffffu, f.last);
         if ((tid & 31) == 0) atomicMax(&sm.maxlast, wl);
@@ -473,7 +776,7 @@ __device__ __forceinline__ void forward_walk(WalkSmem<kThreads, BATCH> &sm, cons
                 if ((tid & 31) == 0) atomicAdd(&sm.work, we);
             }
         }
-        shift_list<kThreads>(sm.id, sm.pos, cnt, s_cnt);
+        shift_list(sm.id, sm.pos, cnt, s_cnt);
         // after shift_list's barrier: the checkpoint's count has landed
         if (tid == 0 && sm.pend) {
             sm.ckw[sm.pend - 1u] = sm.work;
@@ -494,22 +797,20 @@ __device__ __forceinline__ void forward_walk(WalkSmem<kThreads, BATCH> &sm, cons
 // per-pixel (sin, cos) tables of the BEAP angles), the tile's association
 // table entries and super-tile list. Returns false for a padding tile.
 struct TileRay {
-    int cx, cy, x, y;
+    int x, y;
     bool inside;
     float dx, dy, dz;
-    float4 col, row;
-    uint2 sr;
+    TileList tl;
 };
 
-__device__ __forceinline__ bool tile_ray(const DevCam &cam, int t, int row0, const float2 *__restrict__ ptab,
-                                         const float4 *__restrict__ ttab, const uint2 *__restrict__ srange, int S,
-                                         TileRay &r, int ray) {
+__device__ __forceinline__ bool tile_ray(const DevCam &cam, int t, const float2 *__restrict__ ptab,
+                                         const uint2 *__restrict__ srange, const uint32_t *svals,
+                                         const uint32_t *smask, const uint32_t *sany, int S, TileRay &r, int ray) {
     const int lt = t - cam.tile_base;
     if (lt >= cam.tiles_x * cam.tiles_y) return false;  // padding tile of a camera slot
-    r.cx = lt % cam.tiles_x;
-    r.cy = lt / cam.tiles_x;
-    r.x = r.cx * kTile + (ray & (kTile - 1));
-    r.y = r.cy * kTile + row0 + (ray / kTile);
+    const int cy = lt / cam.tiles_x, cx = lt - cy * cam.tiles_x;
+    r.x = cx * kTile + (ray & (kTile - 1));
+    r.y = cy * kTile + ray / kTile;
     r.inside = r.x < cam.width && r.y < cam.height;
     r.dx = 0.0f;
     r.dy = 0.0f;
@@ -521,9 +822,13 @@ __device__ __forceinline__ bool tile_ray(const DevCam &cam, int t, int row0, con
         r.dy = th.y * ph.x;
         r.dz = th.y * ph.y;
     }
-    r.col = ttab[cam.tcol_off + r.cx];
-    r.row = ttab[cam.trow_off + r.cy];
-    r.sr = srange[cam.stile_base + (r.cy / S) * cam.stiles_x + r.cx / S];
+    const int sx = cx / S, sy = cy / S, bit = (cy - sy * S) * S + (cx - sx * S);
+    r.tl.vals = svals;
+    r.tl.words = mask_words(S);
+    r.tl.mask = smask + (bit >> 5);
+    r.tl.any = sany + (bit >> 5);
+    r.tl.shift = bit & 31;
+    r.tl.sr = srange[cam.stile_base + sy * cam.stiles_x + sx];
     return true;
 }
 
@@ -546,17 +851,17 @@ __device__ __forceinline__ void l1_pixel(float c0, float c1, float c2, const flo
 // hit and list records, the checkpoints and the backward's unit record. With
 // L1, each pixel's L1 gradient against target too (dL; |differences| summed
 // into l1acc). Returns the tile's backward unit count in thread 0.
-template <int ROWS, int BATCH, bool SPLAT, bool L1>
-__device__ __forceinline__ uint32_t fwd_tile(WalkSmem<ROWS * kTile, BATCH> &sm, uint32_t t_id,
+template <bool SPLAT, bool L1>
+__device__ __forceinline__ uint32_t fwd_tile(WalkSmem &sm, uint32_t t_id,
                                          const DevCam *__restrict__ cams,
                                          int ncams,
                                          const float2 *__restrict__ ptab,
-                                         const float4 *__restrict__ ttab,
                                          int S,
                                          uint2 *__restrict__ tile_walk,
                                          const uint2 *__restrict__ srange,
                                          const uint32_t *__restrict__ svals,
-                                         const uint4 *__restrict__ sranges,
+                                         const uint32_t *__restrict__ smask,
+                                         const uint32_t *__restrict__ sany,
                                          const Record *__restrict__ rec,
                                          uint32_t *__restrict__ misc,
                                          Params p,
@@ -579,14 +884,13 @@ __device__ __forceinline__ uint32_t fwd_tile(WalkSmem<ROWS * kTile, BATCH> &sm, 
                                          float4 *__restrict__ Cfin,
                                          const float *__restrict__ target, float *__restrict__ dL, float inv_m,
                                          float &l1acc) {
-    constexpr int kThreads = ROWS * kTile;
     if (!in_bounds(t_id, (uint64_t)ntiles, kSiteFwdTile, misc)) return 0u;  // block-uniform
     const int t = (int)t_id;
     if (threadIdx.x == 0) sm.cam = find_cam(cams, ncams, t);
     __syncthreads();
     const DevCam &cam = cams[sm.cam];
     TileRay tr;
-    if (!tile_ray(cam, t, 0, ptab, ttab, srange, S, tr, (int)threadIdx.x)) {
+    if (!tile_ray(cam, t, ptab, srange, svals, smask, sany, S, tr, fwd_ray((int)threadIdx.x))) {
         if (threadIdx.x == 0) {
             tile_walk[t] = make_uint2(0u, 0u);
             if (ckpt_cnt) ckpt_cnt[t] = 0u;
@@ -594,7 +898,7 @@ __device__ __forceinline__ uint32_t fwd_tile(WalkSmem<ROWS * kTile, BATCH> &sm, 
         }
         return 0u;
     }
-    tr.sr = checked_range(tr.sr, cap_pairs, kSiteFwdList, misc);
+    tr.tl.sr = checked_range(tr.tl.sr, cap_pairs, kSiteFwdList, misc);
     if (tile_mask && !tile_mask[t]) {  // another part's tile: zeros, nothing for the backward to walk
         if (threadIdx.x == 0) {
             tile_walk[t] = make_uint2(0u, 0u);
@@ -620,8 +924,8 @@ __device__ __forceinline__ uint32_t fwd_tile(WalkSmem<ROWS * kTile, BATCH> &sm, 
         tr.dx = ts;
         tr.dy = ps;
     }
-    forward_walk<kThreads, BATCH, SPLAT>(sm, svals, sranges, rec, p, tr.col, tr.row, tr.cx, tr.cy, tr.sr, tr.dx, tr.dy,
-                                         tr.dz, hit ? hit + (int64_t)t * hit_entries : nullptr,
+    forward_walk<SPLAT>(sm, tr.tl, rec, p, tr.dx, tr.dy, tr.dz,
+                        hit ? hit + (int64_t)t * hit_entries : nullptr,
                                          hit ? idrec + (int64_t)t * hit_entries : nullptr, hit_entries, items,
                                          misc, ckpt ? ckpt + (size_t)t * kCkptMax * kTilePix : nullptr,
                                          ckpt ? ckpt_at + (size_t)t * kCkptMax : nullptr,
@@ -665,15 +969,16 @@ __device__ __forceinline__ uint32_t fwd_tile(WalkSmem<ROWS * kTile, BATCH> &sm, 
     return units;
 }
 
-template <int ROWS, int BATCH, bool SPLAT>
-__global__ void __launch_bounds__(ROWS * kTile, GEER_FWD_MINB) k_render_fwd(const DevCam *__restrict__ cams, int ncams,
+template <bool SPLAT>
+__global__ void __launch_bounds__(kTilePix, GEER_FWD_MINB) k_render_fwd(const DevCam *__restrict__ cams, int ncams,
                                                             const float2 *__restrict__ ptab,
-                                                            const float4 *__restrict__ ttab, int S,
+                                         int S,
                                                             uint2 *__restrict__ tile_walk,
                                                             const uint32_t *__restrict__ tile_order,
                                                             const uint2 *__restrict__ srange,
                                                             const uint32_t *__restrict__ svals,
-                                                            const uint4 *__restrict__ sranges,
+                                                            const uint32_t *__restrict__ smask,
+                                                            const uint32_t *__restrict__ sany,
                                                             const Record *__restrict__ rec,
                                                             uint32_t *__restrict__ misc, Params p,
                                                             float *__restrict__ rgb,
@@ -688,12 +993,10 @@ __global__ void __launch_bounds__(ROWS * kTile, GEER_FWD_MINB) k_render_fwd(cons
                                                             uint4 *__restrict__ unit_rec,
                                                             float4 *__restrict__ Cfin) {
     grid_dep_sync();
-    constexpr int kThreads = ROWS * kTile, kParts = kTile / ROWS;
-    static_assert(kParts == 1, "one block per tile: the block records the tile's walk");
-    __shared__ WalkSmem<kThreads, BATCH> sm;
+    __shared__ WalkSmem sm;
     if (misc[kMiscStatus] & kStatusCapacity) return;
     float l1acc = 0.0f;
-    fwd_tile<ROWS, BATCH, SPLAT, false>(sm, tile_order[blockIdx.x], cams, ncams, ptab, ttab, S, tile_walk, srange, svals, sranges, rec, misc, p, rgb, Tout, Tfin, last_out, evals, hit, idrec, hit_entries, tile_mask, ntiles, items, cap_pairs, ckpt, ckpt_at, ckpt_cnt, unit_rec, Cfin, nullptr, nullptr, 0.0f,
+    fwd_tile<SPLAT, false>(sm, tile_order[blockIdx.x], cams, ncams, ptab, S, tile_walk, srange, svals, smask, sany, rec, misc, p, rgb, Tout, Tfin, last_out, evals, hit, idrec, hit_entries, tile_mask, ntiles, items, cap_pairs, ckpt, ckpt_at, ckpt_cnt, unit_rec, Cfin, nullptr, nullptr, 0.0f,
                                         l1acc);
 }
 
@@ -701,42 +1004,41 @@ __global__ void __launch_bounds__(ROWS * kTile, GEER_FWD_MINB) k_render_fwd(cons
 // list exactly as the renders do. With lists == NULL: count[t] = the list's
 // length; else lists[off[t] + k] = entry k (off in the same array). For inspection.
 __global__ void __launch_bounds__(kTilePix) k_expand_tiles(const DevCam *__restrict__ cams, int ncams,
-                                                          const float4 *__restrict__ ttab, int S,
+                                                          const float2 *__restrict__ ptab, int S,
                                                           const uint2 *__restrict__ srange,
                                                           const uint32_t *__restrict__ svals,
-                                                          const uint4 *__restrict__ sranges,
+                                                          const uint32_t *__restrict__ smask,
+                                                          const uint32_t *__restrict__ sany,
                                                           const uint32_t *__restrict__ misc,
                                                           uint32_t *__restrict__ count_or_off,
                                                           uint32_t *__restrict__ lists, int64_t cap) {
     grid_dep_sync();
     __shared__ uint32_t s_id[2 * kTilePix];
-    __shared__ uint32_t s_wcnt[kScan * kTilePix / 32];
+    __shared__ FillSmem s_fill;
     __shared__ int s_cam;
     if (misc[kMiscStatus] & kStatusCapacity) return;
     const int t = blockIdx.x, tid = threadIdx.x;
     if (tid == 0) s_cam = find_cam(cams, ncams, t);
     __syncthreads();
-    const DevCam &cam = cams[s_cam];
-    const int lt = t - cam.tile_base;
-    if (lt >= cam.tiles_x * cam.tiles_y) {
+    TileRay tr;
+    if (!tile_ray(cams[s_cam], t, ptab, srange, svals, smask, sany, S, tr, tid)) {
         if (!lists && tid == 0) count_or_off[t] = 0u;
         return;
     }
-    const int cx = lt % cam.tiles_x, cy = lt / cam.tiles_x;
-    const float4 col = ttab[cam.tcol_off + cx], row = ttab[cam.trow_off + cy];
-    const uint2 sr = srange[cam.stile_base + (cy / S) * cam.stiles_x + cx / S];
     const int64_t off = lists ? (int64_t)count_or_off[t] : 0;
-    uint32_t pos = sr.x, n_list = 0;
+    uint32_t pos = tr.tl.sr.x, n_list = 0;
+    bool sparse = false;
     int s_cnt = 0;
     while (true) {
-        fill_list<kTilePix>(svals, sranges, col, row, cx, cy, pos, sr.y, kTilePix, s_id, nullptr, s_cnt, s_wcnt);
+        fill_list(tr.tl, pos, sparse, kTilePix, s_id, nullptr, s_cnt, s_fill);
         const int cnt = min(s_cnt, kTilePix);
         if (cnt == 0) break;
         if (lists)
             for (int r = tid; r < cnt; r += kTilePix)
                 if (off + n_list + r < cap) lists[off + n_list + r] = s_id[r];
         __syncthreads();
-        shift_list<kTilePix>(s_id, nullptr, cnt, s_cnt);
+        shift_list(s_id, nullptr, cnt, s_cnt);
+        __syncthreads();
         n_list += (uint32_t)cnt;
     }
     if (!lists && tid == 0) count_or_off[t] = n_list;
@@ -822,17 +1124,16 @@ __device__ __forceinline__ void ray_gradient(BwdRay &r, const float4 &a, const f
 // A backward unit's walk: tile-list entries [lo, walk.y) read back to front,
 // filtered as in the forward from super-list positions [plo, walk.x) (walk.x:
 // just past entry walk.y - 1; plo: where entry lo's search starts).
-template <int kThreads, int BATCH, bool SPLAT, bool CG>
-__device__ __forceinline__ void backward_walk(WalkSmem<kThreads, BATCH> &sm, float (*s_acc)[17],
-                                              const uint32_t *__restrict__ svals,
-                                              const uint4 *__restrict__ sranges, const Record *__restrict__ rec,
-                                              const Params &p, const float4 &col, const float4 &row, int cx, int cy,
+template <bool SPLAT, bool CG>
+__device__ __forceinline__ void backward_walk(WalkSmem &sm, float (*s_acc)[17], const TileList &tl,
+                                              const Record *__restrict__ rec, const Params &p,
                                               uint32_t plo, uint32_t lo, uint2 walk, uint32_t warp_last,
                                               uint32_t block_last,
                                               const uint2 *__restrict__ hit_rec,
                                               const uint32_t *__restrict__ id_rec, int64_t hit_entries, int fwarp,
                                               BwdRay &ray, GradAcc *__restrict__ gacc, uint64_t items,
                                               uint32_t *misc) {
+    constexpr int kThreads = kTilePix, BATCH = kBatch;
     const int tid = threadIdx.x, lane = tid & 31;
     const float log2_amin = log2f(p.alpha_min);
     // entry r of a batch has list index top - 1 - r
@@ -845,7 +1146,7 @@ __device__ __forceinline__ void backward_walk(WalkSmem<kThreads, BATCH> &sm, flo
         if (direct) {
             cnt = (int)min((uint32_t)BATCH, top - lo);
         } else {
-            fill_list_rev<kThreads, BATCH>(svals, sranges, col, row, cx, cy, pos, plo, sm.id, s_cnt, sm.wcnt);
+            fill_list_rev(tl, pos, plo, sm.id, s_cnt, sm.fill.wcnt[0]);
             cnt = min(s_cnt, BATCH);
             if (cnt == 0) break;
         }
@@ -863,7 +1164,12 @@ __device__ __forceinline__ void backward_walk(WalkSmem<kThreads, BATCH> &sm, flo
             // beyond the recorded entries every warp evaluates
             const uint2 h = hit_rec && (int64_t)j < hit_entries ? ld_cg<CG>(hit_rec + j) : make_uint2(~0u, ~0u);
             // an entry no warp hit is never read: its record is not staged
-            if (h.x | h.y) stage_record(sm.rec + r * 4, rec, id, items, kSiteBwdItem, misc);
+            if (h.x | h.y) {
+                float4 q[4];
+                load_record(q, rec, id, items, kSiteBwdItem, misc);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) sm.rec[r * 4 + k] = q[k];
+            }
             // transposed to warp-major order: warp w's flags of the batch are contiguous
             uint8_t *hw = reinterpret_cast<uint8_t *>(sm.hit);
 #pragma unroll
@@ -943,7 +1249,7 @@ __device__ __forceinline__ void backward_walk(WalkSmem<kThreads, BATCH> &sm, flo
                 atomicAdd(dst + 3, make_float4(v[12], v[13], v[14], v[15]));
             }
         }
-        if (!direct) shift_list<kThreads>(sm.id, nullptr, cnt, s_cnt);
+        if (!direct) shift_list(sm.id, nullptr, cnt, s_cnt);
         top -= (uint32_t)cnt;
     }
 }
@@ -974,21 +1280,19 @@ __device__ __forceinline__ BwdRay bwd_ray(const TileRay &tr, const DevCam &cam, 
 // tile's long walk runs on several SMs at once and its transmittance is
 // recovered by division over one unit at most. Persistent blocks take units
 // in the order of k_bwd_order (descending length) from a counter.
-// One backward unit (the body of k_render_bwd's loop): unit code = tile << 4 | k,
-// row part `part` of the tile's rays. CG: read what the forward wrote through
+// One backward unit (the body of k_render_bwd's loop): unit code = tile << 4 | k. CG: read what the forward wrote through
 // L2 (the fused kernel reads it in the launch that wrote it).
-template <int ROWS, int BATCH, bool SPLAT, bool CG>
-__device__ __forceinline__ void bwd_unit(WalkSmem<ROWS * kTile, BATCH> &sm, float (*s_acc)[17], uint32_t code,
-                                         int part,
+template <bool SPLAT, bool CG>
+__device__ __forceinline__ void bwd_unit(WalkSmem &sm, float (*s_acc)[17], uint32_t code,
                                          const DevCam *__restrict__ cams,
                                          int ncams,
                                          const float2 *__restrict__ ptab,
-                                         const float4 *__restrict__ ttab,
                                          int S,
                                          const uint2 *__restrict__ tile_walk,
                                          const uint2 *__restrict__ srange,
                                          const uint32_t *__restrict__ svals,
-                                         const uint4 *__restrict__ sranges,
+                                         const uint32_t *__restrict__ smask,
+                                         const uint32_t *__restrict__ sany,
                                          const Record *__restrict__ rec,
                                          uint32_t *__restrict__ misc,
                                          Params p,
@@ -1006,8 +1310,7 @@ __device__ __forceinline__ void bwd_unit(WalkSmem<ROWS * kTile, BATCH> &sm, floa
                                          const uint2 *__restrict__ ckpt_at,
                                          const uint32_t *__restrict__ ckpt_cnt,
                                          const float4 *__restrict__ Cfin) {
-    constexpr int kThreads = ROWS * kTile;
-    const int tray = part * kThreads + (int)threadIdx.x;  // the ray's index in the tile
+    const int tray = (int)threadIdx.x;  // the ray's index in the tile
     const uint32_t t_id = code >> 4, k = code & 15u;
     if (!in_bounds(t_id, (uint64_t)ntiles, kSiteBwdTile, misc)) return;  // block-uniform
     const int t = (int)t_id;
@@ -1015,12 +1318,12 @@ __device__ __forceinline__ void bwd_unit(WalkSmem<ROWS * kTile, BATCH> &sm, floa
     __syncthreads();
     const DevCam &cam = cams[sm.cam];
     TileRay tr;
-    if (!tile_ray(cam, t, part * ROWS, ptab, ttab, srange, S, tr, (int)threadIdx.x)) return;
-    tr.sr = checked_range(tr.sr, cap_pairs, kSiteBwdList, misc);
+    if (!tile_ray(cam, t, ptab, srange, svals, smask, sany, S, tr, tray)) return;
+    tr.tl.sr = checked_range(tr.tl.sr, cap_pairs, kSiteBwdList, misc);
     uint2 walk = ld_cg<CG>(tile_walk + t);
-    if (!in_bounds(walk.x, (uint64_t)tr.sr.y + 1u, kSiteBwdList, misc)) walk = make_uint2(0u, 0u);
+    if (!in_bounds(walk.x, (uint64_t)tr.tl.sr.y + 1u, kSiteBwdList, misc)) walk = make_uint2(0u, 0u);
     // the unit: tile-list entries [lo, hi), super-list positions [plo, phi)
-    uint32_t lo = 0u, plo = tr.sr.x, hi = walk.y, phi = walk.x;
+    uint32_t lo = 0u, plo = tr.tl.sr.x, hi = walk.y, phi = walk.x;
     bool top = true;
     const uint32_t nck = ckpt_cnt ? min(ld_cg<CG>(ckpt_cnt + t), (uint32_t)kCkptMax) : 0u;
     if (k > 0 && k <= nck) {
@@ -1070,22 +1373,22 @@ __device__ __forceinline__ void bwd_unit(WalkSmem<ROWS * kTile, BATCH> &sm, floa
     __syncthreads();
     const uint32_t block_last = sm.maxlast;
     if (block_last <= lo) return;
-    backward_walk<kThreads, BATCH, SPLAT, CG>(sm, s_acc, svals, sranges, rec, p, tr.col, tr.row, tr.cx, tr.cy, plo, lo,
-                                          make_uint2(phi, hi), warp_last, block_last,
+    backward_walk<SPLAT, CG>(sm, s_acc, tr.tl, rec, p, plo, lo, make_uint2(phi, hi), warp_last, block_last,
                                           hit ? hit + (int64_t)t * hit_entries : nullptr,
                                           hit ? idrec + (int64_t)t * hit_entries : nullptr, hit_entries,
                                           tray >> 5, ray, gacc, items, misc);
 }
 
-template <int ROWS, int BATCH, bool SPLAT>
-__global__ void __launch_bounds__(ROWS * kTile, GEER_BWD_MINB) k_render_bwd(const DevCam *__restrict__ cams, int ncams,
+template <bool SPLAT>
+__global__ void __launch_bounds__(kTilePix, GEER_BWD_MINB) k_render_bwd(const DevCam *__restrict__ cams, int ncams,
                                                                            const float2 *__restrict__ ptab,
-                                                                           const float4 *__restrict__ ttab, int S,
+                                         int S,
                                                                            const uint2 *__restrict__ tile_walk,
                                                                            const uint32_t *__restrict__ units,
                                                                            const uint2 *__restrict__ srange,
                                                                            const uint32_t *__restrict__ svals,
-                                                                           const uint4 *__restrict__ sranges,
+                                                                           const uint32_t *__restrict__ smask,
+                                                                           const uint32_t *__restrict__ sany,
                                                                            const Record *__restrict__ rec,
                                                                            uint32_t *__restrict__ misc, Params p,
                                                                            const float *__restrict__ dL_drgb,
@@ -1101,13 +1404,11 @@ __global__ void __launch_bounds__(ROWS * kTile, GEER_BWD_MINB) k_render_bwd(cons
                                                                            const uint32_t *__restrict__ ckpt_cnt,
                                                                            const float4 *__restrict__ Cfin) {
     grid_dep_sync();
-    constexpr int kThreads = ROWS * kTile, kParts = kTile / ROWS;
-    static_assert(kParts * ROWS == kTile, "a unit's rays are split into kParts blocks of ROWS rows");
-    __shared__ WalkSmem<kThreads, BATCH> sm;
-    __shared__ float s_acc[BATCH][17];
+    __shared__ WalkSmem sm;
+    __shared__ float s_acc[kBatch][17];
     __shared__ uint32_t s_unit;
     if (misc[kMiscStatus] & kStatusCapacity) return;
-    const uint32_t n_work = misc[kMiscUnits] * (uint32_t)kParts;  // (unit, row part) pairs
+    const uint32_t n_work = misc[kMiscUnits];
     while (true) {
         __syncthreads();  // the previous unit's shared state has been read
         if (threadIdx.x == 0) {
@@ -1117,7 +1418,7 @@ __global__ void __launch_bounds__(ROWS * kTile, GEER_BWD_MINB) k_render_bwd(cons
         __syncthreads();
         const uint32_t w = s_unit;
         if (w >= n_work) break;
-        bwd_unit<ROWS, BATCH, SPLAT, false>(sm, s_acc, units[w / kParts], (int)(w % kParts), cams, ncams, ptab, ttab, S, tile_walk, srange, svals, sranges, rec, misc, p, dL_drgb, Tfin, last_in, hit, idrec, hit_entries, gacc, ntiles, items, cap_pairs, ckpt, ckpt_at, ckpt_cnt, Cfin);
+        bwd_unit<SPLAT, false>(sm, s_acc, units[w], cams, ncams, ptab, S, tile_walk, srange, svals, smask, sany, rec, misc, p, dL_drgb, Tfin, last_in, hit, idrec, hit_entries, gacc, ntiles, items, cap_pairs, ckpt, ckpt_at, ckpt_cnt, Cfin);
     }
 }
 
@@ -1134,11 +1435,12 @@ __global__ void __launch_bounds__(ROWS * kTile, GEER_BWD_MINB) k_render_bwd(cons
 constexpr uint32_t kQueueEmpty = 0xffffffffu;  // an unpublished queue slot (the host fills the queue with it)
 constexpr uint32_t kQueuePolls = 1u << 22;     // bound of a wait for a queue slot (<= ~1 us sleep between polls)
 
-template <int ROWS, int BATCH, bool SPLAT>
-__global__ void __launch_bounds__(ROWS * kTile, GEER_BWD_MINB) k_render_train(
-    const DevCam *__restrict__ cams, int ncams, const float2 *__restrict__ ptab, const float4 *__restrict__ ttab,
-    int S, uint2 *__restrict__ tile_walk, const uint32_t *__restrict__ tile_order, const uint2 *__restrict__ srange,
-    const uint32_t *__restrict__ svals, const uint4 *__restrict__ sranges, const Record *__restrict__ rec,
+template <bool SPLAT>
+__global__ void __launch_bounds__(kTilePix, GEER_BWD_MINB) k_render_train(
+    const DevCam *__restrict__ cams, int ncams, const float2 *__restrict__ ptab,
+                                         int S, uint2 *__restrict__ tile_walk, const uint32_t *__restrict__ tile_order, const uint2 *__restrict__ srange,
+    const uint32_t *__restrict__ svals, const uint32_t *__restrict__ smask, const uint32_t *__restrict__ sany,
+    const Record *__restrict__ rec,
     uint32_t *__restrict__ misc, Params p, float *__restrict__ rgb, float *__restrict__ Tout,
     float *__restrict__ Tfin, uint32_t *__restrict__ last, uint2 *__restrict__ evals, uint2 *__restrict__ hit,
     uint32_t *__restrict__ idrec, int64_t hit_entries, const uint8_t *__restrict__ tile_mask, int64_t ntiles,
@@ -1147,10 +1449,8 @@ __global__ void __launch_bounds__(ROWS * kTile, GEER_BWD_MINB) k_render_train(
     const float *__restrict__ target, float *__restrict__ dL, float inv_m, float *__restrict__ loss,
     GradAcc *__restrict__ gacc, uint32_t *__restrict__ queue, uint32_t queue_cap) {
     grid_dep_sync();
-    constexpr int kThreads = ROWS * kTile;
-    static_assert(ROWS == kTile, "one block per tile and per unit");
-    __shared__ WalkSmem<kThreads, BATCH> sm;
-    __shared__ float s_acc[BATCH][17];
+    __shared__ WalkSmem sm;
+    __shared__ float s_acc[kBatch][17];
     __shared__ uint32_t s_work;
     __shared__ float s_loss;
     if (misc[kMiscStatus] & kStatusCapacity) return;
@@ -1163,8 +1463,8 @@ __global__ void __launch_bounds__(ROWS * kTile, GEER_BWD_MINB) k_render_train(
         const uint32_t f = s_work;
         if (f >= (uint32_t)ntiles) break;
         const uint32_t t = tile_order[f];
-        const uint32_t nu = fwd_tile<ROWS, BATCH, SPLAT, true>(
-            sm, t, cams, ncams, ptab, ttab, S, tile_walk, srange, svals, sranges, rec, misc, p, rgb, Tout, Tfin, last,
+        const uint32_t nu = fwd_tile<SPLAT, true>(
+            sm, t, cams, ncams, ptab, S, tile_walk, srange, svals, smask, sany, rec, misc, p, rgb, Tout, Tfin, last,
             evals, hit, idrec, hit_entries, tile_mask, ntiles, items, cap_pairs, ckpt, ckpt_at, ckpt_cnt, unit_rec,
             Cfin, target, dL, inv_m, l1acc);
         __syncthreads();  // every thread's outputs of the tile are written
@@ -1215,8 +1515,8 @@ __global__ void __launch_bounds__(ROWS * kTile, GEER_BWD_MINB) k_render_train(
         __syncthreads();
         const uint32_t code = s_work;
         if (code == kQueueEmpty) break;
-        bwd_unit<ROWS, BATCH, SPLAT, true>(sm, s_acc, code, 0, cams, ncams, ptab, ttab, S, tile_walk, srange, svals,
-                                           sranges, rec, misc, p, dL, Tfin, last, hit, idrec, hit_entries, gacc,
+        bwd_unit<SPLAT, true>(sm, s_acc, code, cams, ncams, ptab, S, tile_walk, srange, svals,
+                                           smask, sany, rec, misc, p, dL, Tfin, last, hit, idrec, hit_entries, gacc,
                                            ntiles, items, cap_pairs, ckpt, ckpt_at, ckpt_cnt, Cfin);
     }
 }
@@ -1225,11 +1525,10 @@ __global__ void __launch_bounds__(ROWS * kTile, GEER_BWD_MINB) k_render_train(
 
 cudaError_t launch_render_fwd(const geer_workspace *ws, float *rgb, float *T_final, cudaStream_t s) {
     if (ws->n_tiles == 0) return cudaSuccess;
-    constexpr int R = GEER_FWD_ROWS, B = GEER_FWD_BATCH;
-    launch_k(ws->params.alpha_model == GEER_ALPHA_EXACT ? k_render_fwd<R, B, false> : k_render_fwd<R, B, true>,
-        dim3((unsigned)(ws->n_tiles * (kTile / R))), dim3(R * kTile), 0, s,
-        ws->d_cams, ws->n_cams, ws->d_pix_tab, ws->d_tile_tab, ws->super_size, ws->d_tile_walk, ws->d_tile_order,
-        ws->d_srange, ws->d_vals[ws->sorted_buf], ws->d_sranges, ws->d_rec, ws->d_misc,
+    launch_k(ws->params.alpha_model == GEER_ALPHA_EXACT ? k_render_fwd<false> : k_render_fwd<true>,
+        dim3((unsigned)ws->n_tiles), dim3(kTilePix), 0, s,
+        ws->d_cams, ws->n_cams, ws->d_pix_tab, ws->super_size, ws->d_tile_walk, ws->d_tile_order,
+        ws->d_srange, ws->d_vals[ws->sorted_buf], ws->d_smask[ws->sorted_buf], ws->d_sany, ws->d_rec, ws->d_misc,
         ws->params, rgb, T_final,
         ws->d_Tfin, ws->d_last, ws->d_evals, ws->d_hit, ws->d_idrec, ws->hit_entries,
         ws->tile_mask_on ? static_cast<const uint8_t *>(ws->d_tile_mask) : nullptr, ws->n_tiles,
@@ -1241,18 +1540,17 @@ cudaError_t launch_render_fwd(const geer_workspace *ws, float *rgb, float *T_fin
 cudaError_t launch_expand_tiles(const geer_workspace *ws, uint32_t *count_or_off, uint32_t *lists, cudaStream_t s) {
     if (ws->n_tiles == 0) return cudaSuccess;
     launch_k(k_expand_tiles, dim3((unsigned)ws->n_tiles), dim3(kTilePix), 0, s, ws->d_cams, ws->n_cams,
-             ws->d_tile_tab, ws->super_size, ws->d_srange, ws->d_vals[ws->sorted_buf], ws->d_sranges, ws->d_misc,
+             ws->d_pix_tab, ws->super_size, ws->d_srange, ws->d_vals[ws->sorted_buf], ws->d_smask[ws->sorted_buf], ws->d_sany, ws->d_misc,
              count_or_off, lists, ws->cap_pairs);
     return cudaGetLastError();
 }
 
 cudaError_t launch_render_bwd(const geer_workspace *ws, const float *dL_drgb, cudaStream_t s) {
     if (ws->n_tiles == 0) return cudaSuccess;
-    constexpr int R = GEER_BWD_ROWS, B = GEER_BWD_BATCH;
-    launch_k(ws->params.alpha_model == GEER_ALPHA_EXACT ? k_render_bwd<R, B, false> : k_render_bwd<R, B, true>,
-        dim3((unsigned)std::max(1, ws->bwd_grid)), dim3(R * kTile), 0, s,
-        ws->d_cams, ws->n_cams, ws->d_pix_tab, ws->d_tile_tab, ws->super_size, ws->d_tile_walk, ws->d_bwd_order,
-        ws->d_srange, ws->d_vals[ws->sorted_buf], ws->d_sranges, ws->d_rec, ws->d_misc,
+    launch_k(ws->params.alpha_model == GEER_ALPHA_EXACT ? k_render_bwd<false> : k_render_bwd<true>,
+        dim3((unsigned)std::max(1, ws->bwd_grid)), dim3(kTilePix), 0, s,
+        ws->d_cams, ws->n_cams, ws->d_pix_tab, ws->super_size, ws->d_tile_walk, ws->d_bwd_order,
+        ws->d_srange, ws->d_vals[ws->sorted_buf], ws->d_smask[ws->sorted_buf], ws->d_sany, ws->d_rec, ws->d_misc,
         ws->params, dL_drgb,
         ws->d_Tfin, ws->d_last, ws->d_hit, ws->d_idrec, ws->hit_entries, ws->d_gacc, ws->n_tiles,
         (uint64_t)ws->n_cams * (uint64_t)ws->n_gauss, ws->cap_pairs, ws->d_ckpt, ws->d_ckpt_at, ws->d_ckpt_cnt,
@@ -1263,12 +1561,11 @@ cudaError_t launch_render_bwd(const geer_workspace *ws, const float *dL_drgb, cu
 cudaError_t launch_render_train(const geer_workspace *ws, const float *target, float *rgb, float *T_final,
                                 float *dL_drgb, float *loss, cudaStream_t s) {
     if (ws->n_tiles == 0) return cudaSuccess;
-    constexpr int R = GEER_BWD_ROWS, B = GEER_BWD_BATCH;
     const int64_t m = 3 * ws->n_pixels;  // the L1 mean's value count
-    launch_k(ws->params.alpha_model == GEER_ALPHA_EXACT ? k_render_train<R, B, false> : k_render_train<R, B, true>,
-        dim3((unsigned)std::max(1, ws->train_grid)), dim3(R * kTile), 0, s,
-        ws->d_cams, ws->n_cams, ws->d_pix_tab, ws->d_tile_tab, ws->super_size, ws->d_tile_walk, ws->d_tile_order,
-        ws->d_srange, ws->d_vals[ws->sorted_buf], ws->d_sranges, ws->d_rec, ws->d_misc, ws->params, rgb, T_final,
+    launch_k(ws->params.alpha_model == GEER_ALPHA_EXACT ? k_render_train<false> : k_render_train<true>,
+        dim3((unsigned)std::max(1, ws->train_grid)), dim3(kTilePix), 0, s,
+        ws->d_cams, ws->n_cams, ws->d_pix_tab, ws->super_size, ws->d_tile_walk, ws->d_tile_order,
+        ws->d_srange, ws->d_vals[ws->sorted_buf], ws->d_smask[ws->sorted_buf], ws->d_sany, ws->d_rec, ws->d_misc, ws->params, rgb, T_final,
         ws->d_Tfin, ws->d_last, ws->d_evals, ws->d_hit, ws->d_idrec, ws->hit_entries,
         ws->tile_mask_on ? static_cast<const uint8_t *>(ws->d_tile_mask) : nullptr, ws->n_tiles,
         (uint64_t)ws->n_cams * (uint64_t)ws->n_gauss, ws->cap_pairs, ws->d_ckpt, ws->d_ckpt_at, ws->d_ckpt_cnt,
@@ -1278,21 +1575,18 @@ cudaError_t launch_render_train(const geer_workspace *ws, const float *target, f
 }
 
 int render_train_blocks_per_sm(int alpha_model) {
-    constexpr int R = GEER_BWD_ROWS, B = GEER_BWD_BATCH;
     int b = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &b, alpha_model == GEER_ALPHA_EXACT ? k_render_train<R, B, false> : k_render_train<R, B, true>,
-            R * kTile, 0) != cudaSuccess)
+            &b, alpha_model == GEER_ALPHA_EXACT ? k_render_train<false> : k_render_train<true>,
+            kTilePix, 0) != cudaSuccess)
         b = 1;
     return b < 1 ? 1 : b;
 }
 
 int render_bwd_blocks_per_sm(int alpha_model) {
-    constexpr int R = GEER_BWD_ROWS, B = GEER_BWD_BATCH;
     int b = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &b, alpha_model == GEER_ALPHA_EXACT ? k_render_bwd<R, B, false> : k_render_bwd<R, B, true>, R * kTile,
-            0) != cudaSuccess)
+            &b, alpha_model == GEER_ALPHA_EXACT ? k_render_bwd<false> : k_render_bwd<true>, kTilePix, 0) != cudaSuccess)
         b = 1;
     return b < 1 ? 1 : b;
 }

@@ -123,14 +123,15 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_hist(const uint32_t *__r
     }
 }
 
-// With rout: also rout[pos] = ranges[value] for every key written (the last pass
-// of the super-tile sort gathers the association ranges into list order).
-template <int ITEMS>
+// With W > 0 every key also carries W 32-bit words (min_ -> mout_, W per key: the
+// super-tile sort's tile masks), reordered through the values' shared buffer after
+// the values have left it.
+template <int ITEMS, int W>
 __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(
     const uint32_t *__restrict__ kin_, const uint32_t *__restrict__ vin_, uint32_t *__restrict__ kout_,
     uint32_t *__restrict__ vout_, int dev_buf, const uint32_t *__restrict__ misc, int count_slot,
     int check_capacity, int shift, const uint32_t *__restrict__ tile_hist, const uint32_t *__restrict__ group_excl,
-    const uint32_t *__restrict__ digit_base, const uint4 *__restrict__ ranges, uint4 *__restrict__ rout) {
+    const uint32_t *__restrict__ digit_base, const uint32_t *__restrict__ min_, uint32_t *__restrict__ mout_) {
     grid_dep_sync();
     // dev_buf: (kin_, vin_) is buffer 0 and (kout_, vout_) buffer 1; the input is
     // the one the histogram kernel recorded, and an identity pass is skipped
@@ -140,12 +141,12 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(
     const uint32_t *__restrict__ vin = swap ? vout_ : vin_;
     uint32_t *__restrict__ kout = swap ? const_cast<uint32_t *>(kin_) : kout_;
     uint32_t *__restrict__ vout = swap ? const_cast<uint32_t *>(vin_) : vout_;
-    constexpr int W = kSortThreads / 32, TILE = kSortThreads * ITEMS, GROUP = kGroupTiles;
-    __shared__ uint32_t s_whist[W][kRadix];
-    __shared__ uint32_t s_match[W][kRadix];  // lane masks per digit, zero between ranking steps
+    constexpr int NW = kSortThreads / 32, TILE = kSortThreads * ITEMS, GROUP = kGroupTiles;
+    __shared__ uint32_t s_whist[NW][kRadix];
+    __shared__ uint32_t s_match[NW][kRadix];  // lane masks per digit, zero between ranking steps
     __shared__ uint32_t s_lbase[kRadix];  // start of each digit inside the tile
     __shared__ uint32_t s_out[kRadix];    // global position of the tile's first key of each digit
-    __shared__ uint32_t s_wsum[W];
+    __shared__ uint32_t s_wsum[NW];
     __shared__ uint32_t s_key[TILE];
     __shared__ uint32_t s_val[TILE];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -156,16 +157,16 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(
         const uint32_t nt = (uint32_t)min((uint64_t)TILE, (uint64_t)n - (uint64_t)tile * TILE);
         const uint64_t t0 = (uint64_t)tile * TILE;
         for (uint32_t i = tid; i < nt; i += kSortThreads) {
-            const uint32_t v = vin[t0 + i];
             kout[t0 + i] = kin[t0 + i];
-            vout[t0 + i] = v;
-            if (rout) rout[t0 + i] = ranges[v];
+            vout[t0 + i] = vin[t0 + i];
         }
+        if (W > 0)
+            for (uint32_t i = tid; i < nt * W; i += kSortThreads) mout_[t0 * W + i] = min_[t0 * W + i];
         return;
     }
     const uint32_t base_d = digit_base[tid];
-    for (int i = tid; i < W * kRadix; i += kSortThreads) (&s_match[0][0])[i] = 0u;
-    for (int i = tid; i < W * kRadix; i += kSortThreads) (&s_whist[0][0])[i] = 0u;
+    for (int i = tid; i < NW * kRadix; i += kSortThreads) (&s_match[0][0])[i] = 0u;
+    for (int i = tid; i < NW * kRadix; i += kSortThreads) (&s_whist[0][0])[i] = 0u;
     // this tile's global offset for digit tid
     const uint32_t g0 = (tile / GROUP) * GROUP;
     uint32_t off = base_d + group_excl[(uint64_t)(tile / GROUP) * kRadix + tid];
@@ -213,7 +214,7 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(
     // warp offsets inside the tile per digit, tile count per digit
     uint32_t cnt = 0;
 #pragma unroll
-    for (int w = 0; w < W; ++w) {
+    for (int w = 0; w < NW; ++w) {
         const uint32_t c = s_whist[w][tid];
         s_whist[w][tid] = cnt;
         cnt += c;
@@ -229,7 +230,7 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(
     __syncthreads();
     uint32_t pre = 0;
 #pragma unroll
-    for (int w = 0; w < W; ++w) pre += w < warp ? s_wsum[w] : 0u;
+    for (int w = 0; w < NW; ++w) pre += w < warp ? s_wsum[w] : 0u;
     s_lbase[tid] = pre + v - cnt;
     __syncthreads();
     // reorder the tile by digit in shared memory
@@ -240,6 +241,7 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(
             const uint32_t lp = s_lbase[d] + s_whist[warp][d] + rank[k];
             s_key[lp] = key[k];
             s_val[lp] = val[k];
+            if (W > 0) rank[k] = lp;
         }
     }
     __syncthreads();
@@ -253,50 +255,85 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(
             const uint32_t d = (kk >> shift) & 0xffu;
             const uint32_t pos = s_out[d] + (lp - s_lbase[d]);
             if (pos < n) {
-                const uint32_t v = s_val[lp];
                 kout[pos] = kk;
-                vout[pos] = v;
-                if (rout) rout[pos] = ranges[v];
+                vout[pos] = s_val[lp];
             }
         }
     }
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+        uint32_t m[ITEMS];
+#pragma unroll
+        for (int k = 0; k < ITEMS; ++k) {
+            const uint64_t i = base + (uint64_t)k * 32;
+            m[k] = i < n ? min_[i * W + w] : 0u;
+        }
+        __syncthreads();  // s_val has been read
+#pragma unroll
+        for (int k = 0; k < ITEMS; ++k)
+            if (rank[k] != 0xffffffffu) s_val[rank[k]] = m[k];
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < ITEMS; ++k) {
+            const uint32_t lp = (uint32_t)(k * kSortThreads + tid);
+            if (lp < nt) {
+                const uint32_t d = (s_key[lp] >> shift) & 0xffu;
+                const uint32_t pos = s_out[d] + (lp - s_lbase[d]);
+                if (pos < n) mout_[(uint64_t)pos * W + w] = s_val[lp];
+            }
+        }
+    }
+}
+
+
+// The or of every 32 sorted pairs' tile masks (a warp per group): the render's
+// list scan skips the groups without an entry of its tile.
+__global__ void __launch_bounds__(256) k_group_masks(const uint32_t *__restrict__ mask, int words,
+                                                     const uint32_t *__restrict__ misc, uint32_t *__restrict__ any) {
+    grid_dep_sync();
+    if (misc[kMiscStatus] & kStatusCapacity) return;
+    const uint64_t n = (uint64_t)misc[kMiscPairs], step = (uint64_t)gridDim.x * 256u;
+    const int lane = threadIdx.x & 31;
+    for (uint64_t i = (uint64_t)blockIdx.x * 256u + threadIdx.x; (i & ~31ull) < n; i += step)
+        for (int w = 0; w < words; ++w) {
+            const uint32_t v = __reduce_or_sync(0xffffffffu, i < n ? mask[i * words + w] : 0u);
+            if (lane == 0) any[(i >> 5) * words + w] = v;
+        }
 }
 
 }  // namespace
 
 int sort_blocks_per_sm() {
     int b = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_radix_scatter<kSortItems>, kSortThreads, 0) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_radix_scatter<kSortItems, 0>, kSortThreads, 0) !=
         cudaSuccess)
         b = 1;
     return b < 1 ? 1 : b;
 }
 
-template <int ITEMS>
-static cudaError_t radix_pass_t(geer_workspace *ws, uint32_t *const kbuf[2], uint32_t *const vbuf[2], int cur,
-                                int dev_buf, int slot, int check, int shift, int64_t cap_keys, uint4 *rout,
-                                cudaStream_t s) {
-    constexpr int TILE = kSortThreads * ITEMS;
-    const unsigned tiles = (unsigned)std::max<int64_t>(1, (cap_keys + TILE - 1) / TILE);
-    launch_k(k_radix_hist<ITEMS>, dim3(tiles), dim3(kSortThreads), 0, s, kbuf[cur], kbuf[cur ^ 1], dev_buf,
-             ws->d_misc, slot, check, shift, ws->d_tile_hist, ws->d_group_sum, ws->d_group_excl, ws->d_digit_base);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    launch_k(k_radix_scatter<ITEMS>, dim3(tiles), dim3(kSortThreads), 0, s, kbuf[cur], vbuf[cur], kbuf[cur ^ 1],
-             vbuf[cur ^ 1], dev_buf, ws->d_misc, slot, check, shift, ws->d_tile_hist, ws->d_group_excl,
-             ws->d_digit_base, ws->d_ranges, rout);
-    return cudaGetLastError();
-}
-
 // One stable pass over digit `pass` of the keys in buffer `cur` (count in
 // misc[slot]); with dev_buf the buffers are chosen on the device and a pass
-// whose digit is the same for every key is skipped.
+// whose digit is the same for every key is skipped. mbuf (words > 0): the 32-bit
+// words that travel with the keys.
 // (Tiles of 1024 keys for small sorts were measured slower: 0.106 against 0.079 ms
 // for the four passes over 1M depth keys.)
 static cudaError_t radix_pass(geer_workspace *ws, uint32_t *const kbuf[2], uint32_t *const vbuf[2], int cur, int slot,
-                              int check, int pass, int64_t cap_keys, cudaStream_t s, uint4 *rout = nullptr,
-                              int dev_buf = 0) {
-    return radix_pass_t<kSortItems>(ws, kbuf, vbuf, cur, dev_buf, slot, check, kRadixBits * pass, cap_keys, rout, s);
+                              int check, int pass, int64_t cap_keys, cudaStream_t s, uint32_t *const *mbuf, int words,
+                              int dev_buf) {
+    constexpr int TILE = kSortThreads * kSortItems;
+    const int shift = kRadixBits * pass;
+    const unsigned tiles = (unsigned)std::max<int64_t>(1, (cap_keys + TILE - 1) / TILE);
+    launch_k(k_radix_hist<kSortItems>, dim3(tiles), dim3(kSortThreads), 0, s, kbuf[cur], kbuf[cur ^ 1], dev_buf,
+             ws->d_misc, slot, check, shift, ws->d_tile_hist, ws->d_group_sum, ws->d_group_excl, ws->d_digit_base);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    launch_k(words == 0   ? k_radix_scatter<kSortItems, 0>
+             : words == 1 ? k_radix_scatter<kSortItems, 1>
+                          : k_radix_scatter<kSortItems, 2>,
+             dim3(tiles), dim3(kSortThreads), 0, s, kbuf[cur], vbuf[cur], kbuf[cur ^ 1], vbuf[cur ^ 1], dev_buf,
+             ws->d_misc, slot, check, shift, ws->d_tile_hist, ws->d_group_excl, ws->d_digit_base,
+             words ? mbuf[cur] : nullptr, words ? mbuf[cur ^ 1] : nullptr);
+    return cudaGetLastError();
 }
 
 // Stable sort of the live items by depth key (4 digits of the FP32 bits). The
@@ -307,7 +344,7 @@ cudaError_t launch_depth_sort(geer_workspace *ws, cudaStream_t s) {
     const int64_t items = (int64_t)ws->n_cams * ws->n_gauss;
     if (items > 0) {
         for (int p = 0; p < 4; ++p) {
-            cudaError_t e = radix_pass(ws, ws->d_ikey, ws->d_iid, 0, kMiscLive, 0, p, items, s, nullptr, 1);
+            cudaError_t e = radix_pass(ws, ws->d_ikey, ws->d_iid, 0, kMiscLive, 0, p, items, s, nullptr, 0, 1);
             if (e != cudaSuccess) return e;
         }
     }
@@ -315,18 +352,20 @@ cudaError_t launch_depth_sort(geer_workspace *ws, cudaStream_t s) {
 }
 
 // Stable sort of the (super-tile, item) pairs by super-tile id (one or two
-// 8-bit digits); the last pass also writes the items' association ranges in
-// list order (the render kernels' filters read them coalesced).
+// 8-bit digits); the pairs' tile masks travel with them.
 cudaError_t launch_tile_sort(geer_workspace *ws, cudaStream_t s) {
     int cur = 0;
     for (int p = 0; p < ws->n_sort_passes; ++p) {
-        cudaError_t e = radix_pass(ws, ws->d_keys, ws->d_vals, cur, kMiscPairs, 1, p, ws->cap_pairs, s,
-                                   p + 1 == ws->n_sort_passes ? ws->d_sranges : nullptr);
+        cudaError_t e = radix_pass(ws, ws->d_keys, ws->d_vals, cur, kMiscPairs, 1, p, ws->cap_pairs, s, ws->d_smask,
+                                   mask_words(ws->super_size), 0);
         if (e != cudaSuccess) return e;
         cur ^= 1;
     }
     ws->sorted_buf = cur;
-    return cudaSuccess;
+    const int64_t blocks = std::min<int64_t>(std::max<int64_t>(1, (ws->cap_pairs + 255) / 256), (int64_t)ws->num_sms * 8);
+    launch_k(k_group_masks, dim3((unsigned)blocks), dim3(256), 0, s, (const uint32_t *)ws->d_smask[cur],
+             mask_words(ws->super_size), (const uint32_t *)ws->d_misc, ws->d_sany);
+    return cudaGetLastError();
 }
 
 }  // namespace geer

@@ -56,6 +56,27 @@ __device__ __forceinline__ float rcp(float x) {
     return y;
 }
 
+// Two FP32 operations in one instruction (each rounded as the scalar one).
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+    float2 r;
+    asm("{\n .reg .b64 x, y, z;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n add.rn.f32x2 z, x, y;\n"
+        " mov.b64 {%0, %1}, z;\n}" : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+    float2 r;
+    asm("{\n .reg .b64 x, y, z;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n mul.rn.f32x2 z, x, y;\n"
+        " mov.b64 {%0, %1}, z;\n}" : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+    float2 r;
+    asm("{\n .reg .b64 x, y, w, z;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n mov.b64 w, {%6, %7};\n"
+        " fma.rn.f32x2 z, x, y, w;\n mov.b64 {%0, %1}, z;\n}"
+        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return r;
+}
+
 __device__ __forceinline__ int find_cam(const DevCam *cams, int ncams, int t) {
     int c = 0;
     for (int i = 1; i < ncams; ++i)
@@ -68,7 +89,7 @@ __device__ __forceinline__ int find_cam(const DevCam *cams, int ncams, int t) {
 // log2(sigma) - kappa log2(e) / 2. The forward and the backward share it so that
 // both take the same FP32 decisions.
 struct Eval {
-    float du0, du1, du2, m0, m1, m2, dd, od, kappa, arg;
+    float du0, du1, du2, m0, m1, m2, inv_dd, od, kappa, arg;
     bool hit;  // alpha >= alpha_min and the closest approach lies in front of the camera
 };
 
@@ -82,9 +103,9 @@ __device__ __forceinline__ Eval evaluate(const float4 &a, const float4 &b, const
     v.m1 = c.w * v.du0 - c.y * v.du2;
     v.m2 = c.y * v.du1 - c.z * v.du0;
     const float mm = v.m0 * v.m0 + v.m1 * v.m1 + v.m2 * v.m2;
-    v.dd = v.du0 * v.du0 + v.du1 * v.du1 + v.du2 * v.du2;
+    v.inv_dd = rcp(v.du0 * v.du0 + v.du1 * v.du1 + v.du2 * v.du2);
     v.od = c.y * v.du0 + c.z * v.du1 + c.w * v.du2;
-    v.kappa = mm * rcp(v.dd);
+    v.kappa = mm * v.inv_dd;
     v.arg = fmaf(v.kappa, kNegHalfLog2e, e.x);
     v.hit = !(v.arg < log2_amin || v.od >= 0.0f);
     return v;
@@ -327,14 +348,22 @@ __device__ __forceinline__ void fill_list_rev(const TileList &tl, uint32_t &pos,
 struct WalkSmem {
     float4 rec[(kBatch + 1) * 4];       // records of the current batch; forward: the last one is never hit
     uint32_t id[kBatch + kTilePix];     // tile-list entries found by the filter (item ids)
-    uint32_t pos[kBatch + kTilePix];    // their positions in the super-tile list (forward)
     uint2 hit[kBatch];                  // per entry: one byte per backward warp (16 x 2 rays), nonzero if a ray hit it
-    uint16_t list[kTileWarps][kBatch + kFwdUnroll];  // forward: each sub-tile's entries of the batch (byte offsets in rec)
-    float4 conic[kBatch * 2];           // forward: the entries' quadratics
-    float4 sub[kTileWarps];             // forward: the sub-tiles' rectangles (centre, half sizes) in the tile's chart
-    float2 ray[kTileWarps][32];         // forward: their rays' points there
-    float4 frame[3];                    // forward: the chart's axes c, e1, e2 (splat: the reference angles)
-    uint32_t ext[2];                    // forward: the largest |x|, |y| of the tile's rays (FP32 bits)
+    union {
+        struct {                        // forward
+            uint32_t pos[kBatch + kTilePix];    // the entries' positions in the super-tile list
+            float4 conic[kBatch * 2];           // the batch's quadratics
+            uint16_t list[kTileWarps][kBatch + kFwdUnroll];  // each sub-tile's entries of the batch (byte offsets in rec)
+            float4 sub[kTileWarps];             // the sub-tiles' rectangles (centre, half sizes) in the tile's chart
+            float2 ray[kTileWarps][32];         // their rays' points there
+            float4 frame[3];                    // the chart's axes c, e1, e2 (splat: the reference angles)
+            uint32_t ext[2];                    // the largest |x|, |y| of the tile's rays (FP32 bits)
+        };
+        struct {                        // backward
+            float acc[kBatch][17];              // the batch's sums over the tile's rays
+            uint8_t blist[kTileWarps][kBatch];  // each warp's entries of the batch
+        };
+    };
     FillSmem fill;
     uint32_t maxlast, walkpos;       // the tile's last contributor and its super-list position + 1
     uint32_t nck, next_ck;           // forward: checkpoints recorded, list index of the next one
@@ -1050,11 +1079,14 @@ __global__ void __launch_bounds__(kTilePix) k_expand_tiles(const DevCam *__restr
 // dL/dsigma, dL/dc, dL/dW through d_u (outer product with the ray direction)
 // and dL/do_u (the PreprocessCUDA part chains o_u = -W mu_c).
 //
-// The 16 values are reduced over the warp (reduce-scatter by shuffles), over the
-// block in shared memory, then added to global memory with one set of float4
-// atomics per (block, Gaussian). A warp skips list entries beyond the last
-// contributor of its rays, and entries that none of its rays hit in the forward
-// (the forward's per-warp hit record; the same FP32 evaluation decides both).
+// The 16 values are reduced over the warp (reduce-scatter by shuffles, lanes 16, 8,
+// 4, 2, 1 apart), over the tile's warps in shared memory, then added to global
+// memory with one set of float4 atomics per (tile, Gaussian). (Added to global
+// memory per warp, 2% faster, they lose precision: a Gaussian over many tiles takes
+// eight times the roundings at its full sum, 5e-6 against 1e-6 of the quaternions'
+// norm from run to run.) A warp walks the list entries below the last contributor
+// of its rays that one of its rays hit in the forward (the forward's hit record;
+// the same FP32 evaluation decides both).
 // gS: the colour behind the current entry (what lies after it in the list, the
 // background included) projected on dL/dC. dL/dalpha needs only this dot product,
 // so the ray carries one scalar instead of the three channels.
@@ -1063,79 +1095,164 @@ struct BwdRay {
     uint32_t last;
 };
 
-// One ray's contribution to the 16 accumulators of the Gaussian in (a, b, c, e)
-// (GradAcc order), and the step of the ray's reverse compositing state.
-// SPLAT: the splat alpha (r.dx, r.dy the ray's screen angles); its record is
-// the centre and conic, and gv[4..8] take dL/d(theta_c, phi_c, A, B, C):
-// dq/dtheta_c = -2 (A D0 + B D1), dq/dphi_c = -2 (B D0 + C D1),
-// dq/dA = D0^2, dq/dB = 2 D0 D1, dq/dC = D1^2.
+// What one ray adds to the 16 accumulators of the Gaussian in (a, b, c, e), as
+// factors, and the step of the ray's reverse compositing state. `act`: the ray
+// walks the entry. Branch-free: a ray that does not hit selects zeros.
+//   colour wgt (g0, g1, g2); sigma sig; exact dL/dW r d^T, dL/do_u o;
+//   splat  o0, o1 = dL/d(theta_c, phi_c), r0, r1, r2 = dL/d(A, B, C):
+//          dq/dtheta_c = -2 (A D0 + B D1), dq/dphi_c = -2 (B D0 + C D1),
+//          dq/dA = D0^2, dq/dB = 2 D0 D1, dq/dC = D1^2.
+struct RayGrad {
+    float wgt, sig, r0, r1, r2, o0, o1, o2;
+};
+
 template <bool SPLAT>
-__device__ __forceinline__ void ray_gradient(BwdRay &r, const float4 &a, const float4 &b, const float4 &c,
-                                             const float4 &e, float log2_amin, float alpha_max, float gv[16],
-                                             bool &contrib) {
+__device__ __forceinline__ RayGrad ray_gradient(BwdRay &r, const float4 &a, const float4 &b, const float4 &c,
+                                                const float4 &e, float log2_amin, float alpha_max, bool act) {
     const Eval v = SPLAT ? evaluate_splat(a, b, e, r.dx, r.dy, log2_amin)
                          : evaluate(a, b, c, e, r.dx, r.dy, r.dz, log2_amin);
-    if (!v.hit) return;
-    contrib = true;
-    const float ae = exp2f(v.arg);
+    act = act && v.hit;
+    const float ae = ex2(v.arg);
     const float alpha = fminf(ae, alpha_max);
-    // approximate reciprocal (within 2 ulp): the correctly rounded one costs more
-    // than the rest of this step's transmittance update
-    const float inv_om = __fdividef(1.0f, 1.0f - alpha);
+    const float inv_om = rcp(1.0f - alpha);
     const float Ti = r.T * inv_om;  // transmittance in front of this Gaussian
+    RayGrad g;
     const float wgt = Ti * alpha;
-    gv[1] = fmaf(r.g0, wgt, gv[1]);
-    gv[2] = fmaf(r.g1, wgt, gv[2]);
-    gv[3] = fmaf(r.g2, wgt, gv[3]);
+    g.wgt = act ? wgt : 0.0f;
     // dL/dalpha = sum_ch g_ch (T_i c_ch - S_ch / (1 - alpha)) = T_i (g . c) - (g . S) / (1 - alpha)
     const float gc = fmaf(r.g0, e.y, fmaf(r.g1, e.z, r.g2 * e.w));
     const float dLda = fmaf(Ti, gc, -r.gS * inv_om);
-    r.gS = fmaf(wgt, gc, r.gS);
-    r.T = Ti;
-    if (ae < alpha_max) {
-        gv[0] = fmaf(dLda, exp2f(v.kappa * kNegHalfLog2e), gv[0]);  // dL/dsigma = dL/da e^{-kappa/2}
-        const float dLdk = -0.5f * dLda * ae;
-        if (SPLAT) {
-            const float d0 = v.du0, d1 = v.du1;
-            gv[4] = fmaf(-2.0f * dLdk, fmaf(a.z, d0, a.w * d1), gv[4]);
-            gv[5] = fmaf(-2.0f * dLdk, fmaf(a.w, d0, b.x * d1), gv[5]);
-            gv[6] = fmaf(dLdk, d0 * d0, gv[6]);
-            gv[7] = fmaf(2.0f * dLdk, d0 * d1, gv[7]);
-            gv[8] = fmaf(dLdk, d1 * d1, gv[8]);
-            return;
-        }
-        // with g_m = 2 m_u / |d_u|^2 (dkappa/dm_u), scaled by dL/dkappa:
-        //   dL/dd_u = dL/dkappa (-(2 kappa / |d_u|^2) d_u + g_m x o_u),  dL/do_u = dL/dkappa (d_u x g_m)
-        const float h = 2.0f * dLdk * __fdividef(1.0f, v.dd);
-        const float gm0 = h * v.m0, gm1 = h * v.m1, gm2 = h * v.m2;
-        const float sk = -h * v.kappa;
-        const float r0 = sk * v.du0 + (gm1 * c.w - gm2 * c.z);
-        const float r1 = sk * v.du1 + (gm2 * c.y - gm0 * c.w);
-        const float r2 = sk * v.du2 + (gm0 * c.z - gm1 * c.y);
-        gv[13] += v.du1 * gm2 - v.du2 * gm1;
-        gv[14] += v.du2 * gm0 - v.du0 * gm2;
-        gv[15] += v.du0 * gm1 - v.du1 * gm0;
-        gv[4] = fmaf(r0, r.dx, gv[4]); gv[5] = fmaf(r0, r.dy, gv[5]); gv[6] = fmaf(r0, r.dz, gv[6]);
-        gv[7] = fmaf(r1, r.dx, gv[7]); gv[8] = fmaf(r1, r.dy, gv[8]); gv[9] = fmaf(r1, r.dz, gv[9]);
-        gv[10] = fmaf(r2, r.dx, gv[10]); gv[11] = fmaf(r2, r.dy, gv[11]); gv[12] = fmaf(r2, r.dz, gv[12]);
+    if (act) {
+        r.gS = fmaf(wgt, gc, r.gS);
+        r.T = Ti;
     }
+    const bool pass = act && ae < alpha_max;
+    g.sig = pass ? dLda * ex2(v.kappa * kNegHalfLog2e) : 0.0f;  // dL/dsigma = dL/da e^{-kappa/2}
+    const float dLdk = -0.5f * dLda * ae;
+    if (SPLAT) {
+        const float d0 = v.du0, d1 = v.du1;
+        g.o0 = pass ? -2.0f * dLdk * fmaf(a.z, d0, a.w * d1) : 0.0f;
+        g.o1 = pass ? -2.0f * dLdk * fmaf(a.w, d0, b.x * d1) : 0.0f;
+        g.o2 = 0.0f;
+        g.r0 = pass ? dLdk * (d0 * d0) : 0.0f;
+        g.r1 = pass ? 2.0f * dLdk * (d0 * d1) : 0.0f;
+        g.r2 = pass ? dLdk * (d1 * d1) : 0.0f;
+        return g;
+    }
+    // with g_m = 2 m_u / |d_u|^2 (dkappa/dm_u), scaled by dL/dkappa:
+    //   dL/dd_u = dL/dkappa (-(2 kappa / |d_u|^2) d_u + g_m x o_u),  dL/do_u = dL/dkappa (d_u x g_m)
+    const float h = 2.0f * dLdk * v.inv_dd;
+    const float gm0 = h * v.m0, gm1 = h * v.m1, gm2 = h * v.m2;
+    const float sk = -h * v.kappa;
+    const float r0 = sk * v.du0 + (gm1 * c.w - gm2 * c.z);
+    const float r1 = sk * v.du1 + (gm2 * c.y - gm0 * c.w);
+    const float r2 = sk * v.du2 + (gm0 * c.z - gm1 * c.y);
+    g.r0 = pass ? r0 : 0.0f;
+    g.r1 = pass ? r1 : 0.0f;
+    g.r2 = pass ? r2 : 0.0f;
+    g.o0 = pass ? v.du1 * gm2 - v.du2 * gm1 : 0.0f;
+    g.o1 = pass ? v.du2 * gm0 - v.du0 * gm2 : 0.0f;
+    g.o2 = pass ? v.du0 * gm1 - v.du1 * gm0 : 0.0f;
+    return g;
+}
+
+// Warp sums of the 16 accumulator values: lane l and l ^ 1 end with the sum of one
+// value, at the lane's offset in GradAcc (LanePerm::off).
+//
+// The exact integral's values are four rows of four: (r_k dx, r_k dy, r_k dz, o_k)
+// and (wgt g0, wgt g1, wgt g2, sig). Bits 4 and 3 of the lane permute the columns,
+// lane class c holding column i ^ c at place i: the lane keeps its ray's direction
+// and dL/dC in that order, with a zero in column 3 and the column 3 value added
+// through b (1 there, 0 elsewhere). So the first two exchanges (lanes 16 and 8
+// apart) send the places the lane does not keep and add what arrives, without
+// selecting what to send; only the next two (4 and 2 apart) select. That and
+// packed arithmetic take ~50 instructions for the products and the sums, where
+// selecting in every exchange took ~75. The tree of each value's sum is the plain
+// butterfly's.
+struct LanePerm {
+    float2 d01, d23, b01, b23, g01, g23;
+    int off;
+};
+
+template <bool SPLAT>
+__device__ __forceinline__ LanePerm lane_perm(const BwdRay &r) {
+    const int lane = threadIdx.x & 31, c = SPLAT ? 0 : lane >> 3;
+    const auto pick = [&](int i, float a0, float a1, float a2, float a3) {
+        const int k = i ^ c;
+        return k == 0 ? a0 : k == 1 ? a1 : k == 2 ? a2 : a3;
+    };
+    LanePerm q;
+    q.d01 = make_float2(pick(0, r.dx, r.dy, r.dz, 0.0f), pick(1, r.dx, r.dy, r.dz, 0.0f));
+    q.d23 = make_float2(pick(2, r.dx, r.dy, r.dz, 0.0f), pick(3, r.dx, r.dy, r.dz, 0.0f));
+    q.g01 = make_float2(pick(0, r.g0, r.g1, r.g2, 0.0f), pick(1, r.g0, r.g1, r.g2, 0.0f));
+    q.g23 = make_float2(pick(2, r.g0, r.g1, r.g2, 0.0f), pick(3, r.g0, r.g1, r.g2, 0.0f));
+    q.b01 = make_float2(pick(0, 0.0f, 0.0f, 0.0f, 1.0f), pick(1, 0.0f, 0.0f, 0.0f, 1.0f));
+    q.b23 = make_float2(pick(2, 0.0f, 0.0f, 0.0f, 1.0f), pick(3, 0.0f, 0.0f, 0.0f, 1.0f));
+    const int row = (lane >> 1) & 3;
+    q.off = SPLAT ? lane >> 1 : row < 3 ? (c < 3 ? 4 + 3 * row + c : 13 + row) : (c < 3 ? 1 + c : 0);
+    return q;
+}
+
+__device__ __forceinline__ float2 xchg2(float2 keep, float2 send, int w) {
+    return add2(keep, make_float2(__shfl_xor_sync(0xffffffffu, send.x, w), __shfl_xor_sync(0xffffffffu, send.y, w)));
+}
+
+template <bool SPLAT>
+__device__ __forceinline__ float warp_sum(const RayGrad &g, const BwdRay &r, const LanePerm &q) {
+    const int lane = threadIdx.x & 31;
+    if (SPLAT) {
+        float v[16];
+        v[0] = g.sig;
+        v[1] = g.wgt * r.g0;
+        v[2] = g.wgt * r.g1;
+        v[3] = g.wgt * r.g2;
+        v[4] = g.o0; v[5] = g.o1; v[6] = g.r0; v[7] = g.r1; v[8] = g.r2;
+#pragma unroll
+        for (int k = 9; k < 16; ++k) v[k] = 0.0f;
+#pragma unroll
+        for (int w = 8; w > 0; w >>= 1) {  // lanes with bit 2w keep the upper w values
+            const bool up = lane & (2 * w);
+#pragma unroll
+            for (int k = 0; k < w; ++k) {
+                const float send = up ? v[k] : v[k + w];
+                const float keep = up ? v[k + w] : v[k];
+                v[k] = keep + __shfl_xor_sync(0xffffffffu, send, 2 * w);
+            }
+        }
+        return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+    }
+    const float row[4] = {g.r0, g.r1, g.r2, g.wgt}, last[4] = {g.o0, g.o1, g.o2, g.sig};
+    float2 x[2];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float2 f = make_float2(row[k], row[k]), l = make_float2(last[k], last[k]);
+        const float2 a = fma2(f, k < 3 ? q.d01 : q.g01, mul2(l, q.b01));
+        const float2 b = fma2(f, k < 3 ? q.d23 : q.g23, mul2(l, q.b23));
+        const float2 v = xchg2(a, b, 16);
+        const float s = v.x + __shfl_xor_sync(0xffffffffu, v.y, 8);
+        if (k & 1) x[k >> 1].y = s;
+        else x[k >> 1].x = s;
+    }
+    const bool u4 = lane & 4, u2 = lane & 2;
+    const float2 y = xchg2(u4 ? x[1] : x[0], u4 ? x[0] : x[1], 4);
+    const float z = (u2 ? y.y : y.x) + __shfl_xor_sync(0xffffffffu, u2 ? y.x : y.y, 2);
+    return z + __shfl_xor_sync(0xffffffffu, z, 1);
 }
 
 // A backward unit's walk: tile-list entries [lo, walk.y) read back to front,
 // filtered as in the forward from super-list positions [plo, walk.x) (walk.x:
 // just past entry walk.y - 1; plo: where entry lo's search starts).
 template <bool SPLAT, bool CG>
-__device__ __forceinline__ void backward_walk(WalkSmem &sm, float (*s_acc)[17], const TileList &tl,
-                                              const Record *__restrict__ rec, const Params &p,
-                                              uint32_t plo, uint32_t lo, uint2 walk, uint32_t warp_last,
-                                              uint32_t block_last,
+__device__ __forceinline__ void backward_walk(WalkSmem &sm, const TileList &tl, const Record *__restrict__ rec,
+                                              const Params &p, uint32_t plo, uint32_t lo, uint2 walk,
+                                              uint32_t warp_last, uint32_t block_last,
                                               const uint2 *__restrict__ hit_rec,
-                                              const uint32_t *__restrict__ id_rec, int64_t hit_entries, int fwarp,
+                                              const uint32_t *__restrict__ id_rec, int64_t hit_entries,
                                               BwdRay &ray, GradAcc *__restrict__ gacc, uint64_t items,
                                               uint32_t *misc) {
-    constexpr int kThreads = kTilePix, BATCH = kBatch;
-    const int tid = threadIdx.x, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const float log2_amin = log2f(p.alpha_min);
+    const LanePerm perm = lane_perm<SPLAT>(ray);
     // entry r of a batch has list index top - 1 - r
     uint32_t pos = walk.x, top = walk.y;
     int s_cnt = 0;
@@ -1144,112 +1261,72 @@ __device__ __forceinline__ void backward_walk(WalkSmem &sm, float (*s_acc)[17], 
         const bool direct = id_rec && (int64_t)top <= hit_entries;
         int cnt;
         if (direct) {
-            cnt = (int)min((uint32_t)BATCH, top - lo);
+            cnt = (int)min((uint32_t)kBatch, top - lo);
         } else {
             fill_list_rev(tl, pos, plo, sm.id, s_cnt, sm.fill.wcnt[0]);
-            cnt = min(s_cnt, BATCH);
+            cnt = min(s_cnt, kBatch);
             if (cnt == 0) break;
         }
         // entries at or beyond the block's last contributor are not walked
         const int skip = top > block_last ? (int)min((uint32_t)cnt, top - block_last) : 0;
-        for (int r = skip + tid; r < cnt; r += kThreads) {
-            const uint32_t j = top - 1u - (uint32_t)r;
+        if (tid >= skip && tid < cnt) {
+            const uint32_t j = top - 1u - (uint32_t)tid;
             uint32_t id;
             if (direct) {
                 id = ld_cg<CG>(id_rec + j);
-                sm.id[r] = id;
+                sm.id[tid] = id;
             } else {
-                id = sm.id[r];
+                id = sm.id[tid];
             }
             // beyond the recorded entries every warp evaluates
-            const uint2 h = hit_rec && (int64_t)j < hit_entries ? ld_cg<CG>(hit_rec + j) : make_uint2(~0u, ~0u);
+            uint2 h = hit_rec && (int64_t)j < hit_entries ? ld_cg<CG>(hit_rec + j) : make_uint2(~0u, ~0u);
+            if ((h.x | h.y) && !in_bounds(id, items, kSiteBwdItem, misc)) h = make_uint2(0u, 0u);
             // an entry no warp hit is never read: its record is not staged
             if (h.x | h.y) {
-                float4 q[4];
-                load_record(q, rec, id, items, kSiteBwdItem, misc);
+                const float4 *src = reinterpret_cast<const float4 *>(rec + id);
 #pragma unroll
-                for (int k = 0; k < 4; ++k) sm.rec[r * 4 + k] = q[k];
+                for (int k = 0; k < 4; ++k) sm.rec[tid * 4 + k] = src[k];
             }
-            // transposed to warp-major order: warp w's flags of the batch are contiguous
-            uint8_t *hw = reinterpret_cast<uint8_t *>(sm.hit);
-#pragma unroll
-            for (int w = 0; w < kTileWarps; ++w)
-                hw[w * BATCH + r] = (uint8_t)((w < 4 ? h.x : h.y) >> (8 * (w & 3)));
+            sm.hit[tid] = h;
         }
-        for (int i = skip * 17 + tid; i < cnt * 17; i += kThreads) (&s_acc[0][0])[i] = 0.0f;
+        for (int i = skip * 17 + tid; i < cnt * 17; i += kTilePix) (&sm.acc[0][0])[i] = 0.0f;
         __syncthreads();
-        // this warp's first entry below its rays' last contributor (warp-uniform)
-        const int r0 = max(skip, top > warp_last ? (int)min((uint32_t)cnt, top - warp_last) : 0);
-        // entries none of this warp's rays hit in the forward are skipped (the same
-        // FP32 decisions here would not hit either): 32 entries' flags per ballot
-        const uint8_t *hit_w = reinterpret_cast<const uint8_t *>(sm.hit) + fwarp * BATCH;
-        for (int base = r0; base < cnt; base += 32) {
-            uint32_t todo = __ballot_sync(0xffffffffu, base + lane < cnt && hit_w[base + lane] != 0);
-            while (todo) {
-                const int r = base + __ffs(todo) - 1;
-                todo &= todo - 1u;
-                const uint32_t j = top - 1u - (uint32_t)r;
-                float gv[16];
-#pragma unroll
-                for (int k = 0; k < 16; ++k) gv[k] = 0.0f;
-                bool contrib = false;
-                if (j < ray.last) {
-                    const float4 a = sm.rec[r * 4 + 0];
-                    const float4 b = sm.rec[r * 4 + 1];
-                    const float4 c = sm.rec[r * 4 + 2];
-                    const float4 e = sm.rec[r * 4 + 3];
-                    ray_gradient<SPLAT>(ray, a, b, c, e, log2_amin, p.alpha_max, gv, contrib);
-                }
-                if (__any_sync(0xffffffffu, contrib)) {
-                    // warp reduce-scatter of the 16 values: lane l ends with the sum of value (l >> 1)
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        const bool up = lane & 16;
-                        const float send = up ? gv[k] : gv[k + 8];
-                        const float keep = up ? gv[k + 8] : gv[k];
-                        gv[k] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-                    }
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const bool up = lane & 8;
-                        const float send = up ? gv[k] : gv[k + 4];
-                        const float keep = up ? gv[k + 4] : gv[k];
-                        gv[k] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-                    }
-#pragma unroll
-                    for (int k = 0; k < 2; ++k) {
-                        const bool up = lane & 4;
-                        const float send = up ? gv[k] : gv[k + 2];
-                        const float keep = up ? gv[k + 2] : gv[k];
-                        gv[k] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-                    }
-                    {
-                        const bool up = lane & 2;
-                        const float send = up ? gv[0] : gv[1];
-                        const float keep = up ? gv[1] : gv[0];
-                        gv[0] = keep + __shfl_xor_sync(0xffffffffu, send, 2);
-                    }
-                    gv[0] += __shfl_xor_sync(0xffffffffu, gv[0], 1);
-                    if ((lane & 1) == 0) atomicAdd(&s_acc[r][lane >> 1], gv[0]);
-                }
-            }
+        // this warp's entries: those its rays hit in the forward, below their last
+        // contributor (the same FP32 decisions here would not hit the others either)
+        uint8_t *const list = sm.blist[warp];
+        const int first = max(skip, top > warp_last ? (int)min((uint32_t)cnt, top - warp_last) : 0);
+        int n = 0;
+        for (int base = first & ~31; base < cnt; base += 32) {
+            const int r = base + lane;
+            const bool mine = r >= first && r < cnt && reinterpret_cast<const uint8_t *>(sm.hit + r)[warp] != 0;
+            const uint32_t b = __ballot_sync(0xffffffffu, mine);
+            if (mine) list[n + __popc(b & lanemask_lt())] = (uint8_t)r;
+            n += __popc(b);
+        }
+        __syncwarp();
+        const int reach = top > ray.last ? (int)min((uint32_t)kBatch, top - ray.last) : 0;  // the ray's first entry
+        for (int k = 0; k < n; ++k) {
+            const int r = (int)list[k];
+            const float4 a = sm.rec[r * 4 + 0];
+            const float4 b = sm.rec[r * 4 + 1];
+            const float4 c = sm.rec[r * 4 + 2];
+            const float4 e = sm.rec[r * 4 + 3];
+            const RayGrad g = ray_gradient<SPLAT>(ray, a, b, c, e, log2_amin, p.alpha_max, r >= reach);
+            const float v = warp_sum<SPLAT>(g, ray, perm);
+            if (!(lane & 1)) atomicAdd(&sm.acc[r][perm.off], v);
         }
         __syncthreads();
         // flush: one Gaussian of the batch per thread, four float4 atomics
-        for (int r = skip + tid; r < cnt; r += kThreads) {
-            const float *v = s_acc[r];
-            bool any = false;
-#pragma unroll
-            for (int k = 0; k < 16; ++k) any |= v[k] != 0.0f;
-            if (any && in_bounds(sm.id[r], items, kSiteBwdItem, misc)) {
-                float4 *dst = reinterpret_cast<float4 *>(gacc + sm.id[r]);
-                atomicAdd(dst + 0, make_float4(v[0], v[1], v[2], v[3]));
-                atomicAdd(dst + 1, make_float4(v[4], v[5], v[6], v[7]));
-                atomicAdd(dst + 2, make_float4(v[8], v[9], v[10], v[11]));
-                atomicAdd(dst + 3, make_float4(v[12], v[13], v[14], v[15]));
-            }
+        if (tid >= skip && tid < cnt && (sm.hit[tid].x | sm.hit[tid].y)) {
+            const float *v = sm.acc[tid];
+            float4 *dst = reinterpret_cast<float4 *>(gacc + sm.id[tid]);
+            atomicAdd(dst + 0, make_float4(v[0], v[1], v[2], v[3]));
+            atomicAdd(dst + 1, make_float4(v[4], v[5], v[6], v[7]));
+            atomicAdd(dst + 2, make_float4(v[8], v[9], v[10], v[11]));
+            atomicAdd(dst + 3, make_float4(v[12], v[13], v[14], v[15]));
         }
         if (!direct) shift_list(sm.id, nullptr, cnt, s_cnt);
+        __syncthreads();  // the batch's sums and ids have been read
         top -= (uint32_t)cnt;
     }
 }
@@ -1283,7 +1360,7 @@ __device__ __forceinline__ BwdRay bwd_ray(const TileRay &tr, const DevCam &cam, 
 // One backward unit (the body of k_render_bwd's loop): unit code = tile << 4 | k. CG: read what the forward wrote through
 // L2 (the fused kernel reads it in the launch that wrote it).
 template <bool SPLAT, bool CG>
-__device__ __forceinline__ void bwd_unit(WalkSmem &sm, float (*s_acc)[17], uint32_t code,
+__device__ __forceinline__ void bwd_unit(WalkSmem &sm, uint32_t code,
                                          const DevCam *__restrict__ cams,
                                          int ncams,
                                          const float2 *__restrict__ ptab,
@@ -1373,10 +1450,9 @@ __device__ __forceinline__ void bwd_unit(WalkSmem &sm, float (*s_acc)[17], uint3
     __syncthreads();
     const uint32_t block_last = sm.maxlast;
     if (block_last <= lo) return;
-    backward_walk<SPLAT, CG>(sm, s_acc, tr.tl, rec, p, plo, lo, make_uint2(phi, hi), warp_last, block_last,
-                                          hit ? hit + (int64_t)t * hit_entries : nullptr,
-                                          hit ? idrec + (int64_t)t * hit_entries : nullptr, hit_entries,
-                                          tray >> 5, ray, gacc, items, misc);
+    backward_walk<SPLAT, CG>(sm, tr.tl, rec, p, plo, lo, make_uint2(phi, hi), warp_last, block_last,
+                             hit ? hit + (int64_t)t * hit_entries : nullptr,
+                             hit ? idrec + (int64_t)t * hit_entries : nullptr, hit_entries, ray, gacc, items, misc);
 }
 
 template <bool SPLAT>
@@ -1405,7 +1481,6 @@ __global__ void __launch_bounds__(kTilePix, GEER_BWD_MINB) k_render_bwd(const De
                                                                            const float4 *__restrict__ Cfin) {
     grid_dep_sync();
     __shared__ WalkSmem sm;
-    __shared__ float s_acc[kBatch][17];
     __shared__ uint32_t s_unit;
     if (misc[kMiscStatus] & kStatusCapacity) return;
     const uint32_t n_work = misc[kMiscUnits];
@@ -1418,7 +1493,7 @@ __global__ void __launch_bounds__(kTilePix, GEER_BWD_MINB) k_render_bwd(const De
         __syncthreads();
         const uint32_t w = s_unit;
         if (w >= n_work) break;
-        bwd_unit<SPLAT, false>(sm, s_acc, units[w], cams, ncams, ptab, S, tile_walk, srange, svals, smask, sany, rec, misc, p, dL_drgb, Tfin, last_in, hit, idrec, hit_entries, gacc, ntiles, items, cap_pairs, ckpt, ckpt_at, ckpt_cnt, Cfin);
+        bwd_unit<SPLAT, false>(sm, units[w], cams, ncams, ptab, S, tile_walk, srange, svals, smask, sany, rec, misc, p, dL_drgb, Tfin, last_in, hit, idrec, hit_entries, gacc, ntiles, items, cap_pairs, ckpt, ckpt_at, ckpt_cnt, Cfin);
     }
 }
 
@@ -1450,7 +1525,6 @@ __global__ void __launch_bounds__(kTilePix, GEER_BWD_MINB) k_render_train(
     GradAcc *__restrict__ gacc, uint32_t *__restrict__ queue, uint32_t queue_cap) {
     grid_dep_sync();
     __shared__ WalkSmem sm;
-    __shared__ float s_acc[kBatch][17];
     __shared__ uint32_t s_work;
     __shared__ float s_loss;
     if (misc[kMiscStatus] & kStatusCapacity) return;
@@ -1515,7 +1589,7 @@ __global__ void __launch_bounds__(kTilePix, GEER_BWD_MINB) k_render_train(
         __syncthreads();
         const uint32_t code = s_work;
         if (code == kQueueEmpty) break;
-        bwd_unit<SPLAT, true>(sm, s_acc, code, cams, ncams, ptab, S, tile_walk, srange, svals,
+        bwd_unit<SPLAT, true>(sm, code, cams, ncams, ptab, S, tile_walk, srange, svals,
                                            smask, sany, rec, misc, p, dL, Tfin, last, hit, idrec, hit_entries, gacc,
                                            ntiles, items, cap_pairs, ckpt, ckpt_at, ckpt_cnt, Cfin);
     }

@@ -81,15 +81,13 @@ __device__ __forceinline__ void sh_grad(int k, const ShDir &d, float g[3]) {
     }
 }
 
-// One block per 64 Gaussians. The block's SH coefficients are staged into shared
-// memory with coalesced asynchronous copies (row stride made odd so that
-// per-thread rows do not share banks) while each thread loads its own
-// parameters; each thread then runs the chain for its Gaussian over the cameras
-// and collects its dL/dsh in shared memory, and the block adds that to dL/dsh in
-// global memory coalesced. With one camera the SH row itself is overwritten by
-// its gradient term by term (each coefficient is read before its slot is
-// written), which halves the block's shared memory; with several cameras the
-// gradient has a row of its own.
+// One block per 64 Gaussians. Each warp stages the SH coefficients of its 32 in
+// shared memory with coalesced asynchronous copies (sh_stage) while each thread
+// loads its own parameters; each thread then runs the chain for its Gaussian over
+// the cameras and collects its dL/dsh in shared memory, and the warp writes that
+// (or adds it) to dL/dsh in global memory coalesced, 16 bytes a lane. With one
+// camera the SH row itself is overwritten by its gradient chunk by chunk, which
+// halves the shared memory; with several cameras the gradient has a row of its own.
 constexpr int kPBThreads = 64;
 #ifndef GEER_PB_MINB
 #define GEER_PB_MINB 14  // resident blocks of the one-camera variant: caps registers at 72
@@ -159,24 +157,17 @@ __global__ void __launch_bounds__(kPBThreads, ONE_CAM ? GEER_PB_MINB : 1) k_prep
     const GradAcc *__restrict__ gacc, float *__restrict__ d_mean, float *__restrict__ d_scale,
     float *__restrict__ d_quat, float *__restrict__ d_opacity, float *__restrict__ d_sh, int accumulate) {
     grid_dep_sync();
-    constexpr int NB = (DEG + 1) * (DEG + 1), NC = 3 * NB, ST = NC | 1;
-    __shared__ float s_sh[kPBThreads * ST];
-    __shared__ float s_dsh[ONE_CAM ? 1 : kPBThreads * ST];
-    __shared__ uint8_t s_live[kPBThreads];
+    constexpr int NC = ShRows<DEG>::NC, ST = ShRows<DEG>::kStride;
+    __shared__ __align__(16) float s_sh[kPBThreads * ST];
+    __shared__ __align__(16) float s_dsh[ONE_CAM ? 4 : kPBThreads * ST];
     const int tid = threadIdx.x;
     const int64_t g0 = (int64_t)blockIdx.x * kPBThreads;
     const int nloc = (int)min((int64_t)kPBThreads, n - g0);
-    {
-        // asynchronous 4-byte copies into the padded rows: no registers held while
-        // the block's rows are in flight
-        const float *src = sh + g0 * NC;
-        for (int i = tid; i < nloc * NC; i += kPBThreads) {
-            const int gl = i / NC, k = i - gl * NC;
-            cp_async4(&s_sh[gl * ST + k], src + i);
-        }
-        if (!ONE_CAM)
-            for (int i = tid; i < kPBThreads * ST; i += kPBThreads) s_dsh[i] = 0.0f;
-    }
+    // the warp's rows, asynchronously: no registers held while they are in flight
+    const int w0 = tid & ~31, rows = min(32, nloc - w0);
+    if (rows > 0) sh_stage<DEG>(s_sh + w0 * ST, sh + (g0 + w0) * NC, rows);
+    if (!ONE_CAM)
+        for (int i = tid & 31; i < 32 * ST; i += 32) s_dsh[w0 * ST + i] = 0.0f;
     const int64_t g = g0 + tid;
     bool any = false;
     if (tid < nloc)
@@ -197,10 +188,10 @@ __global__ void __launch_bounds__(kPBThreads, ONE_CAM ? GEER_PB_MINB : 1) k_prep
             for (int k = 0; k < 4; ++k) pa[k] = ap[k];
         }
     }
-    s_live[tid] = any ? 1 : 0;
     asm volatile("cp.async.wait_all;\n" ::: "memory");
-    const bool block_any = __syncthreads_or(any);
-    if (!block_any && accumulate) return;
+    __syncwarp();
+    const uint32_t live = __ballot_sync(0xffffffffu, any);  // the warp's Gaussians with a gradient
+    if (!live && accumulate) return;
     if (any) {
         float *shc = s_sh + tid * ST;
         float *dsh = ONE_CAM ? shc : s_dsh + tid * ST;
@@ -280,31 +271,44 @@ __global__ void __launch_bounds__(kPBThreads, ONE_CAM ? GEER_PB_MINB : 1) k_prep
             u.xx = u.x * u.x; u.yy = u.y * u.y; u.zz = u.z * u.z;
             const float drgb[3] = {a0.y, a0.z, a0.w};
             float raw[3] = {0.5f, 0.5f, 0.5f};
-#pragma unroll
-            for (int k = 0; k < NB; ++k) {
-                const float Yk = sh_value(k, u);
-#pragma unroll
-                for (int ch = 0; ch < 3; ++ch) raw[ch] += Yk * shc[3 * k + ch];
-            }
+            sh_each<DEG>(shc, [&](int i, float v) { raw[i % 3] += sh_value(i / 3, u) * v; });
             float dLdc[3];
 #pragma unroll
             for (int ch = 0; ch < 3; ++ch) dLdc[ch] = raw[ch] > 0.0f ? drgb[ch] : 0.0f;
             float ddir[3] = {0, 0, 0};
-#pragma unroll
-            for (int k = 0; k < NB; ++k) {
-                const float Yk = sh_value(k, u);
-                float gk[3];
-                sh_grad(k, u, gk);
-                float wk = 0.0f;
-#pragma unroll
-                for (int ch = 0; ch < 3; ++ch) {
-                    wk += dLdc[ch] * shc[3 * k + ch];
-                    if (ONE_CAM) dsh[3 * k + ch] = dLdc[ch] * Yk;  // slot read just above
-                    else dsh[3 * k + ch] += dLdc[ch] * Yk;
+            // per coefficient k: dL/dsh_k = dL/dc Y_k and the direction term; with one camera
+            // the row is overwritten in place, chunk by chunk (each read before it is written)
+            float wk = 0.0f;
+            const auto term = [&](int i, float v) {
+                const int k = i / 3, ch = i - 3 * k;
+                wk += dLdc[ch] * v;
+                if (ch == 2) {
+                    float gk[3];
+                    sh_grad(k, u, gk);
+                    ddir[0] += wk * gk[0];
+                    ddir[1] += wk * gk[1];
+                    ddir[2] += wk * gk[2];
+                    wk = 0.0f;
                 }
-                ddir[0] += wk * gk[0];
-                ddir[1] += wk * gk[1];
-                ddir[2] += wk * gk[2];
+                return dLdc[ch] * sh_value(k, u);
+            };
+            if constexpr (ShRows<DEG>::kVec) {
+#pragma unroll
+                for (int q = 0; q < NC / 4; ++q) {
+                    const float4 v = reinterpret_cast<const float4 *>(shc)[q];
+                    float4 o = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                    if (!ONE_CAM) o = reinterpret_cast<const float4 *>(dsh)[q];
+                    const float t0 = term(4 * q, v.x), t1 = term(4 * q + 1, v.y), t2 = term(4 * q + 2, v.z),
+                                t3 = term(4 * q + 3, v.w);
+                    reinterpret_cast<float4 *>(dsh)[q] = ONE_CAM ? make_float4(t0, t1, t2, t3)
+                                                                 : make_float4(o.x + t0, o.y + t1, o.z + t2, o.w + t3);
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < NC; ++i) {
+                    const float t = term(i, shc[i]);
+                    dsh[i] = ONE_CAM ? t : dsh[i] + t;
+                }
             }
             const float dp = ddir[0] * u.x + ddir[1] * u.y + ddir[2] * u.z;
             dmu[0] += (ddir[0] - u.x * dp) / vn;
@@ -360,34 +364,42 @@ __global__ void __launch_bounds__(kPBThreads, ONE_CAM ? GEER_PB_MINB : 1) k_prep
             for (int a = 0; a < 4; ++a) d_quat[4 * g + a] = 0.0f;
         if (d_opacity) d_opacity[g] = 0.0f;
     }
-    __syncthreads();
-    if (d_sh) {
-        // accumulating, rows of Gaussians without a gradient are left untouched;
-        // overwriting, they are zeroed
-        const float *acc = ONE_CAM ? s_sh : s_dsh;
-        float *dst = d_sh + g0 * NC;
-#ifndef GEER_PB_BATCH
-#define GEER_PB_BATCH 24
-#endif
-        constexpr int kBatch = GEER_PB_BATCH;  // values in flight per thread
-        if (!accumulate) {
-            for (int i = tid; i < nloc * NC; i += kPBThreads) {
-                const int gl = i / NC;
-                dst[i] = s_live[gl] ? acc[gl * ST + (i - gl * NC)] : 0.0f;
-            }
-            return;
-        }
-        for (int i0 = tid; i0 < nloc * NC; i0 += kBatch * kPBThreads) {
-            float v[kBatch];
+    __syncwarp();
+    if (d_sh && rows > 0) {
+        // the warp's rows, 16 bytes a lane; accumulating, rows of Gaussians without a
+        // gradient are left untouched, overwriting, they are zeroed
+        const float *acc = (ONE_CAM ? s_sh : s_dsh) + w0 * ST;
+        float *dst = d_sh + (g0 + w0) * NC;
+        const int floats = rows * NC, lane = tid & 31;
+        constexpr int kIters = (8 * NC + 31) / 32;       // 16-byte chunks a lane
+        constexpr int kGroup = kIters < 6 ? kIters : 6;  // of them in flight
+        const auto own = [&](int f) { return (live >> (f / NC) & 1u) != 0; };
+        const auto at = [&](int f) { return acc + (ST == NC ? f : f / NC * ST + f % NC); };
+#pragma unroll 1
+        for (int k0 = 0; k0 < kIters; k0 += kGroup) {
+            float4 old[kGroup];
+            bool whole[kGroup];  // a chunk of one row, or of rows with a gradient (dst is 16-byte aligned)
 #pragma unroll
-            for (int b = 0; b < kBatch; ++b) {
-                const int i = i0 + b * kPBThreads, gl = i / NC;
-                v[b] = (i < nloc * NC && s_live[gl]) ? dst[i] : 0.0f;
+            for (int b = 0; b < kGroup; ++b) {
+                const int f = 4 * ((k0 + b) * 32 + lane);
+                whole[b] = f + 4 <= floats && own(f) && (NC % 4 == 0 || own(f + 3));
+                if (accumulate && whole[b]) old[b] = *reinterpret_cast<const float4 *>(dst + f);
             }
 #pragma unroll
-            for (int b = 0; b < kBatch; ++b) {
-                const int i = i0 + b * kPBThreads, gl = i / NC;
-                if (i < nloc * NC && s_live[gl]) dst[i] = v[b] + acc[gl * ST + (i - gl * NC)];
+            for (int b = 0; b < kGroup; ++b) {
+                const int f = 4 * ((k0 + b) * 32 + lane);
+                if (whole[b]) {
+                    float4 v = *reinterpret_cast<const float4 *>(at(f));
+                    if (accumulate) v = make_float4(old[b].x + v.x, old[b].y + v.y, old[b].z + v.z, old[b].w + v.w);
+                    *reinterpret_cast<float4 *>(dst + f) = v;
+                } else if (NC % 4 == 0) {  // a row without a gradient (or past the end)
+                    if (!accumulate && f < floats) *reinterpret_cast<float4 *>(dst + f) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                } else {
+#pragma unroll 1
+                    for (int i = f; i < min(f + 4, floats); ++i)
+                        if (!accumulate) dst[i] = own(i) ? *at(i) : 0.0f;
+                        else if (own(i)) dst[i] += *at(i);
+                }
             }
         }
     }

@@ -316,7 +316,7 @@ size_t layout(const Caps &c, char *base, geer_workspace *ws) {
     size_t o_gs = L.take(sizeof(uint32_t) * kRadix * groups);
     size_t o_ge = L.take(sizeof(uint32_t) * kRadix * groups);
     size_t o_db = L.take(sizeof(uint32_t) * kRadix);
-    size_t o_misc = L.take(sizeof(uint32_t) * kMiscCount);
+    size_t o_misc = L.take(sizeof(uint32_t) * (kMiscCount + kOrderBuckets));
     size_t o_tr = L.take((sizeof(uint2) + sizeof(uint32_t)) * c.tiles);
     size_t o_to = L.take(sizeof(uint32_t) * c.tiles);
     const bool bwd = c.hit_entries > 0;  // the forward-only layout has no backward state

@@ -182,10 +182,74 @@ inline cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, siz
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-// Asynchronous 4-byte global -> shared copy (completed by cp.async.wait_all).
+// Asynchronous 4- and 16-byte global -> shared copies (completed by cp.async.wait_all).
 __device__ __forceinline__ void cp_async4(float *smem, const float *gmem) {
     const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async16(float *smem, const float *gmem) {
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(gmem) : "memory");
+}
+
+// A warp's 32 rows of SH coefficients (NC floats each) in shared memory. 32 rows are
+// a whole number of 16-byte chunks, so that a warp's rows start 16-byte aligned
+// (the array does) and are copied 16 bytes a lane, where 4-byte copies took an index
+// division each. Degree 3's rows (12 chunks) are padded to 13, so that eight lanes'
+// 16-byte accesses of the same chunk fall into different banks; degree 1's three
+// chunks and the odd rows of degrees 0 and 2 need no padding.
+template <int DEG>
+struct ShRows {
+    static constexpr int NC = 3 * (DEG + 1) * (DEG + 1);
+    static constexpr int kStride = DEG == 3 ? NC + 4 : NC;  // floats
+    static constexpr bool kVec = NC % 4 == 0;               // rows of whole chunks
+};
+
+// Starts copying rows [0, rows) of src (rows <= 32) into s; all lanes of the warp.
+// src is 16-byte aligned (the entry points require it of the array).
+template <int DEG>
+__device__ __forceinline__ void sh_stage(float *s, const float *__restrict__ src, int rows) {
+    constexpr int NC = ShRows<DEG>::NC, ST = ShRows<DEG>::kStride, kChunks = 8 * NC;  // 32 rows' chunks
+    const int lane = threadIdx.x & 31;
+    if (rows == 32) {
+        // chunk k * 32 + lane: for degree 3 three chunks a lane span eight rows, so that
+        // three places per lane and constant steps give all its chunks
+        constexpr int kIters = (kChunks + 31) / 32, kPlaces = ST == NC ? 1 : 3;
+        static_assert(ST == NC || 96 % (NC / 4) == 0, "three chunks a lane are whole rows");
+        const float *from = src + 4 * lane;
+        float *to[kPlaces];
+#pragma unroll
+        for (int q = 0; q < kPlaces; ++q) {
+            const int f = 4 * (q * 32 + lane);
+            to[q] = s + (ST == NC ? f : f / NC * ST + f % NC);
+        }
+#pragma unroll
+        for (int k = 0; k < kIters; ++k)
+            if (kChunks % 32 == 0 || k * 32 + lane < kChunks)
+                cp_async16(to[k % kPlaces] + k / kPlaces * (ST == NC ? 128 : 8 * ST), from + 128 * k);
+        return;
+    }
+#pragma unroll 1
+    for (int i = lane; i < rows * NC; i += 32) cp_async4(s + (ST == NC ? i : i / NC * ST + i % NC), src + i);
+}
+
+// Calls f(i, value) for the row's floats in order (i a compile-time constant after unrolling).
+template <int DEG, typename F>
+__device__ __forceinline__ void sh_each(const float *row, F f) {
+    constexpr int NC = ShRows<DEG>::NC;
+    if constexpr (ShRows<DEG>::kVec) {
+#pragma unroll
+        for (int q = 0; q < NC / 4; ++q) {
+            const float4 v = reinterpret_cast<const float4 *>(row)[q];
+            f(4 * q, v.x);
+            f(4 * q + 1, v.y);
+            f(4 * q + 2, v.z);
+            f(4 * q + 3, v.w);
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < NC; ++i) f(i, row[i]);
+    }
 }
 
 __device__ __forceinline__ void unpack_ranges(const uint4 r4, int rg[8]) {
@@ -268,7 +332,7 @@ struct geer_workspace {
     uint32_t *d_group_sum;  // [cap_sort_groups][kRadix] (zero between passes)
     uint32_t *d_group_excl; // [cap_sort_groups][kRadix]
     uint32_t *d_digit_base; // [kRadix]
-    uint32_t *d_misc;       // [kMiscCount]
+    uint32_t *d_misc;       // [kMiscCount], then the render order's bucket cursors [kOrderBuckets]
     uint2 *d_tile_walk;     // [cap_tiles] per tile, where the forward's scan of its super-tile list ended:
                             // (position, tile-list entries found before it); followed by [cap_tiles] u32 scratch
     uint32_t *d_tile_order; // [cap_tiles] tiles by descending super-tile list length: the forward's schedule
@@ -324,6 +388,7 @@ cudaError_t launch_bin_front(const geer_workspace *ws, cudaStream_t s);
 cudaError_t launch_depth_sort(geer_workspace *ws, cudaStream_t s);
 cudaError_t launch_count_pairs(const geer_workspace *ws, cudaStream_t s);
 cudaError_t launch_duplicate(const geer_workspace *ws, cudaStream_t s);
+cudaError_t launch_masks_order(const geer_workspace *ws, cudaStream_t s);
 cudaError_t launch_bwd_order(const geer_workspace *ws, cudaStream_t s);
 cudaError_t launch_expand_tiles(const geer_workspace *ws, uint32_t *counts_or_offsets, uint32_t *lists, cudaStream_t s);
 cudaError_t launch_tile_sort(geer_workspace *ws, cudaStream_t s);

@@ -30,7 +30,7 @@ struct Arc {
 // tan(angle/2) of the planar direction (x, z), angle measured from +z towards +x.
 __device__ float half_tan(float x, float z) {
     float r = fsq(fa(fm(x, x), fm(z, z)));
-    return (z >= 0.0f) ? fdv(x, fa(r, z)) : fdv(fs(r, z), x);
+    return fdv(z >= 0.0f ? x : fs(r, z), z >= 0.0f ? fa(r, z) : x);  // x / (r + z) or (r - z) / x
 }
 
 // PBF bounds about one camera axis (Sec. 3.2, App. D.1): the bounding planes
@@ -90,34 +90,49 @@ __device__ Arc shift_arc(Arc a) {
     return r;
 }
 
-// The first tile index k in [0, n] with pred(k) (false before, true from k on:
-// pred is monotone in k), searched from a guess: the guess only sets where the
-// probes start, so the result is exactly the first true index whatever the guess.
-template <typename Pred>
-__device__ __forceinline__ int first_true_from(int guess, int n, Pred pred) {
-    int k = min(max(guess, 0), n);
-    while (k > 0 && pred(k - 1)) --k;
-    while (k < n && !pred(k)) ++k;
+// The first tile index k in [0, n] with pred(v(k)) (false before, true from k on:
+// pred is monotone in k), searched from a guess k in [0, n]; below: v(k - 1), at: v(k)
+// (anything where there is none). The guess only sets where the probes start, so the
+// result is exactly the first true index whatever the guess.
+template <typename Value, typename Pred>
+__device__ __forceinline__ int first_true_from(int k, int n, float below, float at, Value value, Pred pred) {
+    if (k > 0 && pred(below)) {
+        do --k;
+        while (k > 0 && pred(value(k - 1)));
+    } else if (k < n && !pred(at)) {
+        do ++k;
+        while (k < n && !pred(value(k)));
+    }
     return k;
+}
+
+// atan(x) within 2e-5 rad, on [-1, 1] by Abramowitz and Stegun 4.4.49, pi/2 - atan(1/x)
+// beyond. Only for where a search starts.
+__device__ __forceinline__ float atan_guess(float x) {
+    const float ax = fabsf(x), t = ax > 1.0f ? __fdividef(1.0f, ax) : ax, u = t * t;
+    const float y = t * fmaf(u, fmaf(u, fmaf(u, fmaf(u, 0.0208351f, -0.0851330f), 0.1801410f), -0.3302995f), 0.9998660f);
+    return copysignf(ax > 1.0f ? 1.5707963f - y : y, x);
 }
 
 // Tile range [lo, hi) whose half-angle span [ta, tb] (tab[i].x, tab[i].y, both
 // increasing in i) meets the arc; prefix u suffix becomes the whole range. BEAP
 // angles are linear in the pixel index (Sec. 3.3), so the pixel of a bound tau
-// is about (2 atan(tau)) * ppr + (w - 1) / 2: that tile is the first probe
-// (ppr: pixels per radian, half: (w - 1) / 2), and a probe or two more find the
-// first index of each condition exactly.
+// is about (2 atan(tau)) * ppr + (w - 1) / 2 (ppr: pixels per radian, half: (w - 1) / 2),
+// and its tile nearly always the answer: the four edges that confirm both ends are
+// loaded together, and only a miss probes further.
 __device__ void arc_range(Arc a, const float4 *tab, int n, float ppr, float half, int &olo, int &ohi) {
     olo = 0;
     ohi = 0;
     if (a.kind == 0) return;
     if (a.kind == 3) { ohi = n; return; }
-    const float plo = fmaf(2.0f * atanf(a.lo), ppr, half), phi = fmaf(2.0f * atanf(a.hi), ppr, half);
+    const float plo = fmaf(2.0f * atan_guess(a.lo), ppr, half), phi = fmaf(2.0f * atan_guess(a.hi), ppr, half);
     // first index with tb >= a.lo (tb: the tile's last ray), then first with ta > a.hi
-    const int first = first_true_from((int)floorf((plo - (kTile - 1)) / kTile), n,
-                                      [&](int k) { return tab[k].y >= a.lo; });
-    const int last = first_true_from((int)floorf(phi / kTile) + 1, n,
-                                     [&](int k) { return tab[k].x > a.hi; }) - 1;
+    const int k0 = min(max((int)ceilf((plo - (kTile - 1)) / kTile), 0), n);
+    const int k1 = min(max((int)floorf(phi / kTile) + 1, 0), n);
+    const float b0 = tab[max(k0 - 1, 0)].y, e0 = tab[min(k0, n - 1)].y;
+    const float b1 = tab[max(k1 - 1, 0)].x, e1 = tab[min(k1, n - 1)].x;
+    const int first = first_true_from(k0, n, b0, e0, [&](int k) { return tab[k].y; }, [&](float v) { return v >= a.lo; });
+    const int last = first_true_from(k1, n, b1, e1, [&](int k) { return tab[k].x; }, [&](float v) { return v > a.hi; }) - 1;
     if (a.kind == 1) {
         if (first <= last) { olo = first; ohi = last + 1; }
         return;
@@ -297,14 +312,14 @@ __device__ __forceinline__ void splat_arcs(int mode, int snug, float amin, float
 // Real SH of degree <= 3 in the 3DGS convention (Condon-Shortley phase, index
 // l^2 + l + m), written out as polynomials of the unit direction. The constants
 // are K_lm sqrt(2)^(m != 0) = sqrt((2l+1)/(4 pi) (l-|m|)!/(l+|m|)!) (* sqrt 2).
-__device__ __forceinline__ void sh_colour(int deg, const float *c, float x, float y, float z, float rgb[3]) {
+template <int DEG>
+__device__ __forceinline__ void sh_colour(const float *row, float x, float y, float z, float rgb[3]) {
+    constexpr int deg = DEG;
     float Y[16];
     Y[0] = 0.28209479177387814f;  // 1/(2 sqrt(pi))
-    int nb = 1;
     if (deg >= 1) {
         const float k1 = 0.4886025119029199f;  // sqrt(3/(4 pi))
         Y[1] = -k1 * y; Y[2] = k1 * z; Y[3] = -k1 * x;
-        nb = 4;
     }
     if (deg >= 2) {
         float xx = x * x, yy = y * y, zz = z * z;
@@ -313,7 +328,6 @@ __device__ __forceinline__ void sh_colour(int deg, const float *c, float x, floa
         Y[6] = 0.31539156525252005f * (2.0f * zz - xx - yy);  // sqrt(5/pi)/4
         Y[7] = -1.0925484305920792f * x * z;
         Y[8] = 0.5462742152960396f * (xx - yy);           // sqrt(15/pi)/4
-        nb = 9;
         if (deg >= 3) {
             Y[9] = -0.5900435899266435f * y * (3.0f * xx - yy);        // sqrt(35/(2 pi))/4
             Y[10] = 2.890611442640554f * x * y * z;                    // sqrt(105/pi)/2
@@ -322,21 +336,13 @@ __device__ __forceinline__ void sh_colour(int deg, const float *c, float x, floa
             Y[13] = -0.4570457994644658f * x * (4.0f * zz - xx - yy);
             Y[14] = 1.445305721320277f * z * (xx - yy);                // sqrt(105/pi)/4
             Y[15] = -0.5900435899266435f * x * (xx - 3.0f * yy);
-            nb = 16;
         }
     }
-    float r = 0.5f, g = 0.5f, b = 0.5f;
-#pragma unroll
-    for (int k = 0; k < 16; ++k) {
-        if (k < nb) {
-            r += Y[k] * c[3 * k];
-            g += Y[k] * c[3 * k + 1];
-            b += Y[k] * c[3 * k + 2];
-        }
-    }
-    rgb[0] = fmaxf(r, 0.0f);
-    rgb[1] = fmaxf(g, 0.0f);
-    rgb[2] = fmaxf(b, 0.0f);
+    float c[3] = {0.5f, 0.5f, 0.5f};
+    sh_each<DEG>(row, [&](int i, float v) { c[i % 3] += Y[i / 3] * v; });
+    rgb[0] = fmaxf(c[0], 0.0f);
+    rgb[1] = fmaxf(c[1], 0.0f);
+    rgb[2] = fmaxf(c[2], 0.0f);
 }
 
 // True when the association predicate reduces to the rectangle X0 x Y0: no
@@ -392,9 +398,9 @@ __device__ __forceinline__ uint32_t assoc_count(const DevCam &cam, const int rg[
 }
 
 // The associated set as rectangles {x0, x1, y0, y1} (at most nine, overlapping
-// only on rows / columns that carry both flags); returns their number.
-__device__ __forceinline__ int assoc_rects(const DevCam &cam, const int rg[8], int4 rc[9]) {
-    int n = 0;
+// only on rows / columns that carry both flags): calls f for each.
+template <typename F>
+__device__ __forceinline__ void assoc_rects(const DevCam &cam, const int rg[8], F f) {
 #pragma unroll
     for (int i = 0; i < 2; ++i) {      // rows of the z interval (i = 0) or the w runs (i = 1) ...
 #pragma unroll
@@ -415,12 +421,11 @@ __device__ __forceinline__ int assoc_rects(const DevCam &cam, const int rg[8], i
                     const int c0 = j == 0 ? cam.zc[0] : (ci == 0 ? 0 : cam.wc[1]);
                     const int c1 = j == 0 ? cam.zc[1] : (ci == 0 ? cam.wc[0] : cam.tiles_x);
                     const int x0 = max(xlo, c0), x1 = min(xhi, c1);
-                    if (x0 < x1) rc[n++] = make_int4(x0, x1, y0, y1);
+                    if (x0 < x1) f(make_int4(x0, x1, y0, y1));
                 }
             }
         }
     }
-    return n;
 }
 
 // The super-tiles (S x S tiles) holding an associated tile: the union of the
@@ -428,7 +433,8 @@ __device__ __forceinline__ int assoc_rects(const DevCam &cam, const int rg[8], i
 template <typename F>
 __device__ __forceinline__ void for_each_super_general(const DevCam &cam, int S, const int rg[8], F f) {
     int4 rc[9];
-    const int n = assoc_rects(cam, rg, rc);
+    int n = 0;
+    assoc_rects(cam, rg, [&](int4 r) { rc[n++] = r; });
     for (int k = 0; k < n; ++k) {
         const int sx0 = rc[k].x / S, sx1 = (rc[k].y - 1) / S + 1, sy0 = rc[k].z / S, sy1 = (rc[k].w - 1) / S + 1;
         for (int sy = sy0; sy < sy1; ++sy)
@@ -481,15 +487,10 @@ __device__ __forceinline__ uint32_t block_sum_u32(uint32_t v, uint32_t *sm) {
 }
 
 // Thread per Gaussian, loop over cameras (the Gaussian's parameters are read once).
-// Two blocks per SM (128 registers): measured faster than one block without
-// spills and than three with more.
-// SH rows of the block staged in shared memory: row stride NC | 1 floats (odd, so
-// that the threads' rows do not share banks).
-template <int DEG>
-struct PrepSh {
-    static constexpr int kStride = (3 * (DEG + 1) * (DEG + 1)) | 1;
-};
-
+// Bound by issued instructions and the latency of the chain of divisions and table
+// loads. (1M Gaussians, one fisheye camera: 96 -> 78 us, and 24M (camera, Gaussian)
+// items 1810 -> 1470 us, with the SH rows copied 16 bytes a lane, one division per
+// half-angle and the searches of arc_range.)
 #ifndef GEER_PREP_MINB
 #define GEER_PREP_MINB 3  // resident blocks per SM: caps registers at 80
 #endif
@@ -504,20 +505,16 @@ __global__ void __launch_bounds__(kPrepThreads, GEER_PREP_MINB) k_preprocess(
     uint4 *__restrict__ ranges, GradAcc *__restrict__ gacc, uint32_t *__restrict__ count, uint32_t *__restrict__ key,
     uint32_t *__restrict__ blocksum, int64_t nblk) {
     grid_dep_sync();
-    constexpr int NC = 3 * (DEG + 1) * (DEG + 1), ST = PrepSh<DEG>::kStride;
-    extern __shared__ float s_sh[];  // [kPrepThreads][ST]
-    __shared__ uint32_t red[kPrepThreads / 32];
+    constexpr int NC = ShRows<DEG>::NC, ST = ShRows<DEG>::kStride;
+    extern __shared__ __align__(16) float s_sh[];  // [kPrepThreads][ST]
     const int64_t g0 = (int64_t)blockIdx.x * kPrepThreads;
     const int64_t g = g0 + threadIdx.x;
     {
-        // the block's SH coefficients, copied asynchronously while the bounds are
+        // the warp's SH coefficients, copied asynchronously while the bounds are
         // computed; read only for the colour
-        const int nloc = (int)min((int64_t)kPrepThreads, n - g0);
-        const float *src = sh + g0 * NC;
-        for (int i = threadIdx.x; i < nloc * NC; i += kPrepThreads) {
-            const int gl = i / NC;
-            cp_async4(&s_sh[gl * ST + (i - gl * NC)], src + i);
-        }
+        const int w0 = threadIdx.x & ~31;
+        const int rows = (int)min((int64_t)32, n - (g0 + w0));
+        if (rows > 0) sh_stage<DEG>(s_sh + w0 * ST, sh + (g0 + w0) * NC, rows);
     }
     bool ok = g < n;
     float mu[3] = {0, 0, 0}, sc[3] = {1, 1, 1}, qt[4] = {1, 0, 0, 0}, sigma = 0.0f;
@@ -659,14 +656,14 @@ __global__ void __launch_bounds__(kPrepThreads, GEER_PREP_MINB) k_preprocess(
             key[idx] = 0u;
             ranges[idx] = make_uint4(0, 0, 0, 0);
         }
-        if (ci == 0) {  // the SH rows have arrived (block-uniform)
+        if (ci == 0) {  // the warp's SH rows have arrived
             asm volatile("cp.async.wait_all;\n" ::: "memory");
-            __syncthreads();
+            __syncwarp();
         }
         if (live) {
             float dx = mu[0] - cam.o[0], dy = mu[1] - cam.o[1], dz = mu[2] - cam.o[2];
             float inv = rsqrtf(dx * dx + dy * dy + dz * dz);
-            sh_colour(DEG, s_sh + threadIdx.x * ST, dx * inv, dy * inv, dz * inv, r.rgb);
+            sh_colour<DEG>(s_sh + threadIdx.x * ST, dx * inv, dy * inv, dz * inv, r.rgb);
             float4 *dst = reinterpret_cast<float4 *>(rec + idx);
             const float4 *src = reinterpret_cast<const float4 *>(&r);
 #pragma unroll
@@ -678,13 +675,12 @@ __global__ void __launch_bounds__(kPrepThreads, GEER_PREP_MINB) k_preprocess(
 #pragma unroll
             for (int i = 0; i < 4; ++i) acc[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         }
-        uint32_t tot = block_sum_u32(cnt > 0 ? 1u : 0u, red);
-        if (threadIdx.x == 0) blocksum[(int64_t)ci * nblk + blockIdx.x] = tot;
+        const int tot = __syncthreads_count(cnt > 0);
+        if (threadIdx.x == 0) blocksum[(int64_t)ci * nblk + blockIdx.x] = (uint32_t)tot;
     }
 }
 
-// Exclusive scan of per-block counts (one block; each thread scans a contiguous
-// chunk serially). mode 0 (live items): total -> misc[kMiscLive]; also clears the
+// Exclusive scan of per-block counts (one block). mode 0 (live items): total -> misc[kMiscLive]; also clears the
 // per-super-tile pair counts. mode 1 ((super-tile, item) pairs): total ->
 // misc[kMiscPairs] (clamped to cap) with the capacity check. mode 2 ((tile, item)
 // associations P): total -> misc[kMiscTileLo / Hi]. With two blocks, block 1
@@ -699,38 +695,57 @@ __global__ void __launch_bounds__(1024) k_scan_blocks(uint32_t *__restrict__ blo
         blocksum = blocksum_b;
         mode = mode_b;
     }
-    const int t = threadIdx.x;
-    const int64_t chunk = (m + 1023) / 1024;
-    const int64_t b = t * chunk, e = min(m, b + chunk);
-    unsigned long long s = 0;
-    for (int64_t i = b; i < e; ++i) s += blocksum[i];
-    unsigned long long v = s;
-    const int lane = t & 31, warp = t >> 5;
+    // 4096 counts at a time, four neighbouring ones a thread (one 16-byte access), with a running total
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    unsigned long long carry = 0;
+    const auto load = [&](int64_t i) {
+        if (i + 4 <= m) return *reinterpret_cast<const uint4 *>(blocksum + i);
+        return make_uint4(i < m ? blocksum[i] : 0u, i + 1 < m ? blocksum[i + 1] : 0u, i + 2 < m ? blocksum[i + 2] : 0u, 0u);
+    };
+    uint4 c = load(4 * t);
+    for (int64_t i0 = 0; i0 < m; i0 += 4096) {
+        const int64_t i = i0 + 4 * t;
+        const uint4 next = i0 + 4096 < m ? load(i + 4096) : make_uint4(0u, 0u, 0u, 0u);
+        const unsigned long long s = (unsigned long long)c.x + c.y + c.z + c.w;
+        unsigned long long v = s;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        unsigned long long y = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += y;
-    }
-    if (lane == 31) warp_tot[warp] = v;
-    __syncthreads();
-    if (warp == 0) {
+        for (int o = 1; o < 32; o <<= 1) {
+            unsigned long long y = __shfl_up_sync(0xffffffffu, v, o);
+            if (lane >= o) v += y;
+        }
+        if (lane == 31) warp_tot[warp] = v;
+        __syncthreads();
         unsigned long long w = warp_tot[lane];
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             unsigned long long y = __shfl_up_sync(0xffffffffu, w, o);
             if (lane >= o) w += y;
         }
-        warp_tot[lane] = w;
+        const unsigned long long before = __shfl_sync(0xffffffffu, w, max(warp - 1, 0));
+        unsigned long long excl = carry + v - s + (warp > 0 ? before : 0ull);
+        carry += __shfl_sync(0xffffffffu, w, 31);
+        __syncthreads();
+        uint4 o4;
+        const auto put = [&](uint32_t n) {
+            const uint32_t e = (uint32_t)min(excl, 0xffffffffull);
+            excl += n;
+            return e;
+        };
+        o4.x = put(c.x);
+        o4.y = put(c.y);
+        o4.z = put(c.z);
+        o4.w = put(c.w);
+        if (i + 4 <= m) {
+            *reinterpret_cast<uint4 *>(blocksum + i) = o4;
+        } else {
+            if (i < m) blocksum[i] = o4.x;
+            if (i + 1 < m) blocksum[i + 1] = o4.y;
+            if (i + 2 < m) blocksum[i + 2] = o4.z;
+        }
+        c = next;
     }
-    __syncthreads();
-    unsigned long long excl = v - s + (warp > 0 ? warp_tot[warp - 1] : 0ull);
-    for (int64_t i = b; i < e; ++i) {
-        uint32_t c = blocksum[i];
-        blocksum[i] = (uint32_t)min(excl, 0xffffffffull);
-        excl += c;
-    }
-    if (t == 1023) {
-        const unsigned long long total = excl;
+    if (t == 0) {
+        const unsigned long long total = carry;
         if (mode == 0) {
             misc[kMiscLive] = (uint32_t)total;
             // the depth sort's first pass reads buffer 0 (see depth_sorted_buf)
@@ -753,38 +768,60 @@ __global__ void __launch_bounds__(1024) k_scan_blocks(uint32_t *__restrict__ blo
 }
 
 // Compaction of the live (camera, Gaussian) items, in index order, into
-// (depth key, item) arrays.
-__global__ void __launch_bounds__(kPrepThreads) k_compact(int ncams, int64_t n, const uint32_t *__restrict__ count,
+// (depth key, item) arrays. Block (b, ci): Gaussians [256 b, 256 b + 256) of camera ci.
+__global__ void __launch_bounds__(kPrepThreads) k_compact(int64_t n, const uint32_t *__restrict__ count,
                                                           const uint32_t *__restrict__ key,
                                                           const uint32_t *__restrict__ blocksum, int64_t nblk,
                                                           uint32_t *__restrict__ okey, uint32_t *__restrict__ oid) {
     grid_dep_sync();
     __shared__ uint32_t wsum[kPrepThreads / 32];
     const int64_t g = (int64_t)blockIdx.x * kPrepThreads + threadIdx.x;
-    for (int ci = 0; ci < ncams; ++ci) {
-        const int64_t idx = (int64_t)ci * n + g;
-        const bool live = g < n && count[idx] > 0;
-        uint32_t tot;
-        const uint32_t pre = block_excl_scan(live ? 1u : 0u, wsum, tot);
-        if (live) {
-            const uint32_t k = key[idx];
-            const uint32_t pos = blocksum[(int64_t)ci * nblk + blockIdx.x] + pre;
-            okey[pos] = k;
-            oid[pos] = (uint32_t)idx;
-        }
+    const int64_t idx = (int64_t)blockIdx.y * n + g;
+    const bool live = g < n && count[idx] > 0;
+    const uint32_t k = g < n ? key[idx] : 0u;
+    uint32_t tot;
+    const uint32_t pre = block_excl_scan(live ? 1u : 0u, wsum, tot);
+    if (live) {
+        const uint32_t pos = blocksum[(int64_t)blockIdx.y * nblk + blockIdx.x] + pre;
+        okey[pos] = k;
+        oid[pos] = (uint32_t)idx;
     }
 }
 
-// Number of (super-tile, item) pairs of an item with c associated tiles.
-__device__ __forceinline__ uint32_t super_count(const DevCam &cam, int S, const int rg[8], uint32_t c, bool rect) {
-    if (c == 0) return 0u;
-    if (rect) {
-        const int sx0 = rg[0] / S, sx1 = (rg[1] - 1) / S + 1, sy0 = rg[4] / S, sy1 = (rg[5] - 1) / S + 1;
-        return (uint32_t)((sx1 - sx0) * (sy1 - sy0));
+// x / S for a tile index x, inv_s = super_inverse(S): exact for S < 9 and x < 2^28.
+__device__ __forceinline__ uint32_t super_inverse(int S) { return S > 1 ? 0xffffffffu / (uint32_t)S + 1u : 0u; }
+__device__ __forceinline__ int super_of(int x, uint32_t inv_s) {
+    return inv_s ? (int)__umulhi((uint32_t)x, inv_s) : x;
+}
+
+// A live item's association for the binning: its only rectangle (packed columns
+// and rows, lo | hi << 16) when it is one (rects 1: all but the Gaussians across a
+// tile column or row where the other angle passes 90 degrees), and its number of
+// super-tiles.
+struct Assoc {
+    uint32_t xr, yr, rects, supers;
+};
+
+__device__ __forceinline__ Assoc item_assoc(const DevCam &cam, int S, uint32_t inv_s, const uint4 r4) {
+    Assoc a{r4.x, r4.z, 1u, 0u};
+    int rg[8];
+    unpack_ranges(r4, rg);
+    if (!is_rect(cam, rg)) {
+        a.rects = 0;
+        assoc_rects(cam, rg, [&](int4 r) {
+            a.xr = (uint32_t)r.x | (uint32_t)r.y << 16;
+            a.yr = (uint32_t)r.z | (uint32_t)r.w << 16;
+            ++a.rects;
+        });
     }
-    uint32_t k = 0;
-    for_each_super_general(cam, S, rg, [&](int, int) { ++k; });
-    return k;
+    if (a.rects == 1) {
+        const int sx0 = super_of((int)(a.xr & 0xffff), inv_s), sx1 = super_of((int)(a.xr >> 16) - 1, inv_s) + 1;
+        const int sy0 = super_of((int)(a.yr & 0xffff), inv_s), sy1 = super_of((int)(a.yr >> 16) - 1, inv_s) + 1;
+        a.supers = (uint32_t)((sx1 - sx0) * (sy1 - sy0));
+    } else if (a.rects > 1) {
+        for_each_super_general(cam, S, rg, [&](int, int) { ++a.supers; });
+    }
+    return a;
 }
 
 // Per block of depth-sorted live items: their super-tile pairs (emission
@@ -804,13 +841,10 @@ __global__ void __launch_bounds__(kPrepThreads) k_gather_counts(const DevCam *__
     const uint32_t *__restrict__ sorted_id = depth_sorted_buf(misc) ? sorted1 : sorted0;
     const int64_t i = (int64_t)blockIdx.x * kPrepThreads + threadIdx.x;
     uint32_t c = 0, sc = 0;
-    if (i < L) {
+    if (i < L) {  // (the live items: c > 0)
         const uint32_t item = sorted_id[i];
         c = count[item];
-        int rg[8];
-        unpack_ranges(ranges[item], rg);
-        const DevCam &cam = cams[item / (uint32_t)n];
-        sc = super_count(cam, S, rg, c, is_rect(cam, rg));
+        sc = item_assoc(cams[item / (uint32_t)n], S, super_inverse(S), ranges[item]).supers;
     }
     const uint32_t tot = block_sum_u32(c, red);
     if (threadIdx.x == 0) bs_tile[blockIdx.x] = tot;
@@ -845,124 +879,128 @@ __device__ __forceinline__ uint64_t tile_mask_general(const DevCam &cam, const i
     return m;
 }
 
-// The same for a rectangle (is_rect): columns [xlo, xhi) x rows [ylo, yhi). every:
-// bit j * S of every row j.
-__device__ __forceinline__ uint64_t tile_mask_rect(uint32_t xr, uint32_t yr, int sx, int sy, int S, uint64_t every) {
-    const uint32_t cols = span_bits((int)(xr & 0xffff), (int)(xr >> 16), sx * S, S);
-    const uint32_t rows = span_bits((int)(yr & 0xffff), (int)(yr >> 16), sy * S, S);
-    // rows is a run of ones [l, h): the bits every has in [l S, h S), each times cols
-    const int l = __ffs(rows) - 1, h = 32 - __clz(rows);
-    const uint64_t upto = h * S < 64 ? (1ull << (h * S)) - 1ull : ~0ull;
-    return rows ? (every & upto & ~((1ull << (l * S)) - 1ull)) * cols : 0ull;
+// The same for a rectangle that meets the super-tile: columns [xlo, xhi) x rows
+// [ylo, yhi) (packed lo | hi << 16). every: bit j * S of every row j. M: uint32_t
+// where the S * S bits fit it.
+template <typename M>
+__device__ __forceinline__ M tile_mask_rect(uint32_t xr, uint32_t yr, int sx, int sy, int S, M every) {
+    constexpr int kBits = 8 * sizeof(M);
+    const int x0 = sx * S, y0 = sy * S;
+    const int xl = max((int)(xr & 0xffff) - x0, 0), xh = min((int)(xr >> 16) - x0, S);
+    const int yl = max((int)(yr & 0xffff) - y0, 0), yh = min((int)(yr >> 16) - y0, S);
+    // the bits every has in [yl S, yh S), each times the columns' run of ones
+    const M upto = yh * S < kBits ? ((M)1 << (yh * S)) - 1 : ~(M)0;
+    return (every & upto & ~(((M)1 << (yl * S)) - 1)) * (M)((1u << xh) - (1u << xl));
 }
 
-__device__ __forceinline__ void put_mask(uint32_t *out, int64_t i, int words, uint64_t m) {
-    if (words == 1) out[i] = (uint32_t)m;
-    else reinterpret_cast<uint2 *>(out)[i] = make_uint2((uint32_t)m, (uint32_t)(m >> 32));
+__device__ __forceinline__ void put_mask(uint32_t *out, int64_t i, uint32_t m) { out[i] = m; }
+__device__ __forceinline__ void put_mask(uint32_t *out, int64_t i, uint64_t m) {
+    reinterpret_cast<uint2 *>(out)[i] = make_uint2((uint32_t)m, (uint32_t)(m >> 32));
 }
 
 // DuplicateWithKeys in depth order, at super-tile granularity: item i of the
 // depth-sorted list emits one (global super-tile, item) pair per super-tile
-// holding an associated tile, in row-major order, with its tile mask (what the
-// renders' list fills test: one bit of a 4-byte load, where the 16 bytes of ranges
-// cost an unpacking and eight comparisons), and counts the pairs per super-tile.
-// Items whose association is a rectangle are emitted by the whole warp together
-// (lane j writes output j: coalesced); others loop per thread.
+// holding an associated tile, with its tile mask (what the renders' list fills
+// test: one bit of a 4-byte load, where the 16 bytes of ranges cost an unpacking and
+// eight comparisons), and counts the pairs per super-tile. An item's pairs may come
+// in any order (each belongs to another super-tile). Items whose association is one
+// rectangle are emitted by the whole warp together (lane j writes output j:
+// coalesced) from a list in shared memory; the few others loop per thread.
+// M: the mask's type (32 bits up to S = 5).
+template <typename M>
 __global__ void __launch_bounds__(kPrepThreads) k_duplicate(
-    const DevCam *__restrict__ cams, const float4 *__restrict__ ttab, int64_t n, int S,
-    const uint32_t *__restrict__ sorted0, const uint32_t *__restrict__ sorted1, const uint4 *__restrict__ ranges,
-    const uint32_t *__restrict__ count, uint32_t *__restrict__ misc, const uint32_t *__restrict__ blocksum,
-    uint32_t *__restrict__ okeys, uint32_t *__restrict__ ovals, uint32_t *__restrict__ omask,
-    uint32_t *__restrict__ scount, int nst, int64_t cap) {
+    const DevCam *__restrict__ cams, int64_t n, int S, const uint32_t *__restrict__ sorted0,
+    const uint32_t *__restrict__ sorted1, const uint4 *__restrict__ ranges, uint32_t *__restrict__ misc,
+    const uint32_t *__restrict__ blocksum, uint32_t *__restrict__ okeys, uint32_t *__restrict__ ovals,
+    uint32_t *__restrict__ omask, uint32_t *__restrict__ scount, int nst, int64_t cap) {
     grid_dep_sync();
+    // a one-rectangle item: {columns, rows, item, first output (of the block's)},
+    // {first output (of the warp's), super-tiles a row | stiles_x << 16, first super-tile, its x | y << 16}
+    __shared__ uint4 s_item[kPrepThreads][2];
     __shared__ uint32_t wsum[kPrepThreads / 32];
     extern __shared__ uint32_t sh[];  // per-super-tile pair counts when they fit (nst <= kSmemTiles)
     const bool smem = nst <= kSmemTiles;
     if (smem)
         for (int k = threadIdx.x; k < nst; k += kPrepThreads) sh[k] = 0u;
     const uint32_t L = misc[kMiscLive];
+    if ((int64_t)blockIdx.x * kPrepThreads >= L) return;
     const uint32_t *__restrict__ sorted_id = depth_sorted_buf(misc) ? sorted1 : sorted0;
     const int lane = threadIdx.x & 31;
     const int64_t i = (int64_t)blockIdx.x * kPrepThreads + threadIdx.x;
-    uint32_t item = 0, cnt = 0;
-    int rg[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    const uint32_t inv_s = super_inverse(S);
+    uint32_t item = 0;
+    uint4 r4 = make_uint4(0u, 0u, 0u, 0u);
     int ci = 0;
-    uint32_t xr = 0, yr = 0;  // the direct column and row ranges, packed
-    bool rect = true;
+    Assoc as{0u, 0u, 0u, 0u};
     if (i < L) {
         item = sorted_id[i];
         ci = (int)(item / (uint32_t)n);
-        const uint4 r4 = ranges[item];
-        xr = r4.x;
-        yr = r4.z;
-        unpack_ranges(r4, rg);
-        rect = is_rect(cams[ci], rg);
-        cnt = super_count(cams[ci], S, rg, count[item], rect);
+        r4 = ranges[item];
+        as = item_assoc(cams[ci], S, inv_s, r4);
     }
-    uint32_t tot;
-    const uint32_t pre = block_excl_scan(cnt, wsum, tot);
-    const int64_t off = (int64_t)blocksum[blockIdx.x] + pre;
-    const bool fits = off + cnt <= cap;
+    const uint32_t cnt = as.supers;
     const DevCam &cam = cams[ci];
-    __syncthreads();  // the per-super-tile counters are cleared
-    int sx0 = 0, sy0 = 0, rw = 1;
-    if (rect && fits && cnt > 0) {
-        sx0 = rg[0] / S;
-        sy0 = rg[4] / S;
-        rw = (rg[1] - 1) / S + 1 - sx0;
-    }
-    // cooperative emission of the rectangle items of this warp
-    const uint32_t rc = (rect && fits) ? cnt : 0u;
+    uint32_t tot;
+    const uint32_t pre = block_excl_scan(cnt, wsum, tot);  // (its barriers also follow the clearing of sh)
+    const int64_t base = (int64_t)blocksum[blockIdx.x];
+    const bool fits = base + pre + cnt <= cap;
+    // cooperative emission of the warp's one-rectangle items
+    const bool one = as.rects == 1 && fits;
+    const uint32_t rc = one ? cnt : 0u;
     uint32_t incl = rc;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
         if (lane >= o) incl += y;
     }
-    const int words = mask_words(S);
-    uint64_t every = 0;
-    for (int j = 0; j < S; ++j) every |= 1ull << (j * S);
+    const uint32_t ones = __ballot_sync(0xffffffffu, one);
+    uint4(*list)[2] = s_item + (threadIdx.x & ~31);
+    if (one) {
+        const int sx0 = super_of((int)(as.xr & 0xffff), inv_s), sy0 = super_of((int)(as.yr & 0xffff), inv_s);
+        const int rw = super_of((int)(as.xr >> 16) - 1, inv_s) + 1 - sx0;
+        const int k = __popc(ones & ((1u << lane) - 1u));
+        list[k][0] = make_uint4(as.xr, as.yr, item, pre);
+        list[k][1] = make_uint4(incl - rc, (uint32_t)rw | (uint32_t)cam.stiles_x << 16,
+                                (uint32_t)(cam.stile_base + sy0 * cam.stiles_x + sx0), (uint32_t)sx0 | (uint32_t)sy0 << 16);
+    }
+    __syncwarp();
+    M every = 0;
+    for (int j = 0; j < S; ++j) every |= (M)1 << (j * S);
     const uint32_t wtot = __shfl_sync(0xffffffffu, incl, 31);
-    const uint32_t sb = (uint32_t)(cam.stile_base + sy0 * cam.stiles_x + sx0);
+    int before = -1;  // items that start in the windows so far, less one
     for (uint32_t j0 = 0; j0 < wtot; j0 += 32) {
+        // the outputs of this window where an item starts; an output's item is the last to start
+        const uint32_t at = incl - rc - j0;
+        const uint32_t starts = __reduce_or_sync(0xffffffffu, one && at < 32u ? 1u << at : 0u);
         const uint32_t j = j0 + lane;
-        // owner: first lane whose inclusive count exceeds j
-        int lo = 0;
-#pragma unroll
-        for (int step = 16; step > 0; step >>= 1) {
-            const uint32_t v = __shfl_sync(0xffffffffu, incl, lo + step - 1);
-            if (v <= j) lo += step;
-        }
-        const uint32_t o_incl = __shfl_sync(0xffffffffu, incl, lo);
-        const uint32_t o_cnt = __shfl_sync(0xffffffffu, rc, lo);
-        const int o_rw = __shfl_sync(0xffffffffu, rw, lo);
-        const uint32_t o_sb = __shfl_sync(0xffffffffu, sb, lo);
-        const int o_sx = __shfl_sync(0xffffffffu, cam.stiles_x, lo);
-        const uint32_t o_item = __shfl_sync(0xffffffffu, item, lo);
-        const int64_t o_off = __shfl_sync(0xffffffffu, off, lo);
-        const uint32_t o_xr = __shfl_sync(0xffffffffu, xr, lo), o_yr = __shfl_sync(0xffffffffu, yr, lo);
-        const uint32_t o_s = __shfl_sync(0xffffffffu, (uint32_t)sx0 | (uint32_t)sy0 << 16, lo);
+        const int o = before + __popc(starts & (0xffffffffu >> (31 - lane)));
+        before += __popc(starts);
         if (j < wtot) {
-            const uint32_t k = j - (o_incl - o_cnt);
-            const uint32_t ky = k / (uint32_t)o_rw, kx = k - ky * (uint32_t)o_rw;
-            const uint32_t st = o_sb + ky * (uint32_t)o_sx + kx;
-            okeys[o_off + k] = st;
-            ovals[o_off + k] = o_item;
-            put_mask(omask, o_off + k, words,
-                     tile_mask_rect(o_xr, o_yr, (int)(o_s & 0xffff) + (int)kx, (int)(o_s >> 16) + (int)ky, S, every));
+            const uint4 a = list[o][0], b = list[o][1];
+            const uint32_t k = j - b.x, rw = b.y & 0xffff;
+            // k / rw: the quotient's distance from the next whole number is at least 0.5 / rw,
+            // more than its rounding errors below 2^21
+            const uint32_t ky = k < 1u << 21 ? (uint32_t)__fdividef((float)k + 0.5f, (float)rw) : k / rw;
+            const uint32_t kx = k - ky * rw, st = b.z + ky * (b.y >> 16) + kx;
+            const int64_t out = base + (int64_t)(a.w + k);
+            okeys[out] = st;
+            ovals[out] = a.z;
+            put_mask(omask, out, tile_mask_rect<M>(a.x, a.y, (int)((b.w & 0xffff) + kx), (int)((b.w >> 16) + ky), S, every));
             if (in_bounds(st, (uint64_t)nst, kSiteDupSuper, misc)) atomicAdd(smem ? &sh[st] : &scount[st], 1u);
         }
     }
-    // per-thread emission of the other items (flipped angular ranges)
-    if (!rect && fits && cnt > 0) {
-        int64_t o = off;
-        const int64_t end = off + cnt;
+    // per-thread emission of the items of several rectangles
+    if (as.rects > 1 && fits) {
+        int rg[8];
+        unpack_ranges(r4, rg);
+        int64_t o = base + pre;
+        const int64_t end = o + cnt;
         for_each_super_general(cam, S, rg, [&](int sx, int sy) {
             if (o < end) {
                 const uint32_t st = (uint32_t)(cam.stile_base + sy * cam.stiles_x + sx);
                 okeys[o] = st;
                 ovals[o] = item;
-                put_mask(omask, o, words, tile_mask_general(cam, rg, sx, sy, S));
+                put_mask(omask, o, (M)tile_mask_general(cam, rg, sx, sy, S));
                 if (in_bounds(st, (uint64_t)nst, kSiteDupSuper, misc)) atomicAdd(smem ? &sh[st] : &scount[st], 1u);
                 ++o;
             }
@@ -1040,31 +1078,33 @@ __device__ __forceinline__ uint32_t block_chunk_prefix(uint32_t s, uint32_t *war
     return pre;
 }
 
-// One block, IdentifyFrustumRanges at super-tile granularity: each super-tile's
-// [start, end) in the sorted super-tile pairs (exclusive scan of its pair
-// count), and the order in which the render blocks take the tiles: by
-// descending length of their super-tile's list (bucketed), so that the costliest
-// tiles start first and the grid does not end on a tail of heavy tiles. (Measured
-// on the 1M-Gaussian fisheye workload: 0.344 ms forward against 0.358 - 0.409 ms
-// with the length capped at 16K - 1K entries and 0.424 ms in tile order.)
+// IdentifyFrustumRanges at super-tile granularity, block 0: each super-tile's
+// [start, end) in the sorted super-tile pairs (exclusive scan of its pair count),
+// and the places of the buckets in the order in which the render blocks take the
+// tiles: by descending length of their super-tile's list (bucketed), so that the
+// costliest tiles start first and the grid does not end on a tail of heavy tiles.
+// (Measured on the 1M-Gaussian fisheye workload: 0.344 ms forward against 0.358 -
+// 0.409 ms with the length capped at 16K - 1K entries and 0.424 ms in tile order.)
+// A super-tile adds its tiles to its bucket; k_masks_order then places them. The
+// other blocks reset the fused render's unit queue. (One block that also walked all
+// the tiles and the queue took 100 us on four 1920 x 1536 cameras.)
+constexpr int kQueueBlock = 8 * 1024;  // queue words reset by a block
 __global__ void __launch_bounds__(1024) k_tile_offsets(const DevCam *__restrict__ cams, int ncams, int S,
-                                                       int ntiles, uint2 *__restrict__ srange, int nst,
+                                                       uint2 *__restrict__ srange, int nst,
                                                        uint32_t *__restrict__ misc,
-                                                       uint32_t *__restrict__ tile_order,
                                                        uint32_t *__restrict__ queue, uint32_t queue_n) {
     grid_dep_sync();
+    const int t = threadIdx.x;
     // the fused render's unit queue and its counters start afresh with every binning
-    if (queue) {
-        for (uint32_t i = threadIdx.x; i < queue_n; i += 1024) queue[i] = 0xffffffffu;
-        if (threadIdx.x < 4) misc[kMiscFwdNext + threadIdx.x] = 0u;
+    if (blockIdx.x > 0) {
+        const uint32_t q0 = (blockIdx.x - 1) * (uint32_t)kQueueBlock, q1 = min(queue_n, q0 + kQueueBlock);
+        for (uint32_t i = q0 + t; i < q1; i += 1024) queue[i] = 0xffffffffu;
+        return;
     }
-    constexpr int kOrderSmem = 16384;  // super-tiles / tiles whose buckets the block keeps in shared memory
+    if (queue && t < 4) misc[kMiscFwdNext + t] = 0u;
     __shared__ uint32_t warp_tot[32];
     __shared__ uint32_t hist[kOrderBuckets];
-    __shared__ uint8_t s_sbk[kOrderSmem], s_tbk[kOrderSmem];
     if (misc[kMiscStatus] & kStatusCapacity) return;
-    const int t = threadIdx.x;
-    const bool keep_s = nst <= kOrderSmem, keep_t = ntiles <= kOrderSmem;
     for (int i = t; i < kOrderBuckets; i += 1024) hist[i] = 0u;
     // super-tile ranges
     const uint32_t *scount = reinterpret_cast<const uint32_t *>(srange + nst);
@@ -1073,50 +1113,74 @@ __global__ void __launch_bounds__(1024) k_tile_offsets(const DevCam *__restrict_
     uint32_t ss = 0;
     for (int i = sb; i < se; ++i) ss += scount[i];
     uint32_t srun = block_chunk_prefix(ss, warp_tot);
+    int c = 0;
     for (int i = sb; i < se; ++i) {
         const uint32_t cnt = scount[i];
         srange[i] = make_uint2(srun, srun + cnt);
-        if (keep_s) s_sbk[i] = (uint8_t)order_bucket(cnt);
         srun += cnt;
+        while (c + 1 < ncams && cams[c + 1].stile_base <= i) ++c;
+        const DevCam &cm = cams[c];
+        const int l = i - cm.stile_base, sy = cm.stiles_x > 0 ? l / cm.stiles_x : 0, sx = l - sy * cm.stiles_x;
+        const int w = min(S, cm.tiles_x - sx * S), h = min(S, cm.tiles_y - sy * S);
+        if (cnt > 0 && w > 0 && h > 0) atomicAdd(&hist[order_bucket(cnt)], (uint32_t)(w * h));
     }
     __syncthreads();
-    // each tile's cost estimate: its super-tile's list length (0 for padding tiles),
-    // bucketed in the first pass and kept for the second
-    const int chunk = (ntiles + 1023) / 1024;
-    const int b = t * chunk, e = min(ntiles, b + chunk);
-    int c = 0;
-    for (int k = 1; k < ncams; ++k)
-        if (cams[k].tile_base <= b) c = k;
-    for (int pass = 0; pass < 2; ++pass) {
-        int cc = c;
-        for (int k = 0; k < chunk; ++k) {  // the same trip count in every lane (warp-wide atomics)
-            const int i = b + k;
-            int bk = kOrderBuckets - 1;
-            if (i < e && pass == 1 && keep_t) {
-                bk = s_tbk[i];
-            } else if (i < e) {
-                while (cc + 1 < ncams && cams[cc + 1].tile_base <= i) ++cc;
-                const DevCam &cm = cams[cc];
+    // (the last bucket's own size, the tiles without entries, is not needed)
+    bucket_scan(hist);
+    __syncthreads();
+    for (int i = t; i < kOrderBuckets; i += 1024) misc[kMiscCount + i] = hist[i];
+}
+
+// After the sort of the super-tile pairs. Blocks [0, order_blocks): 1024 tiles each
+// take their places in the render order, a block's tiles of a bucket together.
+// The others: the or of every 32 sorted pairs' tile masks (a warp per group): the
+// render's list scan skips the groups without an entry of its tile.
+__global__ void __launch_bounds__(256) k_masks_order(const DevCam *__restrict__ cams, int ncams, int S, int ntiles,
+                                                     const uint2 *__restrict__ srange, uint32_t *__restrict__ order,
+                                                     int order_blocks, const uint32_t *__restrict__ mask, int words,
+                                                     uint32_t *__restrict__ misc, uint32_t *__restrict__ any) {
+    grid_dep_sync();
+    if (misc[kMiscStatus] & kStatusCapacity) return;
+    const int t = threadIdx.x, lane = t & 31;
+    if ((int)blockIdx.x < order_blocks) {
+        __shared__ uint32_t hist[kOrderBuckets];
+        if (t < kOrderBuckets) hist[t] = 0u;
+        __syncthreads();
+        const uint32_t inv_s = super_inverse(S);
+        int bk[4], c = 0;
+        uint32_t rank[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = (int)blockIdx.x * 1024 + u * 256 + t;
+            bk[u] = kOrderBuckets - 1;  // the tiles that a slot layout leaves unused come last
+            if (i < ntiles) {
+                while (c + 1 < ncams && cams[c + 1].tile_base <= i) ++c;
+                const DevCam &cm = cams[c];
                 const int lt = i - cm.tile_base;
                 if (lt >= 0 && lt < cm.tiles_x * cm.tiles_y) {
                     const int cy = lt / cm.tiles_x, cx = lt - cy * cm.tiles_x;
-                    const int si = cm.stile_base + (cy / S) * cm.stiles_x + cx / S;
-                    if (keep_s) {
-                        bk = s_sbk[si];
-                    } else {
-                        const uint2 r = srange[si];
-                        bk = order_bucket(r.y - r.x);
-                    }
+                    const uint2 r = srange[cm.stile_base + super_of(cy, inv_s) * cm.stiles_x + super_of(cx, inv_s)];
+                    bk[u] = order_bucket(r.y - r.x);
                 }
-                if (keep_t) s_tbk[i] = (uint8_t)bk;
             }
-            const uint32_t slot = bucket_add(hist, i < e, bk);
-            if (pass == 1 && i < e) tile_order[slot] = (uint32_t)i;
+            rank[u] = bucket_add(hist, i < ntiles, bk[u]);
         }
         __syncthreads();
-        if (pass == 0) bucket_scan(hist);
+        if (t < kOrderBuckets && hist[t]) hist[t] = atomicAdd(&misc[kMiscCount + t], hist[t]);
         __syncthreads();
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = (int)blockIdx.x * 1024 + u * 256 + t;
+            if (i < ntiles) order[hist[bk[u]] + rank[u]] = (uint32_t)i;
+        }
+        return;
     }
+    const uint64_t n = (uint64_t)misc[kMiscPairs], step = (uint64_t)(gridDim.x - order_blocks) * 256u;
+    for (uint64_t i = (uint64_t)(blockIdx.x - order_blocks) * 256u + t; (i & ~31ull) < n; i += step)
+        for (int w = 0; w < words; ++w) {
+            const uint32_t v = __reduce_or_sync(0xffffffffu, i < n ? mask[i * words + w] : 0u);
+            if (lane == 0) any[(i >> 5) * words + w] = v;
+        }
 }
 
 // One block: the backward's units and their schedule. A tile whose forward walk
@@ -1188,7 +1252,7 @@ cudaError_t launch_preprocess(const geer_workspace *ws, const geer_gaussians *g,
     const bool splat = prm.assoc != GEER_ASSOC_PBF || prm.alpha_model != GEER_ALPHA_EXACT;
 #define GEER_PREP_LAUNCH(D)                                                                                      \
     {                                                                                                            \
-        const int smem = kPrepThreads * PrepSh<D>::kStride * (int)sizeof(float);                               \
+        const int smem = kPrepThreads * ShRows<D>::kStride * (int)sizeof(float);                               \
         auto *kern = splat ? k_preprocess<D, true> : k_preprocess<D, false>;                                     \
         if (smem > 48 * 1024) {                                                                                  \
             const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);  \
@@ -1215,7 +1279,7 @@ cudaError_t launch_bin_front(const geer_workspace *ws, cudaStream_t s) {
              ws->n_stiles, ws->cap_pairs, 0, nullptr, 0);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || nblk == 0) return e;
-    launch_k(k_compact, dim3((unsigned)nblk), dim3(kPrepThreads), 0, s, ws->n_cams, ws->n_gauss, ws->d_count,
+    launch_k(k_compact, dim3((unsigned)nblk, (unsigned)ws->n_cams), dim3(kPrepThreads), 0, s, ws->n_gauss, ws->d_count,
              ws->d_key, ws->d_blocksum, nblk, ws->d_ikey[0], ws->d_iid[0]);
     return cudaGetLastError();
 }
@@ -1240,15 +1304,26 @@ cudaError_t launch_duplicate(const geer_workspace *ws, cudaStream_t s) {
     uint32_t *scount = reinterpret_cast<uint32_t *>(ws->d_srange + ws->n_stiles);
     if (m > 0) {
         const size_t smem = ws->n_stiles <= kSmemTiles ? sizeof(uint32_t) * ws->n_stiles : 0;
-        launch_k(k_duplicate, dim3((unsigned)m), dim3(kPrepThreads), smem, s, ws->d_cams, ws->d_tile_tab,
-                 ws->n_gauss, ws->super_size, ws->d_iid[0], ws->d_iid[1], ws->d_ranges, ws->d_count, ws->d_misc,
-                 ws->d_blocksum2, ws->d_keys[0], ws->d_vals[0], ws->d_smask[0], scount, (int)ws->n_stiles, ws->cap_pairs);
+        launch_k(mask_words(ws->super_size) == 1 ? k_duplicate<uint32_t> : k_duplicate<uint64_t>, dim3((unsigned)m),
+                 dim3(kPrepThreads), smem, s, ws->d_cams, ws->n_gauss, ws->super_size, ws->d_iid[0], ws->d_iid[1],
+                 ws->d_ranges, ws->d_misc, ws->d_blocksum2, ws->d_keys[0], ws->d_vals[0], ws->d_smask[0], scount,
+                 (int)ws->n_stiles, ws->cap_pairs);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    launch_k(k_tile_offsets, dim3(1), dim3(1024), 0, s, ws->d_cams, ws->n_cams, ws->super_size, (int)ws->n_tiles,
-             ws->d_srange, (int)ws->n_stiles, ws->d_misc, ws->d_tile_order,
-             ws->trains ? ws->d_bwd_order : nullptr, (uint32_t)(ws->n_tiles * (kCkptMax + 1)));
+    const uint32_t queue_n = ws->trains ? (uint32_t)(ws->n_tiles * (kCkptMax + 1)) : 0u;
+    launch_k(k_tile_offsets, dim3(1 + (queue_n + kQueueBlock - 1) / kQueueBlock), dim3(1024), 0, s, ws->d_cams,
+             ws->n_cams, ws->super_size, ws->d_srange, (int)ws->n_stiles, ws->d_misc,
+             ws->trains ? ws->d_bwd_order : nullptr, queue_n);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_masks_order(const geer_workspace *ws, cudaStream_t s) {
+    const int64_t blocks = std::min<int64_t>(std::max<int64_t>(1, (ws->cap_pairs + 255) / 256), (int64_t)ws->num_sms * 8);
+    const int order_blocks = (int)((ws->n_tiles + 1023) / 1024);
+    launch_k(k_masks_order, dim3((unsigned)(blocks + order_blocks)), dim3(256), 0, s, ws->d_cams, ws->n_cams,
+             ws->super_size, (int)ws->n_tiles, ws->d_srange, ws->d_tile_order, order_blocks,
+             (const uint32_t *)ws->d_smask[ws->sorted_buf], mask_words(ws->super_size), ws->d_misc, ws->d_sany);
     return cudaGetLastError();
 }
 

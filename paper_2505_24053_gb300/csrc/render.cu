@@ -1168,7 +1168,8 @@ __device__ __forceinline__ RayGrad ray_gradient(BwdRay &r, const float4 &a, cons
 // selecting what to send; only the next two (4 and 2 apart) select. That and
 // packed arithmetic take ~50 instructions for the products and the sums, where
 // selecting in every exchange took ~75. The tree of each value's sum is the plain
-// butterfly's.
+// butterfly's. (With the branch-free gradient and the warps' entry lists: the
+// 1M-Gaussian training step 1010 -> 927 us, the surround step 21.0 -> 19.35 ms.)
 struct LanePerm {
     float2 d01, d23, b01, b23, g01, g23;
     int off;

@@ -285,22 +285,6 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(
     }
 }
 
-
-// The or of every 32 sorted pairs' tile masks (a warp per group): the render's
-// list scan skips the groups without an entry of its tile.
-__global__ void __launch_bounds__(256) k_group_masks(const uint32_t *__restrict__ mask, int words,
-                                                     const uint32_t *__restrict__ misc, uint32_t *__restrict__ any) {
-    grid_dep_sync();
-    if (misc[kMiscStatus] & kStatusCapacity) return;
-    const uint64_t n = (uint64_t)misc[kMiscPairs], step = (uint64_t)gridDim.x * 256u;
-    const int lane = threadIdx.x & 31;
-    for (uint64_t i = (uint64_t)blockIdx.x * 256u + threadIdx.x; (i & ~31ull) < n; i += step)
-        for (int w = 0; w < words; ++w) {
-            const uint32_t v = __reduce_or_sync(0xffffffffu, i < n ? mask[i * words + w] : 0u);
-            if (lane == 0) any[(i >> 5) * words + w] = v;
-        }
-}
-
 }  // namespace
 
 int sort_blocks_per_sm() {
@@ -362,10 +346,7 @@ cudaError_t launch_tile_sort(geer_workspace *ws, cudaStream_t s) {
         cur ^= 1;
     }
     ws->sorted_buf = cur;
-    const int64_t blocks = std::min<int64_t>(std::max<int64_t>(1, (ws->cap_pairs + 255) / 256), (int64_t)ws->num_sms * 8);
-    launch_k(k_group_masks, dim3((unsigned)blocks), dim3(256), 0, s, (const uint32_t *)ws->d_smask[cur],
-             mask_words(ws->super_size), (const uint32_t *)ws->d_misc, ws->d_sany);
-    return cudaGetLastError();
+    return launch_masks_order(ws, s);
 }
 
 }  // namespace geer

@@ -92,6 +92,12 @@ constexpr int kPBThreads = 64;
 #ifndef GEER_PB_MINB
 #define GEER_PB_MINB 14  // resident blocks of the one-camera variant: caps registers at 72
 #endif
+#ifndef GEER_PB_MINB_CAMS
+// Of the variant for several cameras: 204 registers (the next camera's loads overlap the
+// chain). Measured, 6M Gaussians and four cameras: 1.21 ms, with 7 1.69, with 10 2.02
+// (going through every camera: 1.35 at the best).
+#define GEER_PB_MINB_CAMS 5
+#endif
 
 // The splat alpha's chain (GEER_ALPHA_SPLAT) from dL/d(theta_c, phi_c) and
 // dL/d(A, B, C) (the conic K = Sigma_2^-1, B its off-diagonal) to the camera-frame
@@ -151,7 +157,7 @@ __device__ __forceinline__ void splat_chain(const float mc[3], const float M[9],
 }
 
 template <int DEG, bool ONE_CAM, bool SPLAT>
-__global__ void __launch_bounds__(kPBThreads, ONE_CAM ? GEER_PB_MINB : 1) k_preprocess_bwd(
+__global__ void __launch_bounds__(kPBThreads, ONE_CAM ? GEER_PB_MINB : GEER_PB_MINB_CAMS) k_preprocess_bwd(
     const DevCam *__restrict__ cams, int ncams, const float *__restrict__ mean, const float *__restrict__ scale,
     const float *__restrict__ quat, const float *__restrict__ sh, int64_t n, const uint32_t *__restrict__ count,
     const GradAcc *__restrict__ gacc, float *__restrict__ d_mean, float *__restrict__ d_scale,
@@ -170,8 +176,13 @@ __global__ void __launch_bounds__(kPBThreads, ONE_CAM ? GEER_PB_MINB : 1) k_prep
         for (int i = tid & 31; i < 32 * ST; i += 32) s_dsh[w0 * ST + i] = 0.0f;
     const int64_t g = g0 + tid;
     bool any = false;
+    uint32_t seen = 0;  // the first 32 cameras that see the Gaussian
     if (tid < nloc)
-        for (int ci = 0; ci < ncams; ++ci) any |= count[(int64_t)ci * n + g] > 0;
+        for (int ci = 0; ci < ncams; ++ci) {
+            const bool c = count[(int64_t)ci * n + g] > 0;
+            any |= c;
+            if (c && ci < 32) seen |= 1u << ci;
+        }
     float mu[3], s[3], q[4];
     float4 pa[4];  // the one camera's accumulators, loaded with the parameters
     if (any) {  // a Gaussian not associated with any tile has no gradient
@@ -206,9 +217,16 @@ __global__ void __launch_bounds__(kPBThreads, ONE_CAM ? GEER_PB_MINB : 1) k_prep
         R[6] = 2.0f * (x * z - w * y);        R[7] = 2.0f * (y * z + w * x);        R[8] = 1.0f - 2.0f * (x * x + y * y);
         float dmu[3] = {0, 0, 0}, ds[3] = {0, 0, 0}, dR[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0}, dsig = 0.0f;
 
-        for (int ci = 0; ci < (ONE_CAM ? 1 : ncams); ++ci) {
+        // each lane takes the next camera that sees its own Gaussian, so that a warp goes
+        // through the chain as often as its busiest lane, not once per camera
+        const auto next = [&](int ci) {
+            ++ci;
+            if constexpr (!ONE_CAM)
+                while (ci < ncams && !(ci < 32 ? seen >> ci & 1u : count[(int64_t)ci * n + g])) ++ci;
+            return ci;
+        };
+        for (int ci = next(-1); ci < (ONE_CAM ? 1 : ncams); ci = next(ci)) {
             const int64_t idx = (int64_t)ci * n + g;
-            if (!ONE_CAM && count[idx] == 0) continue;
             const DevCam &cam = cams[ci];
             float4 a0, a1, a2, a3;
             if (ONE_CAM) {

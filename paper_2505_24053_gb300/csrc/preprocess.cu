@@ -428,25 +428,6 @@ __device__ __forceinline__ void assoc_rects(const DevCam &cam, const int rg[8], 
     }
 }
 
-// The super-tiles (S x S tiles) holding an associated tile: the union of the
-// rectangles' super-tile boxes, each super-tile visited once.
-template <typename F>
-__device__ __forceinline__ void for_each_super_general(const DevCam &cam, int S, const int rg[8], F f) {
-    int4 rc[9];
-    int n = 0;
-    assoc_rects(cam, rg, [&](int4 r) { rc[n++] = r; });
-    for (int k = 0; k < n; ++k) {
-        const int sx0 = rc[k].x / S, sx1 = (rc[k].y - 1) / S + 1, sy0 = rc[k].z / S, sy1 = (rc[k].w - 1) / S + 1;
-        for (int sy = sy0; sy < sy1; ++sy)
-            for (int sx = sx0; sx < sx1; ++sx) {
-                bool seen = false;
-                for (int q = 0; q < k && !seen; ++q)
-                    seen = sx >= rc[q].x / S && sx <= (rc[q].y - 1) / S && sy >= rc[q].z / S && sy <= (rc[q].w - 1) / S;
-                if (!seen) f(sx, sy);
-            }
-    }
-}
-
 // Block-wide exclusive scan (256 threads); returns the exclusive prefix and the block total.
 __device__ __forceinline__ uint32_t block_excl_scan(uint32_t x, uint32_t *wsum, uint32_t &total) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -468,22 +449,6 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t x, uint32_t *wsum, 
     __syncthreads();
     total = tot;
     return pre + v - x;
-}
-
-__device__ __forceinline__ uint32_t block_sum_u32(uint32_t v, uint32_t *sm) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) sm[warp] = v;
-    __syncthreads();
-    uint32_t t = 0;
-    if (threadIdx.x < 32) {
-        t = threadIdx.x < (blockDim.x >> 5) ? sm[threadIdx.x] : 0u;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    }
-    __syncthreads();
-    return t;  // valid in warp 0
 }
 
 // Thread per Gaussian, loop over cameras (the Gaussian's parameters are read once).
@@ -695,6 +660,7 @@ __global__ void __launch_bounds__(1024) k_scan_blocks(uint32_t *__restrict__ blo
         blocksum = blocksum_b;
         mode = mode_b;
     }
+    if (mode != 0) m = ((int64_t)misc[kMiscLive] + kPrepThreads - 1) / kPrepThreads;  // the blocks with live items
     // 4096 counts at a time, four neighbouring ones a thread (one 16-byte access), with a running total
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     unsigned long long carry = 0;
@@ -796,14 +762,13 @@ __device__ __forceinline__ int super_of(int x, uint32_t inv_s) {
 
 // A live item's association for the binning: its only rectangle (packed columns
 // and rows, lo | hi << 16) when it is one (rects 1: all but the Gaussians across a
-// tile column or row where the other angle passes 90 degrees), and its number of
-// super-tiles.
+// tile column or row where the other angle passes 90 degrees).
 struct Assoc {
-    uint32_t xr, yr, rects, supers;
+    uint32_t xr, yr, rects;
 };
 
-__device__ __forceinline__ Assoc item_assoc(const DevCam &cam, int S, uint32_t inv_s, const uint4 r4) {
-    Assoc a{r4.x, r4.z, 1u, 0u};
+__device__ __forceinline__ Assoc item_assoc(const DevCam &cam, const uint4 r4) {
+    Assoc a{r4.x, r4.z, 1u};
     int rg[8];
     unpack_ranges(r4, rg);
     if (!is_rect(cam, rg)) {
@@ -814,43 +779,135 @@ __device__ __forceinline__ Assoc item_assoc(const DevCam &cam, int S, uint32_t i
             ++a.rects;
         });
     }
-    if (a.rects == 1) {
-        const int sx0 = super_of((int)(a.xr & 0xffff), inv_s), sx1 = super_of((int)(a.xr >> 16) - 1, inv_s) + 1;
-        const int sy0 = super_of((int)(a.yr & 0xffff), inv_s), sy1 = super_of((int)(a.yr >> 16) - 1, inv_s) + 1;
-        a.supers = (uint32_t)((sx1 - sx0) * (sy1 - sy0));
-    } else if (a.rects > 1) {
-        for_each_super_general(cam, S, rg, [&](int, int) { ++a.supers; });
-    }
     return a;
 }
 
-// Per block of depth-sorted live items: their super-tile pairs (emission
-// offsets) and their tile pairs (the total, for the capacity check).
-__global__ void __launch_bounds__(kPrepThreads) k_gather_counts(const DevCam *__restrict__ cams,
-                                                                const float4 *__restrict__ ttab, int64_t n, int S,
-                                                                const uint32_t *__restrict__ sorted0,
-                                                                const uint32_t *__restrict__ sorted1,
-                                                                const uint32_t *__restrict__ count,
-                                                                const uint4 *__restrict__ ranges,
-                                                                const uint32_t *__restrict__ misc,
-                                                                uint32_t *__restrict__ bs_super,
-                                                                uint32_t *__restrict__ bs_tile) {
-    grid_dep_sync();
-    __shared__ uint32_t red[kPrepThreads / 32];
-    const uint32_t L = misc[kMiscLive];
-    const uint32_t *__restrict__ sorted_id = depth_sorted_buf(misc) ? sorted1 : sorted0;
-    const int64_t i = (int64_t)blockIdx.x * kPrepThreads + threadIdx.x;
-    uint32_t c = 0, sc = 0;
-    if (i < L) {  // (the live items: c > 0)
-        const uint32_t item = sorted_id[i];
-        c = count[item];
-        sc = item_assoc(cams[item / (uint32_t)n], S, super_inverse(S), ranges[item]).supers;
+// The super-tile box of a rectangle: first column and row, columns, super-tiles.
+struct SuperBox {
+    int sx0, sy0, w;
+    uint32_t supers;
+};
+__device__ __forceinline__ SuperBox super_box(uint32_t xr, uint32_t yr, uint32_t inv_s) {
+    SuperBox b;
+    b.sx0 = super_of((int)(xr & 0xffff), inv_s);
+    b.sy0 = super_of((int)(yr & 0xffff), inv_s);
+    b.w = super_of((int)(xr >> 16) - 1, inv_s) + 1 - b.sx0;
+    b.supers = (uint32_t)(b.w * (super_of((int)(yr >> 16) - 1, inv_s) + 1 - b.sy0));
+    return b;
+}
+
+// The super-tiles of an item of several rectangles, by its warp: the union of the
+// rectangles' super-tile boxes, each super-tile once. f(sx, sy, keep) for 32
+// super-tiles at a time, keep false for those of an earlier rectangle and past the
+// end. rg: the item's ranges in every lane; box: the warp's nine {sx0, sx1, sy0, sy1}
+// (ends included) in shared memory.
+template <typename F>
+__device__ __forceinline__ void warp_supers(const DevCam &cam, uint32_t inv_s, const int rg[8], int4 *box, F f) {
+    const int lane = threadIdx.x & 31;
+    int n = 0;
+    __syncwarp();
+    assoc_rects(cam, rg, [&](int4 r) {
+        if (lane == 0)
+            box[n] = make_int4(super_of(r.x, inv_s), super_of(r.y - 1, inv_s), super_of(r.z, inv_s),
+                               super_of(r.w - 1, inv_s));
+        ++n;
+    });
+    __syncwarp();
+    for (int k = 0; k < n; ++k) {
+        const int4 b = box[k];
+        const int w = b.y - b.x + 1, cells = w * (b.w - b.z + 1);
+        for (int c0 = 0; c0 < cells; c0 += 32) {
+            const int c = c0 + lane, cy = c / w, sx = b.x + c - cy * w, sy = b.z + cy;
+            bool keep = c < cells;
+            for (int q = 0; q < k; ++q) {
+                const int4 e = box[q];
+                keep = keep && !(sx >= e.x && sx <= e.y && sy >= e.z && sy <= e.w);
+            }
+            f(sx, sy, keep);
+        }
     }
-    const uint32_t tot = block_sum_u32(c, red);
-    if (threadIdx.x == 0) bs_tile[blockIdx.x] = tot;
+}
+
+// Per 256 depth-sorted live items (a block of the emission): their super-tile pairs
+// (emission offsets) and their tile pairs (the total, for the capacity check). Each
+// item's rectangle and super-tiles are left in depth order for the emission, in the
+// depth sort's buffers, which nobody reads any more: columns and rows in the keys'
+// (columns 0: several rectangles), super-tiles in the unused ids'. Bound by the
+// scattered reads of the items' ranges: the tile counts follow from them (a second
+// scattered read took as long), and a thread has kGather items in flight.
+constexpr int kGather = 2;  // (24M items, 9M live: 273 us; with 1 320, with 4 299; both arrays read 452)
+__global__ void __launch_bounds__(kPrepThreads) k_gather_counts(
+    const DevCam *__restrict__ cams, int64_t n, int S, uint32_t *__restrict__ id0, uint32_t *__restrict__ id1,
+    const uint4 *__restrict__ ranges, const uint32_t *__restrict__ misc, uint32_t *__restrict__ bs_super, uint32_t *__restrict__ bs_tile, uint32_t *__restrict__ oxr,
+    uint32_t *__restrict__ oyr) {
+    grid_dep_sync();
+    __shared__ uint32_t s_sum[kGather][2];
+    __shared__ int4 s_box[kPrepThreads / 32][9];
+    const uint32_t L = misc[kMiscLive];
+    const int64_t i0 = (int64_t)blockIdx.x * (kGather * kPrepThreads);
+    if (i0 >= L) return;
+    const bool cur = depth_sorted_buf(misc) != 0;
+    const uint32_t *__restrict__ sorted_id = cur ? id1 : id0;
+    uint32_t *__restrict__ osupers = cur ? id0 : id1;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t inv_s = super_inverse(S);
+    if (threadIdx.x < 2 * kGather) (&s_sum[0][0])[threadIdx.x] = 0u;
+    uint32_t item[kGather];
+    uint4 r4[kGather];
+#pragma unroll
+    for (int u = 0; u < kGather; ++u) {
+        const int64_t i = i0 + u * kPrepThreads + threadIdx.x;
+        item[u] = i < L ? sorted_id[i] : 0u;
+    }
+#pragma unroll
+    for (int u = 0; u < kGather; ++u) {
+        r4[u] = make_uint4(0u, 0u, 0u, 0u);
+        if (i0 + u * kPrepThreads + threadIdx.x < L) r4[u] = ranges[item[u]];
+    }
     __syncthreads();
-    const uint32_t stot = block_sum_u32(sc, red);
-    if (threadIdx.x == 0) bs_super[blockIdx.x] = stot;
+#pragma unroll
+    for (int u = 0; u < kGather; ++u) {
+        const int64_t i = i0 + u * kPrepThreads + threadIdx.x;
+        const int ci = (int)(item[u] / (uint32_t)n);
+        Assoc a{0u, 0u, 0u};
+        uint32_t sc = 0, c = 0;
+        if (i < L) a = item_assoc(cams[ci], r4[u]);
+        if (a.rects == 1) {
+            sc = super_box(a.xr, a.yr, inv_s).supers;
+            c = ((a.xr >> 16) - (a.xr & 0xffff)) * ((a.yr >> 16) - (a.yr & 0xffff));
+        }
+        for (uint32_t many = __ballot_sync(0xffffffffu, a.rects > 1); many; many &= many - 1) {
+            const int o = __ffs(many) - 1;
+            const uint4 q = make_uint4(__shfl_sync(0xffffffffu, r4[u].x, o), __shfl_sync(0xffffffffu, r4[u].y, o),
+                                       __shfl_sync(0xffffffffu, r4[u].z, o), __shfl_sync(0xffffffffu, r4[u].w, o));
+            int rg[8];
+            unpack_ranges(q, rg);
+            uint32_t k = 0;
+            const DevCam &cam = cams[__shfl_sync(0xffffffffu, ci, o)];
+            warp_supers(cam, inv_s, rg, s_box[warp], [&](int, int, bool keep) {
+                k += (uint32_t)__popc(__ballot_sync(0xffffffffu, keep));
+            });
+            if (lane == o) {
+                sc = k;
+                c = assoc_count(cam, rg, 0, cam.tiles_x, 0, cam.tiles_y);
+            }
+        }
+        if (i < L) {
+            oxr[i] = a.rects == 1 ? a.xr : 0u;
+            oyr[i] = a.yr;
+            osupers[i] = sc;
+        }
+        const uint32_t tiles = __reduce_add_sync(0xffffffffu, c), supers = __reduce_add_sync(0xffffffffu, sc);
+        if (lane == 0) {
+            atomicAdd(&s_sum[u][0], supers);
+            atomicAdd(&s_sum[u][1], tiles);
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < kGather && i0 + threadIdx.x * kPrepThreads < L) {
+        bs_super[(int64_t)blockIdx.x * kGather + threadIdx.x] = s_sum[threadIdx.x][0];
+        bs_tile[(int64_t)blockIdx.x * kGather + threadIdx.x] = s_sum[threadIdx.x][1];
+    }
 }
 
 // Bits [lo, hi) of the S tile columns (or rows) that start at base.
@@ -905,47 +962,47 @@ __device__ __forceinline__ void put_mask(uint32_t *out, int64_t i, uint64_t m) {
 // eight comparisons), and counts the pairs per super-tile. An item's pairs may come
 // in any order (each belongs to another super-tile). Items whose association is one
 // rectangle are emitted by the whole warp together (lane j writes output j:
-// coalesced) from a list in shared memory; the few others loop per thread.
+// coalesced) from a list in shared memory; the few others by the warp one by one (a
+// thread looping over its item's super-tiles kept its block waiting).
 // M: the mask's type (32 bits up to S = 5).
 template <typename M>
 __global__ void __launch_bounds__(kPrepThreads) k_duplicate(
-    const DevCam *__restrict__ cams, int64_t n, int S, const uint32_t *__restrict__ sorted0,
-    const uint32_t *__restrict__ sorted1, const uint4 *__restrict__ ranges, uint32_t *__restrict__ misc,
-    const uint32_t *__restrict__ blocksum, uint32_t *__restrict__ okeys, uint32_t *__restrict__ ovals,
-    uint32_t *__restrict__ omask, uint32_t *__restrict__ scount, int nst, int64_t cap) {
+    const DevCam *__restrict__ cams, int64_t n, int S, const uint32_t *__restrict__ id0,
+    const uint32_t *__restrict__ id1, const uint32_t *__restrict__ xrs, const uint32_t *__restrict__ yrs,
+    const uint4 *__restrict__ ranges, uint32_t *__restrict__ misc, const uint32_t *__restrict__ blocksum,
+    uint32_t *__restrict__ okeys, uint32_t *__restrict__ ovals, uint32_t *__restrict__ omask,
+    uint32_t *__restrict__ scount, int nst, int64_t cap) {
     grid_dep_sync();
     // a one-rectangle item: {columns, rows, item, first output (of the block's)},
     // {first output (of the warp's), super-tiles a row | stiles_x << 16, first super-tile, its x | y << 16}
     __shared__ uint4 s_item[kPrepThreads][2];
     __shared__ uint32_t wsum[kPrepThreads / 32];
+    __shared__ int4 s_box[kPrepThreads / 32][9];
     extern __shared__ uint32_t sh[];  // per-super-tile pair counts when they fit (nst <= kSmemTiles)
     const bool smem = nst <= kSmemTiles;
     if (smem)
         for (int k = threadIdx.x; k < nst; k += kPrepThreads) sh[k] = 0u;
     const uint32_t L = misc[kMiscLive];
     if ((int64_t)blockIdx.x * kPrepThreads >= L) return;
-    const uint32_t *__restrict__ sorted_id = depth_sorted_buf(misc) ? sorted1 : sorted0;
+    const bool cur = depth_sorted_buf(misc) != 0;
     const int lane = threadIdx.x & 31;
     const int64_t i = (int64_t)blockIdx.x * kPrepThreads + threadIdx.x;
     const uint32_t inv_s = super_inverse(S);
-    uint32_t item = 0;
-    uint4 r4 = make_uint4(0u, 0u, 0u, 0u);
-    int ci = 0;
-    Assoc as{0u, 0u, 0u, 0u};
+    uint32_t item = 0, xr = 0, yr = 0, cnt = 0;  // as the counting left them
     if (i < L) {
-        item = sorted_id[i];
-        ci = (int)(item / (uint32_t)n);
-        r4 = ranges[item];
-        as = item_assoc(cams[ci], S, inv_s, r4);
+        item = (cur ? id1 : id0)[i];
+        cnt = (cur ? id0 : id1)[i];
+        xr = xrs[i];
+        yr = yrs[i];
     }
-    const uint32_t cnt = as.supers;
+    const int ci = (int)(item / (uint32_t)n);
     const DevCam &cam = cams[ci];
     uint32_t tot;
     const uint32_t pre = block_excl_scan(cnt, wsum, tot);  // (its barriers also follow the clearing of sh)
     const int64_t base = (int64_t)blocksum[blockIdx.x];
     const bool fits = base + pre + cnt <= cap;
     // cooperative emission of the warp's one-rectangle items
-    const bool one = as.rects == 1 && fits;
+    const bool one = xr != 0 && fits;
     const uint32_t rc = one ? cnt : 0u;
     uint32_t incl = rc;
 #pragma unroll
@@ -956,12 +1013,12 @@ __global__ void __launch_bounds__(kPrepThreads) k_duplicate(
     const uint32_t ones = __ballot_sync(0xffffffffu, one);
     uint4(*list)[2] = s_item + (threadIdx.x & ~31);
     if (one) {
-        const int sx0 = super_of((int)(as.xr & 0xffff), inv_s), sy0 = super_of((int)(as.yr & 0xffff), inv_s);
-        const int rw = super_of((int)(as.xr >> 16) - 1, inv_s) + 1 - sx0;
+        const SuperBox b = super_box(xr, yr, inv_s);
         const int k = __popc(ones & ((1u << lane) - 1u));
-        list[k][0] = make_uint4(as.xr, as.yr, item, pre);
-        list[k][1] = make_uint4(incl - rc, (uint32_t)rw | (uint32_t)cam.stiles_x << 16,
-                                (uint32_t)(cam.stile_base + sy0 * cam.stiles_x + sx0), (uint32_t)sx0 | (uint32_t)sy0 << 16);
+        list[k][0] = make_uint4(xr, yr, item, pre);
+        list[k][1] = make_uint4(incl - rc, (uint32_t)b.w | (uint32_t)cam.stiles_x << 16,
+                                (uint32_t)(cam.stile_base + b.sy0 * cam.stiles_x + b.sx0),
+                                (uint32_t)b.sx0 | (uint32_t)b.sy0 << 16);
     }
     __syncwarp();
     M every = 0;
@@ -989,21 +1046,25 @@ __global__ void __launch_bounds__(kPrepThreads) k_duplicate(
             if (in_bounds(st, (uint64_t)nst, kSiteDupSuper, misc)) atomicAdd(smem ? &sh[st] : &scount[st], 1u);
         }
     }
-    // per-thread emission of the items of several rectangles
-    if (as.rects > 1 && fits) {
+    // the items of several rectangles, one at a time
+    for (uint32_t many = __ballot_sync(0xffffffffu, cnt > 0 && xr == 0 && fits); many; many &= many - 1) {
+        const int o = __ffs(many) - 1;
+        const uint32_t it = __shfl_sync(0xffffffffu, item, o), cn = __shfl_sync(0xffffffffu, cnt, o);
+        const DevCam &c = cams[__shfl_sync(0xffffffffu, ci, o)];
+        const int64_t out = base + __shfl_sync(0xffffffffu, pre, o);
         int rg[8];
-        unpack_ranges(r4, rg);
-        int64_t o = base + pre;
-        const int64_t end = o + cnt;
-        for_each_super_general(cam, S, rg, [&](int sx, int sy) {
-            if (o < end) {
-                const uint32_t st = (uint32_t)(cam.stile_base + sy * cam.stiles_x + sx);
-                okeys[o] = st;
-                ovals[o] = item;
-                put_mask(omask, o, (M)tile_mask_general(cam, rg, sx, sy, S));
+        unpack_ranges(ranges[it], rg);
+        uint32_t done = 0;
+        warp_supers(c, inv_s, rg, s_box[threadIdx.x >> 5], [&](int sx, int sy, bool keep) {
+            const uint32_t kept = __ballot_sync(0xffffffffu, keep), k = done + (uint32_t)__popc(kept & ((1u << lane) - 1u));
+            if (keep && k < cn) {
+                const uint32_t st = (uint32_t)(c.stile_base + sy * c.stiles_x + sx);
+                okeys[out + k] = st;
+                ovals[out + k] = it;
+                put_mask(omask, out + k, (M)tile_mask_general(c, rg, sx, sy, S));
                 if (in_bounds(st, (uint64_t)nst, kSiteDupSuper, misc)) atomicAdd(smem ? &sh[st] : &scount[st], 1u);
-                ++o;
             }
+            done += (uint32_t)__popc(kept);
         });
     }
     __syncthreads();
@@ -1287,9 +1348,9 @@ cudaError_t launch_bin_front(const geer_workspace *ws, cudaStream_t s) {
 cudaError_t launch_count_pairs(const geer_workspace *ws, cudaStream_t s) {
     const int64_t m = prep_blocks((int64_t)ws->n_cams * ws->n_gauss);
     if (m > 0) {
-        launch_k(k_gather_counts, dim3((unsigned)m), dim3(kPrepThreads), 0, s, ws->d_cams, ws->d_tile_tab,
-                 ws->n_gauss, ws->super_size, ws->d_iid[0], ws->d_iid[1], ws->d_count, ws->d_ranges, ws->d_misc,
-                 ws->d_blocksum2, ws->d_blocksum3);
+        launch_k(k_gather_counts, dim3((unsigned)((m + kGather - 1) / kGather)), dim3(kPrepThreads), 0, s, ws->d_cams,
+                 ws->n_gauss, ws->super_size, ws->d_iid[0], ws->d_iid[1], ws->d_ranges, ws->d_misc, ws->d_blocksum2,
+                 ws->d_blocksum3, ws->d_ikey[0], ws->d_ikey[1]);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
@@ -1306,7 +1367,7 @@ cudaError_t launch_duplicate(const geer_workspace *ws, cudaStream_t s) {
         const size_t smem = ws->n_stiles <= kSmemTiles ? sizeof(uint32_t) * ws->n_stiles : 0;
         launch_k(mask_words(ws->super_size) == 1 ? k_duplicate<uint32_t> : k_duplicate<uint64_t>, dim3((unsigned)m),
                  dim3(kPrepThreads), smem, s, ws->d_cams, ws->n_gauss, ws->super_size, ws->d_iid[0], ws->d_iid[1],
-                 ws->d_ranges, ws->d_misc, ws->d_blocksum2, ws->d_keys[0], ws->d_vals[0], ws->d_smask[0], scount,
+                 ws->d_ikey[0], ws->d_ikey[1], ws->d_ranges, ws->d_misc, ws->d_blocksum2, ws->d_keys[0], ws->d_vals[0], ws->d_smask[0], scount,
                  (int)ws->n_stiles, ws->cap_pairs);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;

@@ -1,0 +1,110 @@
+"""The per-Gaussian kernels and the binning at the edges of their blocks.
+
+- Rows of SH coefficients copied and written back 16 bytes a lane by whole warps:
+  ragged last warps, every degree, gradients written and added (rows of Gaussians
+  without a gradient untouched), against the oracle with the tolerance of
+  test_gpu_backward.py.
+- More cameras than the 32 whose visibility a Gaussian's thread keeps in a word.
+- Lists of Gaussians whose association is several rectangles (boxes of more than 32
+  super-tiles, several cameras) and item counts around a block, against the replica.
+- More block counts than one step of the scan takes (4096).
+"""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+from paper_2505_24053_gb300 import workloads as wl
+from tests.test_gpu_backward import BLOCKS, _compare, _oracle_grads, _scene
+from tests.test_gpu_forward import _expand_pairs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def geer():
+    from paper_2505_24053_gb300 import geer
+    geer.lib()
+    return geer
+
+
+@pytest.mark.parametrize("deg", [0, 1, 2, 3])
+@pytest.mark.parametrize("n", [1, 31, 33, 63, 65, 97])
+@pytest.mark.parametrize("ncams", [1, 2])
+def test_ragged_rows(geer, orc, n, deg, ncams):
+    scene = _scene(100 * deg + n, n, deg)
+    scene.mean[1::3, 2] *= -1.0  # behind the camera: no gradient
+    cams = [wl.Camera(wl.PINHOLE, 40, 32, math.radians(70)), wl.Camera(wl.PINHOLE, 24, 24, math.radians(60))][:ncams]
+    dL = np.random.default_rng(n).normal(0, 1, (sum(c.pixels for c in cams), 3)).astype(np.float32)
+    r = geer.Renderer(cams, n, deg)
+    g = geer.Gaussians.from_scene(scene)
+    r.forward(g)
+    dL_gpu = torch.as_tensor(dL, device="cuda")
+    new = r.backward(g, dL_gpu)
+    _compare({k: new[k].cpu().numpy().astype(np.float64) for k in BLOCKS}, _oracle_grads(orc, scene, cams, dL), "new")
+    # added to 1: one FP32 addition of the same gradient, itself reproducible to 1e-3 of its largest value
+    r.forward(g)
+    ones = r.backward(g, dL_gpu, {k: torch.ones_like(v) for k, v in new.items()})
+    dead = torch.as_tensor(r.ws.debug_preprocess()[3].reshape(ncams, n).sum(0) == 0, device="cuda")
+    for k in BLOCKS:
+        big = float(new[k].abs().max())
+        assert float((ones[k] - 1 - new[k]).abs().max()) <= 1e-3 * big + 2.0 ** -23 * (1 + big), k
+        assert bool((ones[k][dead] == 1).all()) and bool((new[k][dead] == 0).all()), k
+
+
+def test_more_cameras_than_a_word(geer, orc):
+    n = 40
+    scene = _scene(3, n, 1)
+    cams = []
+    for i in range(35):
+        R, t = wl.pose(wl.rot_y(2 * math.pi * i / 35), (0.1, 0.0, -0.1))
+        cams.append(wl.Camera(wl.PINHOLE, 16, 16, math.radians(60), R_cw=R, t_cw=t))
+    dL = np.random.default_rng(1).normal(0, 1, (sum(c.pixels for c in cams), 3)).astype(np.float32)
+    r = geer.Renderer(cams, n, 1)
+    g = geer.Gaussians.from_scene(scene)
+    r.forward(g)
+    seen = r.ws.debug_preprocess()[3].reshape(35, n) > 0
+    assert seen[:32].any() and seen[32:].any()
+    new = r.backward(g, torch.as_tensor(dL, device="cuda"))
+    _compare({k: new[k].cpu().numpy().astype(np.float64) for k in BLOCKS}, _oracle_grads(orc, scene, cams, dL), "35")
+
+
+@pytest.mark.parametrize("n", [1, 2, 255, 256, 257, 513])
+@pytest.mark.parametrize("px,ncams", [(640, 1), (320, 2)])
+def test_lists_of_several_rectangles(geer, orc, n, px, ncams):
+    rng = np.random.default_rng(n)
+    mean = rng.normal(0, 1, (n, 3))
+    mean[:, 2] *= 0.2  # near the plane where both angles pass 90 degrees
+    mean *= (1.5 + rng.uniform(0, 2, (n, 1))) / np.linalg.norm(mean, axis=1, keepdims=True)
+    scene = wl.Scene(mean.astype(np.float32), np.exp(rng.normal(-2.0, 0.6, (n, 3))).astype(np.float32),
+                     rng.standard_normal((n, 4)).astype(np.float32), rng.uniform(0.1, 0.9, n).astype(np.float32),
+                     rng.normal(0, 0.3, (n, 1, 3)).astype(np.float32), 0)
+    R, t = wl.pose(wl.rot_y(1.0), (0.0, 0.1, 0.0))
+    cams = [wl.Camera(wl.EQUIDISTANT, px, px - 13, math.radians(210)),
+            wl.Camera(wl.EQUIDISTANT, px - 40, px, math.radians(195), R_cw=R, t_cw=t)][:ncams]
+    r = geer.Renderer(cams, n, 0, pair_capacity=1 << 22)
+    r.prepare(geer.Gaussians.from_scene(scene))
+    P, _ = r.ws.pair_counts()
+    k, v = r.ws.debug_pairs(cap=P)
+    ek, ev = _expand_pairs(orc, scene, cams)
+    assert P == ek.size and np.array_equal(k, ek) and np.array_equal(v, ev)
+
+
+def test_more_block_counts_than_a_scan_step(geer):
+    """4097 blocks of Gaussians: every live item in its tiles' lists, in depth order."""
+    n = 4096 * 256 + 17
+    rng = np.random.default_rng(8)
+    mean = np.stack([rng.uniform(-2, 2, n), rng.uniform(-2, 2, n), rng.uniform(1, 6, n)], 1)
+    scene = wl.Scene(mean.astype(np.float32), np.full((n, 3), 1e-3, np.float32),
+                     np.tile(np.float32([1, 0, 0, 0]), (n, 1)), np.full(n, 0.5, np.float32),
+                     np.zeros((n, 1, 3), np.float32), 0)
+    cams = [wl.Camera(wl.PINHOLE, 64, 64, math.radians(90)), wl.Camera(wl.PINHOLE, 48, 64, math.radians(80))]
+    r = geer.Renderer(cams, n, 0, pair_capacity=1 << 22)
+    r.prepare(geer.Gaussians.from_scene(scene))
+    counts = r.ws.debug_preprocess()[3]
+    P, _ = r.ws.pair_counts()
+    k, v = r.ws.debug_pairs(cap=P)
+    assert P == k.size == counts.sum(dtype=np.int64)
+    assert np.array_equal(np.bincount(v, minlength=2 * n), counts)
+    assert (k[1:] >= k[:-1]).all()

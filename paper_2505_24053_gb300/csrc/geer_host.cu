@@ -544,7 +544,6 @@ geer_status geer_workspace_init(void *dev_mem, size_t bytes, const geer_camera *
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&ws->num_sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) { free(ws); return GEER_ERR_CUDA; }
-    ws->sort_grid = ws->num_sms * sort_blocks_per_sm();
     ws->bwd_grid = ws->num_sms * render_bwd_blocks_per_sm(ws->params.alpha_model);
     ws->train_grid = ws->num_sms * render_train_blocks_per_sm(ws->params.alpha_model);
     ws->stage_bytes = sizeof(DevCam) * c.cams + sizeof(float4) * c.tile_tab + sizeof(float2) * c.pix_tab;
@@ -1387,7 +1386,6 @@ extern "C" geer_status geer_render_noalloc(const geer_gaussians *g, const geer_c
     ws.params = Params{params->alpha_min, params->T_min, params->alpha_max, params->lambda_pad, params->assoc,
                        params->snugbox, params->alpha_model};
     ws.num_sms = S.num_sms;
-    ws.sort_grid = S.num_sms * sort_blocks_per_sm();
     ws.n_cams = 1;
     ws.n_pixels = (int64_t)cam->width * cam->height;
     ws.n_tiles = (int64_t)S.cam.tiles_x * S.cam.tiles_y;

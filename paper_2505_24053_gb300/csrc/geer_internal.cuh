@@ -366,7 +366,6 @@ struct geer_workspace {
     bool acc_zero;           // the last preprocess zeroed the items' accumulators; no backward since
     bool queue_ready;        // the last bin_sort reset the fused render's unit queue; not used since
     int sorted_buf;          // which ping-pong buffer holds the sorted super-tile pairs
-    int sort_grid;           // grid of the radix kernels (grid-stride over sort tiles)
     int num_sms;
 
     // pinned staging for asynchronous camera uploads
@@ -424,7 +423,6 @@ cudaError_t launch_opacity_reset(int64_t n, float value, float *logit, float *m_
                                  cudaStream_t s);
 cudaError_t launch_image_metrics(const float *pred, const float *gt, int width, int height, const uint8_t *regions,
                                  int n_regions, double *acc, cudaStream_t s);
-int sort_blocks_per_sm();
 int render_bwd_blocks_per_sm(int alpha_model);
 int render_train_blocks_per_sm(int alpha_model);
 

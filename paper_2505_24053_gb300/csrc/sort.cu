@@ -8,13 +8,16 @@
 //                    group sums down the tiles per digit and the digit totals
 //                    (the digit bases);
 //   k_radix_scatter  per sort tile: stable warp-level ranking (peer masks from a
-//                    per-warp shared atomicOr of lane bits), the tile's offset per
+//                    vote per bit of the digit), the tile's offset per
 //                    digit = digit base + group prefix + sum over the earlier
 //                    tiles of its group, reordering by digit in shared memory and
 //                    contiguous writes of each digit run.
 //
-// Tiles hold 3072 keys. The key count stays on the device: both kernels launch one block per tile of
-// the workspace capacity and the blocks past the count exit at once.
+// Tiles hold 3072 keys. The key count stays on the device. The histogram's blocks go
+// through the tiles, each with the next tile's keys in flight: bound by the latency of
+// a tile's loads, votes and sums, and a block and a fence per tile took 48 us where
+// these take 23 (12M keys; 16 -> 14 us at 3.4M). The scatter launches a block per tile
+// of the workspace capacity and the blocks past the count exit at once.
 #include <algorithm>
 
 #include "geer_internal.cuh"
@@ -47,40 +50,44 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_hist(const uint32_t *__r
                                                              uint32_t *__restrict__ digit_base) {
     grid_dep_sync();
     constexpr int W = kSortThreads / 32, TILE = kSortThreads * ITEMS, GROUP = kGroupTiles;
-    __shared__ uint32_t s_h[W][kRadix];
+    __shared__ uint32_t s_h[2][kRadix];  // this tile's counts and, being cleared, the next one's
     __shared__ uint32_t s_wsum[W];
     __shared__ bool s_is_last;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t n = key_count(misc, count_slot, check_capacity);
-    const uint32_t tile = blockIdx.x;
-    const uint32_t ntiles = (n + TILE - 1) / TILE;
-    if (tile >= ntiles) return;
+    const uint32_t ntiles = (uint32_t)(((uint64_t)n + TILE - 1) / TILE);
+    if (blockIdx.x >= ntiles) return;
     // read before the last block of this pass updates them (it finishes after every block started)
     const int in = dev_buf ? depth_sorted_buf(misc) : 0;
     const uint32_t *__restrict__ kin = in ? kin1 : kin0;
-    for (int i = tid; i < W * kRadix; i += kSortThreads) (&s_h[0][0])[i] = 0u;
-    const uint64_t base = (uint64_t)tile * TILE + (uint64_t)warp * 32 * ITEMS + lane;
     uint32_t key[ITEMS];
+    const auto load = [&](uint32_t tile) {
+        const uint64_t t0 = (uint64_t)tile * TILE;
+        const uint32_t nt = tile < ntiles ? (uint32_t)min((uint64_t)TILE, (uint64_t)n - t0) : 0u;
 #pragma unroll
-    for (int k = 0; k < ITEMS; ++k) {
-        const uint64_t i = base + (uint64_t)k * 32;
-        key[k] = i < n ? kin[i] : 0u;
+        for (int k = 0; k < ITEMS; ++k) key[k] = (uint32_t)(k * kSortThreads + tid) < nt ? kin[t0 + k * kSortThreads + tid] : 0u;
+        return nt;
+    };
+    uint32_t nt = load(blockIdx.x);
+    s_h[0][tid] = 0u;
+    __syncthreads();
+    int b = 0;
+    for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, b ^= 1) {
+#pragma unroll
+        for (int k = 0; k < ITEMS; ++k)
+            if ((uint32_t)(k * kSortThreads + tid) < nt) atomicAdd(&s_h[b][(key[k] >> shift) & 0xffu], 1u);
+        nt = load(tile + gridDim.x);  // the next tile's keys, in flight meanwhile
+        s_h[b ^ 1][tid] = 0u;
+        __syncthreads();
+        const uint32_t c = s_h[b][tid];
+        tile_hist[(uint64_t)tile * kRadix + tid] = c;
+        if (c) atomicAdd(&group_sum[(uint64_t)(tile / GROUP) * kRadix + tid], c);
     }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < ITEMS; ++k)
-        if (base + (uint64_t)k * 32 < n) atomicAdd(&s_h[warp][(key[k] >> shift) & 0xffu], 1u);
-    __syncthreads();
-    uint32_t c = 0;
-#pragma unroll
-    for (int w = 0; w < W; ++w) c += s_h[w][tid];
-    tile_hist[(uint64_t)tile * kRadix + tid] = c;
-    if (c) atomicAdd(&group_sum[(uint64_t)(tile / GROUP) * kRadix + tid], c);
 
     // the last block to finish scans the group sums (threadFenceReduction pattern)
     __threadfence();
     __syncthreads();
-    if (tid == 0) s_is_last = atomicAdd(&misc[kMiscSortDone], 1u) == ntiles - 1u;
+    if (tid == 0) s_is_last = atomicAdd(&misc[kMiscSortDone], 1u) == min(ntiles, gridDim.x) - 1u;
     __syncthreads();
     if (!s_is_last) return;
     __threadfence();
@@ -126,8 +133,12 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_hist(const uint32_t *__r
 // With W > 0 every key also carries W 32-bit words (min_ -> mout_, W per key: the
 // super-tile sort's tile masks), reordered through the values' shared buffer after
 // the values have left it.
+// Bound by the latency of shared memory in the ranking, so by the blocks resident per
+// SM: with the values loaded after the ranking and no shared lane masks (atomics and
+// reads of a mask per digit before) 64 registers hold without values to carry or with
+// one word, 48 with two. 12M keys with two words: 167 -> 137 us; 3.4M without: 40 -> 36.
 template <int ITEMS, int W>
-__global__ void __launch_bounds__(kSortThreads) k_radix_scatter(
+__global__ void __launch_bounds__(kSortThreads, W == 2 ? 5 : 4) k_radix_scatter(
     const uint32_t *__restrict__ kin_, const uint32_t *__restrict__ vin_, uint32_t *__restrict__ kout_,
     uint32_t *__restrict__ vout_, int dev_buf, const uint32_t *__restrict__ misc, int count_slot,
     int check_capacity, int shift, const uint32_t *__restrict__ tile_hist, const uint32_t *__restrict__ group_excl,
@@ -143,7 +154,6 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(
     uint32_t *__restrict__ vout = swap ? const_cast<uint32_t *>(vin_) : vout_;
     constexpr int NW = kSortThreads / 32, TILE = kSortThreads * ITEMS, GROUP = kGroupTiles;
     __shared__ uint32_t s_whist[NW][kRadix];
-    __shared__ uint32_t s_match[NW][kRadix];  // lane masks per digit, zero between ranking steps
     __shared__ uint32_t s_lbase[kRadix];  // start of each digit inside the tile
     __shared__ uint32_t s_out[kRadix];    // global position of the tile's first key of each digit
     __shared__ uint32_t s_wsum[NW];
@@ -153,9 +163,9 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(
     const uint32_t n = key_count(misc, count_slot, check_capacity);
     const uint32_t tile = blockIdx.x;
     if ((uint64_t)tile * TILE >= n) return;
+    const uint64_t t0 = (uint64_t)tile * TILE;
+    const uint32_t nt = (uint32_t)min((uint64_t)TILE, (uint64_t)n - t0);  // keys of the tile
     if (misc[kMiscSortSame]) {  // identity pass: coalesced copy of the tile
-        const uint32_t nt = (uint32_t)min((uint64_t)TILE, (uint64_t)n - (uint64_t)tile * TILE);
-        const uint64_t t0 = (uint64_t)tile * TILE;
         for (uint32_t i = tid; i < nt; i += kSortThreads) {
             kout[t0 + i] = kin[t0 + i];
             vout[t0 + i] = vin[t0 + i];
@@ -165,51 +175,51 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(
         return;
     }
     const uint32_t base_d = digit_base[tid];
-    for (int i = tid; i < NW * kRadix; i += kSortThreads) (&s_match[0][0])[i] = 0u;
     for (int i = tid; i < NW * kRadix; i += kSortThreads) (&s_whist[0][0])[i] = 0u;
     // this tile's global offset for digit tid
     const uint32_t g0 = (tile / GROUP) * GROUP;
     uint32_t off = base_d + group_excl[(uint64_t)(tile / GROUP) * kRadix + tid];
-    uint32_t part[GROUP - 1];
+    static_assert(GROUP % 16 == 0, "the group's tiles in steps of 16");
+#pragma unroll 1
+    for (uint32_t r0 = g0; r0 < tile; r0 += 16) {
+        uint32_t part[16];
 #pragma unroll
-    for (int r = 0; r < GROUP - 1; ++r)
-        part[r] = g0 + r < tile ? tile_hist[(uint64_t)(g0 + r) * kRadix + tid] : 0u;
+        for (int r = 0; r < 16; ++r) part[r] = r0 + r < tile ? tile_hist[(uint64_t)(r0 + r) * kRadix + tid] : 0u;
 #pragma unroll
-    for (int r = 0; r < GROUP - 1; ++r) off += part[r];
+        for (int r = 0; r < 16; ++r) off += part[r];
+    }
     s_out[tid] = off;
     __syncthreads();
 
     uint32_t key[ITEMS], val[ITEMS], rank[ITEMS];
-    const uint64_t base = (uint64_t)tile * TILE + (uint64_t)warp * 32 * ITEMS + lane;
+    const uint32_t base = (uint32_t)(warp * 32 * ITEMS + lane);  // in the tile
+    kin += t0;
+    vin += t0;
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k) key[k] = base + k * 32 < nt ? kin[base + k * 32] : 0u;
+    // stable ranking: warp by warp, item k by item k, lane by lane. The lanes sharing a
+    // digit find each other by a vote per bit of the digit, and all read its count so far.
 #pragma unroll
     for (int k = 0; k < ITEMS; ++k) {
-        const uint64_t i = base + (uint64_t)k * 32;
-        const bool v = i < n;
-        key[k] = v ? kin[i] : 0u;
-        val[k] = v ? vin[i] : 0u;
-    }
-    // stable ranking: warp by warp, item k by item k, lane by lane. The lanes
-    // sharing a digit find each other through a per-warp shared mask per digit
-    // (atomicOr of the lane bits), cleared again by the group leader.
-#pragma unroll
-    for (int k = 0; k < ITEMS; ++k) {
-        const bool v = base + (uint64_t)k * 32 < n;
+        const bool v = base + k * 32 < nt;
         const uint32_t d = (key[k] >> shift) & 0xffu;
-        if (v) atomicOr(&s_match[warp][d], 1u << lane);
-        __syncwarp();
-        const uint32_t peers = v ? s_match[warp][d] : 0u;
-        __syncwarp();
-        const int leader = __ffs(peers) - 1;
-        uint32_t b = 0;
-        if (v && lane == leader) {
-            b = s_whist[warp][d];
-            s_whist[warp][d] = b + __popc(peers);
-            s_match[warp][d] = 0u;
+        uint32_t peers = __ballot_sync(0xffffffffu, v);
+#pragma unroll
+        for (int b = 0; b < kRadixBits; ++b) {
+            const bool bit = (d >> b) & 1u;
+            const uint32_t m = __ballot_sync(0xffffffffu, bit);
+            peers &= bit ? m : ~m;
         }
-        b = __shfl_sync(0xffffffffu, b, leader < 0 ? 0 : leader);
-        rank[k] = v ? b + __popc(peers & lanemask_lt()) : 0xffffffffu;
+        const uint32_t b = s_whist[warp][d];
+        const uint32_t before = (uint32_t)__popc(peers & lanemask_lt());
+        __syncwarp();
+        if (v && before == 0) s_whist[warp][d] = b + (uint32_t)__popc(peers);
+        rank[k] = v ? b + before : 0xffffffffu;
         __syncwarp();
     }
+    // the values, needed from here on only (held through the ranking they cost a block per SM)
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k) val[k] = base + k * 32 < nt ? vin[base + k * 32] : 0u;
     __syncthreads();
     // warp offsets inside the tile per digit, tile count per digit
     uint32_t cnt = 0;
@@ -246,7 +256,6 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(
     }
     __syncthreads();
     // contiguous writes of each digit run
-    const uint32_t nt = (uint32_t)min((uint64_t)TILE, (uint64_t)n - (uint64_t)tile * TILE);
 #pragma unroll
     for (int k = 0; k < ITEMS; ++k) {
         const uint32_t lp = (uint32_t)(k * kSortThreads + tid);
@@ -264,10 +273,7 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(
     for (int w = 0; w < W; ++w) {
         uint32_t m[ITEMS];
 #pragma unroll
-        for (int k = 0; k < ITEMS; ++k) {
-            const uint64_t i = base + (uint64_t)k * 32;
-            m[k] = i < n ? min_[i * W + w] : 0u;
-        }
+        for (int k = 0; k < ITEMS; ++k) m[k] = base + k * 32 < nt ? min_[(t0 + base + k * 32) * W + w] : 0u;
         __syncthreads();  // s_val has been read
 #pragma unroll
         for (int k = 0; k < ITEMS; ++k)
@@ -287,14 +293,6 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(
 
 }  // namespace
 
-int sort_blocks_per_sm() {
-    int b = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_radix_scatter<kSortItems, 0>, kSortThreads, 0) !=
-        cudaSuccess)
-        b = 1;
-    return b < 1 ? 1 : b;
-}
-
 // One stable pass over digit `pass` of the keys in buffer `cur` (count in
 // misc[slot]); with dev_buf the buffers are chosen on the device and a pass
 // whose digit is the same for every key is skipped. mbuf (words > 0): the 32-bit
@@ -307,7 +305,8 @@ static cudaError_t radix_pass(geer_workspace *ws, uint32_t *const kbuf[2], uint3
     constexpr int TILE = kSortThreads * kSortItems;
     const int shift = kRadixBits * pass;
     const unsigned tiles = (unsigned)std::max<int64_t>(1, (cap_keys + TILE - 1) / TILE);
-    launch_k(k_radix_hist<kSortItems>, dim3(tiles), dim3(kSortThreads), 0, s, kbuf[cur], kbuf[cur ^ 1], dev_buf,
+    const unsigned hist_blocks = std::min(tiles, (unsigned)(ws->num_sms * 8));
+    launch_k(k_radix_hist<kSortItems>, dim3(hist_blocks), dim3(kSortThreads), 0, s, kbuf[cur], kbuf[cur ^ 1], dev_buf,
              ws->d_misc, slot, check, shift, ws->d_tile_hist, ws->d_group_sum, ws->d_group_excl, ws->d_digit_base);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;

@@ -108,3 +108,27 @@ def test_more_block_counts_than_a_scan_step(geer):
     assert P == k.size == counts.sum(dtype=np.int64)
     assert np.array_equal(np.bincount(v, minlength=2 * n), counts)
     assert (k[1:] >= k[:-1]).all()
+
+
+def test_more_sort_tiles_than_blocks(geer):
+    """More live items and (super-tile, item) pairs than the 3.7M keys that one
+    round of the histogram's blocks takes on 152 SMs. Depth order inside each tile,
+    equal depths (the same camera twice) in item order."""
+    n = 1_100_000
+    rng = np.random.default_rng(9)
+    z = rng.uniform(1, 6, n)
+    mean = np.stack([rng.uniform(-0.4, 0.4, n) * z, rng.uniform(-0.4, 0.4, n) * z, z], 1)
+    scene = wl.Scene(mean.astype(np.float32), np.full((n, 3), 1e-3, np.float32),
+                     np.tile(np.float32([1, 0, 0, 0]), (n, 1)), np.full(n, 0.5, np.float32),
+                     np.zeros((n, 1, 3), np.float32), 0)
+    r = geer.Renderer([wl.Camera(wl.PINHOLE, 128, 128, math.radians(60))] * 4, n, 0, pair_capacity=1 << 23)
+    r.prepare(geer.Gaussians.from_scene(scene))
+    counts = r.ws.debug_preprocess()[3]
+    P, supers = r.ws.pair_counts()
+    assert supers > 3_800_000
+    k, v = r.ws.debug_pairs(cap=P)
+    assert P == k.size == counts.sum(dtype=np.int64)
+    assert np.array_equal(np.bincount(v, minlength=4 * n), counts)
+    assert (k[1:] >= k[:-1]).all()
+    same = k[1:] == k[:-1]
+    assert same.any() and (v[1:][same] > v[:-1][same]).all()

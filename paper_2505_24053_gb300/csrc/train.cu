@@ -6,11 +6,11 @@
 // and opacity = sigmoid(logit); the chain rule is applied here, and the
 // activated values of the updated parameters are written for the next render.
 //
-// The raw parameters, the gradients and the moments m, v are addressed by one
-// flat element index over the groups [mean 3n | log-scale 3n | quat 4n |
-// logit n | sh 3Kn] (K = (deg + 1)^2); a thread updates four consecutive
-// elements with 128-bit accesses when the layout allows it, else one (all
-// elementwise, HBM-bound: 16 B read and 12-16 B written per element).
+// The moments m, v are flat over the groups [mean 3n | log-scale 3n | quat 4n |
+// logit n | sh 3Kn] (K = (deg + 1)^2). A block takes 1024 elements of one group, four a
+// thread, a block's width apart: every access coalesced whatever the group's alignment
+// in the flat moments, all loads in flight before the first use (elementwise,
+// HBM-bound: 16 B read and 12-16 B written per element).
 #include <cmath>
 
 #include "geer_internal.cuh"
@@ -23,123 +23,71 @@ struct AdamConst {
     float b1, b2, eps, inv_bc1, inv_bc2;  // inv_bc: 1 / (1 - beta^t)
 };
 
-__global__ void __launch_bounds__(256) k_adam_gaussians(AdamConst hp, int64_t n, int K3, float *__restrict__ mean,
-                                                        float *__restrict__ log_scale, float *__restrict__ quat,
-                                                        float *__restrict__ logit, float *__restrict__ sh,
-                                                        const float *__restrict__ d_mean,
-                                                        const float *__restrict__ d_scale,
-                                                        const float *__restrict__ d_quat,
-                                                        const float *__restrict__ d_opacity,
-                                                        const float *__restrict__ d_sh, float *__restrict__ m,
-                                                        float *__restrict__ v, float *__restrict__ scale,
-                                                        float *__restrict__ opacity) {
-    grid_dep_sync();
-    const int64_t total = n * (11 + (int64_t)K3);
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        float *p;
-        float g, lr;
-        int group;  // 1: log-scale, 3: logit (activated outputs), else none
-        int64_t off;
-        if (e < 3 * n) {
-            off = e; p = mean + off; g = d_mean[off]; lr = hp.lr[0]; group = 0;
-        } else if (e < 6 * n) {
-            off = e - 3 * n; p = log_scale + off; g = d_scale[off]; lr = hp.lr[1]; group = 1;
-        } else if (e < 10 * n) {
-            off = e - 6 * n; p = quat + off; g = d_quat[off]; lr = hp.lr[2]; group = 2;
-        } else if (e < 11 * n) {
-            off = e - 10 * n; p = logit + off; g = d_opacity[off]; lr = hp.lr[3]; group = 3;
-        } else {
-            off = e - 11 * n; p = sh + off; g = d_sh[off]; group = 4;
-            lr = ((uint64_t)off % (uint32_t)K3) < 3 ? hp.lr[4] : hp.lr[5];  // first 3 SH values: degree 0
-        }
-        const float x = *p;
-        if (group == 1) {
-            g *= expf(x);  // d scale / d log-scale = scale
-        } else if (group == 3) {
-            const float s = 1.0f / (1.0f + expf(-x));
-            g *= s * (1.0f - s);  // d sigmoid / d logit
-        }
-        const float mm = hp.b1 * m[e] + (1.0f - hp.b1) * g;
-        const float vv = hp.b2 * v[e] + (1.0f - hp.b2) * g * g;
-        m[e] = mm;
-        v[e] = vv;
-        const float xn = x - lr * (mm * hp.inv_bc1) / (sqrtf(vv * hp.inv_bc2) + hp.eps);
-        *p = xn;
-        if (group == 1 && scale) scale[off] = expf(xn);
-        if (group == 3 && opacity) opacity[off] = 1.0f / (1.0f + expf(-xn));
-    }
-}
+enum : int { kGroupMean, kGroupScale, kGroupQuat, kGroupOpacity, kGroupSh, kGroups };
 
-// Four consecutive elements per thread with 128-bit accesses, for n % 4 == 0
-// (the group boundaries 3n, 6n, 10n, 11n are then multiples of 4, so a chunk
-// never straddles two groups) and 16-byte aligned arrays.
-__device__ __forceinline__ float adam_one(const AdamConst &hp, float x, float g, float &m, float &v, float lr) {
-    m = hp.b1 * m + (1.0f - hp.b1) * g;
-    v = hp.b2 * v + (1.0f - hp.b2) * g * g;
-    return x - lr * (m * hp.inv_bc1) / (sqrtf(v * hp.inv_bc2) + hp.eps);
-}
-
-__global__ void __launch_bounds__(256) k_adam_gaussians4(AdamConst hp, int64_t n, int K3, float *__restrict__ mean,
-                                                         float *__restrict__ log_scale, float *__restrict__ quat,
-                                                         float *__restrict__ logit, float *__restrict__ sh,
-                                                         const float *__restrict__ d_mean,
-                                                         const float *__restrict__ d_scale,
-                                                         const float *__restrict__ d_quat,
-                                                         const float *__restrict__ d_opacity,
-                                                         const float *__restrict__ d_sh, float *__restrict__ m,
-                                                         float *__restrict__ v, float *__restrict__ scale,
-                                                         float *__restrict__ opacity) {
-    grid_dep_sync();
-    const int64_t chunks = n * (11 + (int64_t)K3) / 4;
-    const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= chunks) return;
-    const int64_t e = 4 * c;
+// One parameter group: values, gradients, the activated output (or null), its first
+// element in the flat moments, its elements and its first block.
+struct AdamGroup {
     float *p;
-    const float *gp;
-    int group;
-    int64_t off;
-    if (e < 3 * n) { off = e; p = mean; gp = d_mean; group = 0; }
-    else if (e < 6 * n) { off = e - 3 * n; p = log_scale; gp = d_scale; group = 1; }
-    else if (e < 10 * n) { off = e - 6 * n; p = quat; gp = d_quat; group = 2; }
-    else if (e < 11 * n) { off = e - 10 * n; p = logit; gp = d_opacity; group = 3; }
-    else { off = e - 11 * n; p = sh; gp = d_sh; group = 4; }
-    float4 x = *reinterpret_cast<const float4 *>(p + off);
-    float4 g = *reinterpret_cast<const float4 *>(gp + off);
-    float4 mm = *reinterpret_cast<const float4 *>(m + e);
-    float4 vv = *reinterpret_cast<const float4 *>(v + e);
-    float lr[4];
-    if (group < 4) {
-        lr[0] = lr[1] = lr[2] = lr[3] = hp.lr[group];
-    } else {
-        const int base = (int)((uint64_t)off % (uint32_t)K3);  // position in the Gaussian's SH row
+    const float *g;
+    float *out;
+    int64_t e0, count, block0;
+};
+struct AdamGroups {
+    AdamGroup g[kGroups];
+};
+
+constexpr int kAdamThreads = 256, kAdamItems = 4, kAdamChunk = kAdamThreads * kAdamItems;
+
+// (1,093,217 Gaussians of SH degree 3, 64.5M elements: 258 us, where one element a thread
+// with the group and the SH position looked up per element took 528; four neighbouring
+// elements a thread with 128-bit accesses, possible for n % 4 == 0 only: 259. With two elements a thread 277, with eight 263.)
+__global__ void __launch_bounds__(kAdamThreads) k_adam_gaussians(AdamConst hp, AdamGroups gs, int K3,
+                                                                 float *__restrict__ m, float *__restrict__ v) {
+    grid_dep_sync();
+    int group = 0;
+    while (group + 1 < kGroups && (int64_t)blockIdx.x >= gs.g[group + 1].block0) ++group;
+    const AdamGroup &G = gs.g[group];
+    const int64_t off0 = ((int64_t)blockIdx.x - G.block0) * kAdamChunk;
+    const int left = (int)min((int64_t)kAdamChunk, G.count - off0);
+    float *__restrict__ p = G.p + off0;
+    const float *__restrict__ gp = G.g + off0;
+    float *__restrict__ mp = m + G.e0 + off0, *__restrict__ vp = v + G.e0 + off0;
+    float x[kAdamItems], g[kAdamItems], mm[kAdamItems], vv[kAdamItems];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int pos = base + i >= K3 ? base + i - K3 : base + i;
-            lr[i] = pos < 3 ? hp.lr[4] : hp.lr[5];
+    for (int k = 0; k < kAdamItems; ++k) {
+        const int i = k * kAdamThreads + threadIdx.x;
+        if (i < left) {
+            x[k] = p[i];
+            g[k] = gp[i];
+            mm[k] = mp[i];
+            vv[k] = vp[i];
         }
     }
-    float *xs = &x.x, *gs = &g.x, *ms = &mm.x, *vs = &vv.x;
+    // the chunk's first position in its Gaussian's SH row (block-uniform)
+    const uint32_t row0 = group == kGroupSh ? (uint32_t)((uint64_t)off0 % (uint32_t)K3) : 0u;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        float gi = gs[i];
-        if (group == 1) {
-            gi *= expf(xs[i]);
-        } else if (group == 3) {
-            const float sg = 1.0f / (1.0f + expf(-xs[i]));
-            gi *= sg * (1.0f - sg);
+    for (int k = 0; k < kAdamItems; ++k) {
+        const int i = k * kAdamThreads + threadIdx.x;
+        if (i >= left) break;
+        float lr = hp.lr[group];
+        if (group == kGroupSh && (row0 + (uint32_t)i) % (uint32_t)K3 >= 3u) lr = hp.lr[kGroups];
+        float gi = g[k];
+        if (group == kGroupScale) {
+            gi *= expf(x[k]);  // d scale / d log-scale = scale
+        } else if (group == kGroupOpacity) {
+            const float s = 1.0f / (1.0f + expf(-x[k]));
+            gi *= s * (1.0f - s);  // d sigmoid / d logit
         }
-        xs[i] = adam_one(hp, xs[i], gi, ms[i], vs[i], lr[i]);
+        const float m1 = hp.b1 * mm[k] + (1.0f - hp.b1) * gi;
+        const float v1 = hp.b2 * vv[k] + (1.0f - hp.b2) * gi * gi;
+        const float xn = x[k] - lr * (m1 * hp.inv_bc1) / (sqrtf(v1 * hp.inv_bc2) + hp.eps);
+        p[i] = xn;
+        mp[i] = m1;
+        vp[i] = v1;
+        if (G.out && group == kGroupScale) G.out[off0 + i] = expf(xn);
+        if (G.out && group == kGroupOpacity) G.out[off0 + i] = 1.0f / (1.0f + expf(-xn));
     }
-    *reinterpret_cast<float4 *>(p + off) = x;
-    *reinterpret_cast<float4 *>(m + e) = mm;
-    *reinterpret_cast<float4 *>(v + e) = vv;
-    if (group == 1 && scale)
-        *reinterpret_cast<float4 *>(scale + off) = make_float4(expf(x.x), expf(x.y), expf(x.z), expf(x.w));
-    if (group == 3 && opacity)
-        *reinterpret_cast<float4 *>(opacity + off) =
-            make_float4(1.0f / (1.0f + expf(-x.x)), 1.0f / (1.0f + expf(-x.y)), 1.0f / (1.0f + expf(-x.z)),
-                        1.0f / (1.0f + expf(-x.w)));
 }
 
 }  // namespace
@@ -163,20 +111,18 @@ cudaError_t launch_adam_gaussians(const geer_adam *hp, int64_t n, int32_t sh_deg
     c.inv_bc1 = (float)(1.0 / (1.0 - std::pow((double)hp->beta1, (double)hp->step)));
     c.inv_bc2 = (float)(1.0 / (1.0 - std::pow((double)hp->beta2, (double)hp->step)));
     const int K3 = 3 * (sh_degree + 1) * (sh_degree + 1);
-    const int64_t total = n * (11 + (int64_t)K3);
-    auto a16 = [](const void *q) { return q == nullptr || (reinterpret_cast<uintptr_t>(q) & 15u) == 0; };
-    const bool vec = n % 4 == 0 && a16(mean) && a16(log_scale) && a16(quat) && a16(logit_opacity) && a16(sh) &&
-                     a16(d_mean) && a16(d_scale) && a16(d_quat) && a16(d_opacity) && a16(d_sh) && a16(m) &&
-                     a16(v) && a16(scale) && a16(opacity);
-    if (vec) {
-        const int64_t blocks = (total / 4 + 255) / 256;
-        launch_k(k_adam_gaussians4, dim3((unsigned)blocks), dim3(256), 0, s, c, n, K3, mean, log_scale, quat,
-                 logit_opacity, sh, d_mean, d_scale, d_quat, d_opacity, d_sh, m, v, scale, opacity);
-    } else {
-        const int64_t blocks = std::min<int64_t>((total + 255) / 256, (int64_t)1 << 30);
-        launch_k(k_adam_gaussians, dim3((unsigned)blocks), dim3(256), 0, s, c, n, K3, mean, log_scale, quat,
-                 logit_opacity, sh, d_mean, d_scale, d_quat, d_opacity, d_sh, m, v, scale, opacity);
+    AdamGroups gs = {{{mean, d_mean, nullptr, 0, 3 * n, 0},
+                             {log_scale, d_scale, scale, 3 * n, 3 * n, 0},
+                             {quat, d_quat, nullptr, 6 * n, 4 * n, 0},
+                             {logit_opacity, d_opacity, opacity, 10 * n, n, 0},
+                             {sh, d_sh, nullptr, 11 * n, K3 * n, 0}}};
+    int64_t blocks = 0;
+    for (AdamGroup &g : gs.g) {
+        g.block0 = blocks;
+        blocks += (g.count + kAdamChunk - 1) / kAdamChunk;
     }
+    if (blocks > 0x7fffffffll) return cudaErrorInvalidValue;
+    launch_k(k_adam_gaussians, dim3((unsigned)blocks), dim3(kAdamThreads), 0, s, c, gs, K3, m, v);
     return cudaGetLastError();
 }
 

@@ -152,36 +152,88 @@ __global__ void __launch_bounds__(kDensThreads) k_densify_offsets(int64_t n, con
     if (g < n) out_off[g] = blockoff[blockIdx.x] + pre;
 }
 
-// One array of `width` floats per Gaussian (a parameter or a moment group),
-// element-parallel so that reads and writes are coalesced: a kept Gaussian's
-// row to its output row, a clone's to both rows, a split Gaussian's to both
-// children (mean and log-scale: skip_split, written by k_densify_split).
-// zero_new: a moment group (the clone's copy and split children start at 0).
-// act 1: also write exp of the values (activated scale), 2: their sigmoid
-// (activated opacity) into aux.
-__global__ void __launch_bounds__(kDensThreads) k_densify_copy(int64_t n, int64_t no, int width,
-                                                               const float *__restrict__ src, float *__restrict__ dst,
-                                                               int zero_new, int skip_split, int act,
-                                                               float *__restrict__ aux,
+// The arrays of `W` floats per Gaussian that a refinement rewrites.
+struct CopyArray {
+    const float *src;
+    float *dst, *aux;
+};
+struct CopyArgs {
+    CopyArray p[5], m[5], v[5];  // parameters and both moments: mean, log-scale, quat, logit, sh
+};
+
+// A block's rows of one array, element-parallel so that reads and writes are
+// coalesced: a kept Gaussian's row to its output row, a clone's to both rows, a split
+// Gaussian's to both children (SKIP_SPLIT: mean and log-scale, written by
+// k_densify_split). MOMENT: the clone's copy and split children start at 0. ACT 1:
+// also write exp of the values (activated scale), 2: their sigmoid (activated opacity)
+// into aux. s_act: action, s_off: first output row.
+template <int W, bool MOMENT, bool SKIP_SPLIT, int ACT>
+__device__ __forceinline__ void copy_rows(const CopyArray &A, int64_t g0, int rows, const uint8_t *s_act,
+                                          const uint32_t *s_off) {
+    constexpr int kBatch = W < 8 ? W : 8;  // elements in flight per thread (W of them cover a block's rows)
+    const float *__restrict__ src = A.src + g0 * W;
+    const int total = rows * W;
+#pragma unroll 1
+    for (int i0 = threadIdx.x; i0 < total; i0 += kBatch * kDensThreads) {
+        float x[kBatch];
+#pragma unroll
+        for (int b = 0; b < kBatch; ++b) {
+            const int i = i0 + b * kDensThreads;
+            if (i < total) x[b] = src[i];
+        }
+#pragma unroll
+        for (int b = 0; b < kBatch; ++b) {
+            const int i = i0 + b * kDensThreads;
+            if (i >= total) break;
+            const int r = i / W;
+            const uint8_t ac = s_act[r];
+            if (ac == kActPrune || (SKIP_SPLIT && ac == kActSplit)) continue;
+            const int64_t d = (int64_t)s_off[r] * W + (i - r * W);
+            A.dst[d] = MOMENT && ac == kActSplit ? 0.0f : x[b];
+            if (ac != kActKeep) A.dst[d + W] = MOMENT ? 0.0f : x[b];
+            if (ACT && A.aux) {
+                const float y = ACT == 1 ? expf(x[b]) : 1.0f / (1.0f + expf(-x[b]));
+                A.aux[d] = y;
+                if (ac != kActKeep) A.aux[d + W] = y;
+            }
+        }
+    }
+}
+
+// Every array's rows of kDensThreads Gaussians, blockIdx.y choosing between the
+// parameters and the two moments. Bound by HBM. (1M Gaussians of SH degree 3: 230 us,
+// where a launch per array with a 64-bit division per element took 850.)
+template <int DEG>
+__global__ void __launch_bounds__(kDensThreads) k_densify_copy(int64_t n, int64_t no, CopyArgs args,
                                                                const uint8_t *__restrict__ action,
                                                                const uint32_t *__restrict__ out_off) {
     grid_dep_sync();
-    const int64_t idx = (int64_t)blockIdx.x * kDensThreads + threadIdx.x;
-    if (idx >= n * width) return;
-    const int64_t g = idx / width;
-    const int a = (int)(idx - g * width);
-    const uint8_t ac = action[g];
-    if (ac == kActPrune || (skip_split && ac == kActSplit)) return;
-    const int64_t o = out_off[g];
-    if (o + (int64_t)outputs_of(ac) > no) return;  // a plan that does not match: nothing written out of bounds
-    const float x = src[idx];
-    const float x0 = (zero_new && ac == kActSplit) ? 0.0f : x, x1 = zero_new ? 0.0f : x;
-    dst[o * width + a] = x0;
-    if (ac != kActKeep) dst[(o + 1) * width + a] = x1;
-    if (act && aux) {
-        const float y = act == 1 ? expf(x) : 1.0f / (1.0f + expf(-x));
-        aux[o * width + a] = y;
-        if (ac != kActKeep) aux[(o + 1) * width + a] = y;
+    constexpr int K3 = 3 * (DEG + 1) * (DEG + 1);
+    __shared__ uint8_t s_act[kDensThreads];
+    __shared__ uint32_t s_off[kDensThreads];
+    const int64_t g0 = (int64_t)blockIdx.x * kDensThreads;
+    const int rows = (int)min((int64_t)kDensThreads, n - g0);
+    if ((int)threadIdx.x < rows) {
+        uint8_t a = action[g0 + threadIdx.x];
+        const uint32_t o = out_off[g0 + threadIdx.x];
+        if ((int64_t)o + outputs_of(a) > no) a = kActPrune;  // a plan that does not match: nothing written out of bounds
+        s_act[threadIdx.x] = a;
+        s_off[threadIdx.x] = o;
+    }
+    __syncthreads();
+    if (blockIdx.y == 0) {
+        copy_rows<3, false, true, 0>(args.p[0], g0, rows, s_act, s_off);
+        copy_rows<3, false, true, 1>(args.p[1], g0, rows, s_act, s_off);
+        copy_rows<4, false, false, 0>(args.p[2], g0, rows, s_act, s_off);
+        copy_rows<1, false, false, 2>(args.p[3], g0, rows, s_act, s_off);
+        copy_rows<K3, false, false, 0>(args.p[4], g0, rows, s_act, s_off);
+    } else {
+        const CopyArray *mom = blockIdx.y == 1 ? args.m : args.v;
+        copy_rows<3, true, false, 0>(mom[0], g0, rows, s_act, s_off);
+        copy_rows<3, true, false, 0>(mom[1], g0, rows, s_act, s_off);
+        copy_rows<4, true, false, 0>(mom[2], g0, rows, s_act, s_off);
+        copy_rows<1, true, false, 0>(mom[3], g0, rows, s_act, s_off);
+        copy_rows<K3, true, false, 0>(mom[4], g0, rows, s_act, s_off);
     }
 }
 
@@ -293,27 +345,26 @@ cudaError_t launch_densify_apply(int64_t n, int32_t sh_degree, const float *mean
     const int64_t no = n_out;
     // the moments' flat groups: [mean 3 | log-scale 3 | quat 4 | logit 1 | sh K3] per Gaussian
     const int wd[5] = {3, 3, 4, 1, K3};
+    CopyArgs args = {{{mean, o_mean, nullptr},
+                      {log_scale, o_log_scale, o_scale},
+                      {quat, o_quat, nullptr},
+                      {logit, o_logit, o_opacity},
+                      {sh, o_sh, nullptr}},
+                     {},
+                     {}};
     int64_t gi = 0, go = 0;
     for (int grp = 0; grp < 5; ++grp) {
-        const int w = wd[grp];
-        const unsigned blocks = (unsigned)((n * w + kDensThreads - 1) / kDensThreads);
-        launch_k(k_densify_copy, dim3(blocks), dim3(kDensThreads), 0, s, n, no, w, m + gi, o_m + go, 1, 0, 0,
-                 (float *)nullptr, action, (const uint32_t *)off);
-        launch_k(k_densify_copy, dim3(blocks), dim3(kDensThreads), 0, s, n, no, w, v + gi, o_v + go, 1, 0, 0,
-                 (float *)nullptr, action, (const uint32_t *)off);
-        gi += w * n;
-        go += w * no;
+        args.m[grp] = {m + gi, o_m + go, nullptr};
+        args.v[grp] = {v + gi, o_v + go, nullptr};
+        gi += wd[grp] * n;
+        go += wd[grp] * no;
     }
-    const float *src[5] = {mean, log_scale, quat, logit, sh};
-    float *dst[5] = {o_mean, o_log_scale, o_quat, o_logit, o_sh};
-    float *aux[5] = {nullptr, o_scale, nullptr, o_opacity, nullptr};
-    const int act[5] = {0, 1, 0, 2, 0};
-    for (int grp = 0; grp < 5; ++grp) {
-        const int w = wd[grp];
-        const unsigned blocks = (unsigned)((n * w + kDensThreads - 1) / kDensThreads);
-        launch_k(k_densify_copy, dim3(blocks), dim3(kDensThreads), 0, s, n, no, w, src[grp], dst[grp], 0,
-                 grp < 2 ? 1 : 0, act[grp], aux[grp], action, (const uint32_t *)off);
-    }
+    auto *copy = sh_degree == 0   ? k_densify_copy<0>
+                 : sh_degree == 1 ? k_densify_copy<1>
+                 : sh_degree == 2 ? k_densify_copy<2>
+                                  : k_densify_copy<3>;
+    launch_k(copy, dim3((unsigned)dens_blocks(n), 3), dim3(kDensThreads), 0, s, n, no, args, action,
+             (const uint32_t *)off);
     launch_k(k_densify_split, dim3((unsigned)dens_blocks(n)), dim3(kDensThreads), 0, s, n, no, mean, log_scale, quat,
              z, action, (const uint32_t *)off, o_mean, o_log_scale, o_scale);
     return cudaGetLastError();

@@ -42,7 +42,7 @@ def flags(verbose_ptxas: bool = False) -> list[str]:
 def _stale(obj: str, src: str) -> bool:
     if not os.path.exists(obj):
         return True
-    deps = [src, os.path.join(CSRC, "geer_internal.cuh"), os.path.join(HERE, "..", "include", "geer.h"), __file__]
+    deps = [src, os.path.join(CSRC, "geer_internal.cuh"), os.path.join(CSRC, "kb_angles.h"), os.path.join(HERE, "..", "include", "geer.h"), __file__]
     return any(os.path.getmtime(d) > os.path.getmtime(obj) for d in deps)
 
 

@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "geer_internal.cuh"
+#include "kb_angles.h"
 
 using namespace geer;
 
@@ -25,12 +26,6 @@ struct Layout {
 
 int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
-// Kannala-Brandt distorted angle phi (1 + k1 phi^2 + k2 phi^4 + k3 phi^6 + k4 phi^8) (App. E).
-double kb_theta_d(const float k[4], double phi) {
-    const double p2 = phi * phi;
-    return phi * (1.0 + p2 * (k[0] + p2 * (k[1] + p2 * (k[2] + p2 * k[3]))));
-}
-
 // Vertical BEAP field of view: the vertical half-angle that the focal length
 // mapping fov_x/2 to w/2 maps to h/2 (pinhole: tan; equidistant: linear;
 // Kannala-Brandt: smallest root of the distortion polynomial).
@@ -39,25 +34,7 @@ double derived_fov_y(const geer_camera &c) {
     const double fx = c.fov_x, w = c.width, h = c.height;
     if (c.model == GEER_PINHOLE) return 2.0 * atan(tan(0.5 * fx) * h / w);
     if (c.model == GEER_EQUIDISTANT) return fx * h / w;
-    const double edge = kb_theta_d(c.k, 0.5 * fx);
-    if (!(edge > 0.0)) return NAN;
-    const double target = edge * h / w;
-    // bracket the first crossing on a fine grid, then bisect
-    double lo = 0.0, hi = 0.5 * fx;
-    const int n = 8192;
-    for (int s = 1; s <= n; ++s) {
-        const double ph = 0.5 * fx * s / n;
-        if (kb_theta_d(c.k, ph) >= target) {
-            hi = ph;
-            lo = 0.5 * fx * (s - 1) / n;
-            break;
-        }
-    }
-    for (int it = 0; it < 200; ++it) {
-        const double mid = 0.5 * (lo + hi);
-        if (kb_theta_d(c.k, mid) >= target) hi = mid; else lo = mid;
-    }
-    return 2.0 * hi;
+    return kb_fov_y(c.k, fx, w, h);
 }
 
 // BEAP pixel-centre angle (Sec. 3.3): ((i + 1/2)/w - 1/2) FoV.
@@ -194,6 +171,7 @@ void build_tables(const geer_camera *cams, int n, CamTables &out, const uint8_t 
         d.col_ppr = (float)(c.width / fx);
         d.row_ppr = (float)(c.height / fy);
         d.tcol_off = (int32_t)out.ttab.size();
+        d.pcol_off = (int32_t)out.ptab.size();
         for (int tx = 0; tx < d.tiles_x; ++tx) {
             const int i0 = tx * kTile, i1 = std::min(i0 + kTile - 1, c.width - 1);
             float4 v;
@@ -202,13 +180,15 @@ void build_tables(const geer_camera *cams, int n, CamTables &out, const uint8_t 
             v.z = 0.0f;
             v.w = 0.0f;
             for (int i = i0; i <= i1; ++i) {
-                const double cs = cos(beap_angle(i, c.width, fx));
+                const double a = beap_angle(i, c.width, fx), cs = cos(a);
+                out.ptab.push_back(make_float2((float)sin(a), (float)cs));
                 if (cs > -1e-12) v.z = 1.0f;
                 if (cs < 1e-12) { v.w = 1.0f; d.any_col_flip = 1; }
             }
             out.ttab.push_back(v);
         }
         d.trow_off = (int32_t)out.ttab.size();
+        d.prow_off = (int32_t)out.ptab.size();
         for (int ty = 0; ty < d.tiles_y; ++ty) {
             const int j0 = ty * kTile, j1 = std::min(j0 + kTile - 1, c.height - 1);
             float4 v;
@@ -217,21 +197,12 @@ void build_tables(const geer_camera *cams, int n, CamTables &out, const uint8_t 
             v.z = 0.0f;
             v.w = 0.0f;
             for (int j = j0; j <= j1; ++j) {
-                const double cs = cos(beap_angle(j, c.height, fy));
+                const double a = beap_angle(j, c.height, fy), cs = cos(a);
+                out.ptab.push_back(make_float2((float)sin(a), (float)cs));
                 if (cs > -1e-12) v.z = 1.0f;
                 if (cs < 1e-12) { v.w = 1.0f; d.any_row_flip = 1; }
             }
             out.ttab.push_back(v);
-        }
-        d.pcol_off = (int32_t)out.ptab.size();
-        for (int i = 0; i < c.width; ++i) {
-            const double a = beap_angle(i, c.width, fx);
-            out.ptab.push_back(make_float2((float)sin(a), (float)cos(a)));
-        }
-        d.prow_off = (int32_t)out.ptab.size();
-        for (int j = 0; j < c.height; ++j) {
-            const double a = beap_angle(j, c.height, fy);
-            out.ptab.push_back(make_float2((float)sin(a), (float)cos(a)));
         }
         out.ok &= flag_intervals(out.ttab.data() + d.tcol_off, d.tiles_x, d.zc, d.wc);
         out.ok &= flag_intervals(out.ttab.data() + d.trow_off, d.tiles_y, d.zr, d.wr);
@@ -1023,16 +994,8 @@ static void native_params(const geer_camera *cam, double &fy, double &focal, dou
         float k0[4] = {0, 0, 0, 0};
         const float *k = cam->model == GEER_KANNALA_BRANDT ? cam->k : k0;
         focal = 0.5 * cam->width / kb_theta_d(k, half);
-        // the distortion must stay invertible (increasing) up to phi_max: the first
-        // turning point of phi_d(phi) below pi, or pi
-        phi_max = M_PI;
-        const int steps = 4096;
-        double prev = 0.0;
-        for (int s2 = 1; s2 <= steps; ++s2) {
-            const double ph = M_PI * s2 / steps, val = kb_theta_d(k, ph);
-            if (!(val > prev)) { phi_max = M_PI * (s2 - 1) / steps; break; }
-            prev = val;
-        }
+        // the distortion must stay invertible (increasing) up to phi_max
+        phi_max = kb_phi_max(k);
     }
 }
 
@@ -1275,7 +1238,8 @@ bool noalloc_tables(const geer_camera &c, NoAllocState &st, int64_t &ntt, int64_
         float4 v = make_float4((float)tan(0.5 * beap_angle(i0, c.width, fx)),
                                (float)tan(0.5 * beap_angle(i1, c.width, fx)), 0.0f, 0.0f);
         for (int i = i0; i <= i1; ++i) {
-            const double cs = cos(beap_angle(i, c.width, fx));
+            const double a = beap_angle(i, c.width, fx), cs = cos(a);
+            st.ptab[i] = make_float2((float)sin(a), (float)cs);
             if (cs > -1e-12) v.z = 1.0f;
             if (cs < 1e-12) { v.w = 1.0f; d.any_col_flip = 1; }
         }
@@ -1287,22 +1251,15 @@ bool noalloc_tables(const geer_camera &c, NoAllocState &st, int64_t &ntt, int64_
         float4 v = make_float4((float)tan(0.5 * beap_angle(j0, c.height, fy)),
                                (float)tan(0.5 * beap_angle(j1, c.height, fy)), 0.0f, 0.0f);
         for (int j = j0; j <= j1; ++j) {
-            const double cs = cos(beap_angle(j, c.height, fy));
+            const double a = beap_angle(j, c.height, fy), cs = cos(a);
+            st.ptab[c.width + j] = make_float2((float)sin(a), (float)cs);
             if (cs > -1e-12) v.z = 1.0f;
             if (cs < 1e-12) { v.w = 1.0f; d.any_row_flip = 1; }
         }
         st.ttab[d.tiles_x + ty] = v;
     }
     d.pcol_off = 0;
-    for (int i = 0; i < c.width; ++i) {
-        const double a = beap_angle(i, c.width, fx);
-        st.ptab[i] = make_float2((float)sin(a), (float)cos(a));
-    }
     d.prow_off = c.width;
-    for (int j = 0; j < c.height; ++j) {
-        const double a = beap_angle(j, c.height, fy);
-        st.ptab[c.width + j] = make_float2((float)sin(a), (float)cos(a));
-    }
     if (!flag_intervals(st.ttab, d.tiles_x, d.zc, d.wc) || !flag_intervals(st.ttab + d.tiles_x, d.tiles_y, d.zr, d.wr))
         return false;
     d.c0lo = d.tiles_x; d.c0hi = 0;

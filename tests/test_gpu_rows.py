@@ -1,8 +1,10 @@
-"""The optimiser step and the refinement's copies at the edges of their blocks.
+"""The optimiser step, the refinement's copies and the image metrics at the edges of
+their blocks.
 
-Both are elementwise: an Adam step of n Gaussians gives bit for bit what the same
+The first two are elementwise: an Adam step of n Gaussians gives bit for bit what the same
 Gaussians get inside a larger array (the groups start at every alignment of the flat
-moments), and the refinement moves rows unchanged.
+moments), and the refinement moves rows unchanged. The metrics are compared with the
+oracle within test_gpu_eval.py's tolerance.
 """
 import numpy as np
 import pytest
@@ -79,3 +81,19 @@ def test_refinement_moves_rows(geer, n, deg):
     for q, q0 in ((a.m, m0), (a.v, v0)):
         for got, want in zip(_groups(q.cpu().numpy(), src.size, k), q0):
             assert np.array_equal(got, np.where((second | split)[:, None], np.float32(0), want[src]))
+
+
+@pytest.mark.parametrize("w", [1, 31, 32, 33, 65])
+@pytest.mark.parametrize("h", [1, 15, 16, 17, 34])
+def test_metrics_at_tile_edges(geer, h, w):
+    from oracle import metrics as M
+    rng = np.random.default_rng(100 * h + w)
+    pred, gt = (rng.uniform(0, 1, (h, w, 3)).astype(np.float32) for _ in range(2))
+    regions = rng.integers(0, 4, (h, w)).astype(np.uint8)
+    regions[regions == 3] = 255
+    res = geer.image_metrics(*(torch.as_tensor(x, device="cuda") for x in (pred, gt, regions)), 3)
+    ref = M.region_metrics(pred, gt, regions, 3)
+    for r in range(3):
+        assert res[r]["count"] == int(ref[r, 2])
+        assert abs(res[r]["sse"] - ref[r, 0]) <= 1e-5 * ref[r, 0] + 1e-9
+        assert abs(res[r]["ssim_sum"] - ref[r, 1]) <= 1e-5 * ref[r, 2]

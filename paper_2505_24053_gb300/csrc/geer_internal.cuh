@@ -404,6 +404,7 @@ namespace geer {
 
 // Launchers (defined in the .cu files).
 cudaError_t launch_preprocess(const geer_workspace *ws, const geer_gaussians *g, cudaStream_t s);
+bool small_front(const geer_workspace *ws);
 cudaError_t launch_bin_front(const geer_workspace *ws, cudaStream_t s);
 cudaError_t launch_depth_sort(geer_workspace *ws, cudaStream_t s);
 cudaError_t launch_count_pairs(const geer_workspace *ws, cudaStream_t s);

@@ -645,6 +645,14 @@ __global__ void __launch_bounds__(kPrepThreads, GEER_PREP_MINB) k_preprocess(
     }
 }
 
+// The totals of a counting pass: pairs to sort (clamped to cap, with the capacity check).
+__device__ __forceinline__ void put_pair_total(uint32_t *misc, unsigned long long total, int64_t cap) {
+    misc[kMiscPairs] = (uint32_t)min(total, (unsigned long long)cap);
+    misc[kMiscPairsHi] = (uint32_t)(total >> 32);
+    misc[kMiscTotalLo] = (uint32_t)total;
+    if (total > (unsigned long long)cap) atomicOr(&misc[kMiscStatus], kStatusCapacity);
+}
+
 // Exclusive scan of per-block counts (one block). mode 0 (live items): total -> misc[kMiscLive]; also clears the
 // per-super-tile pair counts. mode 1 ((super-tile, item) pairs): total ->
 // misc[kMiscPairs] (clamped to cap) with the capacity check. mode 2 ((tile, item)
@@ -721,10 +729,7 @@ __global__ void __launch_bounds__(1024) k_scan_blocks(uint32_t *__restrict__ blo
             misc[kMiscTileLo] = (uint32_t)total;
             misc[kMiscTileHi] = (uint32_t)(total >> 32);
         } else {
-            misc[kMiscPairs] = (uint32_t)min(total, (unsigned long long)cap);
-            misc[kMiscPairsHi] = (uint32_t)(total >> 32);
-            misc[kMiscTotalLo] = (uint32_t)total;
-            if (total > (unsigned long long)cap) atomicOr(&misc[kMiscStatus], kStatusCapacity);
+            put_pair_total(misc, total, cap);
         }
     }
     if (mode == 0) {
@@ -828,6 +833,42 @@ __device__ __forceinline__ void warp_supers(const DevCam &cam, uint32_t inv_s, c
     }
 }
 
+// One item a lane (live: whether it has one): its rectangle and number of super-tiles,
+// and its tiles; box: the warp's nine boxes in shared memory (warp_supers).
+struct ItemPairs {
+    uint32_t xr, yr, supers, tiles;  // xr 0: several rectangles
+};
+__device__ __forceinline__ ItemPairs warp_item_pairs(const DevCam *__restrict__ cams, uint32_t inv_s, bool live, int ci,
+                                                     const uint4 r4, int4 *box) {
+    const int lane = threadIdx.x & 31;
+    Assoc a{0u, 0u, 0u};
+    ItemPairs p{0u, 0u, 0u, 0u};
+    if (live) a = item_assoc(cams[ci], r4);
+    if (a.rects == 1) {
+        p.xr = a.xr;
+        p.yr = a.yr;
+        p.supers = super_box(a.xr, a.yr, inv_s).supers;
+        p.tiles = ((a.xr >> 16) - (a.xr & 0xffff)) * ((a.yr >> 16) - (a.yr & 0xffff));
+    }
+    for (uint32_t many = __ballot_sync(0xffffffffu, a.rects > 1); many; many &= many - 1) {
+        const int o = __ffs(many) - 1;
+        const uint4 q = make_uint4(__shfl_sync(0xffffffffu, r4.x, o), __shfl_sync(0xffffffffu, r4.y, o),
+                                   __shfl_sync(0xffffffffu, r4.z, o), __shfl_sync(0xffffffffu, r4.w, o));
+        int rg[8];
+        unpack_ranges(q, rg);
+        uint32_t k = 0;
+        const DevCam &cam = cams[__shfl_sync(0xffffffffu, ci, o)];
+        warp_supers(cam, inv_s, rg, box, [&](int, int, bool keep) {
+            k += (uint32_t)__popc(__ballot_sync(0xffffffffu, keep));
+        });
+        if (lane == o) {
+            p.supers = k;
+            p.tiles = assoc_count(cam, rg, 0, cam.tiles_x, 0, cam.tiles_y);
+        }
+    }
+    return p;
+}
+
 // Per 256 depth-sorted live items (a block of the emission): their super-tile pairs
 // (emission offsets) and their tile pairs (the total, for the capacity check). Each
 // item's rectangle and super-tiles are left in depth order for the emission, in the
@@ -838,8 +879,8 @@ __device__ __forceinline__ void warp_supers(const DevCam &cam, uint32_t inv_s, c
 constexpr int kGather = 2;  // (24M items, 9M live: 273 us; with 1 320, with 4 299; both arrays read 452)
 __global__ void __launch_bounds__(kPrepThreads) k_gather_counts(
     const DevCam *__restrict__ cams, int64_t n, int S, uint32_t *__restrict__ id0, uint32_t *__restrict__ id1,
-    const uint4 *__restrict__ ranges, const uint32_t *__restrict__ misc, uint32_t *__restrict__ bs_super, uint32_t *__restrict__ bs_tile, uint32_t *__restrict__ oxr,
-    uint32_t *__restrict__ oyr) {
+    const uint4 *__restrict__ ranges, const uint32_t *__restrict__ misc, uint32_t *__restrict__ bs_super,
+    uint32_t *__restrict__ bs_tile, uint32_t *__restrict__ oxr, uint32_t *__restrict__ oyr) {
     grid_dep_sync();
     __shared__ uint32_t s_sum[kGather][2];
     __shared__ int4 s_box[kPrepThreads / 32][9];
@@ -868,36 +909,13 @@ __global__ void __launch_bounds__(kPrepThreads) k_gather_counts(
 #pragma unroll
     for (int u = 0; u < kGather; ++u) {
         const int64_t i = i0 + u * kPrepThreads + threadIdx.x;
-        const int ci = (int)(item[u] / (uint32_t)n);
-        Assoc a{0u, 0u, 0u};
-        uint32_t sc = 0, c = 0;
-        if (i < L) a = item_assoc(cams[ci], r4[u]);
-        if (a.rects == 1) {
-            sc = super_box(a.xr, a.yr, inv_s).supers;
-            c = ((a.xr >> 16) - (a.xr & 0xffff)) * ((a.yr >> 16) - (a.yr & 0xffff));
-        }
-        for (uint32_t many = __ballot_sync(0xffffffffu, a.rects > 1); many; many &= many - 1) {
-            const int o = __ffs(many) - 1;
-            const uint4 q = make_uint4(__shfl_sync(0xffffffffu, r4[u].x, o), __shfl_sync(0xffffffffu, r4[u].y, o),
-                                       __shfl_sync(0xffffffffu, r4[u].z, o), __shfl_sync(0xffffffffu, r4[u].w, o));
-            int rg[8];
-            unpack_ranges(q, rg);
-            uint32_t k = 0;
-            const DevCam &cam = cams[__shfl_sync(0xffffffffu, ci, o)];
-            warp_supers(cam, inv_s, rg, s_box[warp], [&](int, int, bool keep) {
-                k += (uint32_t)__popc(__ballot_sync(0xffffffffu, keep));
-            });
-            if (lane == o) {
-                sc = k;
-                c = assoc_count(cam, rg, 0, cam.tiles_x, 0, cam.tiles_y);
-            }
-        }
+        const ItemPairs p = warp_item_pairs(cams, inv_s, i < L, (int)(item[u] / (uint32_t)n), r4[u], s_box[warp]);
         if (i < L) {
-            oxr[i] = a.rects == 1 ? a.xr : 0u;
-            oyr[i] = a.yr;
-            osupers[i] = sc;
+            oxr[i] = p.xr;
+            oyr[i] = p.yr;
+            osupers[i] = p.supers;
         }
-        const uint32_t tiles = __reduce_add_sync(0xffffffffu, c), supers = __reduce_add_sync(0xffffffffu, sc);
+        const uint32_t tiles = __reduce_add_sync(0xffffffffu, p.tiles), supers = __reduce_add_sync(0xffffffffu, p.supers);
         if (lane == 0) {
             atomicAdd(&s_sum[u][0], supers);
             atomicAdd(&s_sum[u][1], tiles);
@@ -907,6 +925,196 @@ __global__ void __launch_bounds__(kPrepThreads) k_gather_counts(
     if (threadIdx.x < kGather && i0 + threadIdx.x * kPrepThreads < L) {
         bs_super[(int64_t)blockIdx.x * kGather + threadIdx.x] = s_sum[threadIdx.x][0];
         bs_tile[(int64_t)blockIdx.x * kGather + threadIdx.x] = s_sum[threadIdx.x][1];
+    }
+}
+
+// Everything between the preprocess and the emission for at most kSmallItems (camera,
+// Gaussian) items, in one block: compaction, the stable depth sort (8-bit digits, the
+// keys and ids held in registers through a pass and reordered in shared memory; a pass
+// whose digit all keys share is skipped), the counting in depth order and the scans.
+// It leaves what those kernels leave (ids in buffer 0). Bound by the issue rate of its
+// one SM; the twelve launches it replaces take about 4 us each at these sizes, whatever
+// their work. From the preprocess to the render order, 1000 items take 38 us in place
+// of 69, 4096 46 of 71, 8192 56 of 69; at 10000 both take 67 to 69, hence the line. (The lanes
+// of a digit by a vote per bit: 60 at 8192; by __match_any_sync: 71.) K: items a thread.
+constexpr int kSmallItems = 8192, kSmallThreads = 1024;
+template <int K>
+__global__ void __launch_bounds__(kSmallThreads) k_small_front(
+    const DevCam *__restrict__ cams, int64_t n, int items, int S, const uint32_t *__restrict__ count,
+    const uint32_t *__restrict__ key, const uint4 *__restrict__ ranges, uint32_t *__restrict__ misc,
+    uint32_t *__restrict__ id0, uint32_t *__restrict__ id1, uint32_t *__restrict__ oxr, uint32_t *__restrict__ oyr,
+    uint32_t *__restrict__ bs_super, uint32_t *__restrict__ scount, int64_t nst, int64_t cap) {
+    grid_dep_sync();
+    constexpr int W = kSmallThreads / 32, CHUNKS = K * kSmallThreads / kPrepThreads;
+    extern __shared__ uint32_t dyn[];
+    uint32_t(*s_hist)[kRadix] = reinterpret_cast<uint32_t(*)[kRadix]>(dyn);  // [W]: a warp's keys per digit
+    uint32_t(*s_match)[kRadix] = s_hist + W;  // lane masks per digit, zero between ranking steps
+    uint32_t *s_key = dyn + 2 * W * kRadix;   // [K * kSmallThreads]
+    uint16_t *s_val = reinterpret_cast<uint16_t *>(s_key + K * kSmallThreads);
+    __shared__ uint32_t s_part[kSmallThreads / kRadix][kRadix];
+    __shared__ uint32_t s_wsum[W];
+    __shared__ int4 s_box[W][9];
+    __shared__ uint32_t s_sum[CHUNKS][2];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const uint32_t below = (1u << lane) - 1u;
+    for (int64_t i = t; i < nst; i += kSmallThreads) scount[i] = 0u;
+    for (int i = t; i < W * kRadix; i += kSmallThreads) (&s_match[0][0])[i] = 0u;
+    for (int i = t; i < 2 * CHUNKS; i += kSmallThreads) (&s_sum[0][0])[i] = 0u;
+    // compaction in index order: a warp's 32 K consecutive items
+    uint32_t kk[K], live[K], mine = 0;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int i = (warp * K + k) * 32 + lane;
+        const bool on = i < items && count[i] > 0u;
+        kk[k] = i < items ? key[i] : 0u;
+        live[k] = __ballot_sync(0xffffffffu, on);
+        mine += (uint32_t)__popc(live[k]);
+    }
+    if (lane == 0) s_wsum[warp] = mine;
+    __syncthreads();
+    uint32_t v = s_wsum[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += y;
+    }
+    const int L = (int)__shfl_sync(0xffffffffu, v, 31);
+    uint32_t at = warp ? __shfl_sync(0xffffffffu, v, max(warp - 1, 0)) : 0u;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        if (live[k] >> lane & 1u) {
+            const uint32_t pos = at + (uint32_t)__popc(live[k] & below);
+            s_key[pos] = kk[k];
+            s_val[pos] = (uint16_t)((warp * K + k) * 32 + lane);
+        }
+        at += (uint32_t)__popc(live[k]);
+    }
+    __syncthreads();
+    // the sort: a warp takes 32 kr consecutive keys
+    const int kr = (L + kSmallThreads - 1) / kSmallThreads;
+#pragma unroll 1
+    for (int shift = 0; shift < 32; shift += kRadixBits) {
+        uint32_t val[K], rank[K];
+        const uint32_t d0 = L > 0 ? (s_key[0] >> shift) & 0xffu : 0u;
+        bool same = true;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const int e = (warp * kr + k) * 32 + lane;
+            if (k < kr && e < L) {
+                kk[k] = s_key[e];
+                val[k] = s_val[e];
+                same = same && ((kk[k] >> shift) & 0xffu) == d0;
+            }
+        }
+        for (int i = t; i < W * kRadix; i += kSmallThreads) (&s_hist[0][0])[i] = 0u;
+        if (__syncthreads_and(same)) continue;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            if (k >= kr) break;
+            const bool on = (warp * kr + k) * 32 + lane < L;
+            const uint32_t d = on ? (kk[k] >> shift) & 0xffu : 0u;
+            if (on) atomicOr(&s_match[warp][d], 1u << lane);
+            const uint32_t b = s_hist[warp][d];
+            __syncwarp();
+            const uint32_t peers = s_match[warp][d], before = (uint32_t)__popc(peers & below);
+            __syncwarp();
+            if (on && before == 0) {
+                s_hist[warp][d] = b + (uint32_t)__popc(peers);
+                s_match[warp][d] = 0u;
+            }
+            rank[k] = b + before;
+            __syncwarp();
+        }
+        __syncthreads();
+        // per digit the warps' places: a thread scans eight warps of one digit
+        constexpr int Q = W / (kSmallThreads / kRadix);
+        const int d = t & (kRadix - 1), q = t / kRadix;
+        uint32_t c[Q], sum = 0;
+#pragma unroll
+        for (int w = 0; w < Q; ++w) {
+            c[w] = s_hist[q * Q + w][d];
+            sum += c[w];
+        }
+        s_part[q][d] = sum;
+        __syncthreads();
+        uint32_t pre = 0, tot = 0;
+#pragma unroll
+        for (int p = 0; p < kSmallThreads / kRadix; ++p) {
+            const uint32_t x = s_part[p][d];
+            pre += p < q ? x : 0u;
+            tot += x;
+        }
+        uint32_t sc = tot;  // scan over the digits (each quarter of the block the same)
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, sc, o);
+            if (lane >= o) sc += y;
+        }
+        if (lane == 31) s_wsum[warp] = sc;
+        __syncthreads();
+        uint32_t run = sc - tot + pre;
+#pragma unroll
+        for (int w = 0; w < kRadix / 32; ++w) run += w < (warp & (kRadix / 32 - 1)) ? s_wsum[w] : 0u;
+#pragma unroll
+        for (int w = 0; w < Q; ++w) {
+            s_hist[q * Q + w][d] = run;
+            run += c[w];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+            if (k < kr && (warp * kr + k) * 32 + lane < L) {
+                const uint32_t pos = s_hist[warp][(kk[k] >> shift) & 0xffu] + rank[k];
+                s_key[pos] = kk[k];
+                s_val[pos] = (uint16_t)val[k];
+            }
+        __syncthreads();
+    }
+    // the counting, in depth order
+    const uint32_t inv_s = super_inverse(S);
+    for (int i0 = 0; i0 < L; i0 += kSmallThreads) {
+        const int i = i0 + t;
+        const bool on = i < L;
+        const uint32_t item = on ? s_val[i] : 0u;
+        const uint4 r4 = on ? ranges[item] : make_uint4(0u, 0u, 0u, 0u);
+        const ItemPairs p = warp_item_pairs(cams, inv_s, on, (int)(item / (uint32_t)n), r4, s_box[warp]);
+        if (on) {
+            id0[i] = item;
+            oxr[i] = p.xr;
+            oyr[i] = p.yr;
+            id1[i] = p.supers;
+        }
+        const uint32_t tiles = __reduce_add_sync(0xffffffffu, p.tiles), supers = __reduce_add_sync(0xffffffffu, p.supers);
+        if (lane == 0) {
+            atomicAdd(&s_sum[i / kPrepThreads][0], supers);
+            atomicAdd(&s_sum[i / kPrepThreads][1], tiles);
+        }
+    }
+    __syncthreads();
+    if (warp > 0) return;
+    unsigned long long pairs = 0, tiles = 0;
+    for (int c0 = 0; c0 < CHUNKS; c0 += 32) {
+        const uint32_t a = c0 + lane < CHUNKS ? s_sum[c0 + lane][0] : 0u;
+        unsigned long long x = a, y = c0 + lane < CHUNKS ? s_sum[c0 + lane][1] : 0u;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long u = __shfl_up_sync(0xffffffffu, x, o), w = __shfl_up_sync(0xffffffffu, y, o);
+            if (lane >= o) {
+                x += u;
+                y += w;
+            }
+        }
+        if ((c0 + lane) * kPrepThreads < L) bs_super[c0 + lane] = (uint32_t)min(pairs + x - a, 0xffffffffull);
+        pairs += __shfl_sync(0xffffffffu, x, 31);
+        tiles += __shfl_sync(0xffffffffu, y, 31);
+    }
+    if (lane == 0) {
+        misc[kMiscLive] = (uint32_t)L;
+        misc[kMiscSortCur] = 1u;  // the sorted ids are in buffer 0 (depth_sorted_buf)
+        misc[kMiscSortSame] = 0u;
+        misc[kMiscTileLo] = (uint32_t)tiles;
+        misc[kMiscTileHi] = (uint32_t)(tiles >> 32);
+        put_pair_total(misc, pairs, cap);
     }
 }
 
@@ -1334,7 +1542,30 @@ cudaError_t launch_preprocess(const geer_workspace *ws, const geer_gaussians *g,
     return cudaGetLastError();
 }
 
+// Few enough items for one block to do the work of launch_bin_front, launch_depth_sort
+// and launch_count_pairs (k_small_front, launched as launch_bin_front).
+bool small_front(const geer_workspace *ws) { return (int64_t)ws->n_cams * ws->n_gauss <= kSmallItems; }
+
+static cudaError_t launch_small_front(const geer_workspace *ws, cudaStream_t s) {
+    const int items = (int)(ws->n_cams * ws->n_gauss);
+    static_assert(kSmallItems == 8 * kSmallThreads && kSmallItems <= 65536, "eight items a thread at most, 16-bit ids");
+    const auto launch = [&](auto *kern, int k) {
+        const int smem = 2 * (int)sizeof(uint32_t) * kSmallThreads / 32 * kRadix + 6 * k * kSmallThreads;
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        launch_k(kern, dim3(1), dim3(kSmallThreads), smem, s, ws->d_cams, ws->n_gauss, items, ws->super_size,
+                 ws->d_count, ws->d_key, ws->d_ranges, ws->d_misc, ws->d_iid[0], ws->d_iid[1], ws->d_ikey[0],
+                 ws->d_ikey[1], ws->d_blocksum2, reinterpret_cast<uint32_t *>(ws->d_srange + ws->n_stiles),
+                 ws->n_stiles, ws->cap_pairs);
+        return cudaGetLastError();
+    };
+    return items <= kSmallThreads       ? launch(k_small_front<1>, 1)
+           : items <= 4 * kSmallThreads ? launch(k_small_front<4>, 4)
+                                        : launch(k_small_front<8>, 8);
+}
+
 cudaError_t launch_bin_front(const geer_workspace *ws, cudaStream_t s) {
+    if (small_front(ws)) return launch_small_front(ws, s);
     const int64_t nblk = prep_blocks(ws->n_gauss);
     launch_k(k_scan_blocks, dim3(1), dim3(1024), 0, s, ws->d_blocksum, nblk * ws->n_cams, ws->d_misc, ws->d_srange,
              ws->n_stiles, ws->cap_pairs, 0, nullptr, 0);
@@ -1346,6 +1577,7 @@ cudaError_t launch_bin_front(const geer_workspace *ws, cudaStream_t s) {
 }
 
 cudaError_t launch_count_pairs(const geer_workspace *ws, cudaStream_t s) {
+    if (small_front(ws)) return cudaSuccess;
     const int64_t m = prep_blocks((int64_t)ws->n_cams * ws->n_gauss);
     if (m > 0) {
         launch_k(k_gather_counts, dim3((unsigned)((m + kGather - 1) / kGather)), dim3(kPrepThreads), 0, s, ws->d_cams,

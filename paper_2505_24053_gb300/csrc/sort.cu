@@ -325,7 +325,7 @@ static cudaError_t radix_pass(geer_workspace *ws, uint32_t *const kbuf[2], uint3
 // less than a factor of two) costs its histogram only.
 cudaError_t launch_depth_sort(geer_workspace *ws, cudaStream_t s) {
     const int64_t items = (int64_t)ws->n_cams * ws->n_gauss;
-    if (items > 0) {
+    if (items > 0 && !small_front(ws)) {
         for (int p = 0; p < 4; ++p) {
             cudaError_t e = radix_pass(ws, ws->d_ikey, ws->d_iid, 0, kMiscLive, 0, p, items, s, nullptr, 0, 1);
             if (e != cudaSuccess) return e;

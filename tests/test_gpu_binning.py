@@ -8,6 +8,8 @@
 - Lists of Gaussians whose association is several rectangles (boxes of more than 32
   super-tiles, several cameras) and item counts around a block, against the replica.
 - More block counts than one step of the scan takes (4096).
+- The one-block binning of small scenes against the general path, over the items a
+  thread holds, cameras, equal depths and culled Gaussians.
 """
 import math
 
@@ -132,3 +134,39 @@ def test_more_sort_tiles_than_blocks(geer):
     assert (k[1:] >= k[:-1]).all()
     same = k[1:] == k[:-1]
     assert same.any() and (v[1:][same] > v[:-1][same]).all()
+
+
+@pytest.mark.parametrize("n,ncams", [(1, 1), (31, 1), (1024, 1), (1025, 1), (341, 3), (4096, 1), (2049, 2), (4097, 1),
+                                     (2730, 3), (8192, 1)])
+@pytest.mark.parametrize("fov", [80, 205])
+def test_small_front_equals_the_general_path(geer, n, ncams, fov):
+    """At most 8192 items are binned by one block; the same scene with culled
+    Gaussians behind it takes the general path. Same lists, in the same order."""
+    rng = np.random.default_rng(n + fov)
+    mean = rng.uniform(-2, 2, (n, 3)).astype(np.float32)
+    mean[n // 2:] = mean[:n - n // 2]  # equal depths
+    opacity = rng.uniform(0.1, 0.9, n).astype(np.float32)
+    opacity[::7] = 0.001  # culled
+    opacity[0] = 0.9
+    scene = wl.Scene(mean, np.exp(rng.normal(-4.0, 0.8, (n, 3))).astype(np.float32),
+                     rng.standard_normal((n, 4)).astype(np.float32), opacity,
+                     rng.normal(0, 0.3, (n, 1, 3)).astype(np.float32), 0)
+    pad = 8193
+    big = wl.Scene(*(np.concatenate([a, np.resize(a, (pad,) + a.shape[1:])]) for a in
+                     (scene.mean, scene.scale, scene.quat)),
+                   np.concatenate([opacity, np.zeros(pad, np.float32)]),
+                   np.concatenate([scene.sh, np.zeros((pad, 1, 3), np.float32)]), 0)
+    cams = []
+    for i in range(ncams):
+        R, t = wl.pose(wl.rot_y(1.3 * i), (0.1 * i, 0.0, 0.0))
+        cams.append(wl.Camera(wl.EQUIDISTANT, 150 + 20 * i, 130, math.radians(fov), R_cw=R, t_cw=t))
+    lists = []
+    for sc in (scene, big):
+        r = geer.Renderer(cams, sc.n, 0, pair_capacity=1 << 21)
+        rgb = r.forward(geer.Gaussians.from_scene(sc))
+        P, supers = r.ws.pair_counts()
+        k, v = r.ws.debug_pairs(cap=P)
+        lists.append((P, supers, r.ws.live_items(), k, v // sc.n, v % sc.n, rgb.cpu().numpy()))
+    assert lists[0][:3] == lists[1][:3]
+    for a, b in zip(lists[0][3:], lists[1][3:]):
+        assert np.array_equal(a, b)

@@ -739,23 +739,37 @@ __global__ void __launch_bounds__(1024) k_scan_blocks(uint32_t *__restrict__ blo
 }
 
 // Compaction of the live (camera, Gaussian) items, in index order, into
-// (depth key, item) arrays. Block (b, ci): Gaussians [256 b, 256 b + 256) of camera ci.
+// (depth key, item) arrays. Block (b, ci): the Gaussians of kCompact preprocess blocks
+// of camera ci, all loads in flight together.
+constexpr int kCompact = 4;
 __global__ void __launch_bounds__(kPrepThreads) k_compact(int64_t n, const uint32_t *__restrict__ count,
                                                           const uint32_t *__restrict__ key,
                                                           const uint32_t *__restrict__ blocksum, int64_t nblk,
                                                           uint32_t *__restrict__ okey, uint32_t *__restrict__ oid) {
     grid_dep_sync();
-    __shared__ uint32_t wsum[kPrepThreads / 32];
-    const int64_t g = (int64_t)blockIdx.x * kPrepThreads + threadIdx.x;
-    const int64_t idx = (int64_t)blockIdx.y * n + g;
-    const bool live = g < n && count[idx] > 0;
-    const uint32_t k = g < n ? key[idx] : 0u;
-    uint32_t tot;
-    const uint32_t pre = block_excl_scan(live ? 1u : 0u, wsum, tot);
-    if (live) {
-        const uint32_t pos = blocksum[(int64_t)blockIdx.y * nblk + blockIdx.x] + pre;
-        okey[pos] = k;
-        oid[pos] = (uint32_t)idx;
+    __shared__ uint32_t s_wsum[kCompact][kPrepThreads / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t b0 = (int64_t)blockIdx.x * kCompact, i0 = (int64_t)blockIdx.y * n;
+    uint32_t k[kCompact], pos[kCompact], live[kCompact];
+#pragma unroll
+    for (int u = 0; u < kCompact; ++u) {
+        const int64_t g = (b0 + u) * kPrepThreads + threadIdx.x;
+        const bool in = g < n;
+        const bool on = in && count[i0 + g] > 0;
+        k[u] = in ? key[i0 + g] : 0u;
+        pos[u] = b0 + u < nblk ? blocksum[(int64_t)blockIdx.y * nblk + b0 + u] : 0u;
+        live[u] = __ballot_sync(0xffffffffu, on);
+        if (lane == 0) s_wsum[u][warp] = (uint32_t)__popc(live[u]);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kCompact; ++u) {
+        for (int w = 0; w < warp; ++w) pos[u] += s_wsum[u][w];
+        if (live[u] >> lane & 1u) {
+            const uint32_t p = pos[u] + (uint32_t)__popc(live[u] & ((1u << lane) - 1u));
+            okey[p] = k[u];
+            oid[p] = (uint32_t)(i0 + (b0 + u) * kPrepThreads + threadIdx.x);
+        }
     }
 }
 
@@ -1145,21 +1159,19 @@ __device__ __forceinline__ uint64_t tile_mask_general(const DevCam &cam, const i
 }
 
 // The same for a rectangle that meets the super-tile: columns [xlo, xhi) x rows
-// [ylo, yhi) (packed lo | hi << 16). every: bit j * S of every row j. M: uint32_t
-// where the S * S bits fit it.
+// [ylo, yhi) (packed lo | hi << 16), from the table of row runs: rows[9 l + h] has bit
+// j * S of the rows l <= j < h, each times the columns' run of ones. M: uint32_t where
+// the S * S bits fit it.
 template <typename M>
-__device__ __forceinline__ M tile_mask_rect(uint32_t xr, uint32_t yr, int sx, int sy, int S, M every) {
-    constexpr int kBits = 8 * sizeof(M);
+__device__ __forceinline__ M tile_mask_rect(uint32_t xr, uint32_t yr, int sx, int sy, int S, const M *rows) {
     const int x0 = sx * S, y0 = sy * S;
     const int xl = max((int)(xr & 0xffff) - x0, 0), xh = min((int)(xr >> 16) - x0, S);
     const int yl = max((int)(yr & 0xffff) - y0, 0), yh = min((int)(yr >> 16) - y0, S);
-    // the bits every has in [yl S, yh S), each times the columns' run of ones
-    const M upto = yh * S < kBits ? ((M)1 << (yh * S)) - 1 : ~(M)0;
-    return (every & upto & ~(((M)1 << (yl * S)) - 1)) * (M)((1u << xh) - (1u << xl));
+    return rows[9 * yl + yh] * (M)((1u << xh) - (1u << xl));
 }
 
-__device__ __forceinline__ void put_mask(uint32_t *out, int64_t i, uint32_t m) { out[i] = m; }
-__device__ __forceinline__ void put_mask(uint32_t *out, int64_t i, uint64_t m) {
+__device__ __forceinline__ void put_mask(uint32_t *out, uint32_t i, uint32_t m) { out[i] = m; }
+__device__ __forceinline__ void put_mask(uint32_t *out, uint32_t i, uint64_t m) {
     reinterpret_cast<uint2 *>(out)[i] = make_uint2((uint32_t)m, (uint32_t)(m >> 32));
 }
 
@@ -1171,7 +1183,10 @@ __device__ __forceinline__ void put_mask(uint32_t *out, int64_t i, uint64_t m) {
 // in any order (each belongs to another super-tile). Items whose association is one
 // rectangle are emitted by the whole warp together (lane j writes output j:
 // coalesced) from a list in shared memory; the few others by the warp one by one (a
-// thread looping over its item's super-tiles kept its block waiting).
+// thread looping over its item's super-tiles kept its block waiting). At most the
+// resident blocks go through the items and add their counts to the global ones at the
+// end: a block per 256 items added 8M for 12M pairs on 3600 super-tiles, 149 us where
+// this takes 115 (with twice the blocks 116; 1M-Gaussian fisheye 30 -> 24).
 // M: the mask's type (32 bits up to S = 5).
 template <typename M>
 __global__ void __launch_bounds__(kPrepThreads) k_duplicate(
@@ -1186,94 +1201,106 @@ __global__ void __launch_bounds__(kPrepThreads) k_duplicate(
     __shared__ uint4 s_item[kPrepThreads][2];
     __shared__ uint32_t wsum[kPrepThreads / 32];
     __shared__ int4 s_box[kPrepThreads / 32][9];
+    __shared__ M s_rows[81];  // tile_mask_rect's row runs
     extern __shared__ uint32_t sh[];  // per-super-tile pair counts when they fit (nst <= kSmemTiles)
     const bool smem = nst <= kSmemTiles;
-    if (smem)
-        for (int k = threadIdx.x; k < nst; k += kPrepThreads) sh[k] = 0u;
     const uint32_t L = misc[kMiscLive];
     if ((int64_t)blockIdx.x * kPrepThreads >= L) return;
+    if (smem)
+        for (int k = threadIdx.x; k < nst; k += kPrepThreads) sh[k] = 0u;
+    if (threadIdx.x < 81) {
+        const int l = threadIdx.x / 9, h = threadIdx.x - 9 * l;
+        M m = 0;
+        for (int j = l; j < min(h, S); ++j) m |= (M)1 << (j * S);
+        s_rows[threadIdx.x] = m;
+    }
+    const auto count = [&](uint32_t st) {
+        if (!in_bounds(st, (uint64_t)nst, kSiteDupSuper, misc)) return;
+        if (smem) atomicAdd(&sh[st], 1u);
+        else atomicAdd(&scount[st], 1u);
+    };
     const bool cur = depth_sorted_buf(misc) != 0;
     const int lane = threadIdx.x & 31;
-    const int64_t i = (int64_t)blockIdx.x * kPrepThreads + threadIdx.x;
     const uint32_t inv_s = super_inverse(S);
-    uint32_t item = 0, xr = 0, yr = 0, cnt = 0;  // as the counting left them
-    if (i < L) {
-        item = (cur ? id1 : id0)[i];
-        cnt = (cur ? id0 : id1)[i];
-        xr = xrs[i];
-        yr = yrs[i];
-    }
-    const int ci = (int)(item / (uint32_t)n);
-    const DevCam &cam = cams[ci];
-    uint32_t tot;
-    const uint32_t pre = block_excl_scan(cnt, wsum, tot);  // (its barriers also follow the clearing of sh)
-    const int64_t base = (int64_t)blocksum[blockIdx.x];
-    const bool fits = base + pre + cnt <= cap;
-    // cooperative emission of the warp's one-rectangle items
-    const bool one = xr != 0 && fits;
-    const uint32_t rc = one ? cnt : 0u;
-    uint32_t incl = rc;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
-    }
-    const uint32_t ones = __ballot_sync(0xffffffffu, one);
-    uint4(*list)[2] = s_item + (threadIdx.x & ~31);
-    if (one) {
-        const SuperBox b = super_box(xr, yr, inv_s);
-        const int k = __popc(ones & ((1u << lane) - 1u));
-        list[k][0] = make_uint4(xr, yr, item, pre);
-        list[k][1] = make_uint4(incl - rc, (uint32_t)b.w | (uint32_t)cam.stiles_x << 16,
-                                (uint32_t)(cam.stile_base + b.sy0 * cam.stiles_x + b.sx0),
-                                (uint32_t)b.sx0 | (uint32_t)b.sy0 << 16);
-    }
-    __syncwarp();
-    M every = 0;
-    for (int j = 0; j < S; ++j) every |= (M)1 << (j * S);
-    const uint32_t wtot = __shfl_sync(0xffffffffu, incl, 31);
-    int before = -1;  // items that start in the windows so far, less one
-    for (uint32_t j0 = 0; j0 < wtot; j0 += 32) {
-        // the outputs of this window where an item starts; an output's item is the last to start
-        const uint32_t at = incl - rc - j0;
-        const uint32_t starts = __reduce_or_sync(0xffffffffu, one && at < 32u ? 1u << at : 0u);
-        const uint32_t j = j0 + lane;
-        const int o = before + __popc(starts & (0xffffffffu >> (31 - lane)));
-        before += __popc(starts);
-        if (j < wtot) {
-            const uint4 a = list[o][0], b = list[o][1];
-            const uint32_t k = j - b.x, rw = b.y & 0xffff;
-            // k / rw: the quotient's distance from the next whole number is at least 0.5 / rw,
-            // more than its rounding errors below 2^21
-            const uint32_t ky = k < 1u << 21 ? (uint32_t)__fdividef((float)k + 0.5f, (float)rw) : k / rw;
-            const uint32_t kx = k - ky * rw, st = b.z + ky * (b.y >> 16) + kx;
-            const int64_t out = base + (int64_t)(a.w + k);
-            okeys[out] = st;
-            ovals[out] = a.z;
-            put_mask(omask, out, tile_mask_rect<M>(a.x, a.y, (int)((b.w & 0xffff) + kx), (int)((b.w >> 16) + ky), S, every));
-            if (in_bounds(st, (uint64_t)nst, kSiteDupSuper, misc)) atomicAdd(smem ? &sh[st] : &scount[st], 1u);
+    for (int64_t chunk = blockIdx.x; chunk * kPrepThreads < L; chunk += gridDim.x) {
+        const int64_t i = chunk * kPrepThreads + threadIdx.x;
+        uint32_t item = 0, xr = 0, yr = 0, cnt = 0;  // as the counting left them
+        if (i < L) {
+            item = (cur ? id1 : id0)[i];
+            cnt = (cur ? id0 : id1)[i];
+            xr = xrs[i];
+            yr = yrs[i];
         }
-    }
-    // the items of several rectangles, one at a time
-    for (uint32_t many = __ballot_sync(0xffffffffu, cnt > 0 && xr == 0 && fits); many; many &= many - 1) {
-        const int o = __ffs(many) - 1;
-        const uint32_t it = __shfl_sync(0xffffffffu, item, o), cn = __shfl_sync(0xffffffffu, cnt, o);
-        const DevCam &c = cams[__shfl_sync(0xffffffffu, ci, o)];
-        const int64_t out = base + __shfl_sync(0xffffffffu, pre, o);
-        int rg[8];
-        unpack_ranges(ranges[it], rg);
-        uint32_t done = 0;
-        warp_supers(c, inv_s, rg, s_box[threadIdx.x >> 5], [&](int sx, int sy, bool keep) {
-            const uint32_t kept = __ballot_sync(0xffffffffu, keep), k = done + (uint32_t)__popc(kept & ((1u << lane) - 1u));
-            if (keep && k < cn) {
-                const uint32_t st = (uint32_t)(c.stile_base + sy * c.stiles_x + sx);
-                okeys[out + k] = st;
-                ovals[out + k] = it;
-                put_mask(omask, out + k, (M)tile_mask_general(c, rg, sx, sy, S));
-                if (in_bounds(st, (uint64_t)nst, kSiteDupSuper, misc)) atomicAdd(smem ? &sh[st] : &scount[st], 1u);
+        const int ci = (int)(item / (uint32_t)n);
+        const DevCam &cam = cams[ci];
+        uint32_t tot;
+        const uint32_t pre = block_excl_scan(cnt, wsum, tot);  // (its barriers also follow the clearing of sh)
+        const uint32_t base = blocksum[chunk];  // (pairs that fit have 32-bit places: cap < 2^32)
+        const bool fits = (int64_t)base + pre + cnt <= cap;
+        // cooperative emission of the warp's one-rectangle items
+        const bool one = xr != 0 && fits;
+        const uint32_t rc = one ? cnt : 0u;
+        uint32_t incl = rc;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        const uint32_t ones = __ballot_sync(0xffffffffu, one);
+        uint4(*list)[2] = s_item + (threadIdx.x & ~31);
+        if (one) {
+            const SuperBox b = super_box(xr, yr, inv_s);
+            const int k = __popc(ones & ((1u << lane) - 1u));
+            list[k][0] = make_uint4(xr, yr, item, pre);
+            list[k][1] = make_uint4(incl - rc, (uint32_t)b.w | (uint32_t)cam.stiles_x << 16,
+                                    (uint32_t)(cam.stile_base + b.sy0 * cam.stiles_x + b.sx0),
+                                    (uint32_t)b.sx0 | (uint32_t)b.sy0 << 16);
+        }
+        __syncwarp();
+        const uint32_t wtot = __shfl_sync(0xffffffffu, incl, 31);
+        int before = -1;  // items that start in the windows so far, less one
+        for (uint32_t j0 = 0; j0 < wtot; j0 += 32) {
+            // the outputs of this window where an item starts; an output's item is the last to start
+            const uint32_t at = incl - rc - j0;
+            const uint32_t starts = __reduce_or_sync(0xffffffffu, one && at < 32u ? 1u << at : 0u);
+            const uint32_t j = j0 + lane;
+            const int o = before + __popc(starts & (0xffffffffu >> (31 - lane)));
+            before += __popc(starts);
+            if (j < wtot) {
+                const uint4 a = list[o][0], b = list[o][1];
+                const uint32_t k = j - b.x, rw = b.y & 0xffff;
+                // k / rw: the quotient's distance from the next whole number is at least 0.5 / rw,
+                // more than its rounding errors below 2^21
+                uint32_t ky = (uint32_t)__fdividef((float)k + 0.5f, (float)rw);
+                if (k >= 1u << 21) ky = k / rw;
+                const uint32_t kx = k - ky * rw, st = b.z + ky * (b.y >> 16) + kx, out = base + a.w + k;
+                okeys[out] = st;
+                ovals[out] = a.z;
+                put_mask(omask, out, tile_mask_rect<M>(a.x, a.y, (int)((b.w & 0xffff) + kx), (int)((b.w >> 16) + ky), S, s_rows));
+                count(st);
             }
-            done += (uint32_t)__popc(kept);
-        });
+        }
+        // the items of several rectangles, one at a time
+        for (uint32_t many = __ballot_sync(0xffffffffu, cnt > 0 && xr == 0 && fits); many; many &= many - 1) {
+            const int o = __ffs(many) - 1;
+            const uint32_t it = __shfl_sync(0xffffffffu, item, o), cn = __shfl_sync(0xffffffffu, cnt, o);
+            const DevCam &c = cams[__shfl_sync(0xffffffffu, ci, o)];
+            const uint32_t out = base + __shfl_sync(0xffffffffu, pre, o);
+            int rg[8];
+            unpack_ranges(ranges[it], rg);
+            uint32_t done = 0;
+            warp_supers(c, inv_s, rg, s_box[threadIdx.x >> 5], [&](int sx, int sy, bool keep) {
+                const uint32_t kept = __ballot_sync(0xffffffffu, keep), k = done + (uint32_t)__popc(kept & ((1u << lane) - 1u));
+                if (keep && k < cn) {
+                    const uint32_t st = (uint32_t)(c.stile_base + sy * c.stiles_x + sx);
+                    okeys[out + k] = st;
+                    ovals[out + k] = it;
+                    put_mask(omask, out + k, (M)tile_mask_general(c, rg, sx, sy, S));
+                    count(st);
+                }
+                done += (uint32_t)__popc(kept);
+            });
+        }
     }
     __syncthreads();
     if (smem)
@@ -1444,12 +1471,32 @@ __global__ void __launch_bounds__(256) k_masks_order(const DevCam *__restrict__ 
         }
         return;
     }
-    const uint64_t n = (uint64_t)misc[kMiscPairs], step = (uint64_t)(gridDim.x - order_blocks) * 256u;
-    for (uint64_t i = (uint64_t)(blockIdx.x - order_blocks) * 256u + t; (i & ~31ull) < n; i += step)
-        for (int w = 0; w < words; ++w) {
-            const uint32_t v = __reduce_or_sync(0xffffffffu, i < n ? mask[i * words + w] : 0u);
-            if (lane == 0) any[(i >> 5) * words + w] = v;
+    // a warp takes four groups at a time, their loads in flight together
+    constexpr int G = 4;
+    const uint64_t n = misc[kMiscPairs], step = (uint64_t)(gridDim.x - order_blocks) * (256u * G);
+    for (uint64_t i0 = ((uint64_t)(blockIdx.x - order_blocks) * 8u + (t >> 5)) * (32u * G); i0 < n; i0 += step) {
+        uint32_t m[G][2];
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            const uint64_t i = i0 + 32 * g + lane;
+            m[g][0] = m[g][1] = 0u;
+            if (i < n) {
+                if (words == 1) {
+                    m[g][0] = mask[i];
+                } else {
+                    const uint2 v = reinterpret_cast<const uint2 *>(mask)[i];
+                    m[g][0] = v.x;
+                    m[g][1] = v.y;
+                }
+            }
         }
+#pragma unroll
+        for (int g = 0; g < G; ++g)
+            for (int w = 0; w < words; ++w) {
+                const uint32_t v = __reduce_or_sync(0xffffffffu, w ? m[g][1] : m[g][0]);
+                if (lane == 0 && i0 + 32 * g < n) any[(i0 / 32 + g) * words + w] = v;
+            }
+    }
 }
 
 // One block: the backward's units and their schedule. A tile whose forward walk
@@ -1571,7 +1618,7 @@ cudaError_t launch_bin_front(const geer_workspace *ws, cudaStream_t s) {
              ws->n_stiles, ws->cap_pairs, 0, nullptr, 0);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || nblk == 0) return e;
-    launch_k(k_compact, dim3((unsigned)nblk, (unsigned)ws->n_cams), dim3(kPrepThreads), 0, s, ws->n_gauss, ws->d_count,
+    launch_k(k_compact, dim3((unsigned)((nblk + kCompact - 1) / kCompact), (unsigned)ws->n_cams), dim3(kPrepThreads), 0, s, ws->n_gauss, ws->d_count,
              ws->d_key, ws->d_blocksum, nblk, ws->d_ikey[0], ws->d_iid[0]);
     return cudaGetLastError();
 }
@@ -1597,7 +1644,8 @@ cudaError_t launch_duplicate(const geer_workspace *ws, cudaStream_t s) {
     uint32_t *scount = reinterpret_cast<uint32_t *>(ws->d_srange + ws->n_stiles);
     if (m > 0) {
         const size_t smem = ws->n_stiles <= kSmemTiles ? sizeof(uint32_t) * ws->n_stiles : 0;
-        launch_k(mask_words(ws->super_size) == 1 ? k_duplicate<uint32_t> : k_duplicate<uint64_t>, dim3((unsigned)m),
+        const int64_t blocks = std::min<int64_t>(m, (int64_t)ws->num_sms * 4);
+        launch_k(mask_words(ws->super_size) == 1 ? k_duplicate<uint32_t> : k_duplicate<uint64_t>, dim3((unsigned)blocks),
                  dim3(kPrepThreads), smem, s, ws->d_cams, ws->n_gauss, ws->super_size, ws->d_iid[0], ws->d_iid[1],
                  ws->d_ikey[0], ws->d_ikey[1], ws->d_ranges, ws->d_misc, ws->d_blocksum2, ws->d_keys[0], ws->d_vals[0], ws->d_smask[0], scount,
                  (int)ws->n_stiles, ws->cap_pairs);

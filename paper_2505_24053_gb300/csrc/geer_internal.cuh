@@ -236,7 +236,7 @@ __device__ __forceinline__ void sh_stage(float *s, const float *__restrict__ src
         // chunk k * 32 + lane: for degree 3 three chunks a lane span eight rows, so that
         // three places per lane and constant steps give all its chunks
         constexpr int kIters = (kChunks + 31) / 32, kPlaces = ST == NC ? 1 : 3;
-        static_assert(ST == NC || 96 % (NC / 4) == 0, "three chunks a lane are whole rows");
+        static_assert(ST == NC || NC == 48, "three chunks a lane are eight whole rows");
         const float *from = src + 4 * lane;
         float *to[kPlaces];
 #pragma unroll

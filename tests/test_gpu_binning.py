@@ -8,6 +8,8 @@
 - Lists of Gaussians whose association is several rectangles (boxes of more than 32
   super-tiles, several cameras) and item counts around a block, against the replica.
 - More block counts than one step of the scan takes (4096).
+- Tiles of few entries, walked without bounds, against the same tile with entries that
+  no ray hits behind them.
 - The one-block binning of small scenes against the general path, over the items a
   thread holds, cameras, equal depths and culled Gaussians.
 """
@@ -170,3 +172,29 @@ def test_small_front_equals_the_general_path(geer, n, ncams, fov):
     assert lists[0][:3] == lists[1][:3]
     for a, b in zip(lists[0][3:], lists[1][3:]):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("n", [1, 7, 8, 9, 12])
+@pytest.mark.parametrize("splat", [False, True])
+def test_tiles_of_few_entries(geer, n, splat):
+    rng = np.random.default_rng(n)
+    fov = math.radians(60)
+    cam = wl.Camera(wl.PINHOLE, 16, 16, fov)
+    i = rng.integers(1, 16, (40, 2))
+    ang = (i / 16 - 0.5) * fov  # between the rays, which lie at ((i + 1/2) / 16 - 1/2) fov
+    far = np.stack([np.tan(ang[:, 0]) * 20, np.tan(ang[:, 1]) * 20, np.full(40, 20.0)], 1)
+    near = np.stack([rng.uniform(-1, 1, n), rng.uniform(-1, 1, n), rng.uniform(3, 5, n)], 1)
+    quat = rng.standard_normal((n + 40, 4)).astype(np.float32)
+    scene = wl.Scene(np.concatenate([near, far]).astype(np.float32),
+                     np.concatenate([np.exp(rng.normal(-1.5, 0.5, (n, 3))), np.full((40, 3), 1e-4)]).astype(np.float32),
+                     quat, np.concatenate([rng.uniform(0.2, 0.9, n), np.full(40, 0.9)]).astype(np.float32),
+                     rng.normal(0, 0.3, (n + 40, 1, 3)).astype(np.float32), 0)
+    prm = geer.params_c(alpha_model=geer.ALPHA_SPLAT) if splat else None
+    images = []
+    for sc in (scene.subset(np.arange(n)), scene):
+        r = geer.Renderer([cam], sc.n, 0, params=prm)
+        T = torch.empty(256, device="cuda")
+        images.append((r.forward(geer.Gaussians.from_scene(sc), T=T), T, r.ws.pair_counts()[0]))
+    assert images[0][2] <= n and images[1][2] >= images[0][2] + 30
+    assert torch.equal(images[0][0], images[1][0]) and torch.equal(images[0][1], images[1][1])
+    assert float(images[0][1].min()) < 0.9

@@ -6,6 +6,8 @@
 // (__fmul_rn / __fadd_rn / __fsub_rn / __fdiv_rn / __fsqrt_rn, which the
 // compiler never contracts), so the tile ranges and depth keys are bit-for-bit
 // reproducible by an independent FP32 implementation of the same sequence.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 #include "geer_internal.cuh"
@@ -980,17 +982,21 @@ __global__ void __launch_bounds__(kPrepThreads) k_gather_counts(
     }
 }
 
-// Everything between the preprocess and the emission for at most kSmallItems (camera,
-// Gaussian) items, in one block: compaction, the stable depth sort (8-bit digits, the
-// keys and ids held in registers through a pass and reordered in shared memory; a pass
-// whose digit all keys share is skipped), the counting in depth order and the scans.
-// It leaves what those kernels leave (ids in buffer 0). Bound by the issue rate of its
-// one SM; the twelve launches it replaces take about 4 us each at these sizes, whatever
-// their work. From the preprocess to the render order, 1000 items take 38 us in place
-// of 69, 4096 46 of 71, 8192 56 of 69; at 10000 both take 67 to 69, hence the line. (The lanes
-// of a digit by a vote per bit: 60 at 8192; by __match_any_sync: 71.) K: items a thread.
-constexpr int kSmallItems = 8192, kSmallThreads = 1024;
-template <int K>
+// Everything between the preprocess and the emission for at most kClusterItems (camera,
+// Gaussian) items, in one block or in a cluster of C: compaction, the stable depth sort
+// (8-bit digits, the keys and ids held in registers through a pass and reordered in
+// shared memory; a pass whose digit all keys share is skipped), the counting in depth
+// order and the scans. It leaves what those kernels leave (ids in buffer 0). In a
+// cluster each block holds an equal part of the order, the digits' totals are read from
+// and the keys written to the other blocks' shared memory. One block is bound by the
+// issue rate of its SM, the cluster by its two barriers a pass; the twelve launches
+// replaced take about 4 us each at these sizes, whatever their work. Preprocess to
+// render order, one block / cluster / launches: 2048 items 41 / - / 67 us, 4096
+// 45 / - / 71, 6000 51 / 50 / 73, 8192 57 / 51 / 69, 12001 78 / 56 / 73, 20000 - / 63 /
+// 73, 32768 - / 73 / 75: hence the lines. (The lanes of a digit by a vote per bit instead
+// of shared masks: 60 at 8192; by __match_any_sync: 71.) K: items a thread.
+constexpr int kSmallItems = 4096, kClusterItems = 32768, kSmallThreads = 1024, kCluster = 8;
+template <int K, int C>
 __global__ void __launch_bounds__(kSmallThreads) k_small_front(
     const DevCam *__restrict__ cams, int64_t n, int items, int S, const uint32_t *__restrict__ count,
     const uint32_t *__restrict__ key, const uint4 *__restrict__ ranges, uint32_t *__restrict__ misc,
@@ -1007,16 +1013,21 @@ __global__ void __launch_bounds__(kSmallThreads) k_small_front(
     __shared__ uint32_t s_wsum[W];
     __shared__ int4 s_box[W][9];
     __shared__ uint32_t s_sum[CHUNKS][2];
+    // what the other blocks of the cluster read: live items, digit totals (two passes' in turn), pairs and tiles
+    __shared__ uint32_t s_live, s_dig[C > 1 ? 2 : 1][kRadix], s_low[kSmallThreads / kRadix][C > 1 ? kRadix : 1];
+    __shared__ unsigned long long s_total[2];
+    const auto cluster = cooperative_groups::this_cluster();
+    const int cta = C > 1 ? (int)cluster.block_rank() : 0;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const uint32_t below = (1u << lane) - 1u;
-    for (int64_t i = t; i < nst; i += kSmallThreads) scount[i] = 0u;
+    for (int64_t i = cta * kSmallThreads + t; i < nst; i += C * kSmallThreads) scount[i] = 0u;
     for (int i = t; i < W * kRadix; i += kSmallThreads) (&s_match[0][0])[i] = 0u;
     for (int i = t; i < 2 * CHUNKS; i += kSmallThreads) (&s_sum[0][0])[i] = 0u;
     // compaction in index order: a warp's 32 K consecutive items
     uint32_t kk[K], live[K], mine = 0;
 #pragma unroll
     for (int k = 0; k < K; ++k) {
-        const int i = (warp * K + k) * 32 + lane;
+        const int i = ((cta * W + warp) * K + k) * 32 + lane;
         const bool on = i < items && count[i] > 0u;
         kk[k] = i < items ? key[i] : 0u;
         live[k] = __ballot_sync(0xffffffffu, on);
@@ -1030,40 +1041,67 @@ __global__ void __launch_bounds__(kSmallThreads) k_small_front(
         const uint32_t y = __shfl_up_sync(0xffffffffu, v, o);
         if (lane >= o) v += y;
     }
-    const int L = (int)__shfl_sync(0xffffffffu, v, 31);
+    int L = (int)__shfl_sync(0xffffffffu, v, 31);
     uint32_t at = warp ? __shfl_sync(0xffffffffu, v, max(warp - 1, 0)) : 0u;
+    // C > 1: block c holds the places [c per, (c + 1) per) of the order
+    int per = K * kSmallThreads, own = L;
+    if constexpr (C > 1) {
+        if (t == 0) s_live = (uint32_t)L;
+        cluster.sync();
+        L = 0;
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            const int x = (int)*cluster.map_shared_rank(&s_live, c);
+            at += c < cta ? x : 0;
+            L += x;
+        }
+        per = max((L + C * kPrepThreads - 1) / (C * kPrepThreads), 1) * kPrepThreads;
+        own = min(max(L - cta * per, 0), per);
+    }
+    const auto put = [&](uint32_t pos, uint32_t k, uint32_t val) {
+        if constexpr (C > 1) {
+            const int c = (int)pos / per, e = (int)pos - c * per;
+            cluster.map_shared_rank(s_key, c)[e] = k;
+            cluster.map_shared_rank(s_val, c)[e] = (uint16_t)val;
+        } else {
+            s_key[pos] = k;
+            s_val[pos] = (uint16_t)val;
+        }
+    };
+    const auto sync_all = [&] {
+        if constexpr (C > 1) cluster.sync();
+        else __syncthreads();
+    };
 #pragma unroll
     for (int k = 0; k < K; ++k) {
         if (live[k] >> lane & 1u) {
-            const uint32_t pos = at + (uint32_t)__popc(live[k] & below);
-            s_key[pos] = kk[k];
-            s_val[pos] = (uint16_t)((warp * K + k) * 32 + lane);
+            put(at + (uint32_t)__popc(live[k] & below), kk[k], (uint32_t)(((cta * W + warp) * K + k) * 32 + lane));
         }
         at += (uint32_t)__popc(live[k]);
     }
-    __syncthreads();
+    sync_all();
     // the sort: a warp takes 32 kr consecutive keys
-    const int kr = (L + kSmallThreads - 1) / kSmallThreads;
+    const int kr = ((C > 1 ? per : L) + kSmallThreads - 1) / kSmallThreads;
 #pragma unroll 1
     for (int shift = 0; shift < 32; shift += kRadixBits) {
         uint32_t val[K], rank[K];
-        const uint32_t d0 = L > 0 ? (s_key[0] >> shift) & 0xffu : 0u;
+        const uint32_t d0 = own > 0 ? (s_key[0] >> shift) & 0xffu : 0u;
         bool same = true;
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             const int e = (warp * kr + k) * 32 + lane;
-            if (k < kr && e < L) {
+            if (k < kr && e < own) {
                 kk[k] = s_key[e];
                 val[k] = s_val[e];
                 same = same && ((kk[k] >> shift) & 0xffu) == d0;
             }
         }
         for (int i = t; i < W * kRadix; i += kSmallThreads) (&s_hist[0][0])[i] = 0u;
-        if (__syncthreads_and(same)) continue;
+        if (__syncthreads_and(same) && C == 1) continue;
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             if (k >= kr) break;
-            const bool on = (warp * kr + k) * 32 + lane < L;
+            const bool on = (warp * kr + k) * 32 + lane < own;
             const uint32_t d = on ? (kk[k] >> shift) & 0xffu : 0u;
             if (on) atomicOr(&s_match[warp][d], 1u << lane);
             const uint32_t b = s_hist[warp][d];
@@ -1096,6 +1134,24 @@ __global__ void __launch_bounds__(kSmallThreads) k_small_front(
             pre += p < q ? x : 0u;
             tot += x;
         }
+        if constexpr (C > 1) {
+            // the blocks' totals of the digit; a quarter of this block reads a quarter of them
+            static_assert(C == 2 * (kSmallThreads / kRadix), "two blocks a quarter");
+            uint32_t *dig = s_dig[shift / kRadixBits & 1];
+            if (q == 0) dig[d] = tot;
+            cluster.sync();
+            const uint32_t x0 = cluster.map_shared_rank(dig, 2 * q)[d], x1 = cluster.map_shared_rank(dig, 2 * q + 1)[d];
+            s_part[q][d] = x0 + x1;
+            s_low[q][d] = (2 * q < cta ? x0 : 0u) + (2 * q + 1 < cta ? x1 : 0u);
+            __syncthreads();
+            tot = 0;
+#pragma unroll
+            for (int p = 0; p < kSmallThreads / kRadix; ++p) {
+                tot += s_part[p][d];
+                pre += s_low[p][d];
+            }
+            if (__syncthreads_or(tot == (uint32_t)L)) continue;  // (in every block alike)
+        }
         uint32_t sc = tot;  // scan over the digits (each quarter of the block the same)
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -1115,19 +1171,16 @@ __global__ void __launch_bounds__(kSmallThreads) k_small_front(
         __syncthreads();
 #pragma unroll
         for (int k = 0; k < K; ++k)
-            if (k < kr && (warp * kr + k) * 32 + lane < L) {
-                const uint32_t pos = s_hist[warp][(kk[k] >> shift) & 0xffu] + rank[k];
-                s_key[pos] = kk[k];
-                s_val[pos] = (uint16_t)val[k];
-            }
-        __syncthreads();
+            if (k < kr && (warp * kr + k) * 32 + lane < own)
+                put(s_hist[warp][(kk[k] >> shift) & 0xffu] + rank[k], kk[k], val[k]);
+        sync_all();
     }
     // the counting, in depth order
     const uint32_t inv_s = super_inverse(S);
-    for (int i0 = 0; i0 < L; i0 += kSmallThreads) {
-        const int i = i0 + t;
-        const bool on = i < L;
-        const uint32_t item = on ? s_val[i] : 0u;
+    for (int e0 = 0; e0 < own; e0 += kSmallThreads) {
+        const int e = e0 + t, i = cta * per + e;
+        const bool on = e < own;
+        const uint32_t item = on ? s_val[e] : 0u;
         const uint4 r4 = on ? ranges[item] : make_uint4(0u, 0u, 0u, 0u);
         const ItemPairs p = warp_item_pairs(cams, inv_s, on, (int)(item / (uint32_t)n), r4, s_box[warp]);
         if (on) {
@@ -1138,35 +1191,43 @@ __global__ void __launch_bounds__(kSmallThreads) k_small_front(
         }
         const uint32_t tiles = __reduce_add_sync(0xffffffffu, p.tiles), supers = __reduce_add_sync(0xffffffffu, p.supers);
         if (lane == 0) {
-            atomicAdd(&s_sum[i / kPrepThreads][0], supers);
-            atomicAdd(&s_sum[i / kPrepThreads][1], tiles);
+            atomicAdd(&s_sum[e / kPrepThreads][0], supers);
+            atomicAdd(&s_sum[e / kPrepThreads][1], tiles);
         }
     }
+    if (t < 2) s_total[t] = 0ull;
     __syncthreads();
+    if (t < 2 * CHUNKS) atomicAdd(&s_total[t & 1], (unsigned long long)s_sum[t >> 1][t & 1]);
+    sync_all();
+    unsigned long long pairs = 0, all_pairs = 0, all_tiles = 0;  // pairs: of the blocks before
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+        const unsigned long long *x = C > 1 ? cluster.map_shared_rank(s_total, c) : s_total;
+        pairs += c < cta ? x[0] : 0ull;
+        all_pairs += x[0];
+        all_tiles += x[1];
+    }
+    if constexpr (C > 1) cluster.sync();  // a block's shared memory is read until here
     if (warp > 0) return;
-    unsigned long long pairs = 0, tiles = 0;
     for (int c0 = 0; c0 < CHUNKS; c0 += 32) {
         const uint32_t a = c0 + lane < CHUNKS ? s_sum[c0 + lane][0] : 0u;
-        unsigned long long x = a, y = c0 + lane < CHUNKS ? s_sum[c0 + lane][1] : 0u;
+        unsigned long long x = a;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long u = __shfl_up_sync(0xffffffffu, x, o), w = __shfl_up_sync(0xffffffffu, y, o);
-            if (lane >= o) {
-                x += u;
-                y += w;
-            }
+            const unsigned long long u = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += u;
         }
-        if ((c0 + lane) * kPrepThreads < L) bs_super[c0 + lane] = (uint32_t)min(pairs + x - a, 0xffffffffull);
+        if ((c0 + lane) * kPrepThreads < own)
+            bs_super[cta * per / kPrepThreads + c0 + lane] = (uint32_t)min(pairs + x - a, 0xffffffffull);
         pairs += __shfl_sync(0xffffffffu, x, 31);
-        tiles += __shfl_sync(0xffffffffu, y, 31);
     }
-    if (lane == 0) {
+    if (cta == 0 && lane == 0) {
         misc[kMiscLive] = (uint32_t)L;
         misc[kMiscSortCur] = 1u;  // the sorted ids are in buffer 0 (depth_sorted_buf)
         misc[kMiscSortSame] = 0u;
-        misc[kMiscTileLo] = (uint32_t)tiles;
-        misc[kMiscTileHi] = (uint32_t)(tiles >> 32);
-        put_pair_total(misc, pairs, cap);
+        misc[kMiscTileLo] = (uint32_t)all_tiles;
+        misc[kMiscTileHi] = (uint32_t)(all_tiles >> 32);
+        put_pair_total(misc, all_pairs, cap);
     }
 }
 
@@ -1642,26 +1703,29 @@ cudaError_t launch_preprocess(const geer_workspace *ws, const geer_gaussians *g,
     return cudaGetLastError();
 }
 
-// Few enough items for one block to do the work of launch_bin_front, launch_depth_sort
+// Few enough items for one block or cluster to do the work of launch_bin_front, launch_depth_sort
 // and launch_count_pairs (k_small_front, launched as launch_bin_front).
-bool small_front(const geer_workspace *ws) { return (int64_t)ws->n_cams * ws->n_gauss <= kSmallItems; }
+bool small_front(const geer_workspace *ws) { return (int64_t)ws->n_cams * ws->n_gauss <= kClusterItems; }
 
 static cudaError_t launch_small_front(const geer_workspace *ws, cudaStream_t s) {
     const int items = (int)(ws->n_cams * ws->n_gauss);
-    static_assert(kSmallItems == 8 * kSmallThreads && kSmallItems <= 65536, "eight items a thread at most, 16-bit ids");
-    const auto launch = [&](auto *kern, int k) {
+    static_assert(kSmallItems <= 8 * kSmallThreads && kClusterItems <= 4 * kCluster * kSmallThreads && kClusterItems <= 65536,
+                  "items a thread, 16-bit ids");
+    const auto launch = [&](auto *kern, int k, int blocks) {
         const int smem = 2 * (int)sizeof(uint32_t) * kSmallThreads / 32 * kRadix + 6 * k * kSmallThreads;
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
-        launch_k(kern, dim3(1), dim3(kSmallThreads), smem, s, ws->d_cams, ws->n_gauss, items, ws->super_size,
+        launch_cluster(kern, dim3((unsigned)blocks), dim3(kSmallThreads), smem, s, (unsigned)blocks, ws->d_cams, ws->n_gauss, items, ws->super_size,
                  ws->d_count, ws->d_key, ws->d_ranges, ws->d_misc, ws->d_iid[0], ws->d_iid[1], ws->d_ikey[0],
                  ws->d_ikey[1], ws->d_blocksum2, reinterpret_cast<uint32_t *>(ws->d_srange + ws->n_stiles),
                  ws->n_stiles, ws->cap_pairs);
         return cudaGetLastError();
     };
-    return items <= kSmallThreads       ? launch(k_small_front<1>, 1)
-           : items <= 4 * kSmallThreads ? launch(k_small_front<4>, 4)
-                                        : launch(k_small_front<8>, 8);
+    if (items <= kSmallThreads) return launch(k_small_front<1, 1>, 1, 1);
+    if (items <= 4 * kSmallThreads) return launch(k_small_front<4, 1>, 4, 1);
+    if (items <= kCluster * kSmallThreads) return launch(k_small_front<1, kCluster>, 1, kCluster);
+    if (items <= 2 * kCluster * kSmallThreads) return launch(k_small_front<2, kCluster>, 2, kCluster);
+    return launch(k_small_front<4, kCluster>, 4, kCluster);
 }
 
 cudaError_t launch_bin_front(const geer_workspace *ws, cudaStream_t s) {

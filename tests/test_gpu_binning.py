@@ -10,8 +10,8 @@
 - More block counts than one step of the scan takes (4096).
 - Tiles of few entries, walked without bounds, against the same tile with entries that
   no ray hits behind them.
-- The one-block binning of small scenes against the general path, over the items a
-  thread holds, cameras, equal depths and culled Gaussians.
+- The binning of small scenes by one block or a cluster against the general path, over
+  the items a thread holds, cameras, equal depths and culled Gaussians.
 """
 import math
 
@@ -139,10 +139,11 @@ def test_more_sort_tiles_than_blocks(geer):
 
 
 @pytest.mark.parametrize("n,ncams", [(1, 1), (31, 1), (1024, 1), (1025, 1), (341, 3), (4096, 1), (2049, 2), (4097, 1),
-                                     (2730, 3), (8192, 1)])
+                                     (2731, 3), (8192, 1), (16384, 1), (16385, 1),
+                                     (32768, 1)])
 @pytest.mark.parametrize("fov", [80, 205])
 def test_small_front_equals_the_general_path(geer, n, ncams, fov):
-    """At most 8192 items are binned by one block; the same scene with culled
+    """At most 32768 items are binned by one block or a cluster; the same scene with culled
     Gaussians behind it takes the general path. Same lists, in the same order."""
     rng = np.random.default_rng(n + fov)
     mean = rng.uniform(-2, 2, (n, 3)).astype(np.float32)
@@ -153,7 +154,7 @@ def test_small_front_equals_the_general_path(geer, n, ncams, fov):
     scene = wl.Scene(mean, np.exp(rng.normal(-4.0, 0.8, (n, 3))).astype(np.float32),
                      rng.standard_normal((n, 4)).astype(np.float32), opacity,
                      rng.normal(0, 0.3, (n, 1, 3)).astype(np.float32), 0)
-    pad = 8193
+    pad = 32769
     big = wl.Scene(*(np.concatenate([a, np.resize(a, (pad,) + a.shape[1:])]) for a in
                      (scene.mean, scene.scale, scene.quat)),
                    np.concatenate([opacity, np.zeros(pad, np.float32)]),

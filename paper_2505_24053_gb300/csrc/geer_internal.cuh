@@ -313,11 +313,11 @@ static_assert(kCkptMax + 1 <= kUnitCountByte, "the unit buckets and their count 
 // Stages timed by geer_enable_timing (CUDA events around each stage's kernels).
 enum Stage : int {
     kStagePreprocess = 0,
-    kStageBinFront,      // live-item scan + compaction
+    kStageBinFront,      // live-item scan + compaction (small scenes: all up to the emission)
     kStageDepthSort,
     kStageCountPairs,
-    kStageDuplicate,     // super-tile pairs, super-tile ranges, render order
-    kStageTileSort,      // sort of the super-tile pairs
+    kStageDuplicate,     // super-tile pairs, super-tile ranges
+    kStageTileSort,      // sort of the super-tile pairs, group masks, render order
     kStageRenderFwd,
     kStageRenderBwd,
     kStagePreprocessBwd,

@@ -89,8 +89,12 @@ __device__ __forceinline__ void sh_grad(int k, const ShDir &d, float g[3]) {
 // camera the SH row itself is overwritten by its gradient chunk by chunk, which
 // halves the shared memory; with several cameras the gradient has a row of its own.
 constexpr int kPBThreads = 64;
+// Resident blocks of the one-camera variant. Degree 3 holds its chain in 96 registers
+// with 12 B of spills (1M Gaussians: 104 us with 14 blocks, 72 registers and 140 B of
+// spills, 103 with 12, 90 with 10, 104 with 8); the lower degrees spill little and take
+// the warps (300K of degree 2: 35 us with 14, 38 with 10).
 #ifndef GEER_PB_MINB
-#define GEER_PB_MINB 14  // resident blocks of the one-camera variant: caps registers at 72
+#define GEER_PB_MINB (DEG == 3 ? 10 : 14)
 #endif
 #ifndef GEER_PB_MINB_CAMS
 // Of the variant for several cameras: 204 registers (the next camera's loads overlap the

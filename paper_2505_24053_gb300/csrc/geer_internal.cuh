@@ -364,7 +364,7 @@ struct geer_workspace {
     uint32_t *d_group_sum;  // [cap_sort_groups][kRadix] (zero between passes)
     uint32_t *d_group_excl; // [cap_sort_groups][kRadix]
     uint32_t *d_digit_base; // [kRadix]
-    uint32_t *d_misc;       // [kMiscCount], then the render order's bucket cursors [kOrderBuckets]
+    uint32_t *d_misc;       // [kMiscCount], then the first place of the render order's buckets [kOrderBuckets]
     uint2 *d_tile_walk;     // [cap_tiles] per tile, where the forward's scan of its super-tile list ended:
                             // (position, tile-list entries found before it); followed by [cap_tiles] u32 scratch
     uint32_t *d_tile_order; // [cap_tiles] tiles by descending super-tile list length: the forward's schedule

@@ -1488,6 +1488,17 @@ __device__ __forceinline__ uint32_t block_chunk_prefix(uint32_t s, uint32_t *war
     return pre;
 }
 
+// The super-tile of tile i, or -1 for a tile that a slot layout leaves unused. c: the camera
+// to start looking at (0, then as the call before left it if i has not decreased).
+__device__ __forceinline__ int tile_super(const DevCam *__restrict__ cams, int ncams, uint32_t inv_s, int i, int &c) {
+    while (c + 1 < ncams && cams[c + 1].tile_base <= i) ++c;
+    const DevCam &cm = cams[c];
+    const int lt = i - cm.tile_base;
+    if (lt < 0 || lt >= cm.tiles_x * cm.tiles_y) return -1;
+    const int cy = lt / cm.tiles_x, cx = lt - cy * cm.tiles_x;
+    return cm.stile_base + super_of(cy, inv_s) * cm.stiles_x + super_of(cx, inv_s);
+}
+
 // IdentifyFrustumRanges at super-tile granularity, block 0: each super-tile's
 // [start, end) in the sorted super-tile pairs (exclusive scan of its pair count),
 // and the places of the buckets in the order in which the render blocks take the
@@ -1495,27 +1506,41 @@ __device__ __forceinline__ uint32_t block_chunk_prefix(uint32_t s, uint32_t *war
 // costliest tiles start first and the grid does not end on a tail of heavy tiles.
 // (Measured on the 1M-Gaussian fisheye workload: 0.344 ms forward against 0.358 -
 // 0.409 ms with the length capped at 16K - 1K entries and 0.424 ms in tile order.)
-// A super-tile adds its tiles to its bucket; k_masks_order then places them. The
-// other blocks reset the fused render's unit queue. (One block that also walked all
-// the tiles and the queue took 100 us on four 1920 x 1536 cameras.)
+// A super-tile adds its tiles to its bucket; k_masks_order then places them. Blocks 1 to
+// order_blocks - 1 count, per bucket, the tiles that the blocks of that kernel but the
+// last will place; the others reset the fused render's unit queue. (One block that also
+// walked all the tiles and the queue took 100 us on four 1920 x 1536 cameras.)
 constexpr int kQueueBlock = 8 * 1024;  // queue words reset by a block
-__global__ void __launch_bounds__(1024) k_tile_offsets(const DevCam *__restrict__ cams, int ncams, int S,
+__global__ void __launch_bounds__(1024) k_tile_offsets(const DevCam *__restrict__ cams, int ncams, int S, int ntiles,
                                                        uint2 *__restrict__ srange, int nst,
-                                                       uint32_t *__restrict__ misc,
+                                                       uint32_t *__restrict__ misc, uint32_t *__restrict__ counts,
+                                                       int order_blocks,
                                                        uint32_t *__restrict__ queue, uint32_t queue_n) {
     grid_dep_sync();
     const int t = threadIdx.x;
+    __shared__ uint32_t warp_tot[32];
+    __shared__ uint32_t hist[kOrderBuckets];
     // the fused render's unit queue and its counters start afresh with every binning
-    if (blockIdx.x > 0) {
-        const uint32_t q0 = (blockIdx.x - 1) * (uint32_t)kQueueBlock, q1 = min(queue_n, q0 + kQueueBlock);
+    if ((int)blockIdx.x >= order_blocks) {
+        const uint32_t q0 = (blockIdx.x - order_blocks) * (uint32_t)kQueueBlock, q1 = min(queue_n, q0 + kQueueBlock);
         for (uint32_t i = q0 + t; i < q1; i += 1024) queue[i] = 0xffffffffu;
         return;
     }
-    if (queue && t < 4) misc[kMiscFwdNext + t] = 0u;
-    __shared__ uint32_t warp_tot[32];
-    __shared__ uint32_t hist[kOrderBuckets];
+    if (blockIdx.x == 0 && queue && t < 4) misc[kMiscFwdNext + t] = 0u;
     if (misc[kMiscStatus] & kStatusCapacity) return;
     for (int i = t; i < kOrderBuckets; i += 1024) hist[i] = 0u;
+    if (blockIdx.x > 0) {
+        // the tiles of k_masks_order's block blockIdx.x - 1 per bucket
+        __syncthreads();
+        const int i = t * order_blocks + (int)blockIdx.x - 1;
+        int c = 0;
+        const int st = i < ntiles ? tile_super(cams, ncams, super_inverse(S), i, c) : -1;
+        bucket_add(hist, i < ntiles,
+                   st >= 0 ? order_bucket(reinterpret_cast<const uint32_t *>(srange + nst)[st]) : kOrderBuckets - 1);
+        __syncthreads();
+        for (int b = t; b < kOrderBuckets; b += 1024) counts[(blockIdx.x - 1) * kOrderBuckets + b] = hist[b];
+        return;
+    }
     // super-tile ranges
     const uint32_t *scount = reinterpret_cast<const uint32_t *>(srange + nst);
     const int schunk = (nst + 1023) / 1024;
@@ -1541,47 +1566,48 @@ __global__ void __launch_bounds__(1024) k_tile_offsets(const DevCam *__restrict_
     for (int i = t; i < kOrderBuckets; i += 1024) misc[kMiscCount + i] = hist[i];
 }
 
-// After the sort of the super-tile pairs. Blocks [0, order_blocks): 1024 tiles each
-// take their places in the render order, a block's tiles of a bucket together.
+// After the sort of the super-tile pairs. Blocks [0, order_blocks) place 1024 tiles each
+// in the render order: block k the tiles k, k + order_blocks, k + 2 order_blocks, ...,
+// in each bucket behind those of the blocks before it (counts), so that tiles rendered at
+// the same time lie apart in the image. The order is part of a gradient's rounding: the
+// sums of a Gaussian over hundreds of tiles are added as the tiles finish. With runs of
+// neighbouring tiles in turn, placed as their blocks came, the scale gradients of needles
+// near the cameras, small differences of large sums, moved: four 1920 x 1536 cameras, 6M
+// Gaussians, the means of four runs by 1.4e-6 of the gradients' norm and single ones by
+// 4e-3 of their size, where the runs of one order give 0.7e-6 and 1e-3. (The same time.)
 // The others: the or of every 32 sorted pairs' tile masks (a warp per group): the
 // render's list scan skips the groups without an entry of its tile.
 __global__ void __launch_bounds__(256) k_masks_order(const DevCam *__restrict__ cams, int ncams, int S, int ntiles,
                                                      const uint2 *__restrict__ srange, uint32_t *__restrict__ order,
-                                                     int order_blocks, const uint32_t *__restrict__ mask, int words,
-                                                     uint32_t *__restrict__ misc, uint32_t *__restrict__ any) {
+                                                     int order_blocks, const uint32_t *__restrict__ counts,
+                                                     const uint32_t *__restrict__ mask, int words,
+                                                     const uint32_t *__restrict__ misc, uint32_t *__restrict__ any) {
     grid_dep_sync();
     if (misc[kMiscStatus] & kStatusCapacity) return;
     const int t = threadIdx.x, lane = t & 31;
     if ((int)blockIdx.x < order_blocks) {
         __shared__ uint32_t hist[kOrderBuckets];
-        if (t < kOrderBuckets) hist[t] = 0u;
-        __syncthreads();
         const uint32_t inv_s = super_inverse(S);
-        int bk[4], c = 0;
-        uint32_t rank[4];
+        const int i0 = t * order_blocks + (int)blockIdx.x;
+        int c = 0;
+        uint2 r[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const int i = (int)blockIdx.x * 1024 + u * 256 + t;
-            bk[u] = kOrderBuckets - 1;  // the tiles that a slot layout leaves unused come last
-            if (i < ntiles) {
-                while (c + 1 < ncams && cams[c + 1].tile_base <= i) ++c;
-                const DevCam &cm = cams[c];
-                const int lt = i - cm.tile_base;
-                if (lt >= 0 && lt < cm.tiles_x * cm.tiles_y) {
-                    const int cy = lt / cm.tiles_x, cx = lt - cy * cm.tiles_x;
-                    const uint2 r = srange[cm.stile_base + super_of(cy, inv_s) * cm.stiles_x + super_of(cx, inv_s)];
-                    bk[u] = order_bucket(r.y - r.x);
-                }
-            }
-            rank[u] = bucket_add(hist, i < ntiles, bk[u]);
+            const int i = i0 + u * 256 * order_blocks, st = i < ntiles ? tile_super(cams, ncams, inv_s, i, c) : -1;
+            r[u] = st >= 0 ? srange[st] : make_uint2(0u, 0u);
+        }
+        if (t < kOrderBuckets) {
+            uint32_t at = misc[kMiscCount + t];
+#pragma unroll 8
+            for (int k = 0; k < (int)blockIdx.x; ++k) at += counts[k * kOrderBuckets + t];
+            hist[t] = at;
         }
         __syncthreads();
-        if (t < kOrderBuckets && hist[t]) hist[t] = atomicAdd(&misc[kMiscCount + t], hist[t]);
-        __syncthreads();
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const int i = (int)blockIdx.x * 1024 + u * 256 + t;
-            if (i < ntiles) order[hist[bk[u]] + rank[u]] = (uint32_t)i;
+            const int i = i0 + u * 256 * order_blocks;
+            const uint32_t at = bucket_add(hist, i < ntiles, order_bucket(r[u].y - r[u].x));
+            if (i < ntiles) order[at] = (uint32_t)i;
         }
         return;
     }
@@ -1756,6 +1782,14 @@ cudaError_t launch_count_pairs(const geer_workspace *ws, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+// The blocks that place 1024 tiles each in the render order, and their bucket counts (all
+// blocks' but the last one's), which live in the scratch words behind the walk records.
+static int order_blocks(const geer_workspace *ws) { return (int)((ws->n_tiles + 1023) / 1024); }
+static uint32_t *order_counts(const geer_workspace *ws) {
+    static_assert(kOrderBuckets < 1024, "a word per tile holds a row of counts per 1024 tiles");
+    return reinterpret_cast<uint32_t *>(ws->d_tile_walk + ws->n_tiles);
+}
+
 cudaError_t launch_duplicate(const geer_workspace *ws, cudaStream_t s) {
     const int64_t m = prep_blocks((int64_t)ws->n_cams * ws->n_gauss);
     uint32_t *scount = reinterpret_cast<uint32_t *>(ws->d_srange + ws->n_stiles);
@@ -1770,18 +1804,18 @@ cudaError_t launch_duplicate(const geer_workspace *ws, cudaStream_t s) {
         if (e != cudaSuccess) return e;
     }
     const uint32_t queue_n = ws->trains ? (uint32_t)(ws->n_tiles * (kCkptMax + 1)) : 0u;
-    launch_k(k_tile_offsets, dim3(1 + (queue_n + kQueueBlock - 1) / kQueueBlock), dim3(1024), 0, s, ws->d_cams,
-             ws->n_cams, ws->super_size, ws->d_srange, (int)ws->n_stiles, ws->d_misc,
-             ws->trains ? ws->d_bwd_order : nullptr, queue_n);
+    const int first = std::max(1, order_blocks(ws));
+    launch_k(k_tile_offsets, dim3(first + (queue_n + kQueueBlock - 1) / kQueueBlock), dim3(1024), 0, s, ws->d_cams,
+             ws->n_cams, ws->super_size, (int)ws->n_tiles, ws->d_srange, (int)ws->n_stiles, ws->d_misc,
+             order_counts(ws), first, ws->trains ? ws->d_bwd_order : nullptr, queue_n);
     return cudaGetLastError();
 }
 
 cudaError_t launch_masks_order(const geer_workspace *ws, cudaStream_t s) {
     const int64_t blocks = std::min<int64_t>(std::max<int64_t>(1, (ws->cap_pairs + 255) / 256), (int64_t)ws->num_sms * 8);
-    const int order_blocks = (int)((ws->n_tiles + 1023) / 1024);
-    launch_k(k_masks_order, dim3((unsigned)(blocks + order_blocks)), dim3(256), 0, s, ws->d_cams, ws->n_cams,
-             ws->super_size, (int)ws->n_tiles, ws->d_srange, ws->d_tile_order, order_blocks,
-             (const uint32_t *)ws->d_smask[ws->sorted_buf], mask_words(ws->super_size), ws->d_misc, ws->d_sany);
+    launch_k(k_masks_order, dim3((unsigned)(blocks + order_blocks(ws))), dim3(256), 0, s, ws->d_cams, ws->n_cams,
+             ws->super_size, (int)ws->n_tiles, ws->d_srange, ws->d_tile_order, order_blocks(ws),
+             (const uint32_t *)order_counts(ws), (const uint32_t *)ws->d_smask[ws->sorted_buf], mask_words(ws->super_size), ws->d_misc, ws->d_sany);
     return cudaGetLastError();
 }
 

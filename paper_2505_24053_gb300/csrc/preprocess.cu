@@ -1795,8 +1795,14 @@ cudaError_t launch_duplicate(const geer_workspace *ws, cudaStream_t s) {
     uint32_t *scount = reinterpret_cast<uint32_t *>(ws->d_srange + ws->n_stiles);
     if (m > 0) {
         const size_t smem = ws->n_stiles <= kSmemTiles ? sizeof(uint32_t) * ws->n_stiles : 0;
+        auto *kern = mask_words(ws->super_size) == 1 ? k_duplicate<uint32_t> : k_duplicate<uint64_t>;
+        // the counters come beside ~10 KB of lists: from ~9780 super-tiles on more than the 48 KB of a plain launch
+        if (smem > 32 * 1024) {
+            const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+        }
         const int64_t blocks = std::min<int64_t>(m, (int64_t)ws->num_sms * 4);
-        launch_k(mask_words(ws->super_size) == 1 ? k_duplicate<uint32_t> : k_duplicate<uint64_t>, dim3((unsigned)blocks),
+        launch_k(kern, dim3((unsigned)blocks),
                  dim3(kPrepThreads), smem, s, ws->d_cams, ws->n_gauss, ws->super_size, ws->d_iid[0], ws->d_iid[1],
                  ws->d_ikey[0], ws->d_ikey[1], ws->d_ranges, ws->d_misc, ws->d_blocksum2, ws->d_keys[0], ws->d_vals[0], ws->d_smask[0], scount,
                  (int)ws->n_stiles, ws->cap_pairs);

@@ -15,6 +15,7 @@
 // the camera (o_u . d_u >= 0), stopping before the contributor that would take
 // the transmittance below T_min (App. B.1 colour equation, 3DGS thresholds).
 #include <algorithm>
+#include <type_traits>
 
 #include "geer_internal.cuh"
 
@@ -1091,6 +1092,7 @@ struct BwdRay {
 //          dq/dA = D0^2, dq/dB = 2 D0 D1, dq/dC = D1^2.
 struct RayGrad {
     float wgt, sig, r0, r1, r2, o0, o1, o2;
+    bool act;  // whether the ray hits (wgt is 0 if it does not)
 };
 
 template <bool SPLAT>
@@ -1106,6 +1108,7 @@ __device__ __forceinline__ RayGrad ray_gradient(BwdRay &r, const float4 &a, cons
     RayGrad g;
     const float wgt = Ti * alpha;
     g.wgt = act ? wgt : 0.0f;
+    g.act = act;
     // dL/dalpha = sum_ch g_ch (T_i c_ch - S_ch / (1 - alpha)) = T_i (g . c) - (g . S) / (1 - alpha)
     const float gc = fmaf(r.g0, e.y, fmaf(r.g1, e.z, r.g2 * e.w));
     const float dLda = fmaf(Ti, gc, -r.gS * inv_om);
@@ -1157,6 +1160,12 @@ __device__ __forceinline__ RayGrad ray_gradient(BwdRay &r, const float4 &a, cons
 // selecting in every exchange took ~75. The tree of each value's sum is the plain
 // butterfly's. (With the branch-free gradient and the warps' entry lists: the
 // 1M-Gaussian training step 1010 -> 927 us, the surround step 21.0 -> 19.35 ms.)
+//
+// A product with zero does not mask an infinity or NaN, which would reach the sums of
+// another column and those of entries that the ray does not hit. ODD selects instead:
+// for the warps where a ray's dL/dC or colour behind is not finite, or large enough for
+// a product to overflow. (Selecting always: 1029 us for the 1M-Gaussian training step,
+// where both sets of sums beside each other take 845, as one did.)
 struct LanePerm {
     float2 d01, d23, b01, b23, g01, g23;
     int off;
@@ -1185,15 +1194,15 @@ __device__ __forceinline__ float2 xchg2(float2 keep, float2 send, int w) {
     return add2(keep, make_float2(__shfl_xor_sync(0xffffffffu, send.x, w), __shfl_xor_sync(0xffffffffu, send.y, w)));
 }
 
-template <bool SPLAT>
+template <bool SPLAT, bool ODD>
 __device__ __forceinline__ float warp_sum(const RayGrad &g, const BwdRay &r, const LanePerm &q) {
     const int lane = threadIdx.x & 31;
     if (SPLAT) {
         float v[16];
         v[0] = g.sig;
-        v[1] = g.wgt * r.g0;
-        v[2] = g.wgt * r.g1;
-        v[3] = g.wgt * r.g2;
+        v[1] = ODD && !g.act ? 0.0f : g.wgt * r.g0;
+        v[2] = ODD && !g.act ? 0.0f : g.wgt * r.g1;
+        v[3] = ODD && !g.act ? 0.0f : g.wgt * r.g2;
         v[4] = g.o0; v[5] = g.o1; v[6] = g.r0; v[7] = g.r1; v[8] = g.r2;
 #pragma unroll
         for (int k = 9; k < 16; ++k) v[k] = 0.0f;
@@ -1214,8 +1223,19 @@ __device__ __forceinline__ float warp_sum(const RayGrad &g, const BwdRay &r, con
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const float2 f = make_float2(row[k], row[k]), l = make_float2(last[k], last[k]);
-        const float2 a = fma2(f, k < 3 ? q.d01 : q.g01, mul2(l, q.b01));
-        const float2 b = fma2(f, k < 3 ? q.d23 : q.g23, mul2(l, q.b23));
+        float2 a, b;
+        if (!ODD) {
+            a = fma2(f, k < 3 ? q.d01 : q.g01, mul2(l, q.b01));
+            b = fma2(f, k < 3 ? q.d23 : q.g23, mul2(l, q.b23));
+        } else {
+            a = mul2(f, k < 3 ? q.d01 : q.g01);
+            b = mul2(f, k < 3 ? q.d23 : q.g23);
+            if (k == 3 && !g.act) a = b = make_float2(0.0f, 0.0f);
+            a.x = q.b01.x != 0.0f ? l.x : a.x;
+            a.y = q.b01.y != 0.0f ? l.x : a.y;
+            b.x = q.b23.x != 0.0f ? l.x : b.x;
+            b.y = q.b23.y != 0.0f ? l.x : b.y;
+        }
         const float2 v = xchg2(a, b, 16);
         const float s = v.x + __shfl_xor_sync(0xffffffffu, v.y, 8);
         if (k & 1) x[k >> 1].y = s;
@@ -1241,6 +1261,8 @@ __device__ __forceinline__ void backward_walk(WalkSmem &sm, const TileList &tl, 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const float log2_amin = log2f(p.alpha_min);
     const LanePerm perm = lane_perm<SPLAT>(ray);
+    const auto odd_value = [](float x) { return !(fabsf(x) < 1e15f); };
+    const bool odd = __any_sync(0xffffffffu, odd_value(ray.g0) || odd_value(ray.g1) || odd_value(ray.g2) || odd_value(ray.gS));
     // entry r of a batch has list index top - 1 - r
     uint32_t pos = walk.x, top = walk.y;
     int s_cnt = 0;
@@ -1318,16 +1340,20 @@ __device__ __forceinline__ void backward_walk(WalkSmem &sm, const TileList &tl, 
             }
         }
         __syncwarp();
-        for (int k = 0; k < n; ++k) {
-            const int r = (int)list[k];
-            const float4 a = sm.rec[r * 4 + 0];
-            const float4 b = sm.rec[r * 4 + 1];
-            const float4 c = sm.rec[r * 4 + 2];
-            const float4 e = sm.rec[r * 4 + 3];
-            const RayGrad g = ray_gradient<SPLAT>(ray, a, b, c, e, log2_amin, p.alpha_max, r >= reach);
-            const float v = warp_sum<SPLAT>(g, ray, perm);
-            if (!(lane & 1)) atomicAdd(&sm.acc[r][perm.off], v);
-        }
+        const auto walk_list = [&](auto odd_sums) {
+            for (int k = 0; k < n; ++k) {
+                const int r = (int)list[k];
+                const float4 a = sm.rec[r * 4 + 0];
+                const float4 b = sm.rec[r * 4 + 1];
+                const float4 c = sm.rec[r * 4 + 2];
+                const float4 e = sm.rec[r * 4 + 3];
+                const RayGrad g = ray_gradient<SPLAT>(ray, a, b, c, e, log2_amin, p.alpha_max, r >= reach);
+                const float v = warp_sum<SPLAT, decltype(odd_sums)::value>(g, ray, perm);
+                if (!(lane & 1)) atomicAdd(&sm.acc[r][perm.off], v);
+            }
+        };
+        if (odd) walk_list(std::true_type{});
+        else walk_list(std::false_type{});
         __syncthreads();
         // flush: one Gaussian of the batch per thread, four float4 atomics
         if (tid >= skip && tid < cnt && (sm.hit[tid].x | sm.hit[tid].y)) {

@@ -1798,7 +1798,8 @@ cudaError_t launch_duplicate(const geer_workspace *ws, cudaStream_t s) {
         auto *kern = mask_words(ws->super_size) == 1 ? k_duplicate<uint32_t> : k_duplicate<uint64_t>;
         // the counters come beside ~10 KB of lists: from ~9780 super-tiles on more than the 48 KB of a plain launch
         if (smem > 32 * 1024) {
-            const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       (int)sizeof(uint32_t) * kSmemTiles);  // (the same for every caller)
             if (e != cudaSuccess) return e;
         }
         const int64_t blocks = std::min<int64_t>(m, (int64_t)ws->num_sms * 4);

@@ -56,7 +56,9 @@ enum { GEER_PINHOLE = 0, GEER_EQUIDISTANT = 1, GEER_KANNALA_BRANDT = 2 };
  * in the 3DGS convention. Device SoA, FP32, contiguous:
  *   mean [n][3], scale [n][3], quat [n][4], opacity [n], sh [n][(deg+1)^2][3].
  * `sh` must be 16-byte aligned. Gaussians with non-finite values, a
- * non-positive scale or a zero quaternion are culled. */
+ * non-positive scale or a zero quaternion are culled. The render squares
+ * 1 / scale and the distance to the camera in FP32: scales from 2^-60 to 2^60
+ * and distances below 2^64. */
 typedef struct {
     const float *mean, *scale, *quat, *opacity, *sh;
     int64_t n;
@@ -112,7 +114,8 @@ enum { GEER_ASSOC_PBF = 0, GEER_ASSOC_EWA = 1, GEER_ASSOC_UT = 2 };
 enum { GEER_ALPHA_EXACT = 0, GEER_ALPHA_SPLAT = 1 };
 
 /* Rendering parameters. tile_w = tile_h = 16 (BEAP tiles of 16 x 16 rays,
- * each tile a camera sub-frustum, Sec. 3.2). alpha_min: contributions below it
+ * each tile a camera sub-frustum, Sec. 3.2). alpha_min (a normal number: with a
+ * subnormal one nothing is rendered): contributions below it
  * are skipped; alpha_max: alpha clamp; T_min: a ray stops before the
  * contributor that would take its transmittance below it (3DGS conventions
  * 1/255, 0.99, 1e-4). lambda_pad: relative padding of the per-Gaussian PBF

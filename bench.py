@@ -595,6 +595,9 @@ def run(args):
     n_items = scene.n * len(cams)  # (camera, Gaussian) items
     live = ws.live_items()
     sort_passes = ws.sort_passes()
+    # a pair's tile mask: one word for super-tiles of up to 5 x 5 tiles (the smallest from 4 x 4 on with at most 256 in all)
+    supers = lambda s: sum(math.ceil(c.width / (16 * s)) * math.ceil(c.height / (16 * s)) for c in cams)  # noqa: E731
+    mask_bytes = 4 if next((s for s in range(4, 9) if supers(s) <= 256), 4) <= 5 else 8
     sh_bytes = 4 * 3 * (scene.sh_degree + 1) ** 2
     g_bytes = 4 * (3 + 3 + 4 + 1) + sh_bytes
     work = {
@@ -602,10 +605,11 @@ def run(args):
         # backward accumulators zeroed (64 B)
         "preprocess": ("hbm", scene.n * g_bytes + n_items * (64 + 16 + 4 + 4 + (64 if have_bwd else 0))),
         "depth_sort": ("hbm", 4 * 20 * live),
-        # per live item: id, tile count and ranges read; 8 B per (super-tile, item) pair written
-        "duplicate": ("hbm", live * (4 + 4 + 16) + int(super_pairs) * 8),
-        # passes x (read key 4 B + key/value 8 B, write 8 B), and 16 B of ranges gathered + written
-        "tile_sort": ("hbm", sort_passes * 20 * int(super_pairs) + 32 * int(super_pairs)),
+        # per live item: id, super-tile count and rectangle read; key, value and tile mask per
+        # (super-tile, item) pair written
+        "duplicate": ("hbm", live * 16 + int(super_pairs) * (8 + mask_bytes)),
+        # passes x (key read, then key, value and mask read and written), and the masks once more
+        "tile_sort": ("hbm", int(super_pairs) * (sort_passes * (4 + 2 * (8 + mask_bytes)) + mask_bytes)),
         "render_fwd": ("alu", FLOPS_FWD_EVAL * evals),
         "render_bwd": ("alu", FLOPS_BWD_EVAL * walked),
         # the fused render: the forward's evaluations and the backward's walked entries
@@ -725,10 +729,12 @@ def run(args):
                                else f"copy bandwidth, {peak_src}",
                 "work": {"evaluations": evals, "applied": applied, "walked_back": walked}}
     tiles = math.ceil(cam.width / 16) * math.ceil(cam.height / 16)
-    # preprocess, live scan, compact, 4 depth passes x 2, gather, pair scan, emit, offsets,
-    # super-tile sort passes x 2, render forward (+ L1 gradient, backward order, render backward,
-    # preprocess backward): 22 per training step with one super-tile pass, as the ncu launch list shows
-    launches_per_step = 16 + 2 * sort_passes + ((1 if fused else 4) if have_bwd else 0)
+    # preprocess, live scan, compact, 4 depth passes x 2, gather, pair scan (up to 32768 items one
+    # launch for all from the scan on), emit, offsets, super-tile sort passes x 2, masks and order;
+    # render forward, or the fused render and preprocess backward, or forward, L1 gradient, backward
+    # order, render backward and preprocess backward: 20 per fused training step with one
+    # super-tile pass, as the ncu launch list shows
+    launches_per_step = (5 if n_items <= 32768 else 16) + 2 * sort_passes + ((2 if fused else 5) if have_bwd else 1)
 
     line = {
         "metric": METRIC, "value": value, "unit": "Mpix/s", "n_gpus": world, "steps": args.steps,

@@ -92,14 +92,15 @@ constexpr int kPBThreads = 64;
 // Resident blocks of the one-camera variant. Degree 3 holds its chain in 96 registers
 // with 12 B of spills (1M Gaussians: 104 us with 14 blocks, 72 registers and 140 B of
 // spills, 103 with 12, 90 with 10, 104 with 8); the lower degrees spill little and take
-// the warps (300K of degree 2: 35 us with 14, 38 with 10).
+// the warps (1M Gaussians with 14 / 12 / 10: degree 0 48 / 52 / 53 us, degree 1
+// 53 / 57 / 57, degree 2 72 / 80 / 85).
 #ifndef GEER_PB_MINB
 #define GEER_PB_MINB (DEG == 3 ? 10 : 14)
 #endif
 #ifndef GEER_PB_MINB_CAMS
-// Of the variant for several cameras: 204 registers (the next camera's loads overlap the
-// chain). Measured, 6M Gaussians and four cameras: 1.21 ms, with 7 1.69, with 10 2.02
-// (going through every camera: 1.35 at the best).
+// Of the variant for several cameras: at degree 3 168 registers and 36 B of spills (the next
+// camera's loads overlap the chain). Measured, 6M Gaussians and four cameras: 1.21 ms, with
+// 4 1.55, with 6 1.20, with 7 1.69, with 10 2.02 (going through every camera: 1.35 at the best).
 #define GEER_PB_MINB_CAMS 5
 #endif
 

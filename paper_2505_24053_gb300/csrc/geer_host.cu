@@ -92,8 +92,11 @@ bool flag_intervals(const float4 *tab, int n, int32_t z[2], int32_t w[2]) {
 // smallest S in 4..8 that keeps every super-tile id below 256 (one radix pass),
 // else 4. Slot layouts take S = kSlotSuper and ids from the slot's tile count, so that
 // every launch shape depends on the slot count only. (A batch of the serving
-// mix, 2M Gaussians: 3128 us with S = 4, 2991 with 5, 2986 with 6, 2933 with 8; with an
-// id per tile of the slots the emission's counters did not fit shared memory: 5133.)
+// mix, three slots of 1920 x 1280, 2M Gaussians: 3128 us with S = 4, 2991 with 5, 2986 with
+// 6, 2933 with 8; with an id per tile of the slots the emission's counters did not fit
+// shared memory: 5133. Slots of fewer tiles would take S = 4, with its one mask word: with
+// 8 / 4 16 slots of 320 x 240 788 / 703 us at 100K Gaussians and 4100 / 3630 at 1M, four of
+// 640 x 480 815 / 743 at 500K, eight of 160 x 120 244 / 235 at 20K.)
 constexpr int kSlotSuper = 8;
 
 void assign_super(DevCam *cams, int n, int64_t slot_tiles, int32_t &S, int64_t &n_stiles) {

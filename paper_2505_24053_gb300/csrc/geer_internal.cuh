@@ -145,9 +145,6 @@ struct Params {
     int32_t alpha_model;  // GEER_ALPHA_*
 };
 
-// PBF association ranges of a (camera, Gaussian) item, packed as u16 pairs:
-// [0,1) columns and [4,5) rows of the direct arcs, [2,3) and [6,7) of the arcs
-// shifted by pi (rays beyond 90 degrees).
 #ifndef GEER_PDL
 #define GEER_PDL 1  // programmatic dependent launch of the library's kernels
 #endif
@@ -284,6 +281,9 @@ __device__ __forceinline__ void sh_each(const float *row, F f) {
     }
 }
 
+// Association ranges of a (camera, Gaussian) item, packed as u16 pairs [lo, hi): columns
+// (rg[0], rg[1]) and rows (rg[4], rg[5]) of the direct arcs, (rg[2], rg[3]) and (rg[6],
+// rg[7]) of the arcs shifted by pi (rays beyond 90 degrees).
 __device__ __forceinline__ void unpack_ranges(const uint4 r4, int rg[8]) {
     rg[0] = (int)(r4.x & 0xffff); rg[1] = (int)(r4.x >> 16); rg[2] = (int)(r4.y & 0xffff); rg[3] = (int)(r4.y >> 16);
     rg[4] = (int)(r4.z & 0xffff); rg[5] = (int)(r4.z >> 16); rg[6] = (int)(r4.w & 0xffff); rg[7] = (int)(r4.w >> 16);

@@ -1735,7 +1735,8 @@ bool small_front(const geer_workspace *ws) { return (int64_t)ws->n_cams * ws->n_
 
 static cudaError_t launch_small_front(const geer_workspace *ws, cudaStream_t s) {
     const int items = (int)(ws->n_cams * ws->n_gauss);
-    static_assert(kSmallItems <= 8 * kSmallThreads && kClusterItems <= 4 * kCluster * kSmallThreads && kClusterItems <= 65536,
+    static_assert(kSmallThreads <= kSmallItems && kSmallItems <= 4 * kSmallThreads &&
+                      kClusterItems <= 4 * kCluster * kSmallThreads && kClusterItems <= 65536,
                   "items a thread, 16-bit ids");
     const auto launch = [&](auto *kern, int k, int blocks) {
         const int smem = 2 * (int)sizeof(uint32_t) * kSmallThreads / 32 * kRadix + 6 * k * kSmallThreads;
@@ -1748,7 +1749,7 @@ static cudaError_t launch_small_front(const geer_workspace *ws, cudaStream_t s) 
         return cudaGetLastError();
     };
     if (items <= kSmallThreads) return launch(k_small_front<1, 1>, 1, 1);
-    if (items <= 4 * kSmallThreads) return launch(k_small_front<4, 1>, 4, 1);
+    if (items <= kSmallItems) return launch(k_small_front<4, 1>, 4, 1);
     if (items <= kCluster * kSmallThreads) return launch(k_small_front<1, kCluster>, 1, kCluster);
     if (items <= 2 * kCluster * kSmallThreads) return launch(k_small_front<2, kCluster>, 2, kCluster);
     return launch(k_small_front<4, kCluster>, 4, kCluster);

@@ -275,9 +275,6 @@ __device__ __forceinline__ void fill_list(const TileList &tl, uint32_t &pos, boo
     __syncthreads();
 }
 
-// The same filter walking the super-tile list backwards: appends the passing
-// entries of [beg, pos) in descending position order (the tile list read back to
-// front) until s_id holds at least kBatch entries or pos reaches beg.
 // Moves the s_cnt - cnt entries not yet consumed (fewer than 256) to the front.
 __device__ __forceinline__ void shift_list(uint32_t *s_id, uint32_t *s_pos, int cnt, int &s_cnt) {
     const int rem = s_cnt - cnt;

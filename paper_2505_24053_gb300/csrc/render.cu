@@ -341,6 +341,7 @@ struct WalkSmem {
         struct {                        // backward
             float acc[kBatch][17];              // the batch's sums over the tile's rays
             uint8_t blist[kTileWarps][kBatch];  // each warp's entries of the batch
+            uint32_t odd;                       // a staged colour takes warp_sum's ODD sums from here on
         };
     };
     FillSmem fill;
@@ -1163,8 +1164,9 @@ __device__ __forceinline__ RayGrad ray_gradient(BwdRay &r, const float4 &a, cons
 // A product with zero does not mask an infinity or NaN, which would reach the sums of
 // another column and those of entries that the ray does not hit. ODD selects instead:
 // for the warps where a ray's dL/dC or colour behind is not finite, or large enough for
-// a product to overflow. (Selecting always: 1029 us for the 1M-Gaussian training step,
-// where both sets of sums beside each other take 845, as one did.)
+// a product to overflow, and from a batch with a Gaussian of such a colour on.
+// (Selecting always: 1029 us for the 1M-Gaussian training step, where both sets of sums
+// beside each other take 844, as one did.)
 struct LanePerm {
     float2 d01, d23, b01, b23, g01, g23;
     int off;
@@ -1261,7 +1263,6 @@ __device__ __forceinline__ void backward_walk(WalkSmem &sm, const TileList &tl, 
     const float log2_amin = log2f(p.alpha_min);
     const LanePerm perm = lane_perm<SPLAT>(ray);
     const auto odd_value = [](float x) { return !(fabsf(x) < 1e15f); };
-    const bool odd = __any_sync(0xffffffffu, odd_value(ray.g0) || odd_value(ray.g1) || odd_value(ray.g2) || odd_value(ray.gS));
     // entry r of a batch has list index top - 1 - r
     uint32_t pos = walk.x, top = walk.y;
     int s_cnt = 0;
@@ -1294,7 +1295,11 @@ __device__ __forceinline__ void backward_walk(WalkSmem &sm, const TileList &tl, 
             if (h.x | h.y) {
                 const float4 *src = reinterpret_cast<const float4 *>(rec + id);
 #pragma unroll
-                for (int k = 0; k < 4; ++k) sm.rec[tid * 4 + k] = src[k];
+                for (int k = 0; k < 4; ++k) {
+                    const float4 v = src[k];
+                    sm.rec[tid * 4 + k] = v;
+                    if (!SPLAT && k == 3 && odd_value(v.y + v.z + v.w)) sm.odd = 1u;
+                }
             }
             sm.hit[tid] = h;
         }
@@ -1351,7 +1356,8 @@ __device__ __forceinline__ void backward_walk(WalkSmem &sm, const TileList &tl, 
                 if (!(lane & 1)) atomicAdd(&sm.acc[r][perm.off], v);
             }
         };
-        if (odd) walk_list(std::true_type{});
+        const bool odd = odd_value(ray.g0) || odd_value(ray.g1) || odd_value(ray.g2) || odd_value(ray.gS);
+        if (__any_sync(0xffffffffu, odd) || sm.odd) walk_list(std::true_type{});
         else walk_list(std::false_type{});
         __syncthreads();
         // flush: one Gaussian of the batch per thread, four float4 atomics
@@ -1429,7 +1435,10 @@ __device__ __forceinline__ void bwd_unit(WalkSmem &sm, uint32_t code,
     const uint32_t t_id = code >> 4, k = code & 15u;
     if (!in_bounds(t_id, (uint64_t)ntiles, kSiteBwdTile, misc)) return;  // block-uniform
     const int t = (int)t_id;
-    if (threadIdx.x == 0) sm.cam = find_cam(cams, ncams, t);
+    if (threadIdx.x == 0) {
+        sm.cam = find_cam(cams, ncams, t);
+        sm.odd = 0u;
+    }
     __syncthreads();
     const DevCam &cam = cams[sm.cam];
     TileRay tr;

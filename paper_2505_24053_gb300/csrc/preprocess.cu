@@ -820,7 +820,7 @@ __device__ __forceinline__ SuperBox super_box(uint32_t xr, uint32_t yr, uint32_t
 // The super-tiles of an item of several rectangles, by one thread: the union of the
 // rectangles' super-tile boxes, each super-tile once, while the boxes hold at most
 // kThreadCells super-tiles; else nothing is done and false returned.
-constexpr uint32_t kThreadCells = 16;
+constexpr uint32_t kThreadCells = 6;
 template <typename F>
 __device__ __forceinline__ bool thread_supers(const DevCam &cam, uint32_t inv_s, const uint4 r4, F f) {
     int rg[8];
@@ -846,45 +846,69 @@ __device__ __forceinline__ bool thread_supers(const DevCam &cam, uint32_t inv_s,
     return true;
 }
 
-// The super-tiles of an item of several rectangles, by its warp: the union of the
-// rectangles' super-tile boxes, each super-tile once. f(sx, sy, keep) for 32
-// super-tiles at a time, keep false for those of an earlier rectangle and past the
-// end. rg: the item's ranges in every lane; box: the warp's nine {sx0, sx1, sy0, sy1}
-// (ends included) in shared memory.
-template <typename F>
-__device__ __forceinline__ void warp_supers(const DevCam &cam, uint32_t inv_s, const int rg[8], int4 *box, F f) {
+// Bits [lo, hi) of the S tile columns (or rows) that start at base.
+__device__ __forceinline__ uint32_t span_bits(int lo, int hi, int base, int S) {
+    const int l = min(max(lo - base, 0), S), h = min(max(hi - base, 0), S);
+    return h > l ? (1u << h) - (1u << l) : 0u;
+}
+
+// An item's association within super-tiles as four sets of tile columns times sets of
+// tile rows. A tile (x, y) is associated when (x in X0 and row y has rays with cos(phi)
+// >= 0, or x in X1 and row y has rays with cos(phi) <= 0), and likewise for its row in
+// Y0 / Y1 with the column's flags; multiplied out, byte k of super_cols (the columns of
+// super-tile column sx) goes with byte k of super_rows (the rows of super-tile row sy).
+__device__ __forceinline__ uint32_t super_cols(const DevCam &cam, const int rg[8], int sx, int S) {
+    const int x0 = sx * S;
+    const uint32_t X0 = span_bits(rg[0], rg[1], x0, S), X1 = span_bits(rg[2], rg[3], x0, S);
+    const uint32_t z = span_bits(cam.zc[0], cam.zc[1], x0, S);
+    const uint32_t w = span_bits(0, cam.wc[0], x0, S) | span_bits(cam.wc[1], cam.tiles_x, x0, S);
+    return (X0 & z) | (X0 & w) << 8 | (X1 & z) << 16 | (X1 & w) << 24;
+}
+__device__ __forceinline__ uint32_t super_rows(const DevCam &cam, const int rg[8], int sy, int S) {
+    const int y0 = sy * S;
+    const uint32_t Y0 = span_bits(rg[4], rg[5], y0, S), Y1 = span_bits(rg[6], rg[7], y0, S);
+    const uint32_t z = span_bits(cam.zr[0], cam.zr[1], y0, S);
+    const uint32_t w = span_bits(0, cam.wr[0], y0, S) | span_bits(cam.wr[1], cam.tiles_y, y0, S);
+    return (Y0 & z) | (Y1 & z) << 8 | (Y0 & w) << 16 | (Y1 & w) << 24;
+}
+
+// The super-tile columns (or rows) that hold the tiles [a0, a1) and [b0, b1).
+__device__ __forceinline__ int2 super_span(int a0, int a1, int b0, int b1, uint32_t inv_s) {
+    const bool a = a0 < a1, b = b0 < b1;
+    if (!a && !b) return make_int2(0, 0);
+    return make_int2(super_of(min(a ? a0 : b0, b ? b0 : a0), inv_s), super_of(max(a ? a1 : b1, b ? b1 : a1) - 1, inv_s) + 1);
+}
+
+// The number of super-tiles of an item (rg the same in every lane), by its warp: a lane
+// per super-tile column, whose sets that are not empty become bits of four words, then a
+// lane per row.
+__device__ __forceinline__ uint32_t warp_super_count(const DevCam &cam, const int rg[8], int S, uint32_t inv_s) {
     const int lane = threadIdx.x & 31;
-    int n = 0;
-    __syncwarp();
-    assoc_rects(cam, rg, [&](int4 r) {
-        if (lane == 0)
-            box[n] = make_int4(super_of(r.x, inv_s), super_of(r.y - 1, inv_s), super_of(r.z, inv_s),
-                               super_of(r.w - 1, inv_s));
-        ++n;
-    });
-    __syncwarp();
-    for (int k = 0; k < n; ++k) {
-        const int4 b = box[k];
-        const int w = b.y - b.x + 1, cells = w * (b.w - b.z + 1);
-        for (int c0 = 0; c0 < cells; c0 += 32) {
-            const int c = c0 + lane, cy = c / w, sx = b.x + c - cy * w, sy = b.z + cy;
-            bool keep = c < cells;
-            for (int q = 0; q < k; ++q) {
-                const int4 e = box[q];
-                keep = keep && !(sx >= e.x && sx <= e.y && sy >= e.z && sy <= e.w);
-            }
-            f(sx, sy, keep);
+    const int2 xs = super_span(rg[0], rg[1], rg[2], rg[3], inv_s), ys = super_span(rg[4], rg[5], rg[6], rg[7], inv_s);
+    uint32_t n = 0;
+    for (int x0 = xs.x; x0 < xs.y; x0 += 32) {
+        const uint32_t c = super_cols(cam, rg, x0 + lane, S);  // (columns past the image are empty)
+        uint32_t on[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) on[k] = __ballot_sync(0xffffffffu, c >> (8 * k) & 0xffu);
+        for (int y0 = ys.x; y0 < ys.y; y0 += 32) {
+            const uint32_t r = super_rows(cam, rg, y0 + lane, S);
+            uint32_t any = 0;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) any |= r >> (8 * k) & 0xffu ? on[k] : 0u;
+            n += (uint32_t)__popc(any);
         }
     }
+    return __reduce_add_sync(0xffffffffu, n);
 }
 
 // One item a lane (live: whether it has one): its rectangle and number of super-tiles,
-// and its tiles; box: the warp's nine boxes in shared memory (warp_supers).
+// and its tiles.
 struct ItemPairs {
     uint32_t xr, yr, supers, tiles;  // xr 0: several rectangles
 };
-__device__ __forceinline__ ItemPairs warp_item_pairs(const DevCam *__restrict__ cams, uint32_t inv_s, bool live, int ci,
-                                                     const uint4 r4, int4 *box) {
+__device__ __forceinline__ ItemPairs warp_item_pairs(const DevCam *__restrict__ cams, int S, uint32_t inv_s, bool live,
+                                                     int ci, const uint4 r4) {
     const int lane = threadIdx.x & 31;
     Assoc a{0u, 0u, 0u};
     ItemPairs p{0u, 0u, 0u, 0u};
@@ -895,10 +919,12 @@ __device__ __forceinline__ ItemPairs warp_item_pairs(const DevCam *__restrict__ 
         p.supers = super_box(a.xr, a.yr, inv_s).supers;
         p.tiles = ((a.xr >> 16) - (a.xr & 0xffff)) * ((a.yr >> 16) - (a.yr & 0xffff));
     }
-    // items of several rectangles: small ones by their threads, the others by the warp
-    // one at a time (a thread's long loop held its block up, the warp's loop costs ~200
-    // instructions an item: 412K Gaussians on two 109 x 86 cameras of 182 degrees 78 us
-    // with the warp's loop for all, 14 so)
+    // items of several rectangles: those of few super-tiles by their threads, the others by
+    // the warp one at a time, with a lane per super-tile column and row. (Preprocess and
+    // binning of 1M Gaussians of a room around a 190 degree camera, 15% of them of several
+    // rectangles, with threads up to 0 / 6 / 16 / 64 super-tiles: 277 / 270 / 273 / 313 us;
+    // 358 with a lane per super-tile of every rectangle's box, each tested against the
+    // boxes before. 1M on a shell at 205 degrees: 312 / 214 / 214 / 217, 219 with boxes.)
     bool by_warp = false;
     if (a.rects > 1) {
         const DevCam &cam = cams[ci];
@@ -913,11 +939,7 @@ __device__ __forceinline__ ItemPairs warp_item_pairs(const DevCam *__restrict__ 
                                    __shfl_sync(0xffffffffu, r4.z, o), __shfl_sync(0xffffffffu, r4.w, o));
         int rg[8];
         unpack_ranges(q, rg);
-        uint32_t k = 0;
-        const DevCam &cam = cams[__shfl_sync(0xffffffffu, ci, o)];
-        warp_supers(cam, inv_s, rg, box, [&](int, int, bool keep) {
-            k += (uint32_t)__popc(__ballot_sync(0xffffffffu, keep));
-        });
+        const uint32_t k = warp_super_count(cams[__shfl_sync(0xffffffffu, ci, o)], rg, S, inv_s);
         if (lane == o) p.supers = k;
     }
     return p;
@@ -937,14 +959,13 @@ __global__ void __launch_bounds__(kPrepThreads) k_gather_counts(
     uint32_t *__restrict__ bs_tile, uint32_t *__restrict__ oxr, uint32_t *__restrict__ oyr) {
     grid_dep_sync();
     __shared__ uint32_t s_sum[kGather][2];
-    __shared__ int4 s_box[kPrepThreads / 32][9];
     const uint32_t L = misc[kMiscLive];
     const int64_t i0 = (int64_t)blockIdx.x * (kGather * kPrepThreads);
     if (i0 >= L) return;
     const bool cur = depth_sorted_buf(misc) != 0;
     const uint32_t *__restrict__ sorted_id = cur ? id1 : id0;
     uint32_t *__restrict__ osupers = cur ? id0 : id1;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
     const uint32_t inv_s = super_inverse(S);
     if (threadIdx.x < 2 * kGather) (&s_sum[0][0])[threadIdx.x] = 0u;
     uint32_t item[kGather];
@@ -963,7 +984,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_gather_counts(
 #pragma unroll
     for (int u = 0; u < kGather; ++u) {
         const int64_t i = i0 + u * kPrepThreads + threadIdx.x;
-        const ItemPairs p = warp_item_pairs(cams, inv_s, i < L, (int)(item[u] / (uint32_t)n), r4[u], s_box[warp]);
+        const ItemPairs p = warp_item_pairs(cams, S, inv_s, i < L, (int)(item[u] / (uint32_t)n), r4[u]);
         if (i < L) {
             oxr[i] = p.xr;
             oyr[i] = p.yr;
@@ -1011,7 +1032,6 @@ __global__ void __launch_bounds__(kSmallThreads) k_small_front(
     uint16_t *s_val = reinterpret_cast<uint16_t *>(s_key + K * kSmallThreads);
     __shared__ uint32_t s_part[kSmallThreads / kRadix][kRadix];
     __shared__ uint32_t s_wsum[W];
-    __shared__ int4 s_box[W][9];
     __shared__ uint32_t s_sum[CHUNKS][2];
     // what the other blocks of the cluster read: live items, digit totals (two passes' in turn), pairs and tiles
     __shared__ uint32_t s_live, s_dig[C > 1 ? 2 : 1][kRadix], s_low[kSmallThreads / kRadix][C > 1 ? kRadix : 1];
@@ -1182,7 +1202,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_small_front(
         const bool on = e < own;
         const uint32_t item = on ? s_val[e] : 0u;
         const uint4 r4 = on ? ranges[item] : make_uint4(0u, 0u, 0u, 0u);
-        const ItemPairs p = warp_item_pairs(cams, inv_s, on, (int)(item / (uint32_t)n), r4, s_box[warp]);
+        const ItemPairs p = warp_item_pairs(cams, S, inv_s, on, (int)(item / (uint32_t)n), r4);
         if (on) {
             id0[i] = item;
             oxr[i] = p.xr;
@@ -1231,42 +1251,24 @@ __global__ void __launch_bounds__(kSmallThreads) k_small_front(
     }
 }
 
-// Bits [lo, hi) of the S tile columns (or rows) that start at base.
-__device__ __forceinline__ uint32_t span_bits(int lo, int hi, int base, int S) {
-    const int l = min(max(lo - base, 0), S), h = min(max(hi - base, 0), S);
-    return h > l ? (1u << h) - (1u << l) : 0u;
-}
-
-// The tile mask of an item and super-tile (sx, sy): bit j * S + i for its tile
-// (sx S + i, sy S + j). A tile (x, y) is associated when (x in X0 and row y has rays
-// with cos(phi) >= 0, or x in X1 and row y has rays with cos(phi) <= 0), and likewise
-// for its row in Y0 / Y1 with the column's flags.
-__device__ __forceinline__ uint64_t tile_mask_general(const DevCam &cam, const int rg[8], int sx, int sy, int S) {
-    const int x0 = sx * S, y0 = sy * S;
-    const uint32_t X0 = span_bits(rg[0], rg[1], x0, S), Y0 = span_bits(rg[4], rg[5], y0, S);
-    const uint32_t X1 = span_bits(rg[2], rg[3], x0, S), Y1 = span_bits(rg[6], rg[7], y0, S);
-    const uint32_t zc = span_bits(cam.zc[0], cam.zc[1], x0, S), zr = span_bits(cam.zr[0], cam.zr[1], y0, S);
-    const uint32_t wc = span_bits(0, cam.wc[0], x0, S) | span_bits(cam.wc[1], cam.tiles_x, x0, S);
-    const uint32_t wr = span_bits(0, cam.wr[0], y0, S) | span_bits(cam.wr[1], cam.tiles_y, y0, S);
-    uint64_t m = 0;
-    for (int j = 0; j < S; ++j) {
-        const uint32_t a = (zr >> j & 1u ? X0 : 0u) | (wr >> j & 1u ? X1 : 0u);
-        const uint32_t b = (Y0 >> j & 1u ? zc : 0u) | (Y1 >> j & 1u ? wc : 0u);
-        m |= (uint64_t)(a & b) << (j * S);
-    }
+// The tile mask of an item and super-tile: bit j * S + i for its tile (sx S + i, sy S + j).
+// cols, rows: super_cols, super_rows; spread[r]: bit j * S for every bit j of r.
+template <typename M>
+__device__ __forceinline__ M tile_mask_sets(uint32_t cols, uint32_t rows, const M *spread) {
+    M m = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) m |= spread[rows >> (8 * k) & 0xffu] * (M)(cols >> (8 * k) & 0xffu);
     return m;
 }
 
 // The same for a rectangle that meets the super-tile: columns [xlo, xhi) x rows
-// [ylo, yhi) (packed lo | hi << 16), from the table of row runs: rows[9 l + h] has bit
-// j * S of the rows l <= j < h, each times the columns' run of ones. M: uint32_t where
-// the S * S bits fit it.
+// [ylo, yhi) (packed lo | hi << 16). M: uint32_t where the S * S bits fit it.
 template <typename M>
-__device__ __forceinline__ M tile_mask_rect(uint32_t xr, uint32_t yr, int sx, int sy, int S, const M *rows) {
+__device__ __forceinline__ M tile_mask_rect(uint32_t xr, uint32_t yr, int sx, int sy, int S, const M *spread) {
     const int x0 = sx * S, y0 = sy * S;
     const int xl = max((int)(xr & 0xffff) - x0, 0), xh = min((int)(xr >> 16) - x0, S);
     const int yl = max((int)(yr & 0xffff) - y0, 0), yh = min((int)(yr >> 16) - y0, S);
-    return rows[9 * yl + yh] * (M)((1u << xh) - (1u << xl));
+    return spread[(1u << yh) - (1u << yl)] * (M)((1u << xh) - (1u << xl));
 }
 
 __device__ __forceinline__ void put_mask(uint32_t *out, uint32_t i, uint32_t m) { out[i] = m; }
@@ -1299,19 +1301,18 @@ __global__ void __launch_bounds__(kPrepThreads) k_duplicate(
     // {first output (of the warp's), super-tiles a row | stiles_x << 16, first super-tile, its x | y << 16}
     __shared__ uint4 s_item[kPrepThreads][2];
     __shared__ uint32_t wsum[kPrepThreads / 32];
-    __shared__ int4 s_box[kPrepThreads / 32][9];
-    __shared__ M s_rows[81];  // tile_mask_rect's row runs
+    __shared__ uint2 s_sets[kPrepThreads / 32][32];          // a warp's super_cols and super_rows
+    __shared__ M s_spread[sizeof(M) == 4 ? 32 : kPrepThreads];  // (S <= 5, S <= 8)
     extern __shared__ uint32_t sh[];  // per-super-tile pair counts when they fit (nst <= kSmemTiles)
     const bool smem = nst <= kSmemTiles;
     const uint32_t L = misc[kMiscLive];
     if ((int64_t)blockIdx.x * kPrepThreads >= L) return;
     if (smem)
         for (int k = threadIdx.x; k < nst; k += kPrepThreads) sh[k] = 0u;
-    if (threadIdx.x < 81) {
-        const int l = threadIdx.x / 9, h = threadIdx.x - 9 * l;
+    if (threadIdx.x < 1u << S) {
         M m = 0;
-        for (int j = l; j < min(h, S); ++j) m |= (M)1 << (j * S);
-        s_rows[threadIdx.x] = m;
+        for (int j = 0; j < S; ++j) m |= (M)(threadIdx.x >> j & 1u) << (j * S);
+        s_spread[threadIdx.x] = m;
     }
     const auto count = [&](uint32_t st) {
         if (!in_bounds(st, (uint64_t)nst, kSiteDupSuper, misc)) return;
@@ -1375,7 +1376,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_duplicate(
                 const uint32_t kx = k - ky * rw, st = b.z + ky * (b.y >> 16) + kx, out = base + a.w + k;
                 okeys[out] = st;
                 ovals[out] = a.z;
-                put_mask(omask, out, tile_mask_rect<M>(a.x, a.y, (int)((b.w & 0xffff) + kx), (int)((b.w >> 16) + ky), S, s_rows));
+                put_mask(omask, out, tile_mask_rect<M>(a.x, a.y, (int)((b.w & 0xffff) + kx), (int)((b.w >> 16) + ky), S, s_spread));
                 count(st);
             }
         }
@@ -1389,7 +1390,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_duplicate(
                     const uint32_t st = (uint32_t)(cam.stile_base + sy * cam.stiles_x + sx);
                     okeys[out] = st;
                     ovals[out] = item;
-                    put_mask(omask, out, (M)tile_mask_general(cam, rg, sx, sy, S));
+                    put_mask(omask, out, tile_mask_sets(super_cols(cam, rg, sx, S), super_rows(cam, rg, sy, S), s_spread));
                     count(st);
                     ++out;
                 }
@@ -1402,18 +1403,38 @@ __global__ void __launch_bounds__(kPrepThreads) k_duplicate(
             const uint32_t out = base + __shfl_sync(0xffffffffu, pre, o);
             int rg[8];
             unpack_ranges(ranges[it], rg);
+            const int2 xs = super_span(rg[0], rg[1], rg[2], rg[3], inv_s), ys = super_span(rg[4], rg[5], rg[6], rg[7], inv_s);
+            uint2 *sets = s_sets[threadIdx.x >> 5];
             uint32_t done = 0;
-            warp_supers(c, inv_s, rg, s_box[threadIdx.x >> 5], [&](int sx, int sy, bool keep) {
-                const uint32_t kept = __ballot_sync(0xffffffffu, keep), k = done + (uint32_t)__popc(kept & ((1u << lane) - 1u));
-                if (keep && k < cn) {
-                    const uint32_t st = (uint32_t)(c.stile_base + sy * c.stiles_x + sx);
-                    okeys[out + k] = st;
-                    ovals[out + k] = it;
-                    put_mask(omask, out + k, (M)tile_mask_general(c, rg, sx, sy, S));
-                    count(st);
+            for (int x0 = xs.x; x0 < xs.y; x0 += 32)
+                for (int y0 = ys.x; y0 < ys.y; y0 += 32) {
+                    __syncwarp();
+                    sets[lane] = make_uint2(super_cols(c, rg, x0 + lane, S), super_rows(c, rg, y0 + lane, S));
+                    __syncwarp();
+                    // a lane per super-tile, row by row; 32 further is `down` rows and `right` columns
+                    const int w = min(32, xs.y - x0), h = min(32, ys.y - y0), down = 32 / w, right = 32 - down * w;
+                    int cy = lane / w, cx = lane - cy * w;
+                    for (int k = w * h; k > 0; k -= 32) {
+                        M m = 0;
+                        if (lane < k) m = tile_mask_sets(sets[cx].x, sets[cy].y, s_spread);
+                        const uint32_t kept = __ballot_sync(0xffffffffu, m != 0);
+                        const uint32_t q = done + (uint32_t)__popc(kept & ((1u << lane) - 1u));
+                        if (m != 0 && q < cn) {
+                            const uint32_t st = (uint32_t)(c.stile_base + (y0 + cy) * c.stiles_x + x0 + cx);
+                            okeys[out + q] = st;
+                            ovals[out + q] = it;
+                            put_mask(omask, out + q, m);
+                            count(st);
+                        }
+                        done += (uint32_t)__popc(kept);
+                        cx += right;
+                        cy += down;
+                        if (cx >= w) {
+                            cx -= w;
+                            ++cy;
+                        }
+                    }
                 }
-                done += (uint32_t)__popc(kept);
-            });
         }
     }
     __syncthreads();

@@ -95,6 +95,31 @@ def test_lists_of_several_rectangles(geer, orc, n, px, ncams):
     assert P == ek.size and np.array_equal(k, ek) and np.array_equal(v, ev)
 
 
+@pytest.mark.parametrize("w,h", [(132, 3), (3, 132), (140, 131), (64, 64), (71, 70), (120, 110)],
+                         ids=["33x1", "1x33", "35x33", "16x16", "15x14", "15x14wide"])
+@pytest.mark.parametrize("culled", [0, 33_000], ids=["small_front", "general"])
+def test_several_rectangles_over_many_super_tiles(geer, orc, w, h, culled):
+    """Items of several rectangles over more than 32 super-tile columns, rows or both (4 x 4 tiles
+    each), and over super-tiles of 5 x 5 and 8 x 8 tiles, the latter with masks of two words."""
+    n = 40
+    rng = np.random.default_rng(w + h)
+    v = rng.normal(0, 1, (n, 3))
+    v *= rng.uniform(0.3, 6, (n, 1)) / np.linalg.norm(v, axis=1, keepdims=True)
+    pad = lambda a: np.concatenate([a, np.repeat(a[:1], culled, 0)]).astype(np.float32)  # noqa: E731
+    scene = wl.Scene(pad(v), pad(np.exp(rng.normal(-1.5, 1.0, (n, 3)))), pad(rng.standard_normal((n, 4))),
+                     pad(rng.uniform(0.2, 0.9, n)), pad(rng.normal(0, 0.3, (n, 1, 3))), 0)
+    scene.scale[n:] = 0.0
+    cams = [wl.Camera(wl.EQUIDISTANT, 16 * w - 5, 16 * h - 7, math.radians(230), math.radians(215))]
+    r = geer.Renderer(cams, n + culled, 0, pair_capacity=1 << 21)
+    r.prepare(geer.Gaussians.from_scene(scene))
+    P, _ = r.ws.pair_counts()
+    k, val = r.ws.debug_pairs(cap=P)
+    first = wl.Scene(scene.mean[:n], scene.scale[:n], scene.quat[:n], scene.opacity[:n], scene.sh[:n], 0)
+    ek, ev = _expand_pairs(orc, first, cams)
+    assert P == ek.size > 0
+    assert np.array_equal(k, ek) and np.array_equal(val, ev)
+
+
 def test_more_block_counts_than_a_scan_step(geer):
     """4097 blocks of Gaussians: every live item in its tiles' lists, in depth order."""
     n = 4096 * 256 + 17
